@@ -106,7 +106,8 @@ typedef struct {
  * for indexes of 4,194,304 objects and more searched with 384- or 512-byte rows and beam_width <= 64, AUTO
  * keeps the set in a 16 KB hash table of ranks per resident warp instead (exact; small enough to stay
  * in L2, where the bitmap of a large index costs a DRAM read-modify-write per candidate); a query
- * that fills half the table moves to its bitmap slab.  The results do not depend on the form. */
+ * that fills half the table moves to its bitmap slab.  Small batches (frog_search) keep no set at all under
+ * AUTO, only a table of recently evaluated ranks in shared memory.  The results do not depend on the form. */
 #define FROG_VISITED_AUTO 0
 #define FROG_VISITED_BITMAP 1
 #define FROG_VISITED_HASH 2
@@ -145,7 +146,8 @@ int frog_index_info(const frog_index_t* index, frog_index_info_t* out);
 int frog_index_enable_f16(frog_index_t* index);
 
 /* frog_search: batched FROGSearch (Alg. 2, with Alg. 3 once per query and Alg. 4 plus the lazy
- * hash check of Sec. 7.3.2 at every expansion), one query per warp of a persistent kernel.
+ * hash check of Sec. 7.3.2 at every expansion), one query per warp of a persistent kernel; batches of a few
+ * queries per SM (the line depends on the row size) get a CTA per query instead, same results.
  *   queries    DEVICE, nq x d fp32 row-major (d = index dimensionality)
  *   lo, hi     DEVICE, nq int32, inclusive attribute bounds of each query
  *   k          results per query, 1 <= k <= beam_width

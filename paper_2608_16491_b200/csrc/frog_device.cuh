@@ -615,6 +615,68 @@ __device__ __forceinline__ uint32_t merge_batch(uint64_t* pool, uint64_t my_key,
     return first_pos(m1);
 }
 
+// The same merge for up to 32 keys that also lie in shared memory: lane j < n brings keys[j] (any order,
+// copies of pool keys or of each other allowed).  Every lane finds the place of its key with a binary
+// search over the pool and its rank among the new keys by reading them all (broadcast loads); the final
+// positions of the new keys, as one bit mask per 32 positions, tell each position whether it takes a new
+// key or which old one moves there.  The cost hardly depends on the pool size and little on n, and the
+// dependent chain has no shuffle or vote per key.
+template <int EPL>
+__device__ __forceinline__ uint32_t merge_ranked(uint64_t* pool, const uint64_t* keys, int n, int ef_s, int lane) {
+    constexpr int POOL = 32 * EPL;
+    const uint32_t lt_mask = (1u << lane) - 1u;
+    uint64_t key = lane < n ? keys[lane] : KEY_EMPTY;
+    const uint64_t mk = key | 1ull;
+    bool in = mk < (pool[ef_s - 1] | 1ull);             // a full pool rejects what is not better than its worst
+    int p = 0;                                          // pool keys below mk (at most ef_s - 1 if it enters)
+#pragma unroll
+    for (int step = POOL / 2; step > 0; step >>= 1)
+        if ((pool[p + step - 1] | 1ull) < mk) p += step;
+    in = in && (pool[p] | 1ull) != mk;                  // the pool holds it already
+    int r = 0;
+    bool copy = false;
+#pragma unroll 4
+    for (int j = 0; j < n; ++j) {
+        const uint64_t x = keys[j] | 1ull;
+        r += x < mk ? 1 : 0;
+        copy = copy || (x == mk && j < lane);
+    }
+    in = in && !copy;
+    // keys that lie below this one but do not enter: copies only (what the pool rejects lies above)
+    for (uint32_t out = __ballot_sync(FULL, !in && lane < n); out; out &= out - 1) {
+        const uint64_t x = keys[__ffs(out) - 1] | 1ull;
+        r -= x < mk ? 1 : 0;
+    }
+    const int f = p + r;
+    in = in && f < ef_s;
+    int below = 0, m1 = NO_POS;
+    uint64_t take[EPL];
+    int shift[EPL];
+#pragma unroll
+    for (int e = 0; e < EPL; ++e) {
+        const uint32_t F = __reduce_or_sync(FULL, in && (f >> 5) == e ? 1u << (f & 31) : 0u);
+        const bool mine = (F >> lane) & 1u;
+        shift[e] = mine ? -1 : below + __popc(F & lt_mask);
+        below += __popc(F);
+        take[e] = mine ? KEY_EMPTY : pool[lane + 32 * e - shift[e]];
+    }
+    __syncwarp();
+#pragma unroll
+    for (int e = 0; e < EPL; ++e) {
+        const int x = lane + 32 * e;
+        if (x < ef_s && take[e] != KEY_EMPTY) {
+            if (shift[e] > 0) pool[x] = take[e];
+            if (!(take[e] & 1ull)) m1 = min(m1, x);
+        }
+    }
+    if (in) {
+        pool[f] = key;
+        if (!(key & 1ull)) m1 = min(m1, f);
+    }
+    __syncwarp();
+    return first_pos(m1);
+}
+
 // smallest key of the warp under the order key | 1 (KEY_EMPTY if no lane has one)
 __device__ __forceinline__ uint64_t warp_min_key(uint64_t key) {
     const uint32_t hi = (uint32_t)(key >> 32), lo = (uint32_t)key | 1u;

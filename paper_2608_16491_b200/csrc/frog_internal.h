@@ -103,6 +103,8 @@ namespace froghost {
 // frog_search_lean.cu: the trimmed kernel for 384- and 512-byte fp32 rows (null: shape not covered)
 frog_kernel_fn lean_kernel(int ef_s, int budget, int row_bytes, bool table, bool hook, size_t* smem_per_warp,
                            int* warps_per_cta);
+// frog_search_team.cu: one CTA of `warps` warps per query (see there)
+frog_kernel_fn team_kernel(int warps, int ef_s, int q_len, int vis_bits, bool f16, size_t* smem);
 void set_cuda_error(cudaError_t e);
 int resolve_params(const frog_index* ix, int beam_width, const frog_params_t* in, frog_params_t* out);
 bool make_row_tensor_map(const void* base, bool f16, int row_elems, size_t row_bytes, size_t n, CUtensorMap* out);

@@ -602,6 +602,48 @@ int plan_launch(const frog_index* ix, int beam_width, const frog_params_t& P, in
     return FROG_OK;
 }
 
+// One CTA per query (frog_search_team.cu) for batches that leave warps idle, or FROG_ERR_UNSUPPORTED where
+// one warp per query is the better use of the GPU.  The line between them was measured on indexes of
+// 10,000-100,000 objects over batches of 1-4,000 queries (us per call, one warp per query / 8 warps / 4 warps):
+//   384-byte rows, beam 64, B 64     150 queries 286/210/275    300: 345/260/338    600: 343/379/351
+//   512-byte rows, beam 44, B 64     150: 229/168/229           300: 252/185/238    600: 296/262/286
+//   400-byte rows, beam 128, B 16    300: 657/414/507           600: 729/553/531    1,000: 772/871/627   1,500: 784/1229/805
+//   256-byte fp16 rows, beam 64      300: 414/257/316           600: 412/372/354    1,000: 511/575/423   1,500: 521/849/553
+//   3,072-byte rows, beam 192, B 128 300: 4212/1457/2515        600: 4219/1731/2620 1,500: 4841/3874/3025 4,000: 5246/10206/5907
+//   1,536-byte rows, beam 64, B 32   300: 688/231/355           600: 682/315/372    1,500: 778/653/486   4,000: 872/1604/1132
+// so: 8 warps while every query has a CTA of its own at once (2 per SM; 4 per SM for rows of several
+// chunks), then 4 warps up to 8 queries per SM (16 for long rows) except on the rows that the kernel of
+// frog_search_lean.cu covers, which one warp serves well enough.
+int plan_team(const frog_index* ix, int beam_width, const frog_params_t& P, int nq, LaunchPlan* out, int* vis_bits) {
+    const bool f16 = P.storage == FROG_STORAGE_F16;
+    const int q_len = query_len(ix->info.d);
+    const int row_bytes = f16 ? q_len * 2 : ix->info.d_pad * 4;
+    const bool lean = !f16 && ix->has_tmap_f32 && (row_bytes == 384 || row_bytes == 512);
+    const bool long_rows = row_bytes > STAGE_CHUNK;
+    const int per_sm_nq = (nq + ix->sm_count - 1) / ix->sm_count;
+    const int warps = per_sm_nq <= (long_rows ? 4 : 2) ? 8 : 4;
+    if (warps == 4 && (lean || per_sm_nq > (long_rows ? 16 : 8))) return FROG_ERR_UNSUPPORTED;
+    // a table of about 16 ranks per beam slot: smaller ones repeat distances (3,072-byte rows at beam 192:
+    // 1.3x slower with 2,048 ranks than with 4,096), larger ones cost resident CTAs
+    int bits = 10;
+    while (bits < (warps == 8 ? 13 : 12) && (1 << bits) < 16 * beam_width) ++bits;
+    size_t smem = 0;
+    kernel_fn fn = froghost::team_kernel(warps, beam_width, q_len, bits, f16, &smem);
+    if (smem > 227 * 1024) return FROG_ERR_UNSUPPORTED;
+    FROG_CUDA_TRY(cudaFuncSetAttribute((const void*)fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+    int per_sm = 0;
+    FROG_CUDA_TRY(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, (const void*)fn, warps * 32, smem));
+    if (per_sm < 1) return FROG_ERR_UNSUPPORTED;
+    out->fn = fn;
+    out->grid = per_sm * ix->sm_count < nq ? per_sm * ix->sm_count : nq;
+    out->block = warps * 32;
+    out->ctas_per_sm = per_sm;
+    out->smem = smem;
+    out->table = false;
+    *vis_bits = bits;
+    return FROG_OK;
+}
+
 // gather source and stage geometry: a row slot is the row, or its 512-byte chunk
 void set_gather(const frog_index* ix, bool f16, FrogSearchArgs* A) {
     const int d_pad_h = query_len(ix->info.d);
@@ -836,7 +878,13 @@ extern "C" int frog_search_ex(const frog_index_t* index, const float* queries, c
     const int mode = trace ? ((P.debug_flags & 1) ? MODE_PROFILE : MODE_TRACE) : stats ? MODE_COUNT : MODE_FAST;
     bool bitmap = P.visited != FROG_VISITED_HASH;
     LaunchPlan plan;
-    rc = plan_launch(index, beam_width, P, mode, bitmap, nq, &plan);
+    // one CTA per query where that pays; any explicit choice of the visited set, ablation or test hook keeps
+    // the kernels it names
+    int vis_bits = 0;
+    const bool team = mode == MODE_FAST && P.visited == FROG_VISITED_AUTO && !P.eager_hash && !(P.debug_flags & ~(2 | 16)) &&
+                      plan_team(index, beam_width, P, nq, &plan, &vis_bits) == FROG_OK;
+    if (team) bitmap = false;
+    else rc = plan_launch(index, beam_width, P, mode, bitmap, nq, &plan);
     if (rc) return rc;
     cudaStream_t s = static_cast<cudaStream_t>(stream);
     frog_index* mix = const_cast<frog_index*>(index);      // the scratch sets are the index's only mutable part
@@ -902,10 +950,12 @@ extern "C" int frog_search_ex(const frog_index_t* index, const float* queries, c
     A.order = nullptr;
     set_gather(index, P.storage == FROG_STORAGE_F16, &A);
     A.no_copies = (P.debug_flags & 32) ? 1 : 0;             // tests of the error path (see frog.h)
+    if (team) A.hash_bits = vis_bits;
 
-    FROG_CUDA_TRY(cudaMemsetAsync(sc->d_work, 0, 1024, s));
+    // (a team launch whose queries all start at once takes no numbers and needs no order)
+    if (!team || plan.grid < nq) FROG_CUDA_TRY(cudaMemsetAsync(sc->d_work, 0, 1024, s));
     // planning pass (skipped for tiny batches and when its scratch cannot be had)
-    const bool planned = !(P.debug_flags & 2) && nq >= 64 && froghost::ensure_plan(sc, (size_t)nq) == FROG_OK;
+    const bool planned = !(P.debug_flags & 2) && nq >= 64 && (!team || plan.grid < nq) && froghost::ensure_plan(sc, (size_t)nq) == FROG_OK;
     if (planned) {
         int2* ranges = reinterpret_cast<int2*>(sc->d_plan);
         int32_t* order = sc->d_plan + 2 * sc->plan_queries;
