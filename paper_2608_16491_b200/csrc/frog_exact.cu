@@ -1,9 +1,23 @@
 // frog_exact_search: exact filtered kNN (paper Def. 2) by scanning each query's contiguous rank
-// slab (Sec. 4).  One CTA per query; each warp streams batches of 16 consecutive rows through the
-// same distance routine the beam search uses, keeps its own sorted top-k in shared memory, and
-// warp 0 merges the per-warp lists at the end.  Ordering: (squared distance, original object id)
-// ascending, the total order of Def. 2's tie rule (objects with equal attributes are ranked by id, so
-// this differs from rank order only between equidistant objects with different attributes).
+// slab (Sec. 4).  Ordering: (squared distance, original object id) ascending, the total order of Def. 2's
+// tie rule (objects with equal attributes are ranked by id, so this differs from rank order only between
+// equidistant objects with different attributes).
+//
+// A CTA scans a piece of the rows for a GROUP of queries and keeps the k nearest of each:
+//   * a team of 8 lanes holds two rows in registers and computes their distances to every query of the group
+//     (queries in shared memory), so a row is fetched once per group;
+//   * a distance that beats the query's bound goes to the query's buffer; one warp per query merges the
+//     buffer into the query's pool when it fills (a few times per piece) and lowers the bound.  The bound is
+//     shared by all pieces of a query through global memory: whatever exceeds the k-th best of ANY piece
+//     cannot be an answer;
+//   * the last CTA to finish a group merges the pieces' lists.
+// Fewer than EXACT_GROUP_MIN queries are not grouped: every CTA finds the slabs itself and takes an equal
+// share of all rows (one launch).  Otherwise queries are ordered by (width, position), grouped by eight, and
+// the groups' rows are cut into pieces of equal size (two small kernels).  The form with one CTA per query
+// and no scratch remains for captured streams, for rows too long for eight queries in shared memory, and
+// for the case that scratch cannot be had.
+#include <algorithm>
+
 #include "frog_device.cuh"
 #include "frog_internal.h"
 
@@ -12,6 +26,11 @@ using namespace frogdev;
 namespace {
 
 constexpr int EXACT_WARPS = 8;
+constexpr int EXACT_GROUP = 8;           // queries per group = warps per CTA (one merges each query's buffer)
+constexpr int EXACT_GROUP_MIN = 16;      // batches of fewer queries are not grouped
+constexpr int EXACT_STEP = 8 * EXACT_WARPS;    // rows per step of a CTA: two per team
+constexpr int EXACT_BUF = 256;           // keys buffered per query; merged from 64 on, two steps add at most 128
+constexpr int EXACT_BINS = 33 * 32;      // (width class, position) bins that queries are ordered by
 
 struct ExactArgs {
     const int32_t* sorted_attr;
@@ -24,66 +43,504 @@ struct ExactArgs {
     int nq, k;
     int32_t* out_ids;
     float* out_dists;
+    // scratch (see ExactScratch); null for the form with one CTA per query
+    int2* ranges;
+    int32_t* order;
+    int4* jobs;                      // (group, first row, end row, -)
+    int2* groups;                    // (first piece, pieces)
+    unsigned int* counters;          // [0] pieces of this call, [1] next piece, [2..] bins; zero between calls
+    unsigned int* done;              // finished pieces per group (or query); zero between calls
+    unsigned long long* bound;       // per query: k-th best key of any piece; all ones between calls
+    uint64_t* part;                  // per piece and query of the group: k keys
+    int max_pieces, min_rows;
 };
 
+template <int EPL, int G>
+struct ExactSmem {
+    uint64_t* pool;      // G x 32 EPL
+    uint64_t* buf;       // G x EXACT_BUF
+    uint64_t* tau;       // G: keys above it are not wanted
+    int* cnt;            // G: keys in buf
+    int* l;              // G: first rank
+    int* r;              // G: last rank
+    int* id;             // G: query number, -1 = none
+    int* misc;           // 8
+    float4* q;           // G x d_pad floats
+    static constexpr size_t FIXED = (size_t)G * (32 * EPL + EXACT_BUF + 1) * 8 + (size_t)G * 16 + 32;
+    static size_t bytes(int d_pad) { return (FIXED + 15) / 16 * 16 + (size_t)G * d_pad * 4; }
+    __device__ __forceinline__ explicit ExactSmem(unsigned char* base) {
+        pool = reinterpret_cast<uint64_t*>(base);
+        buf = pool + G * 32 * EPL;
+        tau = buf + G * EXACT_BUF;
+        cnt = reinterpret_cast<int*>(tau + G);
+        l = cnt + G;
+        r = l + G;
+        id = r + G;
+        misc = id + G;
+        q = reinterpret_cast<float4*>(base + (FIXED + 15) / 16 * 16);
+    }
+};
+
+// merge query `g`'s buffer into its pool (one warp) and lower its bound
+template <int EPL, int G>
+__device__ __forceinline__ void exact_flush(const ExactArgs& A, const ExactSmem<EPL, G>& S, int g, int lane) {
+    uint64_t* const pool = S.pool + g * 32 * EPL;
+    const int n = S.cnt[g];
+    for (int off = 0; off < n; off += 32)
+        merge_ranked<EPL>(pool, S.buf + g * EXACT_BUF + off, min(32, n - off), A.k, lane);
+    uint64_t kth = pool[A.k - 1];
+    if (A.bound && S.id[g] >= 0) {
+        unsigned long long seen = 0;
+        if (lane == 0) {
+            if (n > 0 && kth != KEY_EMPTY) atomicMin(A.bound + S.id[g], (unsigned long long)kth);
+            seen = __ldcg(A.bound + S.id[g]);
+        }
+        seen = __shfl_sync(FULL, seen, 0);
+        kth = min(kth, (uint64_t)seen);
+    }
+    __syncwarp();
+    if (lane == 0) {
+        S.tau[g] = kth;
+        S.cnt[g] = 0;
+    }
+}
+
+// The rows [row0, row1) of the group whose slabs and queries are in S; the pools hold the result.
+// Bounded by fp32 issue where rows are shared (8 queries) and by row bytes where they are not.
+template <int EPL, int G>
+__device__ __forceinline__ void exact_scan(const ExactArgs& A, const ExactSmem<EPL, G>& S, int row0, int row1) {
+    const int lane = lane_id(), warp = threadIdx.x >> 5;
+    const int team = lane >> 3, sub = lane & 7;
+    const int groups = A.d_pad >> 2;
+    for (int b = row0; b < row1;) {
+        // rows that no query wants are jumped over
+        int next = row1;
+        bool any = false;
+#pragma unroll
+        for (int g = 0; g < G; ++g) {
+            any = any || (S.l[g] < b + 2 * EXACT_STEP && S.r[g] >= b);
+            if (S.l[g] >= b && S.l[g] <= S.r[g]) next = min(next, S.l[g]);
+        }
+        if (!any) { b = next; continue; }
+#pragma unroll 1
+        for (int half = 0; half < 2; ++half) {
+            const int base = b + half * EXACT_STEP + warp * 8;
+            unsigned int cover = 0;                          // queries that want one of the 8 rows
+#pragma unroll
+            for (int g = 0; g < G; ++g)
+                if (S.l[g] < min(base + 8, row1) && S.r[g] >= base) cover |= 1u << g;
+            if (base >= row1 || cover == 0) continue;
+            const int rowA = base + team, rowB = rowA + 4;
+            const bool vA = rowA < row1, vB = rowB < row1;
+            const float4* pA = reinterpret_cast<const float4*>(A.vectors + (size_t)rowA * (size_t)A.d_pad);
+            const float4* pB = reinterpret_cast<const float4*>(A.vectors + (size_t)rowB * (size_t)A.d_pad);
+            float acc[2][G];
+#pragma unroll
+            for (int g = 0; g < G; ++g) acc[0][g] = acc[1][g] = 0.f;
+#pragma unroll 1
+            for (int g0 = 0; g0 < groups; g0 += 32) {
+                float4 xa[4], xb[4];
+#pragma unroll
+                for (int c = 0; c < 4; ++c) {
+                    const int i = g0 + 8 * c + sub;
+                    xa[c] = xb[c] = make_float4(0.f, 0.f, 0.f, 0.f);
+                    if (vA && i < groups) xa[c] = __ldg(pA + i);
+                    if (vB && i < groups) xb[c] = __ldg(pB + i);
+                }
+#pragma unroll
+                for (int g = 0; g < G; ++g) {
+                    if ((cover >> g) & 1u) {
+                        const float4* qv = S.q + g * groups;
+#pragma unroll
+                        for (int c = 0; c < 4; ++c) {
+                            const int i = g0 + 8 * c + sub;
+                            if (i < groups) {
+                                const float4 q = qv[i];
+                                float t;
+                                t = xa[c].x - q.x; acc[0][g] = fmaf(t, t, acc[0][g]);
+                                t = xb[c].x - q.x; acc[1][g] = fmaf(t, t, acc[1][g]);
+                                t = xa[c].y - q.y; acc[0][g] = fmaf(t, t, acc[0][g]);
+                                t = xb[c].y - q.y; acc[1][g] = fmaf(t, t, acc[1][g]);
+                                t = xa[c].z - q.z; acc[0][g] = fmaf(t, t, acc[0][g]);
+                                t = xb[c].z - q.z; acc[1][g] = fmaf(t, t, acc[1][g]);
+                                t = xa[c].w - q.w; acc[0][g] = fmaf(t, t, acc[0][g]);
+                                t = xb[c].w - q.w; acc[1][g] = fmaf(t, t, acc[1][g]);
+                            }
+                        }
+                    }
+                }
+            }
+            // the butterfly 4, 2, 1 over the team, every lane handing on the sums it does not keep: after
+            // partner distance 4 a lane has one row, after 2 half of the queries, after 1 a quarter
+            const bool up4 = (sub & 4) != 0;
+            float s1[G];
+#pragma unroll
+            for (int g = 0; g < G; ++g) {
+                const float give = up4 ? acc[0][g] : acc[1][g], keep = up4 ? acc[1][g] : acc[0][g];
+                s1[g] = keep + __shfl_xor_sync(FULL, give, 4);
+            }
+            const int row = up4 ? rowB : rowA;
+            constexpr int NK = G >= 4 ? G / 4 : 1;
+            float fin[NK];
+            int g_lo = 0;
+            bool emits = row < row1;
+            if (G >= 4) {
+                const bool up2 = (sub & 2) != 0, up1 = (sub & 1) != 0;
+                float s2[G / 2 > 0 ? G / 2 : 1];
+#pragma unroll
+                for (int g = 0; g < G / 2; ++g) {
+                    const float give = up2 ? s1[g] : s1[g + G / 2], keep = up2 ? s1[g + G / 2] : s1[g];
+                    s2[g] = keep + __shfl_xor_sync(FULL, give, 2);
+                }
+#pragma unroll
+                for (int g = 0; g < G / 4; ++g) {
+                    const float give = up1 ? s2[g] : s2[g + G / 4], keep = up1 ? s2[g + G / 4] : s2[g];
+                    fin[g] = keep + __shfl_xor_sync(FULL, give, 1);
+                }
+                g_lo = (up2 ? G / 2 : 0) + (up1 ? G / 4 : 0);
+            } else {
+                float a = s1[0] + __shfl_xor_sync(FULL, s1[0], 2);
+                fin[0] = a + __shfl_xor_sync(FULL, a, 1);
+                emits = emits && (sub & 3) == 0;
+            }
+#pragma unroll
+            for (int x = 0; x < NK; ++x) {
+                const int g = g_lo + x;
+                const uint64_t tau = S.tau[g];
+                if (emits && row >= S.l[g] && row <= S.r[g] && __float_as_uint(fin[x]) <= (uint32_t)(tau >> 32)) {
+                    const uint64_t key = make_key(fin[x], (uint32_t)__ldg(A.rank2id + row), 1u);
+                    if (key < tau) S.buf[g * EXACT_BUF + atomicAdd(&S.cnt[g], 1)] = key;
+                }
+            }
+        }
+        b += 2 * EXACT_STEP;
+        __syncthreads();
+        bool full = false;
+#pragma unroll
+        for (int g = 0; g < G; ++g) full = full || S.cnt[g] >= 64;
+        __syncthreads();
+        if (full) {
+            if (warp < G) exact_flush<EPL, G>(A, S, warp, lane);
+            __syncthreads();
+        }
+    }
+    if (warp < G) exact_flush<EPL, G>(A, S, warp, lane);
+    __syncthreads();
+}
+
 template <int EPL>
-__global__ void __launch_bounds__(EXACT_WARPS * 32)
+__device__ __forceinline__ void exact_output(const ExactArgs& A, const uint64_t* pool, int q, int lane) {
+    for (int j = lane; j < A.k; j += 32) {
+        const uint64_t key = pool[j];
+        int32_t oid = -1;
+        float dist = __int_as_float(0x7F800000);
+        if (key != KEY_EMPTY) {
+            oid = (int32_t)key_rank(key);
+            dist = __fsqrt_rn(key_dist2(key));
+        }
+        A.out_ids[(size_t)q * A.k + j] = oid;
+        A.out_dists[(size_t)q * A.k + j] = dist;
+    }
+}
+
+// One piece: queries S.id[] with slabs S.l/S.r, rows [row0, row1), `pieces` pieces from `first` on belong to
+// the group, whose count of finished pieces is *done.
+template <int EPL, int G>
+__device__ __forceinline__ void exact_piece(const ExactArgs& A, const ExactSmem<EPL, G>& S, int row0, int row1, int piece,
+                                            int first, int pieces, unsigned int* done) {
+    const int lane = lane_id(), warp = threadIdx.x >> 5;
+    for (int g = 0; g < G; ++g) {
+        float* qf = reinterpret_cast<float*>(S.q) + (size_t)g * A.d_pad;
+        const float* src = A.queries + (size_t)max(S.id[g], 0) * A.d;
+        for (int i = threadIdx.x; i < A.d_pad; i += EXACT_WARPS * 32) qf[i] = i < A.d && S.id[g] >= 0 ? __ldg(src + i) : 0.f;
+    }
+    for (int i = threadIdx.x; i < G * 32 * EPL; i += EXACT_WARPS * 32) S.pool[i] = KEY_EMPTY;
+    if (threadIdx.x < G) {
+        S.cnt[threadIdx.x] = 0;
+        S.tau[threadIdx.x] = A.bound && S.id[threadIdx.x] >= 0 ? (uint64_t)__ldcg(A.bound + S.id[threadIdx.x]) : KEY_EMPTY;
+    }
+    __syncthreads();
+    exact_scan<EPL, G>(A, S, row0, row1);
+    if (pieces > 1) {
+        if (warp < G) {
+            const uint64_t tau = S.tau[warp];              // keys above it lose to another piece's
+            uint64_t* out = A.part + ((size_t)piece * G + warp) * A.k;
+            for (int j = lane; j < A.k; j += 32) {
+                const uint64_t key = S.pool[warp * 32 * EPL + j];
+                __stcg(reinterpret_cast<unsigned long long*>(out + j), (unsigned long long)(key <= tau ? key : KEY_EMPTY));
+            }
+        }
+        __threadfence();
+        __syncthreads();
+        if (threadIdx.x == 0) S.misc[0] = atomicAdd(done, 1u) == (unsigned int)pieces - 1u;
+        __syncthreads();
+        if (!S.misc[0]) return;
+        __threadfence();
+        if (warp < G && S.id[warp] >= 0) {
+            uint64_t* const pool = S.pool + warp * 32 * EPL;
+            uint64_t* const buf = S.buf + warp * EXACT_BUF;
+            uint64_t tau = min((uint64_t)__ldcg(A.bound + S.id[warp]), pool[A.k - 1]);
+            int c = 0;
+            for (int p = first; p < first + pieces; ++p) {
+                if (p == piece) continue;
+                const unsigned long long* in = reinterpret_cast<const unsigned long long*>(A.part) + ((size_t)p * G + warp) * A.k;
+                for (int off = 0; off < A.k; off += 32) {
+                    const uint64_t key = off + lane < A.k ? (uint64_t)__ldcg(in + off + lane) : KEY_EMPTY;
+                    const uint32_t M = __ballot_sync(FULL, key != KEY_EMPTY && key <= tau);
+                    if ((M >> lane) & 1u) buf[c + __popc(M & ((1u << lane) - 1u))] = key;
+                    c += __popc(M);
+                    __syncwarp();
+                    if (c >= 32) {
+                        for (int x = 0; x < c; x += 32) merge_ranked<EPL>(pool, buf + x, min(32, c - x), A.k, lane);
+                        tau = min(tau, pool[A.k - 1]);
+                        c = 0;
+                        __syncwarp();
+                    }
+                    if (M != FULL) break;                   // the list is ascending
+                }
+            }
+            if (c > 0) merge_ranked<EPL>(pool, buf, c, A.k, lane);
+            __syncwarp();
+        }
+        __syncthreads();
+        if (threadIdx.x == 0) *done = 0u;                   // leave the scratch as it was found
+        if (threadIdx.x < G && S.id[threadIdx.x] >= 0) A.bound[S.id[threadIdx.x]] = ~0ull;
+    } else if (A.bound && threadIdx.x < G && S.id[threadIdx.x] >= 0) {
+        A.bound[S.id[threadIdx.x]] = ~0ull;
+    }
+    if (warp < G && S.id[warp] >= 0) exact_output<EPL>(A, S.pool + warp * 32 * EPL, S.id[warp], lane);
+    __syncthreads();
+}
+
+// One CTA per query, no scratch.
+template <int EPL>
+__global__ void __launch_bounds__(EXACT_WARPS * 32, 2)
 frog_exact_kernel(const ExactArgs A) {
     extern __shared__ __align__(16) unsigned char smem_raw[];
-    constexpr int POOL = 32 * EPL;
-    const int lane = lane_id();
-    const int warp = threadIdx.x >> 5;
-    const int q = blockIdx.x;
-    float4* qs = reinterpret_cast<float4*>(smem_raw);
-    uint64_t* pools = reinterpret_cast<uint64_t*>(smem_raw + (size_t)A.d_pad * 4);
-    uint64_t* pool = pools + (size_t)warp * POOL;
-
-    {
-        float* qf = reinterpret_cast<float*>(qs);
-        const float* src = A.queries + (size_t)q * A.d;
-        for (int i = threadIdx.x; i < A.d_pad; i += blockDim.x) qf[i] = i < A.d ? __ldg(src + i) : 0.f;
-        for (int i = lane; i < POOL; i += 32) pool[i] = KEY_EMPTY;
-    }
+    const ExactSmem<EPL, 1> S(smem_raw);
+    const int q = blockIdx.x, lane = lane_id();
     const int32_t lo = __ldg(A.lo + q), hi = __ldg(A.hi + q);
     int l_q, r_q;
     warp_rank_interval(A.sorted_attr, A.n, lo, hi, lane, l_q, r_q);
-    const int w = (lo > hi) ? 0 : (r_q - l_q + 1);
-    __syncthreads();
-
-    for (int b0 = warp * 16; b0 < w; b0 += EXACT_WARPS * 16) {
-        const int cnt = min(16, w - b0);
-        const uint32_t rank = (uint32_t)(l_q + b0 + (lane & 15));
-        float d2 = batch_dist2<4>(A.vectors, A.d_pad, qs, rank, cnt, lane);
-        uint64_t key = KEY_EMPTY;
-        if (lane < cnt) key = make_key(d2, (uint32_t)__ldg(A.rank2id + rank), 1u);   // keyed by object id
-        // (merge_batch itself rejects candidates not better than the current k-th best)
-        merge_batch<EPL>(pool, key, A.k, lane);
+    if (lo > hi) r_q = l_q - 1;
+    if (threadIdx.x == 0) {
+        S.l[0] = l_q;
+        S.r[0] = r_q;
+        S.id[0] = q;
     }
     __syncthreads();
+    exact_piece<EPL, 1>(A, S, l_q, r_q + 1, 0, 0, 1, nullptr);
+}
+
+// Fewer than EXACT_GROUP_MIN queries: all rows cut into equal pieces, at most one per CTA.
+template <int EPL>
+__global__ void __launch_bounds__(EXACT_WARPS * 32, 2)
+frog_exact_few_kernel(const ExactArgs A) {
+    extern __shared__ __align__(16) unsigned char smem_raw[];
+    __shared__ int2 slab[EXACT_GROUP_MIN];
+    const ExactSmem<EPL, 1> S(smem_raw);
+    const int lane = lane_id(), warp = threadIdx.x >> 5;
+    for (int q = warp; q < A.nq; q += EXACT_WARPS) {
+        const int32_t lo = __ldg(A.lo + q), hi = __ldg(A.hi + q);
+        int l_q, r_q;
+        warp_rank_interval(A.sorted_attr, A.n, lo, hi, lane, l_q, r_q);
+        if (lane == 0) slab[q] = make_int2(l_q, max(0, lo > hi ? 0 : r_q - l_q + 1));
+    }
+    __syncthreads();
+    long long rows = 0;
+    for (int q = 0; q < A.nq; ++q) rows += slab[q].y;
+    // the pieces of a query but its last are full, so nq extra ones at most
+    const int share = max((int)gridDim.x - A.nq, 1);
+    int size = (int)max((rows + share - 1) / share, (long long)A.min_rows);
+    size = (size + EXACT_STEP - 1) / EXACT_STEP * EXACT_STEP;
+    int first = 0;
+    for (int q = 0; q < A.nq; ++q) {
+        const int pieces = max(1, (int)(((long long)slab[q].y + size - 1) / size));
+        const int p = (int)blockIdx.x - first;
+        if (p >= 0 && p < pieces) {
+            if (threadIdx.x == 0) {
+                S.l[0] = slab[q].x;
+                S.r[0] = slab[q].x + slab[q].y - 1;
+                S.id[0] = q;
+            }
+            const int row0 = slab[q].x + p * size, row1 = min(row0 + size, slab[q].x + slab[q].y);
+            __syncthreads();
+            exact_piece<EPL, 1>(A, S, row0, row1, (int)blockIdx.x, first, pieces, A.done + q);
+            return;
+        }
+        first += pieces;
+    }
+}
+
+// The pieces that frog_exact_cut_kernel listed, for groups of eight queries.
+template <int EPL>
+__global__ void __launch_bounds__(EXACT_WARPS * 32, 2)
+frog_exact_group_kernel(const ExactArgs A) {
+    extern __shared__ __align__(16) unsigned char smem_raw[];
+    const ExactSmem<EPL, EXACT_GROUP> S(smem_raw);
+    for (;;) {
+        if (threadIdx.x == 0) S.misc[1] = (int)atomicAdd(A.counters + 1, 1u);
+        __syncthreads();
+        const int piece = S.misc[1];
+        if (piece >= (int)__ldcg(A.counters)) break;
+        const int4 job = A.jobs[piece];
+        const int2 gp = A.groups[job.x];
+        if (threadIdx.x < EXACT_GROUP) {
+            const int i = job.x * EXACT_GROUP + threadIdx.x;
+            const int q = i < A.nq ? A.order[i] : -1;
+            const int2 lr = q >= 0 ? A.ranges[q] : make_int2(1, 0);
+            S.id[threadIdx.x] = q;
+            S.l[threadIdx.x] = lr.x;
+            S.r[threadIdx.x] = lr.y;
+        }
+        __syncthreads();
+        exact_piece<EPL, EXACT_GROUP>(A, S, job.y, job.z, piece, gp.x, gp.y, A.done + job.x);
+        __syncthreads();
+    }
+}
+
+// bin of a query: widest first, then by position, so that the queries of a group share rows
+__device__ __forceinline__ int exact_bin(const int2& lr, int n) {
+    const int w = lr.y - lr.x + 1;
+    return (w <= 0 ? 32 : __clz(w)) * 32 + (w <= 0 ? 0 : (int)((long long)lr.x * 32 / n));
+}
+
+// slabs of the queries and the histogram of their bins (one warp per query)
+__global__ void __launch_bounds__(256)
+frog_exact_plan_kernel(const ExactArgs A) {
+    const int q = (int)((blockIdx.x * blockDim.x + threadIdx.x) >> 5);
+    const int lane = lane_id();
+    if (q >= A.nq) return;
+    const int32_t lo = __ldg(A.lo + q), hi = __ldg(A.hi + q);
+    int l_q, r_q;
+    warp_rank_interval(A.sorted_attr, A.n, lo, hi, lane, l_q, r_q);
+    if (lane == 0) {
+        const int2 lr = lo > hi || r_q < l_q ? make_int2(1, 0) : make_int2(l_q, r_q);
+        A.ranges[q] = lr;
+        atomicAdd(A.counters + 2 + exact_bin(lr, A.n), 1u);
+    }
+}
+
+// rows that a group's slabs cover (l ascending), and the row where `skip` of them lie below
+__device__ __forceinline__ int exact_covered(const int2* s, int cnt) {
+    int total = 0, end = 0;
+    for (int i = 0; i < cnt; ++i) {
+        if (s[i].y < s[i].x) continue;
+        total += max(0, s[i].y + 1 - max(s[i].x, end));
+        end = max(end, s[i].y + 1);
+    }
+    return total;
+}
+__device__ __forceinline__ int exact_cut(const int2* s, int cnt, int skip) {
+    int end = 0;
+    for (int i = 0; i < cnt; ++i) {
+        if (s[i].y < s[i].x) continue;
+        const int from = max(s[i].x, end), len = max(0, s[i].y + 1 - from);
+        if (skip < len) return from + skip;
+        skip -= len;
+        end = max(end, s[i].y + 1);
+    }
+    return end;
+}
+
+// order of the queries, and the groups' rows cut into pieces of equal size (one CTA)
+__global__ void __launch_bounds__(1024)
+frog_exact_cut_kernel(const ExactArgs A) {
+    __shared__ unsigned int start[2048];
+    __shared__ unsigned int warp_sum[32];
+    __shared__ unsigned long long rows;
+    __shared__ unsigned int pieces;
+    const int t = threadIdx.x, lane = lane_id(), warp = t >> 5;
+    if (t == 0) { rows = 0; pieces = 0; }
+    // exclusive scan of the bins, two per thread
+    const unsigned int a = 2 * t < EXACT_BINS ? A.counters[2 + 2 * t] : 0u;
+    const unsigned int b = 2 * t + 1 < EXACT_BINS ? A.counters[3 + 2 * t] : 0u;
+    unsigned int x = a + b;
+    for (int o = 1; o < 32; o <<= 1) {
+        const unsigned int y = __shfl_up_sync(FULL, x, o);
+        if (lane >= o) x += y;
+    }
+    if (lane == 31) warp_sum[warp] = x;
+    __syncthreads();
     if (warp == 0) {
-        for (int ow = 1; ow < EXACT_WARPS; ++ow) {
-            const uint64_t* other = pools + (size_t)ow * POOL;
-            for (int j0 = 0; j0 < A.k; j0 += 32) {
-                uint64_t key = (j0 + lane < A.k) ? other[j0 + lane] : KEY_EMPTY;
-                merge_batch<EPL>(pool, key, A.k, lane);
-            }
+        unsigned int s = warp_sum[lane];
+        for (int o = 1; o < 32; o <<= 1) {
+            const unsigned int y = __shfl_up_sync(FULL, s, o);
+            if (lane >= o) s += y;
         }
-        __syncwarp();
-        for (int j = lane; j < A.k; j += 32) {
-            uint64_t key = pool[j];
-            int32_t oid = -1;
-            float dist = __int_as_float(0x7F800000);
-            if (key != KEY_EMPTY) {
-                oid = (int32_t)key_rank(key);
-                dist = __fsqrt_rn(key_dist2(key));
-            }
-            A.out_ids[(size_t)q * A.k + j] = oid;
-            A.out_dists[(size_t)q * A.k + j] = dist;
+        warp_sum[lane] = s;
+    }
+    __syncthreads();
+    const unsigned int before = (warp ? warp_sum[warp - 1] : 0u) + x - a - b;
+    start[2 * t] = before;
+    start[2 * t + 1] = before + a;
+    if (2 * t < EXACT_BINS) A.counters[2 + 2 * t] = 0u;          // leave the bins empty
+    if (2 * t + 1 < EXACT_BINS) A.counters[3 + 2 * t] = 0u;
+    __syncthreads();
+    for (int q = t; q < A.nq; q += 1024) A.order[atomicAdd(&start[exact_bin(A.ranges[q], A.n)], 1u)] = q;
+    __syncthreads();
+    const int groups = (A.nq + EXACT_GROUP - 1) / EXACT_GROUP;
+    auto slabs = [&](int g, int2* s) -> int {
+        const int cnt = min(EXACT_GROUP, A.nq - g * EXACT_GROUP);
+        for (int i = 0; i < cnt; ++i) {
+            const int2 lr = A.ranges[A.order[g * EXACT_GROUP + i]];
+            int j = i;
+            for (; j > 0 && s[j - 1].x > lr.x; --j) s[j] = s[j - 1];
+            s[j] = lr;
         }
+        return cnt;
+    };
+    for (int g = t; g < groups; g += 1024) {
+        int2 s[EXACT_GROUP];
+        const int c = exact_covered(s, slabs(g, s));
+        A.groups[g] = make_int2(c, 0);
+        atomicAdd(&rows, (unsigned long long)c);
+    }
+    __syncthreads();
+    // a group of several pieces has at most twice its rows' share of them, so max_pieces is never exceeded
+    const long long want = ((long long)rows * 2 + A.max_pieces - 1) / A.max_pieces;
+    long long size = want > A.min_rows ? want : A.min_rows;
+    size = (size + 2 * EXACT_STEP - 1) / (2 * EXACT_STEP) * (2 * EXACT_STEP);
+    // groups of several pieces first: their piece numbers address the partial lists
+    for (int pass = 0; pass < 2; ++pass) {
+        for (int g = t; g < groups; g += 1024) {
+            const int2 have = A.groups[g];
+            const int c = have.x, np = max(1, (int)(((long long)c + size - 1) / size));
+            if ((np > 1) != (pass == 0) || (pass == 1 && have.y != 0)) continue;
+            int2 s[EXACT_GROUP];
+            const int cnt = slabs(g, s);
+            const unsigned int first = atomicAdd(&pieces, (unsigned int)np);
+            int from = exact_cut(s, cnt, 0);
+            for (int p = 0; p < np; ++p) {
+                const int to = p + 1 < np ? exact_cut(s, cnt, (int)((long long)(p + 1) * size)) : exact_cut(s, cnt, c);
+                A.jobs[first + p] = make_int4(g, from, to, 0);
+                from = to;
+            }
+            A.groups[g] = make_int2((int)first, np);
+        }
+        __syncthreads();
+    }
+    if (t == 0) {
+        A.counters[0] = pieces;
+        A.counters[1] = 0u;
     }
 }
 
 typedef void (*exact_fn)(const ExactArgs);
+
+template <template <int> class K>
+exact_fn exact_pick(int k) {
+    return k <= 32 ? K<1>::fn() : k <= 64 ? K<2>::fn() : k <= 128 ? K<4>::fn() : k <= 256 ? K<8>::fn() : K<16>::fn();
+}
+template <int EPL> struct OnePerQuery { static exact_fn fn() { return frog_exact_kernel<EPL>; } };
+template <int EPL> struct Few { static exact_fn fn() { return frog_exact_few_kernel<EPL>; } };
+template <int EPL> struct Grouped { static exact_fn fn() { return frog_exact_group_kernel<EPL>; } };
+
+template <int G>
+size_t exact_smem(int k, int d_pad) {
+    return k <= 32 ? ExactSmem<1, G>::bytes(d_pad) : k <= 64 ? ExactSmem<2, G>::bytes(d_pad)
+         : k <= 128 ? ExactSmem<4, G>::bytes(d_pad) : k <= 256 ? ExactSmem<8, G>::bytes(d_pad) : ExactSmem<16, G>::bytes(d_pad);
+}
 
 }  // namespace
 
@@ -94,16 +551,8 @@ extern "C" int frog_exact_search(const frog_index_t* index, const float* queries
     if (nq == 0) return FROG_OK;
     if (!queries || !lo || !hi || !out_ids || !out_dists) return FROG_ERR_INVALID_ARG;
     FROG_CUDA_TRY(cudaSetDevice(index->info.device));
-    exact_fn fn;
-    int pool_slots;
-    if (k <= 32) { fn = frog_exact_kernel<1>; pool_slots = 32; }
-    else if (k <= 64) { fn = frog_exact_kernel<2>; pool_slots = 64; }
-    else if (k <= 128) { fn = frog_exact_kernel<4>; pool_slots = 128; }
-    else if (k <= 256) { fn = frog_exact_kernel<8>; pool_slots = 256; }
-    else { fn = frog_exact_kernel<16>; pool_slots = 512; }
-    size_t smem = (size_t)index->info.d_pad * 4 + (size_t)EXACT_WARPS * pool_slots * 8;
-    FROG_CUDA_TRY(cudaFuncSetAttribute((const void*)fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
-    ExactArgs A;
+    cudaStream_t s = static_cast<cudaStream_t>(stream);
+    ExactArgs A{};
     A.sorted_attr = index->d_sorted_attr;
     A.rank2id = index->d_rank2id;
     A.vectors = index->d_vectors;
@@ -117,7 +566,56 @@ extern "C" int frog_exact_search(const frog_index_t* index, const float* queries
     A.k = k;
     A.out_ids = out_ids;
     A.out_dists = out_dists;
-    fn<<<nq, EXACT_WARPS * 32, smem, static_cast<cudaStream_t>(stream)>>>(A);
+    auto ready = [&](exact_fn fn, size_t smem) {
+        return cudaFuncSetAttribute((const void*)fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    };
+    cudaStreamCaptureStatus capture = cudaStreamCaptureStatusNone;
+    FROG_CUDA_TRY(cudaStreamIsCapturing(s, &capture));
+    const bool few = nq < EXACT_GROUP_MIN;
+    const size_t smem = few ? exact_smem<1>(k, A.d_pad) : exact_smem<EXACT_GROUP>(k, A.d_pad);
+    if (capture == cudaStreamCaptureStatusNone && smem <= 227 * 1024) {
+        const exact_fn fn = few ? exact_pick<Few>(k) : exact_pick<Grouped>(k);
+        FROG_CUDA_TRY(ready(fn, smem));
+        int per_sm = 0;
+        FROG_CUDA_TRY(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, (const void*)fn, EXACT_WARPS * 32, smem));
+        const int grid = std::max(per_sm, 1) * index->sm_count;
+        const int groups = few ? nq : (nq + EXACT_GROUP - 1) / EXACT_GROUP;
+        // enough pieces to even out their ends; fewer for long result lists, whose partial lists they multiply
+        const int max_pieces = few ? grid : grid * (k <= 128 ? 16 : 8);
+        frog_index* mix = const_cast<frog_index*>(index);      // the scratch sets are the index's only mutable part
+        std::lock_guard<std::mutex> lock(mix->mu);
+        FrogScratch* sc = nullptr;
+        const int rc = froghost::acquire_scratch(mix, s, &sc);
+        if (rc) return rc;
+        froghost::ExactScratch X;
+        const size_t lists = (size_t)max_pieces * (few ? 1 : EXACT_GROUP) * k;
+        if (froghost::ensure_exact(sc, (size_t)nq, (size_t)groups, (size_t)max_pieces + groups, lists, EXACT_BINS + 2, &X) == FROG_OK) {
+            A.ranges = static_cast<int2*>(X.ranges);
+            A.order = X.order;
+            A.jobs = static_cast<int4*>(X.jobs);
+            A.groups = static_cast<int2*>(X.groups);
+            A.counters = X.counters;
+            A.done = X.done;
+            A.bound = X.bound;
+            A.part = X.part;
+            A.max_pieces = max_pieces;
+            A.min_rows = few ? 256 : 512;
+            if (!few) {
+                frog_exact_plan_kernel<<<(nq * 32 + 255) / 256, 256, 0, s>>>(A);
+                frog_exact_cut_kernel<<<1, 1024, 0, s>>>(A);
+            }
+            fn<<<grid, EXACT_WARPS * 32, smem, s>>>(A);
+            FROG_CUDA_TRY(cudaGetLastError());
+            FROG_CUDA_TRY(cudaEventRecord(sc->done, s));
+            sc->stream = s;
+            sc->tick = ++mix->tick;
+            return FROG_OK;
+        }
+    }
+    const size_t smem1 = exact_smem<1>(k, A.d_pad);
+    const exact_fn one = exact_pick<OnePerQuery>(k);
+    FROG_CUDA_TRY(ready(one, smem1));
+    one<<<nq, EXACT_WARPS * 32, smem1, s>>>(A);
     FROG_CUDA_TRY(cudaGetLastError());
     return FROG_OK;
 }

@@ -21,6 +21,8 @@ struct FrogScratch {
     size_t table_bytes = 0;
     int32_t* d_plan = nullptr;       // per query: rank interval (2 ints) and processing order (1 int)
     size_t plan_queries = 0;
+    char* d_exact = nullptr;         // scratch of the exact scan (ExactScratch), grown on demand
+    size_t exact_bytes = 0, exact_queries = 0, exact_groups = 0, exact_jobs = 0, exact_lists = 0;
     cudaEvent_t done = nullptr;
     cudaEvent_t k_begin = nullptr, k_end = nullptr;   // around the search kernel of the last timed launch
     bool k_timed = false;
@@ -112,6 +114,18 @@ int acquire_scratch(frog_index* ix, cudaStream_t s, FrogScratch** out);
 int ensure_bitmap(const frog_index* ix, FrogScratch* sc, size_t slots);
 int ensure_table(FrogScratch* sc, size_t slots, int bits);
 int ensure_plan(FrogScratch* sc, size_t nq);
+// Scratch of one exact scan.  At rest `counters` and `done` are zero and `bound` is all ones.
+struct ExactScratch {
+    void* ranges;              // int2 per query
+    int32_t* order;            // per query
+    void* jobs;                // int4 per piece
+    void* groups;              // int2 per group
+    unsigned int* counters;
+    unsigned int* done;        // per group
+    unsigned long long* bound; // per query
+    uint64_t* part;            // keys of the pieces' lists
+};
+int ensure_exact(FrogScratch* sc, size_t nq, size_t groups, size_t jobs, size_t lists, size_t counters, ExactScratch* out);
 }  // namespace froghost
 
 #define FROG_CUDA_TRY(expr)                                  \

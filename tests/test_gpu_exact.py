@@ -1,0 +1,95 @@
+"""The exact filtered scan: grouped, split and one-CTA-per-query forms against the oracle's slab scan, at the
+edges of its pieces, pools and row lengths."""
+import numpy as np
+import pytest
+
+import oracle
+
+pytestmark = pytest.mark.gpu
+
+torch = pytest.importorskip("torch")
+
+
+def _index(libs, tmp, n, d, seed):
+    rng = np.random.default_rng(seed)
+    base = rng.integers(0, 6, (n, d)).astype(np.float32)                # many equal distances: ties by id
+    attrs = rng.integers(0, max(1, n // 3), n).astype(np.int32)
+    path = str(tmp / ("e%d_%d.idx" % (n, d)))
+    libs.build_index_gpu(base, attrs, path, m=4, ef_c=4, patience=1, n_inv=30)
+    return base, attrs, path
+
+
+def _queries(base, attrs, nq, seed, narrow):
+    rng = np.random.default_rng(seed)
+    n, d = base.shape
+    q = (rng.integers(0, 60, (nq, d)) / 10).astype(np.float32)
+    w = np.maximum(1, (n * 2.0 ** -rng.uniform(0, narrow, nq)).astype(int))
+    a = np.sort(attrs)
+    s = (rng.random(nq) * (n - w + 1)).astype(int)
+    lo, hi = a[s].copy(), a[s + w - 1].copy()
+    lo[0], hi[0] = a[0], a[-1]
+    if nq > 1:
+        lo[1], hi[1] = 5, 4                                              # empty
+    if nq > 2:
+        lo[2] = hi[2] = a[-1]
+    return q, lo.astype(np.int32), hi.astype(np.int32)
+
+
+def _check(gix, ix, q, lo, hi, k, graph=False):
+    dev = [torch.from_numpy(x).cuda() for x in (q, lo, hi)]
+    if graph:
+        out = (torch.empty((len(lo), k), dtype=torch.int32, device="cuda"), torch.empty((len(lo), k), device="cuda"))
+        g = torch.cuda.CUDAGraph()
+        with torch.cuda.graph(g):
+            gix.exact_search(*dev, k, out_ids=out[0], out_dists=out[1])
+        g.replay()
+    else:
+        out = gix.exact_search(*dev, k)
+    torch.cuda.synchronize()
+    ids, dists = oracle.exact_slab(ix, q, lo, hi, k, mode=1)[:2]
+    assert np.array_equal(out[0].cpu().numpy(), ids)
+    assert np.array_equal(out[1].cpu().numpy().view(np.uint32), np.asarray(dists, np.float32).view(np.uint32))
+
+
+@pytest.mark.parametrize("n,d", [(1, 3), (130, 16), (5000, 32), (20011, 50), (9000, 128), (3000, 300), (700, 6000)])
+def test_matches_the_oracle(libs, tmp_path, n, d):
+    base, attrs, path = _index(libs, tmp_path, n, d, n)
+    ix = oracle.load_index(path)
+    gix = libs.Index.load(path)
+    for nq, narrow in ((1, 0), (6, 3), (15, 10), (16, 10), (17, 1), (203, 7)):
+        q, lo, hi = _queries(base, attrs, nq, nq, narrow)
+        for k in (1, 10, 33, 100) if n < 20000 else (10, 100):
+            _check(gix, ix, q, lo, hi, k)
+    q, lo, hi = _queries(base, attrs, 40, 7, 4)
+    for k in (64, 65, 129, 257, 512):
+        _check(gix, ix, q, lo, hi, k)
+        _check(gix, ix, q[:3], lo[:3], hi[:3], k)
+    gix.close()
+
+
+def test_groups_with_gaps_streams_and_capture(libs, tmp_path):
+    """Slabs that share no rows (a group's pieces jump the gaps), calls on two streams, and a captured call."""
+    base, attrs, path = _index(libs, tmp_path, 30000, 24, 11)
+    ix = oracle.load_index(path)
+    gix = libs.Index.load(path)
+    rng = np.random.default_rng(2)
+    q, lo, hi = _queries(base, attrs, 64, 3, 3)
+    a = np.sort(attrs)
+    s = rng.integers(0, 29000, 64)
+    lo[3:], hi[3:] = a[s][3:], a[s + rng.integers(0, 900, 64)][3:]
+    _check(gix, ix, q, lo, hi, 20)
+    _check(gix, ix, q, lo, hi, 20, graph=True)
+    _check(gix, ix, q[:5], lo[:5], hi[:5], 20, graph=True)
+    dev = [torch.from_numpy(x).cuda() for x in (q, lo, hi)]
+    want = gix.exact_search(*dev, 20)
+    streams = [torch.cuda.Stream() for _ in range(6)]
+    torch.cuda.synchronize()
+    got = []
+    for i in range(24):
+        with torch.cuda.stream(streams[i % 6]):
+            n = (64, 7)[i % 2]
+            got.append(gix.exact_search(*(x[:n] for x in dev), 20))
+    torch.cuda.synchronize()
+    for g in got:
+        assert torch.equal(g[0], want[0][:len(g[0])]) and torch.equal(g[1], want[1][:len(g[0])])
+    gix.close()
