@@ -105,6 +105,123 @@ __device__ __forceinline__ void exact_flush(const ExactArgs& A, const ExactSmem<
     }
 }
 
+// squares of a row's chunk against a query's, four groups of four elements
+template <bool FULL_CHUNK>
+__device__ __forceinline__ float exact_chunk(float acc, const float4 (&x)[4], const float4* q, int left) {
+#pragma unroll
+    for (int c = 0; c < 4; ++c) {
+        if (FULL_CHUNK || 8 * c < left) {
+            const float4 v = q[8 * c];
+            float t;
+            t = x[c].x - v.x; acc = fmaf(t, t, acc);
+            t = x[c].y - v.y; acc = fmaf(t, t, acc);
+            t = x[c].z - v.z; acc = fmaf(t, t, acc);
+            t = x[c].w - v.w; acc = fmaf(t, t, acc);
+        }
+    }
+    return acc;
+}
+
+// exact_scan for a single query: four rows per team, 16 per warp in flight (bounded by row bytes).
+template <int EPL>
+__device__ __forceinline__ void exact_scan_one(const ExactArgs& A, const ExactSmem<EPL, 1>& S, int row0, int row1) {
+    const int lane = lane_id(), warp = threadIdx.x >> 5;
+    const int team = lane >> 3, sub = lane & 7;
+    const int groups = A.d_pad >> 2;
+    for (int b = row0; b < row1; b += 2 * EXACT_STEP) {
+        const int base = b + warp * 16, end = min(base + 16, row1);
+        if (base < row1) {                                   // warp-uniform
+            const float4* row = reinterpret_cast<const float4*>(A.vectors + (size_t)(base + team) * (size_t)A.d_pad) + sub;
+            float acc[4] = {0.f, 0.f, 0.f, 0.f};
+#pragma unroll 1
+            for (int g0 = 0; g0 < groups; g0 += 32) {
+                float4 x[4][4];
+                const int left = groups - g0 - sub;          // groups of the row from this lane's first on
+                const float4* qv = S.q + g0 + sub;
+                if (g0 + 32 <= groups && end == base + 16) {
+#pragma unroll
+                    for (int r = 0; r < 4; ++r)
+#pragma unroll
+                        for (int c = 0; c < 4; ++c) x[r][c] = __ldg(row + (size_t)r * groups * 4 + g0 + 8 * c);
+#pragma unroll
+                    for (int r = 0; r < 4; ++r) acc[r] = exact_chunk<true>(acc[r], x[r], qv, left);
+                } else {
+#pragma unroll
+                    for (int r = 0; r < 4; ++r)
+#pragma unroll
+                        for (int c = 0; c < 4; ++c) {
+                            x[r][c] = make_float4(0.f, 0.f, 0.f, 0.f);
+                            if (base + 4 * r + team < row1 && 8 * c < left) x[r][c] = __ldg(row + (size_t)r * groups * 4 + g0 + 8 * c);
+                        }
+#pragma unroll
+                    for (int r = 0; r < 4; ++r) acc[r] = exact_chunk<false>(acc[r], x[r], qv, left);
+                }
+            }
+            // the butterfly 4, 2, 1 over the team, every lane handing on the sums it does not keep: half of the
+            // rows after partner distance 4, one row after 2
+            const bool up4 = (sub & 4) != 0, up2 = (sub & 2) != 0;
+            float s1[2];
+#pragma unroll
+            for (int r = 0; r < 2; ++r) {
+                const float give = up4 ? acc[r] : acc[r + 2], keep = up4 ? acc[r + 2] : acc[r];
+                s1[r] = keep + __shfl_xor_sync(FULL, give, 4);
+            }
+            const float give = up2 ? s1[0] : s1[1], keep = up2 ? s1[1] : s1[0];
+            float d = keep + __shfl_xor_sync(FULL, give, 2);
+            d = d + __shfl_xor_sync(FULL, d, 1);
+            const int mine = base + 4 * ((up4 ? 2 : 0) + (up2 ? 1 : 0)) + team;
+            if ((sub & 1) == 0 && mine < row1 && __float_as_uint(d) <= (uint32_t)(S.tau[0] >> 32)) {
+                const uint64_t key = make_key(d, (uint32_t)__ldg(A.rank2id + mine), 1u);
+                if (key < S.tau[0]) S.buf[atomicAdd(&S.cnt[0], 1)] = key;
+            }
+        }
+        __syncthreads();
+        const bool full = S.cnt[0] >= 64;
+        __syncthreads();
+        if (full) {
+            if (warp == 0) exact_flush<EPL, 1>(A, S, 0, lane);
+            __syncthreads();
+        }
+    }
+    if (warp == 0) exact_flush<EPL, 1>(A, S, 0, lane);
+    __syncthreads();
+}
+
+// merge what may be among the k best of the pieces' lists into a single query's pool (one warp); eight loads per
+// lane are in flight at once
+template <int EPL>
+__device__ __forceinline__ void exact_gather(const ExactArgs& A, const ExactSmem<EPL, 1>& S, const unsigned long long* lists, int pieces, int lane) {
+    uint64_t* const pool = S.pool;
+    uint64_t* const buf = S.buf;
+    const unsigned int n = (unsigned int)pieces * (unsigned int)A.k;
+    uint64_t tau = (uint64_t)__ldcg(A.bound + S.id[0]);
+    int c = 0;
+    for (unsigned int off = 0; off < n; off += 256) {
+        uint64_t key[8];
+#pragma unroll
+        for (int i = 0; i < 8; ++i) {
+            const unsigned int x = off + 32 * i + lane;
+            key[i] = KEY_EMPTY;
+            if (x < n) key[i] = (uint64_t)__ldcg(lists + x);
+        }
+#pragma unroll
+        for (int i = 0; i < 8; ++i) {
+            const uint32_t M = __ballot_sync(FULL, key[i] != KEY_EMPTY && key[i] <= tau);
+            if ((M >> lane) & 1u) buf[c + __popc(M & ((1u << lane) - 1u))] = key[i];
+            c += __popc(M);
+            __syncwarp();
+            if (c >= 32) {
+                for (int x = 0; x < c; x += 32) merge_ranked<EPL>(pool, buf + x, min(32, c - x), A.k, lane);
+                tau = min(tau, pool[A.k - 1]);
+                c = 0;
+                __syncwarp();
+            }
+        }
+    }
+    if (c > 0) merge_ranked<EPL>(pool, buf, c, A.k, lane);
+    __syncwarp();
+}
+
 // The rows [row0, row1) of the group whose slabs and queries are in S; the pools hold the result.
 // Bounded by fp32 issue where rows are shared (8 queries) and by row bytes where they are not.
 template <int EPL, int G>
@@ -180,13 +297,13 @@ __device__ __forceinline__ void exact_scan(const ExactArgs& A, const ExactSmem<E
                 s1[g] = keep + __shfl_xor_sync(FULL, give, 4);
             }
             const int row = up4 ? rowB : rowA;
-            constexpr int NK = G >= 4 ? G / 4 : 1;
+            constexpr int NK = G / 4;
             float fin[NK];
             int g_lo = 0;
-            bool emits = row < row1;
-            if (G >= 4) {
+            const bool emits = row < row1;
+            {
                 const bool up2 = (sub & 2) != 0, up1 = (sub & 1) != 0;
-                float s2[G / 2 > 0 ? G / 2 : 1];
+                float s2[G / 2];
 #pragma unroll
                 for (int g = 0; g < G / 2; ++g) {
                     const float give = up2 ? s1[g] : s1[g + G / 2], keep = up2 ? s1[g + G / 2] : s1[g];
@@ -198,10 +315,6 @@ __device__ __forceinline__ void exact_scan(const ExactArgs& A, const ExactSmem<E
                     fin[g] = keep + __shfl_xor_sync(FULL, give, 1);
                 }
                 g_lo = (up2 ? G / 2 : 0) + (up1 ? G / 4 : 0);
-            } else {
-                float a = s1[0] + __shfl_xor_sync(FULL, s1[0], 2);
-                fin[0] = a + __shfl_xor_sync(FULL, a, 1);
-                emits = emits && (sub & 3) == 0;
             }
 #pragma unroll
             for (int x = 0; x < NK; ++x) {
@@ -260,7 +373,8 @@ __device__ __forceinline__ void exact_piece(const ExactArgs& A, const ExactSmem<
         S.tau[threadIdx.x] = A.bound && S.id[threadIdx.x] >= 0 ? (uint64_t)__ldcg(A.bound + S.id[threadIdx.x]) : KEY_EMPTY;
     }
     __syncthreads();
-    exact_scan<EPL, G>(A, S, row0, row1);
+    if constexpr (G == 1) exact_scan_one<EPL>(A, S, row0, row1);
+    else exact_scan<EPL, G>(A, S, row0, row1);
     if (pieces > 1) {
         if (warp < G) {
             const uint64_t tau = S.tau[warp];              // keys above it lose to another piece's
@@ -276,7 +390,10 @@ __device__ __forceinline__ void exact_piece(const ExactArgs& A, const ExactSmem<
         __syncthreads();
         if (!S.misc[0]) return;
         __threadfence();
-        if (warp < G && S.id[warp] >= 0) {
+        if constexpr (G == 1) {
+            // (this piece's own list is read back too: the merge drops what the pool holds)
+            if (warp == 0) exact_gather<EPL>(A, S, reinterpret_cast<const unsigned long long*>(A.part) + (size_t)first * A.k, pieces, lane);
+        } else if (warp < G && S.id[warp] >= 0) {
             uint64_t* const pool = S.pool + warp * 32 * EPL;
             uint64_t* const buf = S.buf + warp * EXACT_BUF;
             uint64_t tau = min((uint64_t)__ldcg(A.bound + S.id[warp]), pool[A.k - 1]);
