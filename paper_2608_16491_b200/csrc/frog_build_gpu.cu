@@ -10,8 +10,7 @@
 //   final        nearest list (m), temporary graph row (RNG selection, vector order) and the
 //                layer's ENC row (same selection in ascending fusion distance, Eq. 3).
 // The selection needs d(c, p) between candidates: the <= 64 candidate rows of an object are staged
-// in shared memory by bulk copies and all pair distances are accumulated there, so the selection
-// itself is a loop over shared-memory look-ups.
+// in shared memory by bulk copies.
 #include <algorithm>
 #include <cmath>
 #include <cstdio>
@@ -274,131 +273,169 @@ pool_kernel(const BuildArgs A) {
     }
 }
 
-// ---- selection: pair distances among the candidates in shared memory, then the RNG rule ------------
+// ---- selection: the RNG rule over the candidates of an object -----------------------------------------
+// The rule visits the candidates in order and keeps c iff d(u,c) < d(c,p) for every kept p.  Here a kept
+// candidate strikes out, in one step, every later one that it rules out: the next one to keep is the first
+// that nobody has struck.  The same set is kept, and of the K (K - 1) / 2 pair distances only those between
+// kept candidates and later ones still standing are computed (about a fifth of 2,016).  A team of 8 lanes
+// per pair; the candidate rows lie in shared memory (bulk copies), or are read from L2 where 64 of them do not fit.
+// Bounded by shared-memory reads of the rows.
 struct SelSmem {
-    uint64_t* keys;     // CAND
-    float* D;           // CAND x CAND, upper triangle used
-    float4* stage;      // CAND rows x STAGE_CHUNK bytes
+    uint64_t* keys;      // CAND
+    double* fus;         // CAND fusion distances
     uint64_t* bar;
-    int* ord;           // CAND: candidate indices in the visiting order
-    int* kept;          // CAND
-    int* pruned;        // CAND
-    double* fus;        // CAND fusion distances
+    uint32_t* dead;      // 3 x 2 words: positions struck out in a round (three rounds take turns)
+    uint8_t* ord;        // CAND: candidate at each position of the visiting order
+    uint8_t* list;       // CAND per warp: positions still standing
+    float4* rows;        // CAND rows (staged form)
 };
-constexpr size_t SEL_BYTES = CAND * 8 + CAND * CAND * 4 + (size_t)CAND * STAGE_CHUNK + 16 + 3 * CAND * 4 + CAND * 8;
+#ifndef SEL_MIN_WARPS
+#define SEL_MIN_WARPS 2
+#endif
+constexpr int SEL_MAX_WARPS = 8;
+constexpr size_t SEL_FIXED = CAND * 8 + CAND * 8 + 16 + 32 + CAND + SEL_MAX_WARPS * CAND;
+static_assert(SEL_FIXED % 16 == 0, "the rows follow at a 16-byte boundary");
+inline size_t sel_bytes(int d_pad, bool staged) { return SEL_FIXED + (staged ? (size_t)CAND * d_pad * 4 : 0); }
 
-// visits ord[0..K) in order, keeps c iff d(u,c) < d(c,p) for every kept p, stops at m, back-fills
-__device__ __forceinline__ int rng_rule(const SelSmem& S, int K, int m, int lane) {
-    int nk = 0, np = 0;
-    for (int t = 0; t < K && nk < m; ++t) {
-        const int ci = S.ord[t];
-        const float dc = key_dist2(S.keys[ci]);
-        bool bad = false;
-        if (lane < nk) {
-            const int p = S.kept[lane];
-            const float dcp = S.D[min(ci, p) * CAND + max(ci, p)];
-            bad = !(dc < dcp);
-        }
-        const bool reject = __any_sync(FULL, bad);
-        if (lane == 0) {
-            if (reject) S.pruned[np] = ci; else S.kept[nk] = ci;
-        }
-        if (reject) ++np; else ++nk;
+// Returns the kept positions (at most m) of ord[0..K) as a mask.  Called by the whole CTA.
+__device__ __forceinline__ uint64_t rng_keep(const SelSmem& S, const char* const rows, const uint64_t* keys, bool staged,
+                                             int row_bytes, int K, int m) {
+    const int lane = lane_id(), warp = threadIdx.x >> 5;
+    const int sub = lane & 7, team = threadIdx.x >> 3, teams = blockDim.x >> 3;
+    uint8_t* const list = S.list + warp * CAND;
+    auto row_of = [&](int c) {
+        return reinterpret_cast<const float4*>(rows + (size_t)(staged ? (uint32_t)c : key_rank(keys[c])) * (size_t)row_bytes);
+    };
+    uint64_t standing = K < 64 ? (1ull << K) - 1ull : ~0ull, kept = 0;
+    int nk = 0;
+    for (int round = 0; standing; ++round) {
+        const int t = __ffsll((long long)standing) - 1;
+        standing &= standing - 1ull;
+        kept |= 1ull << t;
+        if (++nk == m || standing == 0) break;
+        // positions still standing, in order (one copy per warp)
+        const uint32_t lo = (uint32_t)standing, hi = (uint32_t)(standing >> 32), lt = (1u << lane) - 1u;
+        if ((lo >> lane) & 1u) list[__popc(lo & lt)] = (uint8_t)lane;
+        if ((hi >> lane) & 1u) list[__popc(lo) + __popc(hi & lt)] = (uint8_t)(lane + 32);
+        uint32_t* const dead = S.dead + 2 * (round % 3);
+        if (threadIdx.x < 2) S.dead[2 * ((round + 1) % 3) + threadIdx.x] = 0u;
         __syncwarp();
+        const float4* const xc = row_of(S.ord[t]);
+        const int na = __popcll(standing);
+        for (int j0 = 0; j0 < na; j0 += 2 * teams) {            // uniform trip count: the sums need whole warps
+            const int j[2] = {j0 + team, j0 + team + teams};
+            int pos[2], cand[2];
+            const float4* x[2];
+            float d[2] = {0.f, 0.f};
+#pragma unroll
+            for (int i = 0; i < 2; ++i) {
+                pos[i] = list[min(j[i], na - 1)];
+                cand[i] = S.ord[pos[i]];
+                x[i] = row_of(cand[i]);
+            }
+            const bool two = j0 + teams < na;                    // CTA-uniform
+            for (int c0 = 0; c0 < row_bytes; c0 += STAGE_CHUNK) {
+                const int g_lo = c0 >> 4, g_n = min(STAGE_CHUNK, row_bytes - c0) >> 4;
+                float a0 = 0.f, a1 = 0.f;
+#pragma unroll
+                for (int c = 0; c < STAGE_CHUNK / 128; ++c) {
+                    const int g = sub + 8 * c;
+                    if (g < g_n) {
+                        const float4 p = xc[g_lo + g], y = x[0][g_lo + g];
+                        float w;
+                        w = p.x - y.x; a0 = fmaf(w, w, a0);
+                        w = p.y - y.y; a0 = fmaf(w, w, a0);
+                        w = p.z - y.z; a0 = fmaf(w, w, a0);
+                        w = p.w - y.w; a0 = fmaf(w, w, a0);
+                        if (two) {
+                            const float4 z = x[1][g_lo + g];
+                            w = p.x - z.x; a1 = fmaf(w, w, a1);
+                            w = p.y - z.y; a1 = fmaf(w, w, a1);
+                            w = p.z - z.z; a1 = fmaf(w, w, a1);
+                            w = p.w - z.w; a1 = fmaf(w, w, a1);
+                        }
+                    }
+                }
+                a0 += __shfl_xor_sync(FULL, a0, 4);
+                a1 += __shfl_xor_sync(FULL, a1, 4);
+                a0 += __shfl_xor_sync(FULL, a0, 2);
+                a1 += __shfl_xor_sync(FULL, a1, 2);
+                a0 += __shfl_xor_sync(FULL, a0, 1);
+                a1 += __shfl_xor_sync(FULL, a1, 1);
+                d[0] += a0;
+                d[1] += a1;
+            }
+#pragma unroll
+            for (int i = 0; i < 2; ++i)
+                if (sub == 0 && j[i] < na && !(key_dist2(keys[cand[i]]) < d[i])) atomicOr(dead + (pos[i] >> 5), 1u << (pos[i] & 31));
+        }
+        __syncthreads();
+        standing &= ~((uint64_t)dead[0] | (uint64_t)dead[1] << 32);
     }
-    for (int t = 0; t < np && nk < m; ++t) {
-        if (lane == 0) S.kept[nk] = S.pruned[t];
-        ++nk;
-    }
-    __syncwarp();
-    return nk;
+    // round 0 of the next call finds its words zero
+    __syncthreads();
+    if (threadIdx.x < 2) S.dead[threadIdx.x] = 0u;
+    __syncthreads();
+    return kept;
 }
 
-template <bool FINAL>
-__global__ void __launch_bounds__(32)
+template <bool FINAL, bool STAGED>
+__global__ void __launch_bounds__(SEL_MAX_WARPS * 32)
 select_kernel(const BuildArgs A) {
     extern __shared__ __align__(16) unsigned char smem_raw[];
     SelSmem S;
     S.keys = reinterpret_cast<uint64_t*>(smem_raw);
-    S.D = reinterpret_cast<float*>(S.keys + CAND);
-    S.stage = reinterpret_cast<float4*>(S.D + CAND * CAND);
-    S.bar = reinterpret_cast<uint64_t*>(reinterpret_cast<unsigned char*>(S.stage) + (size_t)CAND * STAGE_CHUNK);
-    S.ord = reinterpret_cast<int*>(S.bar + 2);
-    S.kept = S.ord + CAND;
-    S.pruned = S.kept + CAND;
-    S.fus = reinterpret_cast<double*>(S.pruned + CAND);
-    const int lane = lane_id();
-    const int team = lane >> 3, sub = lane & 7;
-    if (lane == 0) mbar_init(S.bar, 1u);
-    __syncwarp();
+    S.fus = reinterpret_cast<double*>(S.keys + CAND);
+    S.bar = reinterpret_cast<uint64_t*>(S.fus + CAND);
+    S.dead = reinterpret_cast<uint32_t*>(S.bar + 2);
+    S.ord = reinterpret_cast<uint8_t*>(S.dead + 8);
+    S.list = S.ord + CAND;
+    S.rows = reinterpret_cast<float4*>(smem_raw + SEL_FIXED);
+    const int lane = lane_id(), tid = threadIdx.x;
+    if (tid == 0) mbar_init(S.bar, 1u);
+    if (tid < 8) S.dead[tid] = 0u;
+    __syncthreads();
     uint32_t phase = 0;
     const uint64_t* cin = FINAL ? A.c2 : A.c1;
     const int row_bytes = A.d_pad * 4;
+    const char* const rows = STAGED ? reinterpret_cast<const char*>(S.rows) : reinterpret_cast<const char*>(A.V);
     for (int u = blockIdx.x; u < A.n; u += gridDim.x) {
-        const uint64_t k0 = cin[(size_t)u * CAND + lane], k1 = cin[(size_t)u * CAND + lane + 32];
-        S.keys[lane] = k0;
-        S.keys[lane + 32] = k1;
+        const uint64_t k0 = cin[(size_t)u * CAND + lane], k1 = cin[(size_t)u * CAND + lane + 32];   // every warp, for K
         const int K = __popc(__ballot_sync(FULL, k0 != KEY_EMPTY)) + __popc(__ballot_sync(FULL, k1 != KEY_EMPTY));
-        for (int i = lane; i < CAND * CAND; i += 32) S.D[i] = 0.f;
-        __syncwarp();
-        // pair distances, accumulated over column chunks of the rows
-        for (int c0 = 0; c0 < row_bytes; c0 += STAGE_CHUNK) {
-            const int cbytes = min(STAGE_CHUNK, row_bytes - c0);
-            __syncwarp();
-            if (lane == 0 && !A.skip_copies) mbar_expect_tx(S.bar, (uint32_t)(K * cbytes));
-            __syncwarp();
-#pragma unroll
-            for (int rr = 0; rr < 2; ++rr) {
-                const int r = lane + 32 * rr;
-                if (r < K && !A.skip_copies)
-                    tma_load_1d(reinterpret_cast<char*>(S.stage) + (size_t)r * STAGE_CHUNK,
-                                reinterpret_cast<const char*>(A.V) + (size_t)key_rank(S.keys[r]) * row_bytes + c0,
-                                (uint32_t)cbytes, S.bar);
-            }
+        if (tid < 32) {
+            S.keys[lane] = k0;
+            S.keys[lane + 32] = k1;
+            S.ord[lane] = (uint8_t)lane;                           // vector-distance order: the keys are ascending
+            S.ord[lane + 32] = (uint8_t)(lane + 32);
+            if (STAGED && lane == 0 && !A.skip_copies) mbar_expect_tx(S.bar, (uint32_t)(K * row_bytes));
+        }
+        __syncthreads();
+        if (STAGED) {
+            for (int r = tid; r < K; r += blockDim.x)
+                if (!A.skip_copies)
+                    tma_load_1d(reinterpret_cast<char*>(S.rows) + (size_t)r * row_bytes,
+                                reinterpret_cast<const char*>(A.V) + (size_t)key_rank(S.keys[r]) * row_bytes, (uint32_t)row_bytes, S.bar);
             wait_copies(A, S.bar, phase);
             phase ^= 1u;
-            const int g_n = cbytes >> 4;
-            for (int i = 0; i + 1 < K; ++i) {
-                const float4* xi = S.stage + i * (STAGE_CHUNK / 16);
-                for (int j0 = i + 1; j0 < K; j0 += 4) {
-                    const int j = j0 + team;
-                    float acc = 0.f;
-                    if (j < K) {
-                        const float4* xj = S.stage + j * (STAGE_CHUNK / 16);
-                        for (int g = sub; g < g_n; g += 8) {
-                            const float4 a = xi[g], b = xj[g];
-                            float t;
-                            t = a.x - b.x; acc = fmaf(t, t, acc);
-                            t = a.y - b.y; acc = fmaf(t, t, acc);
-                            t = a.z - b.z; acc = fmaf(t, t, acc);
-                            t = a.w - b.w; acc = fmaf(t, t, acc);
-                        }
-                    }
-                    acc += __shfl_xor_sync(FULL, acc, 4);
-                    acc += __shfl_xor_sync(FULL, acc, 2);
-                    acc += __shfl_xor_sync(FULL, acc, 1);
-                    if (j < K && sub == 0) S.D[i * CAND + j] += acc;
-                }
-            }
         }
-        __syncwarp();
-        // temporary graph row: RNG rule in vector-distance order (the keys are already ascending)
-        S.ord[lane] = lane;
-        S.ord[lane + 32] = lane + 32;
-        __syncwarp();
-        int nk = rng_rule(S, K, A.m, lane);
+        // temporary graph row: kept candidates in vector-distance order, then the others up to m
+        const uint64_t kept = rng_keep(S, rows, S.keys, STAGED, row_bytes, K, A.m);
+        const int nk = __popcll(kept);
         uint32_t* grow = (FINAL ? A.pg_nxt : A.fwd) + (size_t)u * A.m;
-        if (lane < A.m) grow[lane] = lane < nk ? key_rank(S.keys[S.kept[lane]]) : BOT;
+        for (int i = tid; i < CAND; i += blockDim.x) {
+            const uint64_t below = (1ull << i) - 1ull;
+            const int at = (kept >> i) & 1ull ? __popcll(kept & below) : nk + __popcll(~kept & below);
+            if (i < K && at < A.m) grow[at] = key_rank(S.keys[i]);
+            if (i >= K && i < A.m) grow[i] = BOT;
+        }
         if (FINAL) {
-            if (lane < A.m) {
-                const bool has = lane < K;
-                A.ann_nxt[(size_t)u * A.m + lane] = has ? key_rank(S.keys[lane]) : BOT;
-                A.pd_nxt[(size_t)u * A.m + lane] = has ? key_dist2(S.keys[lane]) : 0.f;
-            }
-            // ENC row: the same rule with the candidates in ascending fusion distance (Eq. 3)
-#pragma unroll
-            for (int rr = 0; rr < 2; ++rr) {
-                const int i = lane + 32 * rr;
+            for (int i = tid; i < CAND; i += blockDim.x) {
+                if (i < A.m) {
+                    const bool has = i < K;
+                    A.ann_nxt[(size_t)u * A.m + i] = has ? key_rank(S.keys[i]) : BOT;
+                    A.pd_nxt[(size_t)u * A.m + i] = has ? key_dist2(S.keys[i]) : 0.f;
+                }
+                // ENC row: the same rule with the candidates in ascending fusion distance (Eq. 3)
                 if (i < K) {
                     const double dv = sqrt((double)key_dist2(S.keys[i]));
                     const double da = fabs((double)u - (double)key_rank(S.keys[i])) * A.inv_span;
@@ -406,48 +443,33 @@ select_kernel(const BuildArgs A) {
                     S.fus[i] = dv * (1.0 - A.beta * (1.0 - za));
                 }
             }
-            __syncwarp();
-#pragma unroll
-            for (int rr = 0; rr < 2; ++rr) {
-                const int i = lane + 32 * rr;
-                if (i < K) {
-                    const double fi = S.fus[i];
-                    const uint32_t ri = key_rank(S.keys[i]);
-                    int pos = 0;
-                    for (int j = 0; j < K; ++j) {
-                        const double fj = S.fus[j];
-                        pos += (fj < fi || (fj == fi && key_rank(S.keys[j]) < ri)) ? 1 : 0;
-                    }
-                    S.ord[pos] = i;
+            __syncthreads();
+            for (int i = tid; i < K; i += blockDim.x) {
+                const double fi = S.fus[i];
+                const uint32_t ri = key_rank(S.keys[i]);
+                int pos = 0;
+                for (int j = 0; j < K; ++j) {
+                    const double fj = S.fus[j];
+                    pos += (fj < fi || (fj == fi && key_rank(S.keys[j]) < ri)) ? 1 : 0;
                 }
+                S.ord[pos] = (uint8_t)i;
             }
-            __syncwarp();
-            if (A.fusion_nearest) {
-                nk = min(K, A.m);                              // the paper's rule: the m fusion-nearest
-                if (lane < nk) S.kept[lane] = S.ord[lane];
-                __syncwarp();
-            } else {
-                nk = rng_rule(S, K, A.m, lane);
+            __syncthreads();
+            const uint64_t all = K < 64 ? (1ull << K) - 1ull : ~0ull;
+            uint64_t enc = A.fusion_nearest ? 0ull : rng_keep(S, rows, S.keys, STAGED, row_bytes, K, A.m);   // 0: the m fusion-nearest
+            uint64_t spare = all & ~enc;
+            for (int x = __popcll(enc); x < A.m && spare; ++x) {
+                enc |= spare & (0ull - spare);
+                spare &= spare - 1ull;
             }
-            // store the kept candidates in ascending fusion distance (their position in ord)
+            // the chosen candidates in ascending fusion distance
             uint32_t* erow = A.enc + ((size_t)u * A.H + A.h) * A.m;
-            int kpos = 0x7FFFFFFF;
-            uint32_t krank = BOT;
-            if (lane < nk) {
-                const int ci = S.kept[lane];
-                krank = key_rank(S.keys[ci]);
-                for (int t = 0; t < K; ++t) if (S.ord[t] == ci) { kpos = t; break; }
+            for (int i = tid; i < CAND; i += blockDim.x) {
+                if ((enc >> i) & 1ull) erow[__popcll(enc & ((1ull << i) - 1ull))] = key_rank(S.keys[S.ord[i]]);
+                if (i >= __popcll(enc) && i < A.m) erow[i] = BOT;
             }
-            int slot = 0;
-            for (int j = 0; j < nk; ++j) {
-                const int pj = __shfl_sync(FULL, kpos, j);
-                slot += (pj < kpos) ? 1 : 0;
-            }
-            if (lane < A.m) erow[lane] = BOT;
-            __syncwarp();
-            if (lane < nk) erow[slot] = krank;
         }
-        __syncwarp();
+        __syncthreads();                                           // everyone is done with the rows and keys
     }
 }
 
@@ -571,12 +593,20 @@ extern "C" int frog_index_build_gpu(const float* vectors, const int32_t* attrs, 
     void (*search_fn)(const BuildArgs) = spool_slots == 32 ? sibling_search_kernel<1>
                                        : spool_slots == 64 ? sibling_search_kernel<2>
                                        : spool_slots == 128 ? sibling_search_kernel<4> : sibling_search_kernel<8>;
-    if (smem_search > 227 * 1024 || SEL_BYTES > 227 * 1024) return FROG_ERR_UNSUPPORTED;
+    if (smem_search > 227 * 1024) return FROG_ERR_UNSUPPORTED;
+    // the selection stages all 64 rows where they fit; about 16 warps per SM share its shared memory, and a CTA
+    // is given more of them the fewer CTAs that leaves room for
+    const bool staged = sel_bytes(d_pad, true) <= 227 * 1024;
+    const size_t smem_sel = sel_bytes(d_pad, staged);
+    const int sel_ctas = std::max<int>(1, (int)(227 * 1024 / (smem_sel + 1024)));
+    const int sel_warps = std::min(SEL_MAX_WARPS, std::max(SEL_MIN_WARPS, 16 / sel_ctas));
+    void (*sel0)(const BuildArgs) = staged ? select_kernel<false, true> : select_kernel<false, false>;
+    void (*sel1)(const BuildArgs) = staged ? select_kernel<true, true> : select_kernel<true, false>;
     FROG_CUDA_TRY(cudaFuncSetAttribute((const void*)leaf_cand_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem_plain));
     FROG_CUDA_TRY(cudaFuncSetAttribute((const void*)pool_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem_plain));
     FROG_CUDA_TRY(cudaFuncSetAttribute((const void*)search_fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem_search));
-    FROG_CUDA_TRY(cudaFuncSetAttribute((const void*)select_kernel<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)SEL_BYTES));
-    FROG_CUDA_TRY(cudaFuncSetAttribute((const void*)select_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)SEL_BYTES));
+    FROG_CUDA_TRY(cudaFuncSetAttribute((const void*)sel0, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem_sel));
+    FROG_CUDA_TRY(cudaFuncSetAttribute((const void*)sel1, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem_sel));
     auto grid_for = [&](const void* fn, int threads, size_t smem, int per_cta) {
         int per_sm = 1;
         cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, fn, threads, smem);
@@ -588,8 +618,8 @@ extern "C" int frog_index_build_gpu(const float* vectors, const int32_t* attrs, 
     const int g_plain = grid_for((const void*)leaf_cand_kernel, BWARPS * 32, smem_plain, BWARPS);
     const int g_pool = grid_for((const void*)pool_kernel, BWARPS * 32, smem_plain, BWARPS);
     const int g_search = grid_for((const void*)search_fn, BWARPS * 32, smem_search, BWARPS);
-    const int g_sel0 = grid_for((const void*)select_kernel<false>, 32, SEL_BYTES, 1);
-    const int g_sel1 = grid_for((const void*)select_kernel<true>, 32, SEL_BYTES, 1);
+    const int g_sel0 = grid_for((const void*)sel0, sel_warps * 32, smem_sel, 1);
+    const int g_sel1 = grid_for((const void*)sel1, sel_warps * 32, smem_sel, 1);
     A.bitmap_words = (((size_t)n + 31) / 32 + 31) & ~(size_t)31;
     if (H > 1 && (rc = buf.alloc(&A.bitmap, (size_t)g_search * BWARPS * A.bitmap_words))) return rc;
 
@@ -599,7 +629,7 @@ extern "C" int frog_index_build_gpu(const float* vectors, const int32_t* attrs, 
         A.h = h;
         if (h == H - 1) leaf_cand_kernel<<<g_plain, BWARPS * 32, smem_plain>>>(A);
         else search_fn<<<g_search, BWARPS * 32, smem_search>>>(A);
-        select_kernel<false><<<g_sel0, 32, SEL_BYTES>>>(A);
+        sel0<<<g_sel0, sel_warps * 32, smem_sel>>>(A);
         FROG_CUDA_TRY(cudaMemsetAsync(A.rev_cnt, 0, ((size_t)n + 1) * 4));
         FROG_CUDA_TRY(cudaMemsetAsync(A.rev_cur, 0, (size_t)n * 4));
         if (reverse_edges) {
@@ -610,7 +640,7 @@ extern "C" int frog_index_build_gpu(const float* vectors, const int32_t* attrs, 
             FROG_CUDA_TRY(cudaMemsetAsync(A.rev_off, 0, ((size_t)n + 1) * 4));      // no incoming sources
         }
         pool_kernel<<<g_pool, BWARPS * 32, smem_plain>>>(A);
-        select_kernel<true><<<g_sel1, 32, SEL_BYTES>>>(A);
+        sel1<<<g_sel1, sel_warps * 32, smem_sel>>>(A);
         FROG_CUDA_TRY(cudaGetLastError());
         std::swap(A.ann_cur, A.ann_nxt);
         std::swap(A.pd_cur, A.pd_nxt);
