@@ -57,8 +57,6 @@ struct BuildArgs {
     uint32_t* rev_off;       // n + 1
     uint32_t* rev_cur;       // n
     uint32_t* rev_src;       // n x m
-    uint32_t* bitmap;        // visited slabs of the sibling searches
-    size_t bitmap_words;
     int h;                   // layer under construction
     int fusion_nearest;      // ENCs = the m fusion-nearest candidates (no RNG rule on them)
     int wait_limit;          // polls a wait on a bulk copy may take before giving up
@@ -76,19 +74,23 @@ struct BWarp {
     float4* q;
     uint64_t* pool;      // CAND keys
     uint64_t* spool;     // search pool (sibling search only)
+    uint64_t* keys;      // keys of one expansion (sibling search only)
     uint32_t* cand;
     uint64_t* bar;
-    float4* stage;
+    float4* stage;       // (sibling search: its table of evaluated ranks)
 };
+constexpr int SEEN_BITS = 10;
+static_assert((4 << SEEN_BITS) == STAGE8, "the table takes the place of the stage buffer");
 __host__ __device__ inline size_t bwarp_bytes(int d_pad, int spool_slots) {
-    return (size_t)d_pad * 4 + CAND * 8 + (size_t)spool_slots * 8 + 32 * 4 + 16 + STAGE8;
+    return (size_t)d_pad * 4 + CAND * 8 + (size_t)spool_slots * 8 + (spool_slots ? 32 * 8 : 0) + 32 * 4 + 16 + STAGE8;
 }
 __device__ __forceinline__ BWarp bwarp_carve(unsigned char* base, int d_pad, int spool_slots) {
     BWarp W;
     W.q = reinterpret_cast<float4*>(base);
     W.pool = reinterpret_cast<uint64_t*>(base + (size_t)d_pad * 4);
     W.spool = W.pool + CAND;
-    W.cand = reinterpret_cast<uint32_t*>(W.spool + spool_slots);
+    W.keys = W.spool + spool_slots;
+    W.cand = reinterpret_cast<uint32_t*>(W.keys + (spool_slots ? 32 : 0));
     W.bar = reinterpret_cast<uint64_t*>(W.cand + 32);
     W.stage = reinterpret_cast<float4*>(W.bar + 2);
     return W;
@@ -144,19 +146,34 @@ leaf_cand_kernel(const BuildArgs A) {
     }
 }
 
-// ---- inner layer: own nearest list + greedy search in the sibling's graph (Alg. 1) ---------------
+// first pool entry after `from` that is neither expanded nor empty (0xFFFF: none)
 template <int EPL>
-__global__ void __launch_bounds__(BWARPS * 32)
+__device__ __forceinline__ uint32_t next_open(const uint64_t* pool, int from, int lane) {
+    for (int e = from >> 5; e < EPL; ++e) {
+        const uint32_t lo = reinterpret_cast<const uint32_t*>(pool + lane + 32 * e)[0];     // flag bit; empty keys have it set
+        const uint32_t M = __ballot_sync(FULL, !(lo & 1u));
+        if (M) return (uint32_t)(32 * e + __ffs(M) - 1);
+    }
+    return 0xFFFFu;
+}
+
+// ---- inner layer: own nearest list + greedy search in the sibling's graph (Alg. 1) ---------------
+// One warp per object, SM full of warps: bounded by instruction issue (65 % of the slots).  Rows are read into
+// registers (eight in flight per warp), only keys that a full pool does not reject are merged, by rank, and the
+// visited set is a table of 1,024 recent ranks in shared memory.  Forgetting is harmless: a vertex evaluated
+// again is in the pool, where the merge drops it and the patience rule does not count it, or lies beyond the
+// worst of the full pool.  100,000 objects of 384 bytes, ten layers: 60 ms (76.8 with rows staged by bulk copies,
+// a bitmap of atomics in L2 and the key-by-key merge; 69 with every new key merged).
+template <int EPL>
+__global__ void __launch_bounds__(BWARPS * 32, 10)      // 96 registers: 60 ms; 72: 68 ms
 sibling_search_kernel(const BuildArgs A) {
     extern __shared__ __align__(16) unsigned char smem_raw[];
     constexpr int SPOOL = 32 * EPL;
     const int lane = lane_id(), warp = threadIdx.x >> 5;
     const BWarp W = bwarp_carve(smem_raw + bwarp_bytes(A.d_pad, SPOOL) * warp, A.d_pad, SPOOL);
-    if (lane == 0) mbar_init(W.bar, 1u);
-    __syncwarp();
-    uint32_t phase = 0;
     const uint32_t lt_mask = (1u << lane) - 1u;
-    uint32_t* bitmap = A.bitmap + (size_t)(blockIdx.x * BWARPS + warp) * A.bitmap_words;
+    uint32_t* const seen = reinterpret_cast<uint32_t*>(W.stage);
+    auto slot_of = [&](uint32_t v) -> uint32_t* { return seen + ((v * 0x9E3779B1u) >> (32 - SEEN_BITS)); };
     const int nwarps = gridDim.x * BWARPS;
     for (int u = blockIdx.x * BWARPS + warp; u < A.n; u += nwarps) {
         int L, R;
@@ -178,16 +195,17 @@ sibling_search_kernel(const BuildArgs A) {
             __syncwarp();
         }
         if (sL <= sR) {
-            for (int i = (sL >> 5) + lane; i <= (sR >> 5); i += 32) bitmap[i] = 0u;
+            const uint4 e4 = make_uint4(BOT, BOT, BOT, BOT);
+            for (int i = lane; i < (1 << SEEN_BITS) / 4; i += 32) reinterpret_cast<uint4*>(seen)[i] = e4;
             __syncwarp();
             const uint32_t ep = (uint32_t)(sL + ((sR - sL) >> 1));            // entry point: middle rank
+            const float d2 = batch_dist2<4>(A.V, A.d_pad, W.q, ep, 1, lane);
             if (lane == 0) {
-                atomicOr(bitmap + (ep >> 5), 1u << (ep & 31));
-                W.cand[0] = ep;
+                *slot_of(ep) = ep;
+                W.keys[0] = make_key(d2, ep, 0u);
             }
             __syncwarp();
-            uint64_t key = cand_keys(A, W, 1, 0u, phase, lane);
-            int first = (int)(merge_batch<EPL>(W.spool, key, A.ef_c, lane) & 0xFFFF);
+            int first = (int)merge_ranked<EPL>(W.spool, W.keys, 1, A.ef_c, lane);
             int pat = A.patience;
             for (int it = 0; first < A.ef_c && it < 4 * A.ef_c; ++it) {
                 const uint32_t x = key_rank(W.spool[first]);
@@ -198,21 +216,36 @@ sibling_search_kernel(const BuildArgs A) {
                 if (lane < A.m) v = __ldg(A.pg_cur + (size_t)x * A.m + lane);
                 bool keep = false;
                 if (v != BOT) {
-                    const uint32_t bit = 1u << (v & 31);
-                    keep = (atomicOr(bitmap + (v >> 5), bit) & bit) == 0;
+                    uint32_t* const slot = slot_of(v);
+                    keep = *slot != v;
+                    if (keep) *slot = v;
                 }
                 const uint32_t M = __ballot_sync(FULL, keep);
                 if (keep) W.cand[__popc(M & lt_mask)] = v;
                 __syncwarp();
-                key = cand_keys(A, W, __popc(M), 0u, phase, lane);
-                const uint64_t best = warp_min_key(key);
-                const bool improved = (best | 1ull) < (mth | 1ull);            // something enters the top m
-                first = (int)(merge_batch<EPL>(W.spool, key, A.ef_c, lane) & 0xFFFF);
+                const int ns = __popc(M);
+                uint64_t key = KEY_EMPTY;
+                if (ns > 0) {
+                    const uint32_t id = W.cand[lane < ns ? lane : 0];
+                    const float d2 = batch_dist2<4>(A.V, A.d_pad, W.q, id, ns, lane);
+                    if (lane < ns) key = make_key(d2, id, 0u);
+                }
+                // only what a full pool does not reject goes through the merge
+                const bool close = (key | 1ull) < (W.spool[A.ef_c - 1] | 1ull);
+                const uint32_t C = __ballot_sync(FULL, close);
+                if (close) W.keys[__popc(C & lt_mask)] = key;
+                __syncwarp();
+                bool entered = false;
+                if (C) first = (int)merge_ranked<EPL>(W.spool, W.keys, __popc(C), A.ef_c, lane, &entered);
+                else first = (int)next_open<EPL>(W.spool, first, lane);
+                // something enters the top m
+                const bool improved = __any_sync(FULL, entered && (W.keys[lane] | 1ull) < (mth | 1ull));
+                __syncwarp();
                 if (improved) pat = A.patience;
                 else if (--pat <= 0) break;
             }
             __syncwarp();
-            key = KEY_EMPTY;
+            uint64_t key = KEY_EMPTY;
             if (lane < A.m) {
                 key = W.spool[lane];
                 if (key != KEY_EMPTY) key |= 1ull;
@@ -279,7 +312,8 @@ pool_kernel(const BuildArgs A) {
 // that nobody has struck.  The same set is kept, and of the K (K - 1) / 2 pair distances only those between
 // kept candidates and later ones still standing are computed (about a fifth of 2,016).  A team of 8 lanes
 // per pair; the candidate rows lie in shared memory (bulk copies), or are read from L2 where 64 of them do not fit.
-// Bounded by shared-memory reads of the rows.
+// Bounded by shared-memory reads of the rows.  100,000 objects of 384 bytes, eleven layers, both selections: 38 ms
+// (212 with one warp per object and all pair distances).
 struct SelSmem {
     uint64_t* keys;      // CAND
     double* fus;         // CAND fusion distances
@@ -289,10 +323,7 @@ struct SelSmem {
     uint8_t* list;       // CAND per warp: positions still standing
     float4* rows;        // CAND rows (staged form)
 };
-#ifndef SEL_MIN_WARPS
-#define SEL_MIN_WARPS 2
-#endif
-constexpr int SEL_MAX_WARPS = 8;
+constexpr int SEL_MIN_WARPS = 2, SEL_MAX_WARPS = 8;      // 384-byte rows: 4 warps are 11 % slower than 2
 constexpr size_t SEL_FIXED = CAND * 8 + CAND * 8 + 16 + 32 + CAND + SEL_MAX_WARPS * CAND;
 static_assert(SEL_FIXED % 16 == 0, "the rows follow at a 16-byte boundary");
 inline size_t sel_bytes(int d_pad, bool staged) { return SEL_FIXED + (staged ? (size_t)CAND * d_pad * 4 : 0); }
@@ -620,8 +651,6 @@ extern "C" int frog_index_build_gpu(const float* vectors, const int32_t* attrs, 
     const int g_search = grid_for((const void*)search_fn, BWARPS * 32, smem_search, BWARPS);
     const int g_sel0 = grid_for((const void*)sel0, sel_warps * 32, smem_sel, 1);
     const int g_sel1 = grid_for((const void*)sel1, sel_warps * 32, smem_sel, 1);
-    A.bitmap_words = (((size_t)n + 31) / 32 + 31) & ~(size_t)31;
-    if (H > 1 && (rc = buf.alloc(&A.bitmap, (size_t)g_search * BWARPS * A.bitmap_words))) return rc;
 
     const size_t edges = nm;
     const int eb = 256, eg = (int)((edges + eb - 1) / eb);

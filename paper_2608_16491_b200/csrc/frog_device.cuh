@@ -621,34 +621,41 @@ __device__ __forceinline__ uint32_t merge_batch(uint64_t* pool, uint64_t my_key,
 // positions of the new keys, as one bit mask per 32 positions, tell each position whether it takes a new
 // key or which old one moves there.  The cost hardly depends on the pool size and little on n, and the
 // dependent chain has no shuffle or vote per key.
-template <int EPL>
-__device__ __forceinline__ uint32_t merge_ranked(uint64_t* pool, const uint64_t* keys, int n, int ef_s, int lane) {
+// `entered` tells a lane whether its key is in the pool now and was not before.
+// UNIQUE: the caller guarantees that there are no copies.
+template <int EPL, bool UNIQUE = false>
+__device__ __forceinline__ uint32_t merge_ranked(uint64_t* pool, const uint64_t* keys, int n, int ef_s, int lane,
+                                                 bool* entered = nullptr) {
     constexpr int POOL = 32 * EPL;
     const uint32_t lt_mask = (1u << lane) - 1u;
     uint64_t key = lane < n ? keys[lane] : KEY_EMPTY;
     const uint64_t mk = key | 1ull;
     bool in = mk < (pool[ef_s - 1] | 1ull);             // a full pool rejects what is not better than its worst
     int p = 0;                                          // pool keys below mk (at most ef_s - 1 if it enters)
+    constexpr int TOP = POOL > 256 ? 256 : POOL > 128 ? 128 : POOL / 2;
 #pragma unroll
-    for (int step = POOL / 2; step > 0; step >>= 1)
-        if ((pool[p + step - 1] | 1ull) < mk) p += step;
-    in = in && (pool[p] | 1ull) != mk;                  // the pool holds it already
+    for (int step = TOP; step > 0; step >>= 1)
+        if (((POOL & (POOL - 1)) == 0 || p + step <= POOL) && (pool[p + step - 1] | 1ull) < mk) p += step;
+    if (!UNIQUE) in = in && (pool[p] | 1ull) != mk;     // the pool holds it already
     int r = 0;
     bool copy = false;
 #pragma unroll 4
     for (int j = 0; j < n; ++j) {
         const uint64_t x = keys[j] | 1ull;
         r += x < mk ? 1 : 0;
-        copy = copy || (x == mk && j < lane);
+        if (!UNIQUE) copy = copy || (x == mk && j < lane);
     }
-    in = in && !copy;
-    // keys that lie below this one but do not enter: copies only (what the pool rejects lies above)
-    for (uint32_t out = __ballot_sync(FULL, !in && lane < n); out; out &= out - 1) {
-        const uint64_t x = keys[__ffs(out) - 1] | 1ull;
-        r -= x < mk ? 1 : 0;
+    if (!UNIQUE) {
+        in = in && !copy;
+        // keys that lie below this one but do not enter: copies only (what the pool rejects lies above)
+        for (uint32_t out = __ballot_sync(FULL, !in && lane < n); out; out &= out - 1) {
+            const uint64_t x = keys[__ffs(out) - 1] | 1ull;
+            r -= x < mk ? 1 : 0;
+        }
     }
     const int f = p + r;
     in = in && f < ef_s;
+    if (entered) *entered = in;
     int below = 0, m1 = NO_POS;
     uint64_t take[EPL];
     int shift[EPL];
@@ -675,14 +682,6 @@ __device__ __forceinline__ uint32_t merge_ranked(uint64_t* pool, const uint64_t*
     }
     __syncwarp();
     return first_pos(m1);
-}
-
-// smallest key of the warp under the order key | 1 (KEY_EMPTY if no lane has one)
-__device__ __forceinline__ uint64_t warp_min_key(uint64_t key) {
-    const uint32_t hi = (uint32_t)(key >> 32), lo = (uint32_t)key | 1u;
-    const uint32_t mhi = __reduce_min_sync(FULL, hi);
-    const uint32_t mlo = __reduce_min_sync(FULL, hi == mhi ? lo : 0xFFFFFFFFu);
-    return ((uint64_t)mhi << 32) | mlo;
 }
 
 // entry point j of a query range: stateless mixer of (seed, l_q, r_q, j), top 32 bits scaled
