@@ -19,6 +19,8 @@
 #include <numeric>
 #include <vector>
 
+#include <sys/stat.h>
+
 #include <thrust/execution_policy.h>
 #include <thrust/scan.h>
 
@@ -504,6 +506,16 @@ select_kernel(const BuildArgs A) {
     }
 }
 
+// rows of the caller's array to their places in rank order, zero-padded to d_pad
+__global__ void rank_rows_kernel(const float* __restrict__ raw, const int32_t* __restrict__ ranks, int d, int d_pad, size_t elems,
+                                 float* __restrict__ out) {
+    for (size_t i = (size_t)blockIdx.x * blockDim.x + threadIdx.x; i < elems; i += (size_t)gridDim.x * blockDim.x) {
+        const size_t r = i / d_pad;
+        const int c = (int)(i - r * d_pad);
+        out[(size_t)ranks[r] * d_pad + c] = c < d ? raw[r * d + c] : 0.f;
+    }
+}
+
 // ---- host side ------------------------------------------------------------------------------------
 bool write_all(FILE* f, const void* p, size_t bytes) {
     const char* c = static_cast<const char*>(p);
@@ -583,13 +595,7 @@ extern "C" int frog_index_build_gpu(const float* vectors, const int32_t* attrs, 
     std::iota(rank2id.begin(), rank2id.end(), 0);
     std::stable_sort(rank2id.begin(), rank2id.end(), [&](int32_t a, int32_t b) { return attrs[a] < attrs[b]; });
     std::vector<int32_t> sorted_attr((size_t)n);
-    std::unique_ptr<float[]> Vh(new (std::nothrow) float[(size_t)n * d_pad]);
-    if (!Vh) return FROG_ERR_NOMEM;
-    for (int64_t r = 0; r < n; ++r) {
-        sorted_attr[r] = attrs[rank2id[r]];
-        std::memcpy(Vh.get() + r * d_pad, vectors + (int64_t)rank2id[r] * d, sizeof(float) * d);
-        for (int j = d; j < d_pad; ++j) Vh[r * d_pad + j] = 0.f;
-    }
+    for (int64_t r = 0; r < n; ++r) sorted_attr[r] = attrs[rank2id[r]];
 
     DeviceBuffers buf;
     BuildArgs A{};
@@ -612,7 +618,23 @@ extern "C" int frog_index_build_gpu(const float* vectors, const int32_t* attrs, 
     // and neither arms the barriers nor issues a copy, so that the give-up path runs with nothing in flight
     A.wait_limit = (P.reserved >> 16) ? (P.reserved >> 16) : (1 << 22);
     A.skip_copies = (P.reserved >> 16) ? 1 : 0;
-    FROG_CUDA_TRY(cudaMemcpy(dV, Vh.get(), (size_t)n * d_pad * 4, cudaMemcpyHostToDevice));
+    {   // rows in rank order, padded, are put together on the device, from slabs of the caller's array of at most 256 MB
+        DeviceBuffers once;
+        float* raw = nullptr;
+        int32_t* ranks = nullptr;
+        const size_t slab = std::min<size_t>((size_t)n, std::max<size_t>(((size_t)64 << 20) / d, 1));
+        if ((rc = once.alloc(&raw, slab * d)) || (rc = once.alloc(&ranks, (size_t)n))) return rc;
+        std::vector<int32_t> rank_of((size_t)n);
+        for (int r = 0; r < n; ++r) rank_of[rank2id[r]] = r;
+        FROG_CUDA_TRY(cudaMemcpy(ranks, rank_of.data(), (size_t)n * 4, cudaMemcpyHostToDevice));
+        for (size_t i0 = 0; i0 < (size_t)n; i0 += slab) {
+            const size_t rows = std::min(slab, (size_t)n - i0), elems = rows * d_pad;
+            FROG_CUDA_TRY(cudaMemcpy(raw, vectors + i0 * d, rows * d * 4, cudaMemcpyHostToDevice));
+            rank_rows_kernel<<<(unsigned)std::min<size_t>((elems + 255) / 256, (size_t)prop.multiProcessorCount * 32), 256>>>(raw, ranks + i0, d, d_pad, elems, dV);
+            FROG_CUDA_TRY(cudaGetLastError());
+        }
+        FROG_CUDA_TRY(cudaDeviceSynchronize());
+    }
     A.V = dV;
     A.n = n; A.d_pad = d_pad; A.H = H; A.m = m; A.ef_c = P.ef_c; A.patience = P.patience;
     A.beta = P.beta; A.gamma = P.gamma; A.inv_span = n > 1 ? 1.0 / (double)(n - 1) : 0.0;
@@ -682,10 +704,6 @@ extern "C" int frog_index_build_gpu(const float* vectors, const int32_t* attrs, 
         if (failed) return FROG_ERR_CUDA;      // a bulk copy never completed: no file is written
     }
 
-    std::unique_ptr<uint32_t[]> ench(new (std::nothrow) uint32_t[nm * H]);
-    if (!ench) return FROG_ERR_NOMEM;
-    FROG_CUDA_TRY(cudaMemcpy(ench.get(), A.enc, nm * H * 4, cudaMemcpyDeviceToHost));
-
     // the index file (same layout as the host builder writes)
     unsigned char hdr[256];
     std::memset(hdr, 0, sizeof(hdr));
@@ -713,9 +731,27 @@ extern "C" int frog_index_build_gpu(const float* vectors, const int32_t* attrs, 
     pos += nn * 4;
     ok = ok && pad_to(f, pos, off_r2i) && write_all(f, rank2id.data(), (size_t)n * 4);
     pos += nn * 4;
-    ok = ok && pad_to(f, pos, off_vec) && write_all(f, Vh.get(), (size_t)n * d_pad * 4);
-    pos += nn * d_pad * 4;
-    ok = ok && pad_to(f, pos, off_enc) && write_all(f, ench.get(), nm * H * 4);
-    if (fclose(f) != 0) ok = false;
-    return ok ? FROG_OK : FROG_ERR_IO;
+    ok = ok && pad_to(f, pos, off_vec) && fflush(f) == 0;
+    rc = ok ? FROG_OK : FROG_ERR_IO;
+    struct stat file;
+    if (ok && fstat(fileno(f), &file) == 0 && S_ISREG(file.st_mode)) {
+        // (the gap before the ENC array reads as zeros)
+        const froghost::FileSection sections[2] = {{off_vec, dV, (size_t)n * d_pad * 4}, {off_enc, A.enc, nm * H * 4}};
+        rc = froghost::transfer_sections(fileno(f), device, sections, 2, false);
+    } else if (ok) {
+        // not a file one can write out of order (a pipe): both arrays through host memory, in order
+        std::unique_ptr<char[]> host(new (std::nothrow) char[std::max((size_t)n * d_pad, nm * H) * 4]);
+        if (!host) rc = FROG_ERR_NOMEM;
+        auto copy = [&](const void* dev, size_t bytes) {
+            const cudaError_t e = cudaMemcpy(host.get(), dev, bytes, cudaMemcpyDeviceToHost);
+            if (e != cudaSuccess) { froghost::set_cuda_error(e); rc = FROG_ERR_CUDA; }
+            else if (!write_all(f, host.get(), bytes)) rc = FROG_ERR_IO;
+        };
+        if (rc == FROG_OK) copy(dV, (size_t)n * d_pad * 4);
+        pos += nn * d_pad * 4;
+        if (rc == FROG_OK && !pad_to(f, pos, off_enc)) rc = FROG_ERR_IO;
+        if (rc == FROG_OK) copy(A.enc, nm * H * 4);
+    }
+    if (fclose(f) != 0 && rc == FROG_OK) rc = FROG_ERR_IO;
+    return rc;
 }

@@ -108,6 +108,13 @@ frog_kernel_fn lean_kernel(int ef_s, int budget, int row_bytes, bool table, bool
 // frog_search_team.cu: one CTA of `warps` warps per query (see there)
 frog_kernel_fn team_kernel(int warps, int ef_s, int q_len, int vis_bits, bool f16, size_t* smem);
 void set_cuda_error(cudaError_t e);
+// a stretch of an index file and the device memory it is read into or written from
+struct FileSection {
+    uint64_t off;
+    void* dev;
+    size_t bytes;
+};
+int transfer_sections(int fd, int device, const FileSection* sections, int count, bool to_device);
 int resolve_params(const frog_index* ix, int beam_width, const frog_params_t* in, frog_params_t* out);
 bool make_row_tensor_map(const void* base, bool f16, int row_elems, size_t row_bytes, size_t n, CUtensorMap* out);
 int acquire_scratch(frog_index* ix, cudaStream_t s, FrogScratch** out);
