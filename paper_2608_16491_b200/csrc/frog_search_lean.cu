@@ -1,4 +1,4 @@
-// The search kernel for the common case: fp32 rows of 384 or 512 bytes (d = 96, 128), an exact
+// The search kernel for the common case: fp32 or fp16 rows of 96 or 128 elements, an exact
 // visited set in global scratch (bitmap slab, or for large indexes a hash table of ranks), rows
 // fetched four at a time by the copy engine's tile::gather4, no counters and no trace.  It
 // computes exactly what frog_search_kernel computes (paper Alg. 2 with Alg. 3 once per query and
@@ -73,6 +73,12 @@ __host__ __device__ constexpr int lean_min_ctas(int epl, int rowb) {
                           : epl == 8 ? FROG_LEAN_MINB_512_P256 : FROG_LEAN_MINB_POOL512);
 }
 
+// Batches of at most LEAN_ROOMY_WARPS queries per SM do not fill those warps; for them the pools of 192 and 256
+// keys over rows of up to 384 bytes come in a second instantiation with the registers of 22 warps, which keeps
+// the pool keys of a merge out of local memory.  3,000 queries, 384-byte rows, beam 160, B 128: 1,245 -> 1,110 us
+// (24 warps: 1,125; 26: 1,145).  Pools of 128 keys hardly spill and are 1 % slower this way.
+constexpr int LEAN_ROOMY_WARPS = 22;
+
 // Scratch builds with -DFROG_LEAN_PROFILE add per-phase cycle counters (summed over all warps into
 // g_lean_prof, read back through frog_debug_lean_profile); the shipped library has none of this.
 #ifdef FROG_LEAN_PROFILE
@@ -82,21 +88,41 @@ __device__ unsigned long long g_lean_prof[8];
 #define LEAN_T(i) do { } while (0)
 #endif
 
-template <int EPL, int ROWB, int CAP>
+// A stored row: its bytes, the bytes of a 4-element group, and how such a group is read.
+template <int N>
+struct RowF32 {
+    static constexpr bool HALF = false;
+    static constexpr int BYTES = N, GROUP = 16, FLOATS = N / 4;
+    static __device__ __forceinline__ float4 group(const char* p) { return *reinterpret_cast<const float4*>(p); }
+};
+template <int N>
+struct RowF16 {
+    static constexpr bool HALF = true;
+    static constexpr int BYTES = N, GROUP = 8, FLOATS = N / 2;
+    static __device__ __forceinline__ float4 group(const char* p) {
+        const uint2 raw = *reinterpret_cast<const uint2*>(p);
+        const float2 lo = __half22float2(*reinterpret_cast<const __half2*>(&raw.x));
+        const float2 hi = __half22float2(*reinterpret_cast<const __half2*>(&raw.y));
+        return make_float4(lo.x, lo.y, hi.x, hi.y);
+    }
+};
+
+template <int EPL, class ROW, int CAP>
 struct Lean {
+    static constexpr int ROWB = ROW::BYTES;
     static constexpr int NSLOT = ROWB <= 384 ? FROG_LEAN_NSLOT_384 : FROG_LEAN_NSLOT_512;   // quads in the ring
     static constexpr int QUAD = 4 * ROWB;                       // bytes of one quad
     static constexpr int POOL = 32 * EPL;
     static constexpr int OFF_POOL = NSLOT * QUAD;
     static constexpr int OFF_CAND = OFF_POOL + POOL * 8;        // <= CAP (64 or 128) ranks + 3 of padding (+ 5 spare)
     static constexpr int OFF_D2 = OFF_CAND + (CAP + 8) * 4;     // squared distances of the <= CAP rows
-    static constexpr int OFF_Q = OFF_D2 + CAP * 4;              // query vector, ROWB bytes
-    static constexpr int OFF_BAR = OFF_Q + ROWB;                // NSLOT mbarriers, then the time-out flag
+    static constexpr int OFF_Q = OFF_D2 + CAP * 4;              // query vector (fp32)
+    static constexpr int OFF_BAR = OFF_Q + ROW::FLOATS * 4;                // NSLOT mbarriers, then the time-out flag
     static constexpr int BYTES = (OFF_BAR + 40 + 127) / 128 * 128;
     static_assert(OFF_CAND % 16 == 0 && OFF_Q % 16 == 0 && OFF_BAR % 8 == 0 && QUAD % 128 == 0, "alignment");
 };
 
-template <int EPL, int ROWB, int CAP>
+template <int EPL, class ROW, int CAP>
 struct LeanSmem {
     char* stage;
     uint64_t* pool;
@@ -106,7 +132,7 @@ struct LeanSmem {
     uint64_t* bar;
     uint32_t* timeout;
     __device__ __forceinline__ explicit LeanSmem(unsigned char* base) {
-        using L = Lean<EPL, ROWB, CAP>;
+        using L = Lean<EPL, ROW, CAP>;
         stage = reinterpret_cast<char*>(base);
         pool = reinterpret_cast<uint64_t*>(base + L::OFF_POOL);
         cand = reinterpret_cast<uint32_t*>(base + L::OFF_CAND);
@@ -123,10 +149,10 @@ struct LeanSmem {
 // then the partial sums are combined by a butterfly with partner distance 4, 2, 1.
 // HOOK (an instantiation of its own, for the test of the error path): no copy is armed or issued and a
 // wait gives up after 64 polls, so every gather ends in the time-out branch without anything in flight.
-template <int EPL, int ROWB, int CAP, bool HOOK = false>
-__device__ __forceinline__ void lean_gather(const FrogSearchArgs& A, const LeanSmem<EPL, ROWB, CAP>& S, int ns,
+template <int EPL, class ROW, int CAP, bool HOOK = false>
+__device__ __forceinline__ void lean_gather(const FrogSearchArgs& A, const LeanSmem<EPL, ROW, CAP>& S, int ns,
                                             uint32_t& ph, int lane) {
-    using L = Lean<EPL, ROWB, CAP>;
+    using L = Lean<EPL, ROW, CAP>;
     const int groups = (ns + 3) >> 2;
     if (lane < 3) S.cand[ns + lane] = (uint32_t)A.n + 1u + (uint32_t)lane;    // rows beyond the tensor: zeros
     __syncwarp();
@@ -144,7 +170,7 @@ __device__ __forceinline__ void lean_gather(const FrogSearchArgs& A, const LeanS
             if (g < groups) issue(g, g);
     }
     const int team = lane >> 3, sub = lane & 7;
-    const char* mine = S.stage + team * ROWB + sub * 16;
+    const char* mine = S.stage + team * ROW::BYTES + sub * ROW::GROUP;
     int slot = 0;
 #pragma unroll 1
     for (int g = 0; g < groups; ++g) {
@@ -153,8 +179,8 @@ __device__ __forceinline__ void lean_gather(const FrogSearchArgs& A, const LeanS
         const char* x = mine + slot * L::QUAD;
         float a = 0.f;
 #pragma unroll
-        for (int c = 0; c < ROWB / 128; ++c) {
-            const float4 xv = *reinterpret_cast<const float4*>(x + c * 128);
+        for (int c = 0; c < ROW::BYTES / (8 * ROW::GROUP); ++c) {
+            const float4 xv = ROW::group(x + c * 8 * ROW::GROUP);
             const float4 qv = S.q[sub + 8 * c];
             float t;
             t = xv.x - qv.x; a = fmaf(t, t, a);
@@ -175,8 +201,8 @@ __device__ __forceinline__ void lean_gather(const FrogSearchArgs& A, const LeanS
 
 // MergeTopEfS of 32 of the ns <= 128 evaluated candidates, those from `off` on (lines 15-17: merging
 // them batch by batch leaves the pool that one merge of all would); returns the first unexpanded position.
-template <int EPL, int ROWB, int CAP>
-__device__ __forceinline__ int lean_merge(const LeanSmem<EPL, ROWB, CAP>& S, int ns, int ef_s, uint32_t new_flag, int off, int lane) {
+template <int EPL, class ROW, int CAP>
+__device__ __forceinline__ int lean_merge(const LeanSmem<EPL, ROW, CAP>& S, int ns, int ef_s, uint32_t new_flag, int off, int lane) {
     const int j = off + lane;
     const uint64_t key = (j < ns) ? make_key(S.d2[j], S.cand[j], new_flag) : KEY_EMPTY;
     return (int)merge_batch<EPL, true>(S.pool, key, ef_s, lane);
@@ -184,20 +210,20 @@ __device__ __forceinline__ int lean_merge(const LeanSmem<EPL, ROWB, CAP>& S, int
 
 // gather + merge out of line, for the places that run once per query (entry points, exact scan) and
 // the rare second batch of an expansion; returns first | parities << 16
-template <int EPL, int ROWB, int CAP, bool HOOK = false>
+template <int EPL, class ROW, int CAP, bool HOOK = false>
 __device__ __noinline__ uint32_t lean_eval_cold(const FrogSearchArgs& A, unsigned char* base, int ns, uint32_t new_flag,
                                                 uint32_t ph) {
-    const LeanSmem<EPL, ROWB, CAP> S(base);
+    const LeanSmem<EPL, ROW, CAP> S(base);
     const int lane = lane_id();
-    lean_gather<EPL, ROWB, CAP, HOOK>(A, S, ns, ph, lane);
-    int first = lean_merge<EPL, ROWB, CAP>(S, ns, A.ef_s, new_flag, 0, lane);
-    for (int off = 32; off < ns; off += 32) first = lean_merge<EPL, ROWB, CAP>(S, ns, A.ef_s, new_flag, off, lane);
+    lean_gather<EPL, ROW, CAP, HOOK>(A, S, ns, ph, lane);
+    int first = lean_merge<EPL, ROW, CAP>(S, ns, A.ef_s, new_flag, 0, lane);
+    for (int off = 32; off < ns; off += 32) first = lean_merge<EPL, ROW, CAP>(S, ns, A.ef_s, new_flag, off, lane);
     return (uint32_t)first | (ph << 16);
 }
-template <int EPL, int ROWB, int CAP>
+template <int EPL, class ROW, int CAP>
 __device__ __noinline__ int lean_merge_cold(unsigned char* base, int ns, int ef_s, uint32_t new_flag, int off) {
-    const LeanSmem<EPL, ROWB, CAP> S(base);
-    return lean_merge<EPL, ROWB, CAP>(S, ns, ef_s, new_flag, off, lane_id());
+    const LeanSmem<EPL, ROW, CAP> S(base);
+    return lean_merge<EPL, ROW, CAP>(S, ns, ef_s, new_flag, off, lane_id());
 }
 
 // Visited check of the cnt <= 64 ranks in en[] (EN order; a longer list is passed in two parts): survivors are compacted, in order, into
@@ -232,15 +258,15 @@ __device__ __forceinline__ int lean_visit_list(const uint32_t* en, int cnt, uint
 // candidate costs no DRAM access; the bitmap's scattered read-modify-writes are what keeps DRAM from the
 // row gathers on large indexes).  The table is exact; a query that fills it half way moves its entries
 // to the warp's bitmap slab and carries on there.
-template <int EPL, int ROWB, bool TABLE, int CAP = 64, bool HOOK = false>
-__global__ void __launch_bounds__(LEAN_WARPS * 32, lean_min_ctas(EPL, ROWB))
+template <int EPL, class ROW, bool TABLE, int CAP = 64, bool HOOK = false, bool ROOMY = false>
+__global__ void __launch_bounds__(LEAN_WARPS * 32, ROOMY ? LEAN_ROOMY_WARPS / LEAN_WARPS : lean_min_ctas(EPL, ROW::BYTES))
 frog_search_lean_kernel(const __grid_constant__ FrogSearchArgs A) {
-    using L = Lean<EPL, ROWB, CAP>;
+    using L = Lean<EPL, ROW, CAP>;
     extern __shared__ __align__(128) unsigned char smem_raw[];
     const int lane = lane_id();
     const int warp = threadIdx.x >> 5;
     unsigned char* base = smem_raw + L::BYTES * warp;
-    const LeanSmem<EPL, ROWB, CAP> S(base);
+    const LeanSmem<EPL, ROW, CAP> S(base);
     if (lane == 0) {
 #pragma unroll
         for (int i = 0; i < L::NSLOT; ++i) mbar_init(S.bar + i, 1u);
@@ -273,7 +299,7 @@ frog_search_lean_kernel(const __grid_constant__ FrogSearchArgs A) {
         {
             float* qf = reinterpret_cast<float*>(base + L::OFF_Q);
             const float* src = A.queries + (size_t)q * A.d;
-            for (int i = lane; i < ROWB / 4; i += 32) qf[i] = i < A.d ? __ldg(src + i) : 0.f;
+            for (int i = lane; i < ROW::FLOATS; i += 32) qf[i] = i < A.d ? __ldg(src + i) : 0.f;
             for (int i = lane; i < L::POOL; i += 32) S.pool[i] = KEY_EMPTY;
         }
         const int32_t lo = __ldg(A.lo + q), hi = __ldg(A.hi + q);
@@ -299,7 +325,7 @@ frog_search_lean_kernel(const __grid_constant__ FrogSearchArgs A) {
                 if (lane < cnt) S.cand[lane] = (uint32_t)(l_q + b0 + lane);
                 if (lane + 32 < cnt) S.cand[lane + 32] = (uint32_t)(l_q + b0 + lane + 32);
                 __syncwarp();
-                ph = lean_eval_cold<EPL, ROWB, CAP, HOOK>(A, base, cnt, 1u, ph) >> 16;
+                ph = lean_eval_cold<EPL, ROW, CAP, HOOK>(A, base, cnt, 1u, ph) >> 16;
                 __syncwarp();
             }
         } else {
@@ -343,7 +369,7 @@ frog_search_lean_kernel(const __grid_constant__ FrogSearchArgs A) {
             if (n_logged >= 0) n_logged = log_ranks(bitmap + A.bitmap_words, A.log_cap, n_logged, S.cand, ns, lane);
             int first;
             {
-                const uint32_t r = lean_eval_cold<EPL, ROWB, CAP, HOOK>(A, base, ns, 0u, ph);
+                const uint32_t r = lean_eval_cold<EPL, ROW, CAP, HOOK>(A, base, ns, 0u, ph);
                 first = (int)(r & 0xFFFFu);
                 ph = r >> 16;
             }
@@ -442,10 +468,10 @@ frog_search_lean_kernel(const __grid_constant__ FrogSearchArgs A) {
                 if (n_logged >= 0) n_logged = log_ranks(bitmap + A.bitmap_words, A.log_cap, n_logged, S.cand, ns, lane);
                 // lines 14-17
                 LEAN_T(1);
-                lean_gather<EPL, ROWB, CAP, HOOK>(A, S, ns, ph, lane);
+                lean_gather<EPL, ROW, CAP, HOOK>(A, S, ns, ph, lane);
                 LEAN_T(2);
-                first = lean_merge<EPL, ROWB, CAP>(S, ns, A.ef_s, 0u, 0, lane);
-                for (int off = 32; off < ns; off += 32) first = lean_merge_cold<EPL, ROWB, CAP>(base, ns, A.ef_s, 0u, off);
+                first = lean_merge<EPL, ROW, CAP>(S, ns, A.ef_s, 0u, 0, lane);
+                for (int off = 32; off < ns; off += 32) first = lean_merge_cold<EPL, ROW, CAP>(base, ns, A.ef_s, 0u, off);
                 LEAN_T(3);
 #ifdef FROG_LEAN_PROFILE
                 t_ph[6] += 1;
@@ -509,28 +535,39 @@ frog_search_lean_kernel(const __grid_constant__ FrogSearchArgs A) {
 // inside the 196 KB carve-out, so that L1 keeps 60 KB; the larger layout was measured 4-9 % slower at
 // B <= 64); budgets up to 128 are instantiated for the pools of 128-256 keys, where they pay (hard,
 // narrow-range batches); other combinations go to the general kernel.
-template <int ROWB>
-frog_kernel_fn lean_pick(int ef_s, int budget, bool table, bool hook, size_t* smem_per_warp) {
+template <int EPL, class ROW, int CAP, bool TABLES>
+frog_kernel_fn lean_fn(bool table, bool roomy, size_t* smem_per_warp) {
+    *smem_per_warp = Lean<EPL, ROW, CAP>::BYTES;
+    if constexpr (EPL >= 6 && EPL <= 8 && ROW::BYTES <= 384) {
+        if (roomy && !table) return frog_search_lean_kernel<EPL, ROW, false, CAP, false, true>;
+    }
+    if constexpr (TABLES && !ROW::HALF) {
+        if (table) return frog_search_lean_kernel<EPL, ROW, true, CAP>;
+    }
+    return table ? nullptr : frog_search_lean_kernel<EPL, ROW, false, CAP>;
+}
+template <class ROW>
+frog_kernel_fn lean_pick(int ef_s, int budget, bool table, bool roomy, bool hook, size_t* smem_per_warp) {
     if (hook) {
-        if (table || budget > 64 || ef_s > 32) return nullptr;
-        *smem_per_warp = Lean<1, ROWB, 64>::BYTES;
-        return frog_search_lean_kernel<1, ROWB, false, 64, true>;
+        if constexpr (ROW::HALF) return nullptr;
+        else {
+            if (table || budget > 64 || ef_s > 32) return nullptr;
+            *smem_per_warp = Lean<1, ROW, 64>::BYTES;
+            return frog_search_lean_kernel<1, ROW, false, 64, true>;
+        }
     }
     if (budget > 64) {
-        if (ef_s <= 64 || ef_s > 256 || (table && ef_s > 128)) return nullptr;
-        if (ef_s <= 128) { *smem_per_warp = Lean<4, ROWB, 128>::BYTES; return table ? frog_search_lean_kernel<4, ROWB, true, 128> : frog_search_lean_kernel<4, ROWB, false, 128>; }
-        if (ef_s <= 192) { *smem_per_warp = Lean<6, ROWB, 128>::BYTES; return frog_search_lean_kernel<6, ROWB, false, 128>; }
-        *smem_per_warp = Lean<8, ROWB, 128>::BYTES;
-        return frog_search_lean_kernel<8, ROWB, false, 128>;
+        if (ef_s <= 64 || ef_s > 256) return nullptr;
+        if (ef_s <= 128) return lean_fn<4, ROW, 128, true>(table, roomy, smem_per_warp);
+        if (ef_s <= 192) return lean_fn<6, ROW, 128, false>(table, roomy, smem_per_warp);
+        return lean_fn<8, ROW, 128, false>(table, roomy, smem_per_warp);
     }
-    if (ef_s <= 32) { *smem_per_warp = Lean<1, ROWB, 64>::BYTES; return table ? frog_search_lean_kernel<1, ROWB, true> : frog_search_lean_kernel<1, ROWB, false>; }
-    if (ef_s <= 64) { *smem_per_warp = Lean<2, ROWB, 64>::BYTES; return table ? frog_search_lean_kernel<2, ROWB, true> : frog_search_lean_kernel<2, ROWB, false>; }
-    if (ef_s <= 128) { *smem_per_warp = Lean<4, ROWB, 64>::BYTES; return table ? frog_search_lean_kernel<4, ROWB, true> : frog_search_lean_kernel<4, ROWB, false>; }
-    if (table) return nullptr;
-    if (ef_s <= 192) { *smem_per_warp = Lean<6, ROWB, 64>::BYTES; return frog_search_lean_kernel<6, ROWB, false>; }
-    if (ef_s <= 256) { *smem_per_warp = Lean<8, ROWB, 64>::BYTES; return frog_search_lean_kernel<8, ROWB, false>; }
-    *smem_per_warp = Lean<16, ROWB, 64>::BYTES;
-    return frog_search_lean_kernel<16, ROWB, false>;
+    if (ef_s <= 32) return lean_fn<1, ROW, 64, true>(table, roomy, smem_per_warp);
+    if (ef_s <= 64) return lean_fn<2, ROW, 64, true>(table, roomy, smem_per_warp);
+    if (ef_s <= 128) return lean_fn<4, ROW, 64, true>(table, roomy, smem_per_warp);
+    if (ef_s <= 192) return lean_fn<6, ROW, 64, false>(table, roomy, smem_per_warp);
+    if (ef_s <= 256) return lean_fn<8, ROW, 64, false>(table, roomy, smem_per_warp);
+    return lean_fn<16, ROW, 64, false>(table, roomy, smem_per_warp);
 }
 
 }  // namespace
@@ -540,12 +577,19 @@ namespace froghost {
 // The lean kernel for this beam width and row size, or null if the shape is not covered (the caller
 // then uses the generic kernel).  Needs the row tensor map and the bitmap visited set.  `table`: the
 // variant whose visited set is the L2-resident hash table (pools of up to 128 keys only); `hook`: the
-// instantiation whose gathers time out by construction (bitmap form, beams up to 32, budgets up to 64).
-frog_kernel_fn lean_kernel(int ef_s, int budget, int row_bytes, bool table, bool hook, size_t* smem_per_warp,
+// instantiation whose gathers time out by construction (bitmap form, beams up to 32, budgets up to 64);
+// `queries_per_sm`: of the batch, 0 = not known (a full GPU).
+frog_kernel_fn lean_kernel(int ef_s, int budget, int row_bytes, bool f16, bool table, bool hook, int queries_per_sm, size_t* smem_per_warp,
                            int* warps_per_cta) {
     *warps_per_cta = LEAN_WARPS;
-    if (row_bytes == 384) return lean_pick<384>(ef_s, budget, table, hook, smem_per_warp);
-    if (row_bytes == 512) return lean_pick<512>(ef_s, budget, table, hook, smem_per_warp);
+    const bool roomy = queries_per_sm > 0 && queries_per_sm <= LEAN_ROOMY_WARPS;
+    if (f16) {
+        if (row_bytes == 192) return lean_pick<RowF16<192>>(ef_s, budget, table, roomy, hook, smem_per_warp);
+        if (row_bytes == 256) return lean_pick<RowF16<256>>(ef_s, budget, table, roomy, hook, smem_per_warp);
+        return nullptr;
+    }
+    if (row_bytes == 384) return lean_pick<RowF32<384>>(ef_s, budget, table, roomy, hook, smem_per_warp);
+    if (row_bytes == 512) return lean_pick<RowF32<512>>(ef_s, budget, table, roomy, hook, smem_per_warp);
     return nullptr;
 }
 

@@ -1,0 +1,48 @@
+"""The short-row search kernel on fp16 rows of 96 and 128 elements, and its instantiations for batches that do not
+fill the GPU, against the CPU oracle.  ``visited=VISITED_BITMAP`` takes it at any batch size."""
+import numpy as np
+import pytest
+
+import oracle
+
+pytestmark = pytest.mark.gpu
+
+torch = pytest.importorskip("torch")
+
+
+# d = 93: a row of 96 elements of which three are padding; 3,300 queries are 23 per SM, 60 are one
+@pytest.mark.parametrize("d,storage,copies", [(93, 1, 1), (96, 1, 55), (128, 1, 1), (128, 1, 55), (96, 0, 1), (96, 0, 55)])
+def test_every_pool(libs, tmp_path, d, storage, copies):
+    rng = np.random.default_rng(d + copies)
+    n = 5000
+    centers = rng.standard_normal((10, d))
+    base = (centers[rng.integers(0, 10, n)] + 0.4 * rng.standard_normal((n, d))).astype(np.float32)
+    attrs = rng.integers(0, n, n).astype(np.int32)
+    path = str(tmp_path / "x.idx")
+    libs.build_index_gpu(base, attrs, path, ef_c=48)
+    ix = oracle.load_index(path)
+    gix = libs.Index.load(path)
+    if storage:
+        gix.enable_f16()
+        ix = oracle.rounded_to_f16(ix)
+    q = (base[rng.integers(0, n, 60)] + 0.2 * rng.standard_normal((60, d))).astype(np.float32)
+    a = np.sort(attrs)
+    w = (n * 2.0 ** -rng.uniform(0, 6, 60)).astype(int)
+    s = (rng.random(60) * (n - w)).astype(int)
+    lo, hi = a[s], a[s + w - 1]
+    dev = [torch.from_numpy(np.ascontiguousarray(np.tile(x, (copies,) + (1,) * (x.ndim - 1)))).cuda() for x in (q, lo, hi)]
+    for ef, budget in ((16, 16), (32, 64), (33, 64), (64, 24), (65, 128), (128, 64), (129, 64), (192, 128), (193, 128),
+                       (256, 64), (257, 64), (512, 32)):
+        ref = oracle.search(ix, q, lo, hi, 10, ef, B=budget)
+        p = libs.Params(budget=budget, storage=storage, visited=libs.VISITED_BITMAP)
+        status = torch.zeros(60 * copies, dtype=torch.int32, device="cuda")
+        ids, dists = gix.search(*dev, 10, ef, params=p, status=status)
+        torch.cuda.synchronize()
+        assert np.array_equal(ids.cpu().numpy(), np.tile(ref.ids, (copies, 1)))
+        assert np.array_equal(dists.cpu().numpy().view(np.uint32), np.tile(ref.dists.view(np.uint32), (copies, 1)))
+        assert np.array_equal(status.cpu().numpy().view(np.uint32), np.tile(ref.status, copies))
+        if copies == 1:
+            q1 = [x[:60] for x in dev]
+            other = gix.search_static(*q1, 10, ef, params=libs.Params(budget=budget, storage=storage))
+            assert torch.equal(other[0], ids) and torch.equal(other[1], dists)
+    gix.close()
