@@ -184,7 +184,9 @@ int frog_search_ex(const frog_index_t* index, const float* queries, const int32_
                    uint32_t* trace, int trace_cap, void* stream);
 
 /* frog_exact_search: exact filtered kNN (Def. 2 of Sec. 2.1) by scanning the contiguous rank
- * slab of each query (Sec. 4: an attribute range is a contiguous rank interval), one CTA per
+ * slab of each query (Sec. 4: an attribute range is a contiguous rank interval).  The rows are cut into
+ * pieces over the whole GPU and, from 16 queries on, shared by groups of eight; that uses scratch of the
+ * index (see frog_search).  Under stream capture, and where scratch cannot be had, one CTA scans each
  * query.  Same buffers and conventions as frog_search; 1 <= k <= FROG_MAX_BEAM_WIDTH.  Used for ground truth
  * and as the pre-filtering reference. */
 int frog_exact_search(const frog_index_t* index, const float* queries, const int32_t* lo, const int32_t* hi,
