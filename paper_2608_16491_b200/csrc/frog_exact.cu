@@ -11,10 +11,10 @@
 //     shared by all pieces of a query through global memory: whatever exceeds the k-th best of ANY piece
 //     cannot be an answer;
 //   * the last CTA to finish a group merges the pieces' lists.
-// Fewer than EXACT_GROUP_MIN queries are not grouped: every CTA finds the slabs itself and takes an equal
-// share of all rows (one launch).  Otherwise queries are ordered by (width, position), grouped by eight, and
-// the groups' rows are cut into pieces of equal size (two small kernels).  The form with one CTA per query
-// and no scratch remains for captured streams, for rows too long for eight queries in shared memory, and
+// Up to EXACT_GROUP_MIN queries are not grouped: all rows are cut into equal pieces, one query each (one launch for
+// fewer than EXACT_PLAN_MIN, else a planning kernel finds the slabs first).  Otherwise queries are ordered by
+// (width, position), grouped by eight, and the groups' rows are cut into pieces of equal size (two small kernels).  The form with one CTA per query
+// and no scratch remains for many queries on small indexes, for captured streams, for rows too long for eight queries in shared memory, and
 // for the case that scratch cannot be had.
 #include <algorithm>
 
@@ -27,7 +27,13 @@ namespace {
 
 constexpr int EXACT_WARPS = 8;
 constexpr int EXACT_GROUP = 8;           // queries per group = warps per CTA (one merges each query's buffer)
-constexpr int EXACT_GROUP_MIN = 16;      // batches of fewer queries are not grouped
+// Grouping costs 35 us of planning and pays for itself from about 200 queries on, whatever the rows (us per call,
+// split / grouped, k = 10): 100,000 x 96: 64 queries 129/235, 100: 168/260, 200: 300/358, 600: 1,075/595;
+// 30,000 x 50: 100: 118/138, 200: 169/170, 600: 372/277; 20,000 x 768: 100: 171/216, 200: 263/252, 600: 677/492.
+constexpr int EXACT_GROUP_MIN = 201;
+// Slabs of so few rows are not worth planning for once there is a query per CTA (5,000 x 96, 600 queries: 111 grouped).
+constexpr int EXACT_SMALL_ROWS = 8192;
+constexpr int EXACT_PLAN_MIN = 17;       // from here on the slabs are found by a planning kernel (100,000 x 96, 16 queries: 49 without)
 constexpr int EXACT_STEP = 8 * EXACT_WARPS;    // rows per step of a CTA: two per team
 constexpr int EXACT_BUF = 256;           // keys buffered per query; merged from 64 on, two steps add at most 128
 constexpr int EXACT_BINS = 33 * 32;      // (width class, position) bins that queries are ordered by
@@ -449,12 +455,12 @@ frog_exact_kernel(const ExactArgs A) {
     exact_piece<EPL, 1>(A, S, l_q, r_q + 1, 0, 0, 1, nullptr);
 }
 
-// Fewer than EXACT_GROUP_MIN queries: all rows cut into equal pieces, at most one per CTA.
+// Fewer than EXACT_PLAN_MIN queries: all rows cut into equal pieces, at most one per CTA.
 template <int EPL>
 __global__ void __launch_bounds__(EXACT_WARPS * 32, 2)
 frog_exact_few_kernel(const ExactArgs A) {
     extern __shared__ __align__(16) unsigned char smem_raw[];
-    __shared__ int2 slab[EXACT_GROUP_MIN];
+    __shared__ int2 slab[EXACT_PLAN_MIN];
     const ExactSmem<EPL, 1> S(smem_raw);
     const int lane = lane_id(), warp = threadIdx.x >> 5;
     for (int q = warp; q < A.nq; q += EXACT_WARPS) {
@@ -486,6 +492,71 @@ frog_exact_few_kernel(const ExactArgs A) {
             return;
         }
         first += pieces;
+    }
+}
+
+// Up to EXACT_GROUP_MIN queries: all rows cut into pieces of equal size, about two per CTA, which evens out their
+// ends.  Every CTA works out the cut for itself from the slabs that the planning kernel found.
+template <int EPL>
+__global__ void __launch_bounds__(EXACT_WARPS * 32, 2)
+frog_exact_split_kernel(const ExactArgs A) {
+    extern __shared__ __align__(16) unsigned char smem_raw[];
+    __shared__ int first[EXACT_GROUP_MIN + 1];               // first piece of each query
+    __shared__ int warp_sum[EXACT_WARPS];
+    __shared__ unsigned long long rows;
+    const ExactSmem<EPL, 1> S(smem_raw);
+    const int lane = lane_id(), warp = threadIdx.x >> 5, t = threadIdx.x;
+    if (t == 0) rows = 0;
+    __syncthreads();
+    auto slab_of = [&](int q) {                              // first rank, rows
+        const int2 lr = A.ranges[q];
+        return make_int2(lr.x, max(0, lr.y - lr.x + 1));
+    };
+    unsigned long long mine = 0;
+    for (int q = t; q < A.nq; q += EXACT_WARPS * 32) mine += (unsigned long long)slab_of(q).y;
+    if (mine) atomicAdd(&rows, mine);
+    __syncthreads();
+    const long long share = 2 * (long long)gridDim.x;
+    long long size = max(((long long)rows + share - 1) / share, (long long)A.min_rows);
+    size = (size + EXACT_STEP - 1) / EXACT_STEP * EXACT_STEP;
+    int before = 0;
+    for (int q0 = 0; q0 < A.nq; q0 += EXACT_WARPS * 32) {
+        const int q = q0 + t;
+        const int np = q < A.nq ? max(1, (int)((slab_of(q).y + size - 1) / size)) : 0;
+        int x = np;
+        for (int o = 1; o < 32; o <<= 1) {
+            const int y = __shfl_up_sync(FULL, x, o);
+            if (lane >= o) x += y;
+        }
+        if (lane == 31) warp_sum[warp] = x;
+        __syncthreads();
+        int add = before;
+        for (int w = 0; w < EXACT_WARPS; ++w) {
+            if (w < warp) add += warp_sum[w];
+            before += warp_sum[w];
+        }
+        if (q < A.nq) first[q] = add + x - np;
+        __syncthreads();
+    }
+    if (t == 0) first[A.nq] = before;
+    __syncthreads();
+    for (int piece = blockIdx.x; piece < first[A.nq]; piece += gridDim.x) {
+        int q = 0, end = A.nq;                               // the last query whose first piece is not beyond this one
+        while (end - q > 1) {
+            const int mid = (q + end) >> 1;
+            if (first[mid] <= piece) q = mid; else end = mid;
+        }
+        const int2 sl = slab_of(q);
+        if (t == 0) {
+            S.l[0] = sl.x;
+            S.r[0] = sl.x + sl.y - 1;
+            S.id[0] = q;
+        }
+        const int p = piece - first[q];
+        const int row0 = sl.x + (int)(p * size), row1 = (int)min((long long)row0 + size, (long long)sl.x + sl.y);
+        __syncthreads();
+        exact_piece<EPL, 1>(A, S, row0, row1, piece, first[q], first[q + 1] - first[q], A.done + q);
+        __syncthreads();
     }
 }
 
@@ -534,7 +605,7 @@ frog_exact_plan_kernel(const ExactArgs A) {
     if (lane == 0) {
         const int2 lr = lo > hi || r_q < l_q ? make_int2(1, 0) : make_int2(l_q, r_q);
         A.ranges[q] = lr;
-        atomicAdd(A.counters + 2 + exact_bin(lr, A.n), 1u);
+        if (A.jobs) atomicAdd(A.counters + 2 + exact_bin(lr, A.n), 1u);
     }
 }
 
@@ -651,6 +722,7 @@ exact_fn exact_pick(int k) {
 }
 template <int EPL> struct OnePerQuery { static exact_fn fn() { return frog_exact_kernel<EPL>; } };
 template <int EPL> struct Few { static exact_fn fn() { return frog_exact_few_kernel<EPL>; } };
+template <int EPL> struct Split { static exact_fn fn() { return frog_exact_split_kernel<EPL>; } };
 template <int EPL> struct Grouped { static exact_fn fn() { return frog_exact_group_kernel<EPL>; } };
 
 template <int G>
@@ -688,17 +760,17 @@ extern "C" int frog_exact_search(const frog_index_t* index, const float* queries
     };
     cudaStreamCaptureStatus capture = cudaStreamCaptureStatusNone;
     FROG_CUDA_TRY(cudaStreamIsCapturing(s, &capture));
-    const bool few = nq < EXACT_GROUP_MIN;
+    const bool few = nq < EXACT_GROUP_MIN, small = !few && index->info.n <= EXACT_SMALL_ROWS;
     const size_t smem = few ? exact_smem<1>(k, A.d_pad) : exact_smem<EXACT_GROUP>(k, A.d_pad);
-    if (capture == cudaStreamCaptureStatusNone && smem <= 227 * 1024) {
-        const exact_fn fn = few ? exact_pick<Few>(k) : exact_pick<Grouped>(k);
+    if (capture == cudaStreamCaptureStatusNone && !small && smem <= 227 * 1024) {
+        const exact_fn fn = nq < EXACT_PLAN_MIN ? exact_pick<Few>(k) : few ? exact_pick<Split>(k) : exact_pick<Grouped>(k);
         FROG_CUDA_TRY(ready(fn, smem));
         int per_sm = 0;
         FROG_CUDA_TRY(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, (const void*)fn, EXACT_WARPS * 32, smem));
         const int grid = std::max(per_sm, 1) * index->sm_count;
         const int groups = few ? nq : (nq + EXACT_GROUP - 1) / EXACT_GROUP;
         // enough pieces to even out their ends; fewer for long result lists, whose partial lists they multiply
-        const int max_pieces = few ? grid : grid * (k <= 128 ? 16 : 8);
+        const int max_pieces = few ? 2 * grid + nq : grid * (k <= 128 ? 16 : 8);
         frog_index* mix = const_cast<frog_index*>(index);      // the scratch sets are the index's only mutable part
         std::lock_guard<std::mutex> lock(mix->mu);
         FrogScratch* sc = nullptr;
@@ -709,7 +781,7 @@ extern "C" int frog_exact_search(const frog_index_t* index, const float* queries
         if (froghost::ensure_exact(sc, (size_t)nq, (size_t)groups, (size_t)max_pieces + groups, lists, EXACT_BINS + 2, &X) == FROG_OK) {
             A.ranges = static_cast<int2*>(X.ranges);
             A.order = X.order;
-            A.jobs = static_cast<int4*>(X.jobs);
+            A.jobs = few ? nullptr : static_cast<int4*>(X.jobs);        // null: no histogram
             A.groups = static_cast<int2*>(X.groups);
             A.counters = X.counters;
             A.done = X.done;
@@ -717,10 +789,8 @@ extern "C" int frog_exact_search(const frog_index_t* index, const float* queries
             A.part = X.part;
             A.max_pieces = max_pieces;
             A.min_rows = few ? 256 : 512;
-            if (!few) {
-                frog_exact_plan_kernel<<<(nq * 32 + 255) / 256, 256, 0, s>>>(A);
-                frog_exact_cut_kernel<<<1, 1024, 0, s>>>(A);
-            }
+            if (!few || nq >= EXACT_PLAN_MIN) frog_exact_plan_kernel<<<(nq * 32 + 255) / 256, 256, 0, s>>>(A);
+            if (!few) frog_exact_cut_kernel<<<1, 1024, 0, s>>>(A);
             fn<<<grid, EXACT_WARPS * 32, smem, s>>>(A);
             FROG_CUDA_TRY(cudaGetLastError());
             FROG_CUDA_TRY(cudaEventRecord(sc->done, s));
