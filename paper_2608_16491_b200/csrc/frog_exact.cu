@@ -31,8 +31,11 @@ constexpr int EXACT_GROUP = 8;           // queries per group = warps per CTA (o
 // split / grouped, k = 10): 100,000 x 96: 64 queries 129/235, 100: 168/260, 200: 300/358, 600: 1,075/595;
 // 30,000 x 50: 100: 118/138, 200: 169/170, 600: 372/277; 20,000 x 768: 100: 171/216, 200: 263/252, 600: 677/492.
 constexpr int EXACT_GROUP_MIN = 201;
-// Slabs of so few rows are not worth planning for once there is a query per CTA (5,000 x 96, 600 queries: 111 grouped).
-constexpr int EXACT_SMALL_ROWS = 8192;
+// Slabs of so few bytes are not worth planning for once there is a query per CTA and lists are short (us, one CTA per
+// query / grouped: 5,000 x 96, 300 queries 93/104, 2,000: 140/163; 8,000 x 128, 600: 169/156, 2,000: 316/349;
+// 8,000 x 384, 600: 275/203; with k = 100 5,000 x 96, 600: 234/160).
+constexpr long long EXACT_SMALL_BYTES = 4500000;
+constexpr int EXACT_SMALL_K = 32;
 constexpr int EXACT_PLAN_MIN = 17;       // from here on the slabs are found by a planning kernel (100,000 x 96, 16 queries: 49 without)
 constexpr int EXACT_STEP = 8 * EXACT_WARPS;    // rows per step of a CTA: two per team
 constexpr int EXACT_BUF = 256;           // keys buffered per query; merged from 64 on, two steps add at most 128
@@ -49,7 +52,7 @@ struct ExactArgs {
     int nq, k;
     int32_t* out_ids;
     float* out_dists;
-    // scratch (see ExactScratch); null for the form with one CTA per query
+    // scratch (see ExactScratch); unused by the form with one CTA per query
     int2* ranges;
     int32_t* order;
     int4* jobs;                      // (group, first row, end row, -)
@@ -95,7 +98,7 @@ __device__ __forceinline__ void exact_flush(const ExactArgs& A, const ExactSmem<
     for (int off = 0; off < n; off += 32)
         merge_ranked<EPL>(pool, S.buf + g * EXACT_BUF + off, min(32, n - off), A.k, lane);
     uint64_t kth = pool[A.k - 1];
-    if (A.bound && S.id[g] >= 0) {
+    if (S.id[g] >= 0) {
         unsigned long long seen = 0;
         if (lane == 0) {
             if (n > 0 && kth != KEY_EMPTY) atomicMin(A.bound + S.id[g], (unsigned long long)kth);
@@ -376,7 +379,7 @@ __device__ __forceinline__ void exact_piece(const ExactArgs& A, const ExactSmem<
     for (int i = threadIdx.x; i < G * 32 * EPL; i += EXACT_WARPS * 32) S.pool[i] = KEY_EMPTY;
     if (threadIdx.x < G) {
         S.cnt[threadIdx.x] = 0;
-        S.tau[threadIdx.x] = A.bound && S.id[threadIdx.x] >= 0 ? (uint64_t)__ldcg(A.bound + S.id[threadIdx.x]) : KEY_EMPTY;
+        S.tau[threadIdx.x] = S.id[threadIdx.x] >= 0 ? (uint64_t)__ldcg(A.bound + S.id[threadIdx.x]) : KEY_EMPTY;
     }
     __syncthreads();
     if constexpr (G == 1) exact_scan_one<EPL>(A, S, row0, row1);
@@ -428,31 +431,70 @@ __device__ __forceinline__ void exact_piece(const ExactArgs& A, const ExactSmem<
         __syncthreads();
         if (threadIdx.x == 0) *done = 0u;                   // leave the scratch as it was found
         if (threadIdx.x < G && S.id[threadIdx.x] >= 0) A.bound[S.id[threadIdx.x]] = ~0ull;
-    } else if (A.bound && threadIdx.x < G && S.id[threadIdx.x] >= 0) {
+    } else if (threadIdx.x < G && S.id[threadIdx.x] >= 0) {
         A.bound[S.id[threadIdx.x]] = ~0ull;
     }
     if (warp < G && S.id[warp] >= 0) exact_output<EPL>(A, S.pool + warp * 32 * EPL, S.id[warp], lane);
     __syncthreads();
 }
 
-// One CTA per query, no scratch.
+// One CTA per query, no scratch: each warp streams batches of 16 rows and keeps a list of its own, warp 0 merges
+// the lists.  32 warps per SM and no barrier in the loop: the better form for many short slabs (see EXACT_SMALL_BYTES).
 template <int EPL>
-__global__ void __launch_bounds__(EXACT_WARPS * 32, 2)
+__global__ void __launch_bounds__(EXACT_WARPS * 32)
 frog_exact_kernel(const ExactArgs A) {
     extern __shared__ __align__(16) unsigned char smem_raw[];
-    const ExactSmem<EPL, 1> S(smem_raw);
-    const int q = blockIdx.x, lane = lane_id();
+    constexpr int POOL = 32 * EPL;
+    const int lane = lane_id();
+    const int warp = threadIdx.x >> 5;
+    const int q = blockIdx.x;
+    float4* qs = reinterpret_cast<float4*>(smem_raw);
+    uint64_t* pools = reinterpret_cast<uint64_t*>(smem_raw + (size_t)A.d_pad * 4);
+    uint64_t* pool = pools + (size_t)warp * POOL;
+
+    {
+        float* qf = reinterpret_cast<float*>(qs);
+        const float* src = A.queries + (size_t)q * A.d;
+        for (int i = threadIdx.x; i < A.d_pad; i += blockDim.x) qf[i] = i < A.d ? __ldg(src + i) : 0.f;
+        for (int i = lane; i < POOL; i += 32) pool[i] = KEY_EMPTY;
+    }
     const int32_t lo = __ldg(A.lo + q), hi = __ldg(A.hi + q);
     int l_q, r_q;
     warp_rank_interval(A.sorted_attr, A.n, lo, hi, lane, l_q, r_q);
-    if (lo > hi) r_q = l_q - 1;
-    if (threadIdx.x == 0) {
-        S.l[0] = l_q;
-        S.r[0] = r_q;
-        S.id[0] = q;
+    const int w = (lo > hi) ? 0 : (r_q - l_q + 1);
+    __syncthreads();
+
+    for (int b0 = warp * 16; b0 < w; b0 += EXACT_WARPS * 16) {
+        const int cnt = min(16, w - b0);
+        const uint32_t rank = (uint32_t)(l_q + b0 + (lane & 15));
+        float d2 = batch_dist2<4>(A.vectors, A.d_pad, qs, rank, cnt, lane);
+        uint64_t key = KEY_EMPTY;
+        if (lane < cnt) key = make_key(d2, (uint32_t)__ldg(A.rank2id + rank), 1u);   // keyed by object id
+        // (merge_batch itself rejects candidates not better than the current k-th best)
+        merge_batch<EPL>(pool, key, A.k, lane);
     }
     __syncthreads();
-    exact_piece<EPL, 1>(A, S, l_q, r_q + 1, 0, 0, 1, nullptr);
+    if (warp == 0) {
+        for (int ow = 1; ow < EXACT_WARPS; ++ow) {
+            const uint64_t* other = pools + (size_t)ow * POOL;
+            for (int j0 = 0; j0 < A.k; j0 += 32) {
+                uint64_t key = (j0 + lane < A.k) ? other[j0 + lane] : KEY_EMPTY;
+                merge_batch<EPL>(pool, key, A.k, lane);
+            }
+        }
+        __syncwarp();
+        for (int j = lane; j < A.k; j += 32) {
+            uint64_t key = pool[j];
+            int32_t oid = -1;
+            float dist = __int_as_float(0x7F800000);
+            if (key != KEY_EMPTY) {
+                oid = (int32_t)key_rank(key);
+                dist = __fsqrt_rn(key_dist2(key));
+            }
+            A.out_ids[(size_t)q * A.k + j] = oid;
+            A.out_dists[(size_t)q * A.k + j] = dist;
+        }
+    }
 }
 
 // Fewer than EXACT_PLAN_MIN queries: all rows cut into equal pieces, at most one per CTA.
@@ -760,7 +802,8 @@ extern "C" int frog_exact_search(const frog_index_t* index, const float* queries
     };
     cudaStreamCaptureStatus capture = cudaStreamCaptureStatusNone;
     FROG_CUDA_TRY(cudaStreamIsCapturing(s, &capture));
-    const bool few = nq < EXACT_GROUP_MIN, small = !few && index->info.n <= EXACT_SMALL_ROWS;
+    const bool few = nq < EXACT_GROUP_MIN;
+    const bool small = !few && k <= EXACT_SMALL_K && index->info.n * A.d_pad * 4 <= EXACT_SMALL_BYTES;
     const size_t smem = few ? exact_smem<1>(k, A.d_pad) : exact_smem<EXACT_GROUP>(k, A.d_pad);
     if (capture == cudaStreamCaptureStatusNone && !small && smem <= 227 * 1024) {
         const exact_fn fn = nq < EXACT_PLAN_MIN ? exact_pick<Few>(k) : few ? exact_pick<Split>(k) : exact_pick<Grouped>(k);
@@ -799,7 +842,8 @@ extern "C" int frog_exact_search(const frog_index_t* index, const float* queries
             return FROG_OK;
         }
     }
-    const size_t smem1 = exact_smem<1>(k, A.d_pad);
+    const int pool_slots = k <= 32 ? 32 : k <= 64 ? 64 : k <= 128 ? 128 : k <= 256 ? 256 : 512;
+    const size_t smem1 = (size_t)A.d_pad * 4 + (size_t)EXACT_WARPS * pool_slots * 8;
     const exact_fn one = exact_pick<OnePerQuery>(k);
     FROG_CUDA_TRY(ready(one, smem1));
     one<<<nq, EXACT_WARPS * 32, smem1, s>>>(A);

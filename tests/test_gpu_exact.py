@@ -1,6 +1,6 @@
 """The exact filtered scan: grouped, split and one-CTA-per-query forms against the oracle's slab scan, at the
 edges of its pieces, pools and row lengths.  From 201 queries on they are grouped (on
-more than 8,192 objects), from 17 on planned by a kernel of their own."""
+small indexes only with k > 32), from 17 on planned by a kernel of their own."""
 import numpy as np
 import pytest
 
@@ -78,18 +78,18 @@ def test_groups_with_gaps_streams_and_capture(libs, tmp_path):
     a = np.sort(attrs)
     s = rng.integers(0, 29000, 1000)
     lo[3:], hi[3:] = a[s][3:], a[s + rng.integers(0, 900, 1000)][3:]
-    _check(gix, ix, q, lo, hi, 20)
-    _check(gix, ix, q, lo, hi, 20, graph=True)
-    _check(gix, ix, q[:5], lo[:5], hi[:5], 20, graph=True)
+    _check(gix, ix, q, lo, hi, 40)
+    _check(gix, ix, q, lo, hi, 40, graph=True)
+    _check(gix, ix, q[:5], lo[:5], hi[:5], 40, graph=True)
     dev = [torch.from_numpy(x).cuda() for x in (q, lo, hi)]
-    want = gix.exact_search(*dev, 20)
+    want = gix.exact_search(*dev, 40)
     streams = [torch.cuda.Stream() for _ in range(6)]
     torch.cuda.synchronize()
     got = []
     for i in range(24):
         with torch.cuda.stream(streams[i % 6]):
             n = (1000, 70, 7)[i % 3]
-            got.append(gix.exact_search(*(x[:n] for x in dev), 20))
+            got.append(gix.exact_search(*(x[:n] for x in dev), 40))
     torch.cuda.synchronize()
     for g in got:
         assert torch.equal(g[0], want[0][:len(g[0])]) and torch.equal(g[1], want[1][:len(g[0])])
