@@ -52,7 +52,7 @@ struct ExactArgs {
     int nq, k;
     int32_t* out_ids;
     float* out_dists;
-    // scratch (see ExactScratch); unused by the form with one CTA per query
+    // scratch (see exact_scratch); unused by the form with one CTA per query
     int2* ranges;
     int32_t* order;
     int4* jobs;                      // (group, first row, end row, -)
@@ -773,6 +773,78 @@ size_t exact_smem(int k, int d_pad) {
          : k <= 128 ? ExactSmem<4, G>::bytes(d_pad) : k <= 256 ? ExactSmem<8, G>::bytes(d_pad) : ExactSmem<16, G>::bytes(d_pad);
 }
 
+// A set for a scan on stream s: the one it used last, an idle one, a new one, or null when all are busy with other
+// streams' scans (the caller does without: a wait for another stream is not made here).  Called with exact_mu held.
+FrogExactSet* exact_set(frog_index* ix, cudaStream_t s) {
+    for (int i = 0; i < ix->n_exact; ++i)
+        if (ix->exact[i].used && ix->exact[i].stream == s) return &ix->exact[i];
+    for (int i = 0; i < ix->n_exact; ++i) {
+        FrogExactSet& set = ix->exact[i];
+        if (!set.used || cudaEventQuery(set.done) == cudaSuccess) return &set;
+        cudaGetLastError();
+    }
+    if (ix->n_exact == FROG_EXACT_SETS) return nullptr;
+    FrogExactSet& set = ix->exact[ix->n_exact];
+    if (cudaEventCreateWithFlags(&set.done, cudaEventDisableTiming) != cudaSuccess) {
+        cudaGetLastError();
+        return nullptr;
+    }
+    ++ix->n_exact;
+    return &set;
+}
+
+// Scratch for `nq` queries in `groups` groups, `jobs` pieces and `lists` partial keys; every part grows to the
+// largest asked for so far.  At rest the bins, `done` and `bound` are as they are set here: the kernels see to it.
+struct ExactScratch {
+    char* ranges;              // int2 per query
+    char* order;               // int per query
+    char* jobs;                // int4 per piece
+    char* groups;              // int2 per group
+    char* counters;            // EXACT_BINS + 2
+    char* done;                // int per group
+    char* bound;               // u64 per query
+    char* part;                // keys of the pieces' lists
+};
+int exact_scratch(FrogExactSet* set, size_t nq, size_t groups, size_t jobs, size_t lists, ExactScratch* out) {
+    const bool fits = set->mem && nq <= set->queries && groups <= set->groups && jobs <= set->jobs && lists <= set->lists;
+    nq = std::max(nq, set->queries);
+    groups = std::max(groups, set->groups);
+    jobs = std::max(jobs, set->jobs);
+    lists = std::max(lists, set->lists);
+    auto up = [](size_t x) { return (x + 255) & ~(size_t)255; };
+    const size_t b_bound = up(nq * 8), b_counters = up((EXACT_BINS + 2) * 4), b_done = up(groups * 4), b_ranges = up(nq * 8),
+                 b_order = up(nq * 4), b_jobs = up(jobs * 16), b_groups = up(groups * 8), b_part = up(lists * 8);
+    if (!fits) {
+        FROG_CUDA_TRY(cudaDeviceSynchronize());
+        if (set->mem) FROG_CUDA_TRY(cudaFree(set->mem));
+        set->mem = nullptr;
+        set->queries = set->groups = set->jobs = set->lists = 0;
+        const cudaError_t e = cudaMalloc(&set->mem, b_bound + b_counters + b_done + b_ranges + b_order + b_jobs + b_groups + b_part);
+        if (e != cudaSuccess) {
+            cudaGetLastError();
+            froghost::set_cuda_error(e);
+            set->mem = nullptr;
+            return FROG_ERR_NOMEM;
+        }
+        FROG_CUDA_TRY(cudaMemset(set->mem, 0xFF, b_bound));
+        FROG_CUDA_TRY(cudaMemset(set->mem + b_bound, 0, b_counters + b_done));
+        FROG_CUDA_TRY(cudaDeviceSynchronize());           // before a launch on any (non-blocking) stream
+        set->queries = nq;
+        set->groups = groups;
+        set->jobs = jobs;
+        set->lists = lists;
+    }
+    out->bound = set->mem;
+    out->counters = out->bound + b_bound;
+    out->done = out->counters + b_counters;
+    out->ranges = out->done + b_done;
+    out->order = out->ranges + b_ranges;
+    out->jobs = out->order + b_order;
+    out->groups = out->jobs + b_jobs;
+    out->part = out->groups + b_groups;
+    return FROG_OK;
+}
+
 }  // namespace
 
 extern "C" int frog_exact_search(const frog_index_t* index, const float* queries, const int32_t* lo,
@@ -815,30 +887,28 @@ extern "C" int frog_exact_search(const frog_index_t* index, const float* queries
         // enough pieces to even out their ends; fewer for long result lists, whose partial lists they multiply
         const int max_pieces = few ? 2 * grid + nq : grid * (k <= 128 ? 16 : 8);
         frog_index* mix = const_cast<frog_index*>(index);      // the scratch sets are the index's only mutable part
-        std::lock_guard<std::mutex> lock(mix->mu);
-        FrogScratch* sc = nullptr;
-        const int rc = froghost::acquire_scratch(mix, s, &sc);
-        if (rc) return rc;
-        froghost::ExactScratch X;
+        std::lock_guard<std::mutex> lock(mix->exact_mu);
+        FrogExactSet* set = exact_set(mix, s);
+        ExactScratch X;
         const size_t lists = (size_t)max_pieces * (few ? 1 : EXACT_GROUP) * k;
-        if (froghost::ensure_exact(sc, (size_t)nq, (size_t)groups, (size_t)max_pieces + groups, lists, EXACT_BINS + 2, &X) == FROG_OK) {
-            A.ranges = static_cast<int2*>(X.ranges);
-            A.order = X.order;
-            A.jobs = few ? nullptr : static_cast<int4*>(X.jobs);        // null: no histogram
-            A.groups = static_cast<int2*>(X.groups);
-            A.counters = X.counters;
-            A.done = X.done;
-            A.bound = X.bound;
-            A.part = X.part;
+        if (set && exact_scratch(set, (size_t)nq, (size_t)groups, (size_t)max_pieces + groups, lists, &X) == FROG_OK) {
+            A.ranges = reinterpret_cast<int2*>(X.ranges);
+            A.order = reinterpret_cast<int32_t*>(X.order);
+            A.jobs = few ? nullptr : reinterpret_cast<int4*>(X.jobs);        // null: no histogram
+            A.groups = reinterpret_cast<int2*>(X.groups);
+            A.counters = reinterpret_cast<unsigned int*>(X.counters);
+            A.done = reinterpret_cast<unsigned int*>(X.done);
+            A.bound = reinterpret_cast<unsigned long long*>(X.bound);
+            A.part = reinterpret_cast<uint64_t*>(X.part);
             A.max_pieces = max_pieces;
             A.min_rows = few ? 256 : 512;
             if (!few || nq >= EXACT_PLAN_MIN) frog_exact_plan_kernel<<<(nq * 32 + 255) / 256, 256, 0, s>>>(A);
             if (!few) frog_exact_cut_kernel<<<1, 1024, 0, s>>>(A);
             fn<<<grid, EXACT_WARPS * 32, smem, s>>>(A);
             FROG_CUDA_TRY(cudaGetLastError());
-            FROG_CUDA_TRY(cudaEventRecord(sc->done, s));
-            sc->stream = s;
-            sc->tick = ++mix->tick;
+            FROG_CUDA_TRY(cudaEventRecord(set->done, s));
+            set->stream = s;
+            set->used = true;
             return FROG_OK;
         }
     }

@@ -196,10 +196,13 @@ extern "C" void frog_index_free(frog_index_t* ix) {
             cudaFree(ix->scratch[i].d_bitmap);
             cudaFree(ix->scratch[i].d_table);
             cudaFree(ix->scratch[i].d_plan);
-            cudaFree(ix->scratch[i].d_exact);
             if (ix->scratch[i].done) cudaEventDestroy(ix->scratch[i].done);
             if (ix->scratch[i].k_begin) cudaEventDestroy(ix->scratch[i].k_begin);
             if (ix->scratch[i].k_end) cudaEventDestroy(ix->scratch[i].k_end);
+        }
+        for (int i = 0; i < ix->n_exact; ++i) {
+            cudaFree(ix->exact[i].mem);
+            cudaEventDestroy(ix->exact[i].done);
         }
         cudaFree(ix->d_stage);
     }

@@ -21,8 +21,6 @@ struct FrogScratch {
     size_t table_bytes = 0;
     int32_t* d_plan = nullptr;       // per query: rank interval (2 ints) and processing order (1 int)
     size_t plan_queries = 0;
-    char* d_exact = nullptr;         // scratch of the exact scan (ExactScratch), grown on demand
-    size_t exact_bytes = 0, exact_queries = 0, exact_groups = 0, exact_jobs = 0, exact_lists = 0;
     cudaEvent_t done = nullptr;
     cudaEvent_t k_begin = nullptr, k_end = nullptr;   // around the search kernel of the last timed launch
     bool k_timed = false;
@@ -30,6 +28,18 @@ struct FrogScratch {
     unsigned long long tick = 0;
 };
 constexpr int FROG_SCRATCH_SETS = 4;
+
+// One set of scratch of the exact scan (ExactScratch), grown on demand.  The scan has sets of its own: what the
+// library reports about the last search on a stream (frog_search_last_status, frog_search_kernel_ms) is kept in the
+// search's sets.
+struct FrogExactSet {
+    char* mem = nullptr;
+    size_t queries = 0, groups = 0, jobs = 0, lists = 0;     // what `mem` is cut for
+    cudaEvent_t done = nullptr;      // end of the last scan that used the set
+    cudaStream_t stream = nullptr;   // and its stream
+    bool used = false;
+};
+constexpr int FROG_EXACT_SETS = 4;
 constexpr int FROG_TABLE_BITS = 12;    // 4,096 ranks = 16 KB per resident warp: 78 MB for a full grid, inside L2
 constexpr int FROG_TABLE_BITS_WIDE = 13;   // beam widths 65..128: 8,192 ranks (a query evaluates ~2,000 there)
 
@@ -46,6 +56,9 @@ struct frog_index {
     int n_scratch = 0;
     unsigned long long tick = 0;     // launch counter, for least-recently-used selection
     std::mutex mu;                   // guards the scratch sets and the order of launches into them
+    FrogExactSet exact[FROG_EXACT_SETS];
+    int n_exact = 0;
+    std::mutex exact_mu;             // the same for the sets of the exact scan
     // Tensor maps of the two row stores for the 4-row gather of the copy engine (box = one row or
     // one 512-byte column chunk of it); absent when the driver entry point is missing or the row
     // shape does not qualify, in which case rows are copied one by one.
@@ -121,18 +134,6 @@ int acquire_scratch(frog_index* ix, cudaStream_t s, FrogScratch** out);
 int ensure_bitmap(const frog_index* ix, FrogScratch* sc, size_t slots);
 int ensure_table(FrogScratch* sc, size_t slots, int bits);
 int ensure_plan(FrogScratch* sc, size_t nq);
-// Scratch of one exact scan.  At rest `counters` and `done` are zero and `bound` is all ones.
-struct ExactScratch {
-    void* ranges;              // int2 per query
-    int32_t* order;            // per query
-    void* jobs;                // int4 per piece
-    void* groups;              // int2 per group
-    unsigned int* counters;
-    unsigned int* done;        // per group
-    unsigned long long* bound; // per query
-    uint64_t* part;            // keys of the pieces' lists
-};
-int ensure_exact(FrogScratch* sc, size_t nq, size_t groups, size_t jobs, size_t lists, size_t counters, ExactScratch* out);
 }  // namespace froghost
 
 #define FROG_CUDA_TRY(expr)                                  \

@@ -847,65 +847,6 @@ int ensure_plan(FrogScratch* sc, size_t nq) {
     return FROG_OK;
 }
 
-// Scratch of the exact scan for `nq` queries in `groups` groups, `jobs` pieces and `lists` partial keys;
-// every part grows to the largest asked for so far.  The kernels leave counters, done and bound as they are
-// set here.
-int ensure_exact(FrogScratch* sc, size_t nq, size_t groups, size_t jobs, size_t lists, size_t counters, ExactScratch* out) {
-    const bool fits = sc->d_exact && nq <= sc->exact_queries && groups <= sc->exact_groups && jobs <= sc->exact_jobs &&
-                      lists <= sc->exact_lists;
-    if (!fits) {
-        nq = nq > sc->exact_queries ? nq : sc->exact_queries;
-        groups = groups > sc->exact_groups ? groups : sc->exact_groups;
-        jobs = jobs > sc->exact_jobs ? jobs : sc->exact_jobs;
-        lists = lists > sc->exact_lists ? lists : sc->exact_lists;
-    } else {
-        nq = sc->exact_queries;
-        groups = sc->exact_groups;
-        jobs = sc->exact_jobs;
-        lists = sc->exact_lists;
-    }
-    auto up = [](size_t x) { return (x + 255) & ~(size_t)255; };
-    const size_t b_bound = up(nq * 8), b_zero = up(counters * 4) + up(groups * 4), b_ranges = up(nq * 8), b_order = up(nq * 4),
-                 b_jobs = up(jobs * 16), b_groups = up(groups * 8), b_part = up(lists * 8);
-    const size_t need = b_bound + b_zero + b_ranges + b_order + b_jobs + b_groups + b_part;
-    if (!fits) {
-        FROG_CUDA_TRY(cudaDeviceSynchronize());
-        if (sc->d_exact) FROG_CUDA_TRY(cudaFree(sc->d_exact));
-        sc->d_exact = nullptr;
-        sc->exact_bytes = sc->exact_queries = sc->exact_groups = sc->exact_jobs = sc->exact_lists = 0;
-        cudaError_t e = cudaMalloc(&sc->d_exact, need);
-        if (e != cudaSuccess) {
-            cudaGetLastError();
-            set_cuda_error(e);
-            return FROG_ERR_NOMEM;
-        }
-        FROG_CUDA_TRY(cudaMemset(sc->d_exact, 0xFF, b_bound));
-        FROG_CUDA_TRY(cudaMemset(sc->d_exact + b_bound, 0, b_zero));
-        FROG_CUDA_TRY(cudaDeviceSynchronize());           // before a launch on any (non-blocking) stream
-        sc->exact_bytes = need;
-        sc->exact_queries = nq;
-        sc->exact_groups = groups;
-        sc->exact_jobs = jobs;
-        sc->exact_lists = lists;
-    }
-    char* p = sc->d_exact;
-    out->bound = reinterpret_cast<unsigned long long*>(p);
-    p += b_bound;
-    out->counters = reinterpret_cast<unsigned int*>(p);
-    out->done = reinterpret_cast<unsigned int*>(p + up(counters * 4));
-    p += b_zero;
-    out->ranges = p;
-    p += b_ranges;
-    out->order = reinterpret_cast<int32_t*>(p);
-    p += b_order;
-    out->jobs = p;
-    p += b_jobs;
-    out->groups = p;
-    p += b_groups;
-    out->part = reinterpret_cast<uint64_t*>(p);
-    return FROG_OK;
-}
-
 }  // namespace froghost
 
 extern "C" int frog_search_launch_info(const frog_index_t* index, int beam_width, const frog_params_t* params,

@@ -94,3 +94,34 @@ def test_groups_with_gaps_streams_and_capture(libs, tmp_path):
     for g in got:
         assert torch.equal(g[0], want[0][:len(g[0])]) and torch.equal(g[1], want[1][:len(g[0])])
     gix.close()
+
+
+def test_reports_about_searches_are_left_alone(libs, tmp_path):
+    """last_status and kernel_ms speak of the last SEARCH on a stream: exact scans, on the same stream or on
+    another, with or without a search before them, change nothing about either."""
+    base, attrs, path = _index(libs, tmp_path, 3000, 16, 5)
+    q, lo, hi = _queries(base, attrs, 300, 6, 3)
+    dev = [torch.from_numpy(x).cuda() for x in (q, lo, hi)]
+    a, b, c = (torch.cuda.Stream() for _ in range(3))
+    torch.cuda.synchronize()
+
+    def refused(call):
+        with pytest.raises(libs.FrogError) as e:
+            call()
+        return e.value.code == 1
+
+    gix = libs.Index.load(path)
+    for n, k in ((3, 10), (100, 10), (300, 40)):
+        gix.exact_search(*(x[:n] for x in dev), k, stream=a)
+        a.synchronize()
+        assert refused(lambda: gix.last_status(stream=a)) and refused(lambda: gix.kernel_ms(stream=a))
+    gix.search(*dev, 10, 32, stream=b, params=libs.Params(debug_flags=16))
+    b.synchronize()
+    ms = gix.kernel_ms(stream=b)
+    for n, k in ((3, 10), (100, 10), (300, 40)):
+        for s in (b, c):
+            gix.exact_search(*(x[:n] for x in dev), k, stream=s)
+            s.synchronize()
+            assert gix.last_status(stream=b) == 0 and gix.kernel_ms(stream=b) == ms
+            assert refused(lambda: gix.last_status(stream=c)) and refused(lambda: gix.kernel_ms(stream=c))
+    gix.close()
