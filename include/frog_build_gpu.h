@@ -30,6 +30,8 @@ extern "C" {
  * resident warp; everything is released before returning.  Returns 0 or a FROG_ERR_* code
  * (1 invalid argument, 2 I/O, 4 out of memory, 5 CUDA error, 6 unsupported parameters).  If a bulk
  * copy of a kernel does not complete within its polling limit the call returns 5 and writes no file.
+ * A regular file gets its header last: what an interrupted or failed build leaves behind, of whatever
+ * length, is refused by frog_index_load.
  * Test hook: a nonzero value v in bits 16..31 of params->reserved makes the kernels issue no copy and
  * give up every wait after v polls, so that this report can be exercised without a fault. */
 int frog_index_build_gpu(const float* vectors, const int32_t* attrs, int64_t n, int32_t d,

@@ -20,6 +20,7 @@
 #include <vector>
 
 #include <sys/stat.h>
+#include <unistd.h>
 
 #include <thrust/execution_policy.h>
 #include <thrust/scan.h>
@@ -726,18 +727,23 @@ extern "C" int frog_index_build_gpu(const float* vectors, const int32_t* attrs, 
     std::memcpy(hdr + 72, offs, sizeof(offs));
     FILE* f = fopen(path, "wb");
     if (!f) return FROG_ERR_IO;
+    struct stat file;
+    const bool regular = fstat(fileno(f), &file) == 0 && S_ISREG(file.st_mode);
+    // The arrays of a regular file are written by several threads, out of order, so the length says nothing about
+    // how far they got: until all of them are there the header is zeros, which frog_index_load refuses.
+    const unsigned char unfinished[256] = {0};
     uint64_t pos = 256;
-    bool ok = write_all(f, hdr, 256) && write_all(f, sorted_attr.data(), (size_t)n * 4);
+    bool ok = write_all(f, regular ? unfinished : hdr, 256) && write_all(f, sorted_attr.data(), (size_t)n * 4);
     pos += nn * 4;
     ok = ok && pad_to(f, pos, off_r2i) && write_all(f, rank2id.data(), (size_t)n * 4);
     pos += nn * 4;
     ok = ok && pad_to(f, pos, off_vec) && fflush(f) == 0;
     rc = ok ? FROG_OK : FROG_ERR_IO;
-    struct stat file;
-    if (ok && fstat(fileno(f), &file) == 0 && S_ISREG(file.st_mode)) {
+    if (ok && regular) {
         // (the gap before the ENC array reads as zeros)
         const froghost::FileSection sections[2] = {{off_vec, dV, (size_t)n * d_pad * 4}, {off_enc, A.enc, nm * H * 4}};
         rc = froghost::transfer_sections(fileno(f), device, sections, 2, false);
+        if (rc == FROG_OK && pwrite(fileno(f), hdr, sizeof(hdr), 0) != (ssize_t)sizeof(hdr)) rc = FROG_ERR_IO;
     } else if (ok) {
         // not a file one can write out of order (a pipe): both arrays through host memory, in order
         std::unique_ptr<char[]> host(new (std::nothrow) char[std::max((size_t)n * d_pad, nm * H) * 4]);

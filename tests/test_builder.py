@@ -170,3 +170,14 @@ def test_odd_dimension_is_zero_padded(libs, cache_dir):
     res = oracle.search(ix, Q, lo, hi, 5, 32)
     gt, _, _ = oracle.exact_slab(ix, Q, lo, hi, 5)
     assert oracle.recall(res.ids, gt) > 0.8
+
+
+def test_a_file_without_its_header_is_refused(libs, tiny, tmp_path):
+    """The GPU builder writes the header last: zeros in its place mean an unfinished file."""
+    data = bytearray(open(tiny[1], "rb").read())
+    data[:256] = bytes(256)
+    p = tmp_path / "unfinished.idx"
+    p.write_bytes(data)
+    with pytest.raises(libs.FrogError) as e:
+        libs.Index.load(str(p))
+    assert e.value.code == 3
