@@ -776,8 +776,10 @@ size_t exact_smem(int k, int d_pad) {
 // A set for a scan on stream s: the one it used last, an idle one, a new one, or null when all are busy with other
 // streams' scans (the caller does without: a wait for another stream is not made here).  Called with exact_mu held.
 FrogExactSet* exact_set(frog_index* ix, cudaStream_t s) {
+    unsigned long long id = 0;
+    if (cudaStreamGetId(s, &id) != cudaSuccess) { cudaGetLastError(); return nullptr; }
     for (int i = 0; i < ix->n_exact; ++i)
-        if (ix->exact[i].used && ix->exact[i].stream == s) return &ix->exact[i];
+        if (ix->exact[i].used && ix->exact[i].stream_id == id) return &ix->exact[i];
     for (int i = 0; i < ix->n_exact; ++i) {
         FrogExactSet& set = ix->exact[i];
         if (!set.used || cudaEventQuery(set.done) == cudaSuccess) return &set;
@@ -907,7 +909,7 @@ extern "C" int frog_exact_search(const frog_index_t* index, const float* queries
             fn<<<grid, EXACT_WARPS * 32, smem, s>>>(A);
             FROG_CUDA_TRY(cudaGetLastError());
             FROG_CUDA_TRY(cudaEventRecord(set->done, s));
-            set->stream = s;
+            FROG_CUDA_TRY(cudaStreamGetId(s, &set->stream_id));
             set->used = true;
             return FROG_OK;
         }

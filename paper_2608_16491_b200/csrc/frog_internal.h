@@ -24,7 +24,10 @@ struct FrogScratch {
     cudaEvent_t done = nullptr;
     cudaEvent_t k_begin = nullptr, k_end = nullptr;   // around the search kernel of the last timed launch
     bool k_timed = false;
-    cudaStream_t stream = nullptr;   // stream of the last launch
+    // Stream of the last launch.  Only the id tells streams apart: a handle may name a new stream after its old one
+    // was destroyed, and the handle cudaStreamPerThread is another stream in every thread.
+    cudaStream_t stream = nullptr;
+    unsigned long long stream_id = 0;
     unsigned long long tick = 0;
 };
 constexpr int FROG_SCRATCH_SETS = 4;
@@ -36,7 +39,7 @@ struct FrogExactSet {
     char* mem = nullptr;
     size_t queries = 0, groups = 0, jobs = 0, lists = 0;     // what `mem` is cut for
     cudaEvent_t done = nullptr;      // end of the last scan that used the set
-    cudaStream_t stream = nullptr;   // and its stream
+    unsigned long long stream_id = 0;   // and its stream
     bool used = false;
 };
 constexpr int FROG_EXACT_SETS = 4;

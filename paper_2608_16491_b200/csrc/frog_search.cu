@@ -746,8 +746,10 @@ bool make_row_tensor_map(const void* base, bool f16, int row_elems, size_t row_b
 // to wait for the set that has been unused the longest.  Called with ix->mu held.
 int acquire_scratch(frog_index* ix, cudaStream_t s, FrogScratch** out) {
     FrogScratch* pick = nullptr;
+    unsigned long long id = 0;
+    FROG_CUDA_TRY(cudaStreamGetId(s, &id));
     for (int i = 0; i < ix->n_scratch && !pick; ++i)
-        if (ix->scratch[i].tick && ix->scratch[i].stream == s) pick = &ix->scratch[i];
+        if (ix->scratch[i].tick && ix->scratch[i].stream_id == id) pick = &ix->scratch[i];
     for (int i = 0; i < ix->n_scratch && !pick; ++i) {
         FrogScratch& sc = ix->scratch[i];
         if (!sc.tick) { pick = &sc; break; }
@@ -776,6 +778,7 @@ int acquire_scratch(frog_index* ix, cudaStream_t s, FrogScratch** out) {
             if (ix->scratch[i].tick < pick->tick) pick = &ix->scratch[i];
         FROG_CUDA_TRY(cudaStreamWaitEvent(s, pick->done, 0));
     }
+    pick->stream_id = id;
     *out = pick;
     return FROG_OK;
 }
@@ -984,38 +987,43 @@ extern "C" int frog_search_ex(const frog_index_t* index, const float* queries, c
     return FROG_OK;
 }
 
+namespace {
+// the set of the last search on stream s, or null.  By handle, which may be that of a stream no longer there, except
+// for the one handle that means another stream in every thread.
+FrogScratch* last_search_on(frog_index* ix, cudaStream_t s) {
+    unsigned long long id = 0;
+    if (s == cudaStreamPerThread && cudaStreamGetId(s, &id) != cudaSuccess) return nullptr;
+    FrogScratch* last = nullptr;
+    for (int i = 0; i < ix->n_scratch; ++i) {
+        FrogScratch& sc = ix->scratch[i];
+        if (sc.tick && sc.stream == s && (s != cudaStreamPerThread || sc.stream_id == id) && (!last || sc.tick > last->tick)) last = &sc;
+    }
+    return last;
+}
+}  // namespace
+
 extern "C" int frog_search_last_status(const frog_index_t* index, void* stream, uint32_t* flags) {
     if (!index || !flags) return FROG_ERR_INVALID_ARG;
     frog_index* mix = const_cast<frog_index*>(index);
     std::lock_guard<std::mutex> lock(mix->mu);
-    cudaStream_t s = static_cast<cudaStream_t>(stream);
-    for (int i = 0; i < mix->n_scratch; ++i) {
-        FrogScratch& sc = mix->scratch[i];
-        if (sc.tick && sc.stream == s) {
-            FROG_CUDA_TRY(cudaEventSynchronize(sc.done));
-            unsigned int word = 0;
-            FROG_CUDA_TRY(cudaMemcpy(&word, sc.d_work + 1, sizeof(word), cudaMemcpyDeviceToHost));
-            *flags = word;
-            return FROG_OK;
-        }
-    }
-    return FROG_ERR_INVALID_ARG;           // no launch on this stream
+    const FrogScratch* sc = last_search_on(mix, static_cast<cudaStream_t>(stream));
+    if (!sc) return FROG_ERR_INVALID_ARG;                  // no launch on this stream
+    FROG_CUDA_TRY(cudaEventSynchronize(sc->done));
+    unsigned int word = 0;
+    FROG_CUDA_TRY(cudaMemcpy(&word, sc->d_work + 1, sizeof(word), cudaMemcpyDeviceToHost));
+    *flags = word;
+    return FROG_OK;
 }
 
 extern "C" int frog_search_kernel_ms(const frog_index_t* index, void* stream, float* ms) {
     if (!index || !ms) return FROG_ERR_INVALID_ARG;
     frog_index* mix = const_cast<frog_index*>(index);
     std::lock_guard<std::mutex> lock(mix->mu);
-    cudaStream_t s = static_cast<cudaStream_t>(stream);
-    for (int i = 0; i < mix->n_scratch; ++i) {
-        FrogScratch& sc = mix->scratch[i];
-        if (sc.tick && sc.stream == s && sc.k_timed) {
-            FROG_CUDA_TRY(cudaEventSynchronize(sc.k_end));
-            FROG_CUDA_TRY(cudaEventElapsedTime(ms, sc.k_begin, sc.k_end));
-            return FROG_OK;
-        }
-    }
-    return FROG_ERR_INVALID_ARG;           // no timed launch on this stream
+    const FrogScratch* sc = last_search_on(mix, static_cast<cudaStream_t>(stream));
+    if (!sc || !sc->k_timed) return FROG_ERR_INVALID_ARG;  // no timed launch on this stream
+    FROG_CUDA_TRY(cudaEventSynchronize(sc->k_end));
+    FROG_CUDA_TRY(cudaEventElapsedTime(ms, sc->k_begin, sc->k_end));
+    return FROG_OK;
 }
 
 extern "C" int frog_search(const frog_index_t* index, const float* queries, const int32_t* lo, const int32_t* hi,

@@ -125,3 +125,59 @@ def test_reports_about_searches_are_left_alone(libs, tmp_path):
             assert gix.last_status(stream=b) == 0 and gix.kernel_ms(stream=b) == ms
             assert refused(lambda: gix.last_status(stream=c)) and refused(lambda: gix.kernel_ms(stream=c))
     gix.close()
+
+
+def test_the_per_thread_stream_is_another_stream_in_every_thread(libs, tmp_path):
+    """Four threads, each on its own per-thread default stream (one handle, four streams): scans and searches of
+    different batches do not share scratch."""
+    import threading
+    import types
+    per_thread = types.SimpleNamespace(cuda_stream=2)
+    base, attrs, path = _index(libs, tmp_path, 30000, 64, 9)
+    gix = libs.Index.load(path)
+    jobs = []
+    for i, nq in enumerate((700, 90, 300, 1500)):
+        dev = [torch.from_numpy(x).cuda() for x in _queries(base, attrs, nq, i, 5)]
+        out = [torch.empty((nq, 20), dtype=t, device="cuda") for t in (torch.int32, torch.float32)]
+        prm = libs.Params(visited=libs.VISITED_BITMAP)
+        want = gix.exact_search(*dev, 20), gix.search(*dev, 20, 24, params=prm)
+        jobs.append((dev, out, prm, want, []))
+    torch.cuda.synchronize()
+    gate = threading.Barrier(4)
+
+    def work(dev, out, prm, want, bad):
+        gate.wait()
+        for i in range(60):
+            if i % 2:
+                gix.exact_search(*dev, 20, out_ids=out[0], out_dists=out[1], stream=per_thread)
+            else:
+                gix.search(*dev, 20, 24, out_ids=out[0], out_dists=out[1], stream=per_thread, params=prm)
+            if i % 10 < 2:
+                torch.cuda.synchronize()
+                w = want[0 if i % 2 else 1]
+                if not (torch.equal(out[0], w[0]) and torch.equal(out[1], w[1])):
+                    bad.append(i)
+        bad.append("done")
+
+    threads = [threading.Thread(target=work, args=j) for j in jobs]
+    for t in threads:
+        t.start()
+    for t in threads:
+        t.join()
+    assert [j[4] for j in jobs] == [["done"]] * 4
+    # what is known about this thread's stream is not known about another's
+    gix.search(*jobs[0][0], 20, 24, stream=per_thread)
+    assert gix.last_status(stream=per_thread) == 0
+    codes = []
+
+    def ask():
+        try:
+            gix.last_status(stream=per_thread)
+        except libs.FrogError as e:
+            codes.append(e.code)
+
+    t = threading.Thread(target=ask)
+    t.start()
+    t.join()
+    assert codes == [1]
+    gix.close()
