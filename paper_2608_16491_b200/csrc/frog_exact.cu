@@ -638,9 +638,9 @@ __device__ __forceinline__ int exact_bin(const int2& lr, int n) {
 // slabs of the queries and the histogram of their bins (one warp per query)
 __global__ void __launch_bounds__(256)
 frog_exact_plan_kernel(const ExactArgs A) {
-    const int q = (int)((blockIdx.x * blockDim.x + threadIdx.x) >> 5);
+    const unsigned int q = blockIdx.x * 8u + (threadIdx.x >> 5);
     const int lane = lane_id();
-    if (q >= A.nq) return;
+    if (q >= (unsigned int)A.nq) return;
     const int32_t lo = __ldg(A.lo + q), hi = __ldg(A.hi + q);
     int l_q, r_q;
     warp_rank_interval(A.sorted_attr, A.n, lo, hi, lane, l_q, r_q);
@@ -879,7 +879,8 @@ extern "C" int frog_exact_search(const frog_index_t* index, const float* queries
     const bool few = nq < EXACT_GROUP_MIN;
     const bool small = !few && k <= EXACT_SMALL_K && index->info.n * A.d_pad * 4 <= EXACT_SMALL_BYTES;
     const size_t smem = few ? exact_smem<1>(k, A.d_pad) : exact_smem<EXACT_GROUP>(k, A.d_pad);
-    if (capture == cudaStreamCaptureStatusNone && !small && smem <= 227 * 1024) {
+    // (the planning kernels count queries in ints with some room)
+    if (capture == cudaStreamCaptureStatusNone && !small && smem <= 227 * 1024 && nq <= 1 << 30) {
         const exact_fn fn = nq < EXACT_PLAN_MIN ? exact_pick<Few>(k) : few ? exact_pick<Split>(k) : exact_pick<Grouped>(k);
         FROG_CUDA_TRY(ready(fn, smem));
         int per_sm = 0;
@@ -904,7 +905,7 @@ extern "C" int frog_exact_search(const frog_index_t* index, const float* queries
             A.part = reinterpret_cast<uint64_t*>(X.part);
             A.max_pieces = max_pieces;
             A.min_rows = few ? 256 : 512;
-            if (!few || nq >= EXACT_PLAN_MIN) frog_exact_plan_kernel<<<(nq * 32 + 255) / 256, 256, 0, s>>>(A);
+            if (!few || nq >= EXACT_PLAN_MIN) frog_exact_plan_kernel<<<(nq - 1) / 8 + 1, 256, 0, s>>>(A);
             if (!few) frog_exact_cut_kernel<<<1, 1024, 0, s>>>(A);
             fn<<<grid, EXACT_WARPS * 32, smem, s>>>(A);
             FROG_CUDA_TRY(cudaGetLastError());

@@ -465,9 +465,9 @@ constexpr int PLAN_HIST = 64, PLAN_CURSOR = 128;   // word offsets in the index'
 __global__ void __launch_bounds__(256)
 frog_plan_kernel(const int32_t* __restrict__ sorted_attr, int n, const int32_t* __restrict__ lo,
                  const int32_t* __restrict__ hi, int nq, int2* __restrict__ ranges, unsigned int* work) {
-    const int q = (int)((blockIdx.x * blockDim.x + threadIdx.x) >> 5);
+    const unsigned int q = blockIdx.x * 8u + (threadIdx.x >> 5);
     const int lane = lane_id();
-    if (q >= nq) return;
+    if (q >= (unsigned int)nq) return;
     const int32_t lo_q = __ldg(lo + q), hi_q = __ldg(hi + q);
     int l_q, r_q;
     warp_rank_interval(sorted_attr, n, lo_q, hi_q, lane, l_q, r_q);        // Sec. 4
@@ -482,15 +482,15 @@ frog_plan_kernel(const int32_t* __restrict__ sorted_attr, int n, const int32_t* 
 __global__ void __launch_bounds__(256)
 frog_order_kernel(const int32_t* __restrict__ lo, const int32_t* __restrict__ hi, int nq,
                   const int2* __restrict__ ranges, int32_t* __restrict__ order, unsigned int* work) {
-    const int q = (int)(blockIdx.x * blockDim.x + threadIdx.x);
-    if (q >= nq) return;
+    const unsigned int q = blockIdx.x * blockDim.x + threadIdx.x;
+    if (q >= (unsigned int)nq) return;
     const int2 lr = ranges[q];
     const int w = (__ldg(lo + q) > __ldg(hi + q)) ? 0 : (lr.y - lr.x + 1);
     const int bucket = w <= 0 ? 0 : 32 - __clz(w);
     unsigned int base = 0;
     for (int b = bucket + 1; b <= 32; ++b) base += work[PLAN_HIST + b];   // queries in heavier buckets
     const unsigned int pos = base + atomicAdd(work + PLAN_CURSOR + bucket, 1u);
-    order[pos] = q;
+    order[pos] = (int32_t)q;
 }
 
 typedef frog_kernel_fn kernel_fn;
@@ -966,8 +966,8 @@ extern "C" int frog_search_ex(const frog_index_t* index, const float* queries, c
     if (planned) {
         int2* ranges = reinterpret_cast<int2*>(sc->d_plan);
         int32_t* order = sc->d_plan + 2 * sc->plan_queries;
-        frog_plan_kernel<<<(nq * 32 + 255) / 256, 256, 0, s>>>(index->d_sorted_attr, A.n, lo, hi, nq, ranges, sc->d_work);
-        frog_order_kernel<<<(nq + 255) / 256, 256, 0, s>>>(lo, hi, nq, ranges, order, sc->d_work);
+        frog_plan_kernel<<<(nq - 1) / 8 + 1, 256, 0, s>>>(index->d_sorted_attr, A.n, lo, hi, nq, ranges, sc->d_work);
+        frog_order_kernel<<<(nq - 1) / 256 + 1, 256, 0, s>>>(lo, hi, nq, ranges, order, sc->d_work);
         A.ranges = ranges;
         A.order = order;
     }

@@ -181,3 +181,23 @@ def test_the_per_thread_stream_is_another_stream_in_every_thread(libs, tmp_path)
     t.join()
     assert codes == [1]
     gix.close()
+
+
+def test_more_queries_than_a_planning_kernel_has_32_bit_threads(libs, tmp_path):
+    """2^27 + 5 queries of one object each (one warp plans a query): as the same queries in small batches."""
+    n, nq = 300_000, (1 << 27) + 5
+    rng = np.random.default_rng(4)
+    base = rng.standard_normal((n, 4)).astype(np.float32)
+    path = str(tmp_path / "many.idx")
+    libs.build_index_gpu(base, np.arange(n, dtype=np.int32), path, m=4, ef_c=4, patience=1, n_inv=12)
+    gix = libs.Index.load(path)
+    g = torch.Generator(device="cuda").manual_seed(1)
+    q = torch.randn(nq, 4, generator=g, device="cuda")
+    lo = torch.randint(0, n, (nq,), generator=g, device="cuda", dtype=torch.int32)
+    some = torch.cat([torch.randint(0, nq, (150,), generator=g, device="cuda"),
+                      torch.tensor([0, 1, 1 << 26, (1 << 26) + 1, 1 << 27, nq - 1], device="cuda")])
+    for call in (lambda *a: gix.exact_search(*a, 1), lambda *a: gix.search(*a, 1, 1)):
+        ids, dists = call(q, lo, lo)
+        want = call(q[some].contiguous(), lo[some].contiguous(), lo[some].contiguous())
+        assert torch.equal(ids[:, 0], lo) and torch.equal(ids[some], want[0]) and torch.equal(dists[some], want[1])
+    gix.close()
