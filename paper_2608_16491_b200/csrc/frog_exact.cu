@@ -773,6 +773,14 @@ size_t exact_smem(int k, int d_pad) {
          : k <= 128 ? ExactSmem<4, G>::bytes(d_pad) : k <= 256 ? ExactSmem<8, G>::bytes(d_pad) : ExactSmem<16, G>::bytes(d_pad);
 }
 
+// While another thread captures a stream, event queries and allocations are refused and spoil its capture, unless the
+// calling thread says that they have nothing to do with it.
+struct NoCaptureOfOurs {
+    cudaStreamCaptureMode mode = cudaStreamCaptureModeRelaxed;
+    NoCaptureOfOurs() { cudaThreadExchangeStreamCaptureMode(&mode); }
+    ~NoCaptureOfOurs() { cudaThreadExchangeStreamCaptureMode(&mode); }
+};
+
 // A set for a scan on stream s: the one it used last, an idle one, a new one, or null when all are busy with other
 // streams' scans (the caller does without: a wait for another stream is not made here).  Called with exact_mu held.
 FrogExactSet* exact_set(frog_index* ix, cudaStream_t s) {
@@ -807,7 +815,7 @@ struct ExactScratch {
     char* bound;               // u64 per query
     char* part;                // keys of the pieces' lists
 };
-int exact_scratch(FrogExactSet* set, size_t nq, size_t groups, size_t jobs, size_t lists, ExactScratch* out) {
+bool exact_scratch(FrogExactSet* set, cudaStream_t s, size_t nq, size_t groups, size_t jobs, size_t lists, ExactScratch* out) {
     const bool fits = set->mem && nq <= set->queries && groups <= set->groups && jobs <= set->jobs && lists <= set->lists;
     nq = std::max(nq, set->queries);
     groups = std::max(groups, set->groups);
@@ -817,20 +825,19 @@ int exact_scratch(FrogExactSet* set, size_t nq, size_t groups, size_t jobs, size
     const size_t b_bound = up(nq * 8), b_counters = up((EXACT_BINS + 2) * 4), b_done = up(groups * 4), b_ranges = up(nq * 8),
                  b_order = up(nq * 4), b_jobs = up(jobs * 16), b_groups = up(groups * 8), b_part = up(lists * 8);
     if (!fits) {
-        FROG_CUDA_TRY(cudaDeviceSynchronize());
-        if (set->mem) FROG_CUDA_TRY(cudaFree(set->mem));
-        set->mem = nullptr;
-        set->queries = set->groups = set->jobs = set->lists = 0;
-        const cudaError_t e = cudaMalloc(&set->mem, b_bound + b_counters + b_done + b_ranges + b_order + b_jobs + b_groups + b_part);
-        if (e != cudaSuccess) {
+        char* mem = nullptr;
+        // (the set's last scan may still be running: on this stream, as a set is taken idle from another)
+        bool ok = cudaMalloc(&mem, b_bound + b_counters + b_done + b_ranges + b_order + b_jobs + b_groups + b_part) == cudaSuccess &&
+                  cudaMemsetAsync(mem, 0xFF, b_bound, s) == cudaSuccess &&
+                  cudaMemsetAsync(mem + b_bound, 0, b_counters + b_done, s) == cudaSuccess &&
+                  (!set->used || cudaEventSynchronize(set->done) == cudaSuccess);
+        if (!ok) {
             cudaGetLastError();
-            froghost::set_cuda_error(e);
-            set->mem = nullptr;
-            return FROG_ERR_NOMEM;
+            cudaFree(mem);
+            return false;                                  // the set stays as it is
         }
-        FROG_CUDA_TRY(cudaMemset(set->mem, 0xFF, b_bound));
-        FROG_CUDA_TRY(cudaMemset(set->mem + b_bound, 0, b_counters + b_done));
-        FROG_CUDA_TRY(cudaDeviceSynchronize());           // before a launch on any (non-blocking) stream
+        cudaFree(set->mem);
+        set->mem = mem;
         set->queries = nq;
         set->groups = groups;
         set->jobs = jobs;
@@ -844,7 +851,7 @@ int exact_scratch(FrogExactSet* set, size_t nq, size_t groups, size_t jobs, size
     out->jobs = out->order + b_order;
     out->groups = out->jobs + b_jobs;
     out->part = out->groups + b_groups;
-    return FROG_OK;
+    return true;
 }
 
 }  // namespace
@@ -891,10 +898,15 @@ extern "C" int frog_exact_search(const frog_index_t* index, const float* queries
         const int max_pieces = few ? 2 * grid + nq : grid * (k <= 128 ? 16 : 8);
         frog_index* mix = const_cast<frog_index*>(index);      // the scratch sets are the index's only mutable part
         std::lock_guard<std::mutex> lock(mix->exact_mu);
-        FrogExactSet* set = exact_set(mix, s);
-        ExactScratch X;
         const size_t lists = (size_t)max_pieces * (few ? 1 : EXACT_GROUP) * k;
-        if (set && exact_scratch(set, (size_t)nq, (size_t)groups, (size_t)max_pieces + groups, lists, &X) == FROG_OK) {
+        FrogExactSet* set = nullptr;
+        ExactScratch X;
+        {
+            const NoCaptureOfOurs relaxed;
+            set = exact_set(mix, s);
+            if (set && !exact_scratch(set, s, (size_t)nq, (size_t)groups, (size_t)max_pieces + groups, lists, &X)) set = nullptr;
+        }
+        if (set) {
             A.ranges = reinterpret_cast<int2*>(X.ranges);
             A.order = reinterpret_cast<int32_t*>(X.order);
             A.jobs = few ? nullptr : reinterpret_cast<int4*>(X.jobs);        // null: no histogram

@@ -201,3 +201,42 @@ def test_more_queries_than_a_planning_kernel_has_32_bit_threads(libs, tmp_path):
         want = call(q[some].contiguous(), lo[some].contiguous(), lo[some].contiguous())
         assert torch.equal(ids[:, 0], lo) and torch.equal(ids[some], want[0]) and torch.equal(dists[some], want[1])
     gix.close()
+
+
+def test_scans_beside_another_threads_capture(libs, tmp_path):
+    """A thread captures a graph; another one scans an index for the first time, which allocates.  The scan works
+    and the capture is not spoilt."""
+    import threading
+    base, attrs, path = _index(libs, tmp_path, 20000, 40, 3)
+    q, lo, hi = _queries(base, attrs, 400, 8, 5)
+    dev = [torch.from_numpy(x).cuda() for x in (q, lo, hi)]
+    gix, side = libs.Index.load(path), torch.cuda.Stream()
+    calls = ((400, 50), (100, 10), (5, 10), (400, 200))
+    want = [[t.cpu() for t in gix.exact_search(*(x[:n] for x in dev), k)] for n, k in calls]
+    gix.close()
+    gix = libs.Index.load(path)
+    parts = [[x[:n].contiguous() for x in dev] for n, _ in calls]
+    out = [[torch.empty((n, k), dtype=t, device="cuda") for t in (torch.int32, torch.float32)] for n, k in calls]
+    x, errors = torch.zeros(1000, device="cuda"), []
+    torch.cuda.synchronize()
+
+    def scan():
+        try:
+            for (n, k), p, o in zip(calls, parts, out):
+                gix.exact_search(*p, k, out_ids=o[0], out_dists=o[1], stream=side)
+        except libs.FrogError as e:
+            errors.append(e)
+
+    graph = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(graph, capture_error_mode="global"):
+        x += 1
+        t = threading.Thread(target=scan)
+        t.start()
+        t.join()
+        x += 1
+    graph.replay()
+    torch.cuda.synchronize()
+    assert not errors and float(x[0]) == 2.0
+    for o, w in zip(out, want):
+        assert torch.equal(o[0].cpu(), w[0]) and torch.equal(o[1].cpu(), w[1])
+    gix.close()
