@@ -185,9 +185,15 @@ int frog_search_ex(const frog_index_t* index, const float* queries, const int32_
 
 /* frog_exact_search: exact filtered kNN (Def. 2 of Sec. 2.1) by scanning the contiguous rank
  * slab of each query (Sec. 4: an attribute range is a contiguous rank interval).  The rows are cut into
- * pieces over the whole GPU and, from 16 queries on, shared by groups of eight; that uses scratch of the
- * index (see frog_search).  Under stream capture, and where scratch cannot be had, one CTA scans each
- * query.  Same buffers and conventions as frog_search; 1 <= k <= FROG_MAX_BEAM_WIDTH.  Used for ground truth
+ * pieces over the whole GPU: of one query each for up to 200 queries, of a group of eight queries that share
+ * them for more.  One CTA per query scans instead, without scratch: more than 200 queries with k <= 32 on an
+ * index of at most 4.5 MB of rows, rows too long for eight queries in shared memory, more than 2^30 queries,
+ * a call under stream capture, and a call whose scratch cannot be had.  The results are the same.
+ * Scratch: an index is loaded with what one stream's scans of up to 2,048 queries with k <= 128 need, but
+ * no more than a quarter of its own size; a scan on another stream, up to four in flight at once, or one that
+ * needs more allocates with cudaMalloc (0.5-3 ms, kept until frog_index_free) -- on indexes of up to 64 MB of
+ * rows only from the second such call on.  None of it is shared with frog_search.
+ * Same buffers and conventions as frog_search; 1 <= k <= FROG_MAX_BEAM_WIDTH.  Used for ground truth
  * and as the pre-filtering reference. */
 int frog_exact_search(const frog_index_t* index, const float* queries, const int32_t* lo, const int32_t* hi,
                       int nq, int k, int32_t* out_ids, float* out_dists, void* stream);

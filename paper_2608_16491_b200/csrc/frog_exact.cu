@@ -36,6 +36,7 @@ constexpr int EXACT_GROUP_MIN = 201;
 // 8,000 x 384, 600: 275/203; with k = 100 5,000 x 96, 600: 234/160).
 constexpr long long EXACT_SMALL_BYTES = 4500000;
 constexpr int EXACT_SMALL_K = 32;
+constexpr size_t EXACT_GROW_BYTES = (size_t)64 << 20;   // see exact_scratch
 constexpr int EXACT_PLAN_MIN = 17;       // from here on the slabs are found by a planning kernel (100,000 x 96, 16 queries: 49 without)
 constexpr int EXACT_STEP = 8 * EXACT_WARPS;    // rows per step of a CTA: two per team
 constexpr int EXACT_BUF = 256;           // keys buffered per query; merged from 64 on, two steps add at most 128
@@ -803,54 +804,82 @@ FrogExactSet* exact_set(frog_index* ix, cudaStream_t s) {
     return &set;
 }
 
-// Scratch for `nq` queries in `groups` groups, `jobs` pieces and `lists` partial keys; every part grows to the
-// largest asked for so far.  At rest the bins, `done` and `bound` are as they are set here: the kernels see to it.
+// How a call's rows are cut, and what that takes of scratch.  A piece holds at least `min_rows` rows of its query or
+// group, or all of them, so that small indexes and small batches need little; only groups (queries, where they are not
+// grouped) of several pieces have partial lists.
+struct ExactCut {
+    size_t groups;             // groups of queries, or queries
+    size_t pieces;             // with partial lists, at most
+    size_t lists;              // their keys
+    int max_pieces, min_rows;
+};
+ExactCut exact_cut_of(size_t n, size_t nq, int k, int grid, bool few) {
+    ExactCut c;
+    c.min_rows = few ? 256 : 512;
+    c.groups = few ? nq : (nq + EXACT_GROUP - 1) / EXACT_GROUP;
+    // enough pieces to even out their ends; fewer for long result lists, whose partial lists they multiply
+    const size_t most = few ? 2 * (size_t)grid + nq : (size_t)grid * (k <= 128 ? 16 : 8);
+    c.max_pieces = (int)most;
+    c.pieces = std::min(most, c.groups * ((n + c.min_rows - 1) / c.min_rows));
+    c.lists = c.pieces * (few ? 1 : EXACT_GROUP) * k;
+    return c;
+}
+
+// Scratch of one call.  At rest the bins, `done` and `bound` are as exact_scratch sets them: the kernels see to it.
 struct ExactScratch {
-    char* ranges;              // int2 per query
-    char* order;               // int per query
-    char* jobs;                // int4 per piece
-    char* groups;              // int2 per group
+    char* bound;               // u64 per query
     char* counters;            // EXACT_BINS + 2
     char* done;                // int per group
-    char* bound;               // u64 per query
+    char* ranges;              // int2 per query
+    char* order;               // int per query
+    char* groups;              // int2 per group
+    char* jobs;                // int4 per piece
     char* part;                // keys of the pieces' lists
 };
-bool exact_scratch(FrogExactSet* set, cudaStream_t s, size_t nq, size_t groups, size_t jobs, size_t lists, ExactScratch* out) {
-    const bool fits = set->mem && nq <= set->queries && groups <= set->groups && jobs <= set->jobs && lists <= set->lists;
-    nq = std::max(nq, set->queries);
-    groups = std::max(groups, set->groups);
-    jobs = std::max(jobs, set->jobs);
-    lists = std::max(lists, set->lists);
-    auto up = [](size_t x) { return (x + 255) & ~(size_t)255; };
-    const size_t b_bound = up(nq * 8), b_counters = up((EXACT_BINS + 2) * 4), b_done = up(groups * 4), b_ranges = up(nq * 8),
-                 b_order = up(nq * 4), b_jobs = up(jobs * 16), b_groups = up(groups * 8), b_part = up(lists * 8);
-    if (!fits) {
+size_t up256(size_t x) { return (x + 255) & ~(size_t)255; }
+size_t exact_rest_bytes(size_t queries) { return up256(queries * 8) + up256((EXACT_BINS + 2) * 4) + up256(queries * 4); }
+size_t exact_bytes(size_t nq, const ExactCut& c, bool few) {
+    return up256(nq * 8) + (few ? 0 : up256(nq * 4) + up256(c.groups * 8) + up256((c.pieces + c.groups) * 16)) + up256(c.lists * 8);
+}
+bool exact_scratch(frog_index* ix, FrogExactSet* set, cudaStream_t s, size_t nq, const ExactCut& c, bool few, ExactScratch* out) {
+    const size_t bytes = exact_bytes(nq, c, few);
+    if (!set->mem || nq > set->queries || bytes > set->bytes) {
+        // Growing takes 0.5-3 ms; on an index this small one scan without scratch costs less than that (up to 64 MB of
+        // rows: 2-3 ms at most for 2,000 queries), so it waits for a second scan that could use it.
+        if (!ix->exact_asked && (size_t)ix->info.n * ix->info.d_pad * 4 <= EXACT_GROW_BYTES) {
+            ix->exact_asked = true;
+            return false;
+        }
+        const size_t new_queries = std::max(nq, set->queries), new_bytes = std::max(bytes, set->bytes);
         char* mem = nullptr;
         // (the set's last scan may still be running: on this stream, as a set is taken idle from another)
-        bool ok = cudaMalloc(&mem, b_bound + b_counters + b_done + b_ranges + b_order + b_jobs + b_groups + b_part) == cudaSuccess &&
-                  cudaMemsetAsync(mem, 0xFF, b_bound, s) == cudaSuccess &&
-                  cudaMemsetAsync(mem + b_bound, 0, b_counters + b_done, s) == cudaSuccess &&
-                  (!set->used || cudaEventSynchronize(set->done) == cudaSuccess);
-        if (!ok) {
+        if (cudaMalloc(&mem, exact_rest_bytes(new_queries) + new_bytes) != cudaSuccess ||
+            (set->used && cudaEventSynchronize(set->done) != cudaSuccess)) {
             cudaGetLastError();
             cudaFree(mem);
             return false;                                  // the set stays as it is
         }
         cudaFree(set->mem);
         set->mem = mem;
-        set->queries = nq;
-        set->groups = groups;
-        set->jobs = jobs;
-        set->lists = lists;
+        set->queries = new_queries;
+        set->bytes = new_bytes;
+        set->clean = false;
     }
     out->bound = set->mem;
-    out->counters = out->bound + b_bound;
-    out->done = out->counters + b_counters;
-    out->ranges = out->done + b_done;
-    out->order = out->ranges + b_ranges;
-    out->jobs = out->order + b_order;
-    out->groups = out->jobs + b_jobs;
-    out->part = out->groups + b_groups;
+    out->counters = out->bound + up256(set->queries * 8);
+    out->done = out->counters + up256((EXACT_BINS + 2) * 4);
+    out->ranges = set->mem + exact_rest_bytes(set->queries);
+    out->order = out->ranges + up256(nq * 8);
+    out->groups = out->order + (few ? 0 : up256(nq * 4));
+    out->jobs = out->groups + (few ? 0 : up256(c.groups * 8));
+    out->part = out->jobs + (few ? 0 : up256((c.pieces + c.groups) * 16));
+    if (!set->clean) {
+        if (cudaMemsetAsync(out->bound, 0xFF, out->counters - out->bound, s) != cudaSuccess ||
+            cudaMemsetAsync(out->counters, 0, out->ranges - out->counters, s) != cudaSuccess) {
+            cudaGetLastError();
+            return false;
+        }
+    }
     return true;
 }
 
@@ -893,18 +922,15 @@ extern "C" int frog_exact_search(const frog_index_t* index, const float* queries
         int per_sm = 0;
         FROG_CUDA_TRY(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, (const void*)fn, EXACT_WARPS * 32, smem));
         const int grid = std::max(per_sm, 1) * index->sm_count;
-        const int groups = few ? nq : (nq + EXACT_GROUP - 1) / EXACT_GROUP;
-        // enough pieces to even out their ends; fewer for long result lists, whose partial lists they multiply
-        const int max_pieces = few ? 2 * grid + nq : grid * (k <= 128 ? 16 : 8);
+        const ExactCut cut = exact_cut_of((size_t)index->info.n, (size_t)nq, k, grid, few);
         frog_index* mix = const_cast<frog_index*>(index);      // the scratch sets are the index's only mutable part
         std::lock_guard<std::mutex> lock(mix->exact_mu);
-        const size_t lists = (size_t)max_pieces * (few ? 1 : EXACT_GROUP) * k;
         FrogExactSet* set = nullptr;
         ExactScratch X;
         {
             const NoCaptureOfOurs relaxed;
             set = exact_set(mix, s);
-            if (set && !exact_scratch(set, s, (size_t)nq, (size_t)groups, (size_t)max_pieces + groups, lists, &X)) set = nullptr;
+            if (set && !exact_scratch(mix, set, s, (size_t)nq, cut, few, &X)) set = nullptr;
         }
         if (set) {
             A.ranges = reinterpret_cast<int2*>(X.ranges);
@@ -915,12 +941,14 @@ extern "C" int frog_exact_search(const frog_index_t* index, const float* queries
             A.done = reinterpret_cast<unsigned int*>(X.done);
             A.bound = reinterpret_cast<unsigned long long*>(X.bound);
             A.part = reinterpret_cast<uint64_t*>(X.part);
-            A.max_pieces = max_pieces;
-            A.min_rows = few ? 256 : 512;
+            A.max_pieces = cut.max_pieces;
+            A.min_rows = cut.min_rows;
+            set->clean = false;                            // until the launches are under way
             if (!few || nq >= EXACT_PLAN_MIN) frog_exact_plan_kernel<<<(nq - 1) / 8 + 1, 256, 0, s>>>(A);
             if (!few) frog_exact_cut_kernel<<<1, 1024, 0, s>>>(A);
             fn<<<grid, EXACT_WARPS * 32, smem, s>>>(A);
             FROG_CUDA_TRY(cudaGetLastError());
+            set->clean = true;
             FROG_CUDA_TRY(cudaEventRecord(set->done, s));
             FROG_CUDA_TRY(cudaStreamGetId(s, &set->stream_id));
             set->used = true;
@@ -934,4 +962,24 @@ extern "C" int frog_exact_search(const frog_index_t* index, const float* queries
     one<<<nq, EXACT_WARPS * 32, smem1, s>>>(A);
     FROG_CUDA_TRY(cudaGetLastError());
     return FROG_OK;
+}
+
+// Scratch for one stream's scans of up to 2,048 queries with k up to 128, but no more than a quarter of the index, so that
+// a first scan has nothing to allocate as a rule.  Not having it is no error.
+void froghost::reserve_exact(frog_index* ix) {
+    const ExactCut cut = exact_cut_of((size_t)ix->info.n, 2048, 128, 2 * ix->sm_count, false);
+    const size_t bytes = std::min(exact_bytes(2048, cut, false), (size_t)ix->info.device_bytes / 4);
+    FrogExactSet& set = ix->exact[0];
+    if (cudaEventCreateWithFlags(&set.done, cudaEventDisableTiming) != cudaSuccess) {
+        cudaGetLastError();
+        return;
+    }
+    ix->n_exact = 1;
+    if (cudaMalloc(&set.mem, exact_rest_bytes(2048) + bytes) != cudaSuccess) {
+        cudaGetLastError();
+        set.mem = nullptr;
+        return;
+    }
+    set.queries = 2048;
+    set.bytes = bytes;
 }

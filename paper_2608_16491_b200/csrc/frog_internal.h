@@ -32,12 +32,12 @@ struct FrogScratch {
 };
 constexpr int FROG_SCRATCH_SETS = 4;
 
-// One set of scratch of the exact scan (ExactScratch), grown on demand.  The scan has sets of its own: what the
-// library reports about the last search on a stream (frog_search_last_status, frog_search_kernel_ms) is kept in the
-// search's sets.
+// One set of scratch of the exact scan.  The scan has sets of its own: what the library reports about the last search
+// on a stream (frog_search_last_status, frog_search_kernel_ms) is kept in the search's sets.
 struct FrogExactSet {
-    char* mem = nullptr;
-    size_t queries = 0, groups = 0, jobs = 0, lists = 0;     // what `mem` is cut for
+    char* mem = nullptr;             // see exact_scratch
+    size_t queries = 0, bytes = 0;   // what `mem` is cut for: queries, bytes of everything that has no state at rest
+    bool clean = false;              // the part that has one is set
     cudaEvent_t done = nullptr;      // end of the last scan that used the set
     unsigned long long stream_id = 0;   // and its stream
     bool used = false;
@@ -61,6 +61,7 @@ struct frog_index {
     std::mutex mu;                   // guards the scratch sets and the order of launches into them
     FrogExactSet exact[FROG_EXACT_SETS];
     int n_exact = 0;
+    bool exact_asked = false;        // a scan would have needed more scratch than there is
     std::mutex exact_mu;             // the same for the sets of the exact scan
     // Tensor maps of the two row stores for the 4-row gather of the copy engine (box = one row or
     // one 512-byte column chunk of it); absent when the driver entry point is missing or the row
@@ -137,6 +138,7 @@ int acquire_scratch(frog_index* ix, cudaStream_t s, FrogScratch** out);
 int ensure_bitmap(const frog_index* ix, FrogScratch* sc, size_t slots);
 int ensure_table(FrogScratch* sc, size_t slots, int bits);
 int ensure_plan(FrogScratch* sc, size_t nq);
+void reserve_exact(frog_index* ix);     // frog_exact.cu: scratch that covers common scans, for a new index
 }  // namespace froghost
 
 #define FROG_CUDA_TRY(expr)                                  \

@@ -45,6 +45,7 @@ def _check(gix, ix, q, lo, hi, k, graph=False):
             gix.exact_search(*dev, k, out_ids=out[0], out_dists=out[1])
         g.replay()
     else:
+        gix.exact_search(*dev, k)                                        # a first call may do without its scratch
         out = gix.exact_search(*dev, k)
     torch.cuda.synchronize()
     ids, dists = oracle.exact_slab(ix, q, lo, hi, k, mode=1)[:2]
@@ -240,3 +241,26 @@ def test_scans_beside_another_threads_capture(libs, tmp_path):
     for o, w in zip(out, want):
         assert torch.equal(o[0].cpu(), w[0]) and torch.equal(o[1].cpu(), w[1])
     gix.close()
+
+
+def test_a_first_scan_of_common_size_allocates_nothing(libs, tmp_path):
+    """The scratch of up to 2,048 queries with k up to 128 comes with the index, as far as a quarter of its size."""
+    base, attrs, path = _index(libs, tmp_path, 50000, 96, 3)
+    ix = oracle.load_index(path)
+    q, lo, hi = _queries(base, attrs, 2048, 8, 6)
+    dev = [torch.from_numpy(x).cuda() for x in (q, lo, hi)]
+    for nq, k in ((1, 10), (16, 128), (200, 128), (500, 10), (2048, 10)):
+        gix = libs.Index.load(path)
+        out = [torch.empty((nq, k), dtype=t, device="cuda") for t in (torch.int32, torch.float32)]
+        part = [x[:nq] for x in dev]
+        if nq == 1:                                         # the library's kernels are loaded
+            gix.exact_search(*(x[:600] for x in dev), 100)
+            gix.exact_search(*(x[:100] for x in dev), 100)
+        torch.cuda.synchronize()
+        before = torch.cuda.mem_get_info()[0]
+        gix.exact_search(*part, k, out_ids=out[0], out_dists=out[1])
+        torch.cuda.synchronize()
+        assert torch.cuda.mem_get_info()[0] == before
+        ids, _ = oracle.exact_slab(ix, q[:nq], lo[:nq], hi[:nq], k, mode=1)[:2]
+        assert np.array_equal(out[0].cpu().numpy(), ids)
+        gix.close()
