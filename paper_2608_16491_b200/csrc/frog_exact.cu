@@ -77,7 +77,7 @@ struct ExactSmem {
     int* misc;           // 8
     float4* q;           // G x d_pad floats
     static constexpr size_t FIXED = (size_t)G * (32 * EPL + EXACT_BUF + 1) * 8 + (size_t)G * 16 + 32;
-    static size_t bytes(int d_pad) { return (FIXED + 15) / 16 * 16 + (size_t)G * d_pad * 4; }
+    static __host__ __device__ size_t bytes(int d_pad) { return (FIXED + 15) / 16 * 16 + (size_t)G * d_pad * 4; }
     __device__ __forceinline__ explicit ExactSmem(unsigned char* base) {
         pool = reinterpret_cast<uint64_t*>(base);
         buf = pool + G * 32 * EPL;
@@ -498,12 +498,22 @@ frog_exact_kernel(const ExactArgs A) {
     }
 }
 
+// what the two kernels that do not group keep behind the scan's shared memory
+struct FewExtra {
+    int2 slab[EXACT_PLAN_MIN];
+};
+struct SplitExtra {
+    unsigned long long rows;
+    int first[EXACT_GROUP_MIN + 1];                          // first piece of each query
+    int warp_sum[EXACT_WARPS];
+};
+
 // Fewer than EXACT_PLAN_MIN queries: all rows cut into equal pieces, at most one per CTA.
 template <int EPL>
 __global__ void __launch_bounds__(EXACT_WARPS * 32, 2)
 frog_exact_few_kernel(const ExactArgs A) {
     extern __shared__ __align__(16) unsigned char smem_raw[];
-    __shared__ int2 slab[EXACT_PLAN_MIN];
+    int2* const slab = reinterpret_cast<FewExtra*>(smem_raw + ExactSmem<EPL, 1>::bytes(A.d_pad))->slab;
     const ExactSmem<EPL, 1> S(smem_raw);
     const int lane = lane_id(), warp = threadIdx.x >> 5;
     for (int q = warp; q < A.nq; q += EXACT_WARPS) {
@@ -544,9 +554,9 @@ template <int EPL>
 __global__ void __launch_bounds__(EXACT_WARPS * 32, 2)
 frog_exact_split_kernel(const ExactArgs A) {
     extern __shared__ __align__(16) unsigned char smem_raw[];
-    __shared__ int first[EXACT_GROUP_MIN + 1];               // first piece of each query
-    __shared__ int warp_sum[EXACT_WARPS];
-    __shared__ unsigned long long rows;
+    SplitExtra& X = *reinterpret_cast<SplitExtra*>(smem_raw + ExactSmem<EPL, 1>::bytes(A.d_pad));
+    unsigned long long& rows = X.rows;
+    int *const first = X.first, *const warp_sum = X.warp_sum;
     const ExactSmem<EPL, 1> S(smem_raw);
     const int lane = lane_id(), warp = threadIdx.x >> 5, t = threadIdx.x;
     if (t == 0) rows = 0;
@@ -914,7 +924,8 @@ extern "C" int frog_exact_search(const frog_index_t* index, const float* queries
     FROG_CUDA_TRY(cudaStreamIsCapturing(s, &capture));
     const bool few = nq < EXACT_GROUP_MIN;
     const bool small = !few && k <= EXACT_SMALL_K && index->info.n * A.d_pad * 4 <= EXACT_SMALL_BYTES;
-    const size_t smem = few ? exact_smem<1>(k, A.d_pad) : exact_smem<EXACT_GROUP>(k, A.d_pad);
+    const size_t smem = !few ? exact_smem<EXACT_GROUP>(k, A.d_pad)
+                             : exact_smem<1>(k, A.d_pad) + (nq < EXACT_PLAN_MIN ? sizeof(FewExtra) : sizeof(SplitExtra));
     // (the planning kernels count queries in ints with some room)
     if (capture == cudaStreamCaptureStatusNone && !small && smem <= 227 * 1024 && nq <= 1 << 30) {
         const exact_fn fn = nq < EXACT_PLAN_MIN ? exact_pick<Few>(k) : few ? exact_pick<Split>(k) : exact_pick<Grouped>(k);

@@ -264,3 +264,17 @@ def test_a_first_scan_of_common_size_allocates_nothing(libs, tmp_path):
         ids, _ = oracle.exact_slab(ix, q[:nq], lo[:nq], hi[:nq], k, mode=1)[:2]
         assert np.array_equal(out[0].cpu().numpy(), ids)
         gix.close()
+
+
+@pytest.mark.parametrize("d", [57300, 57520])
+def test_the_longest_rows_that_fit_one_query(libs, tmp_path, d):
+    """Rows of 229,200 and 230,080 bytes: the scan without pieces needs 2,048 bytes of shared memory besides."""
+    rng = np.random.default_rng(d)
+    base = rng.integers(0, 3, (40, d)).astype(np.float32)
+    path = str(tmp_path / "long.idx")
+    libs.build_index(base, rng.integers(0, 20, 40).astype(np.int32), path, m=4, ef_c=4, n_inv=30)
+    ix, gix = oracle.load_index(path), libs.Index.load(path)
+    for nq in (3, 40):
+        lo = rng.integers(0, 15, nq).astype(np.int32)
+        _check(gix, ix, rng.integers(0, 3, (nq, d)).astype(np.float32), lo, lo + 5, 10)
+    gix.close()
