@@ -647,20 +647,20 @@ extern "C" int frog_index_build_gpu(const float* vectors, const int32_t* attrs, 
     void (*search_fn)(const BuildArgs) = spool_slots == 32 ? sibling_search_kernel<1>
                                        : spool_slots == 64 ? sibling_search_kernel<2>
                                        : spool_slots == 128 ? sibling_search_kernel<4> : sibling_search_kernel<8>;
-    if (smem_search > 227 * 1024) return FROG_ERR_UNSUPPORTED;
+    if (smem_search > froghost::MAX_SMEM) return FROG_ERR_UNSUPPORTED;
     // the selection stages all 64 rows where they fit; about 16 warps per SM share its shared memory, and a CTA
     // is given more of them the fewer CTAs that leaves room for
-    const bool staged = sel_bytes(d_pad, true) <= 227 * 1024;
+    const bool staged = sel_bytes(d_pad, true) <= froghost::MAX_SMEM;
     const size_t smem_sel = sel_bytes(d_pad, staged);
-    const int sel_ctas = std::max<int>(1, (int)(227 * 1024 / (smem_sel + 1024)));
+    const int sel_ctas = std::max<int>(1, (int)(froghost::MAX_SMEM / (smem_sel + 1024)));
     const int sel_warps = std::min(SEL_MAX_WARPS, std::max(SEL_MIN_WARPS, 16 / sel_ctas));
     void (*sel0)(const BuildArgs) = staged ? select_kernel<false, true> : select_kernel<false, false>;
     void (*sel1)(const BuildArgs) = staged ? select_kernel<true, true> : select_kernel<true, false>;
-    FROG_CUDA_TRY(cudaFuncSetAttribute((const void*)leaf_cand_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem_plain));
-    FROG_CUDA_TRY(cudaFuncSetAttribute((const void*)pool_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem_plain));
-    FROG_CUDA_TRY(cudaFuncSetAttribute((const void*)search_fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem_search));
-    FROG_CUDA_TRY(cudaFuncSetAttribute((const void*)sel0, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem_sel));
-    FROG_CUDA_TRY(cudaFuncSetAttribute((const void*)sel1, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem_sel));
+    FROG_CUDA_TRY(froghost::allow_smem(leaf_cand_kernel));
+    FROG_CUDA_TRY(froghost::allow_smem(pool_kernel));
+    FROG_CUDA_TRY(froghost::allow_smem(search_fn));
+    FROG_CUDA_TRY(froghost::allow_smem(sel0));
+    FROG_CUDA_TRY(froghost::allow_smem(sel1));
     auto grid_for = [&](const void* fn, int threads, size_t smem, int per_cta) {
         int per_sm = 1;
         cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, fn, threads, smem);

@@ -917,9 +917,6 @@ extern "C" int frog_exact_search(const frog_index_t* index, const float* queries
     A.k = k;
     A.out_ids = out_ids;
     A.out_dists = out_dists;
-    auto ready = [&](exact_fn fn, size_t smem) {
-        return cudaFuncSetAttribute((const void*)fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    };
     cudaStreamCaptureStatus capture = cudaStreamCaptureStatusNone;
     FROG_CUDA_TRY(cudaStreamIsCapturing(s, &capture));
     const bool few = nq < EXACT_GROUP_MIN;
@@ -927,9 +924,9 @@ extern "C" int frog_exact_search(const frog_index_t* index, const float* queries
     const size_t smem = !few ? exact_smem<EXACT_GROUP>(k, A.d_pad)
                              : exact_smem<1>(k, A.d_pad) + (nq < EXACT_PLAN_MIN ? sizeof(FewExtra) : sizeof(SplitExtra));
     // (the planning kernels count queries in ints with some room)
-    if (capture == cudaStreamCaptureStatusNone && !small && smem <= 227 * 1024 && nq <= 1 << 30) {
+    if (capture == cudaStreamCaptureStatusNone && !small && smem <= froghost::MAX_SMEM && nq <= 1 << 30) {
         const exact_fn fn = nq < EXACT_PLAN_MIN ? exact_pick<Few>(k) : few ? exact_pick<Split>(k) : exact_pick<Grouped>(k);
-        FROG_CUDA_TRY(ready(fn, smem));
+        FROG_CUDA_TRY(froghost::allow_smem(fn));
         int per_sm = 0;
         FROG_CUDA_TRY(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, (const void*)fn, EXACT_WARPS * 32, smem));
         const int grid = std::max(per_sm, 1) * index->sm_count;
@@ -969,7 +966,7 @@ extern "C" int frog_exact_search(const frog_index_t* index, const float* queries
     const int pool_slots = k <= 32 ? 32 : k <= 64 ? 64 : k <= 128 ? 128 : k <= 256 ? 256 : 512;
     const size_t smem1 = (size_t)A.d_pad * 4 + (size_t)EXACT_WARPS * pool_slots * 8;
     const exact_fn one = exact_pick<OnePerQuery>(k);
-    FROG_CUDA_TRY(ready(one, smem1));
+    FROG_CUDA_TRY(froghost::allow_smem(one));
     one<<<nq, EXACT_WARPS * 32, smem1, s>>>(A);
     FROG_CUDA_TRY(cudaGetLastError());
     return FROG_OK;

@@ -119,6 +119,13 @@ struct FrogSearchArgs {
 typedef void (*frog_kernel_fn)(const FrogSearchArgs);
 
 namespace froghost {
+// Every kernel may use what a CTA can have of dynamic shared memory (none has static shared memory).  Always the same
+// limit: set to what a call needs, it would be lowered by one thread between another's setting and its launch.
+constexpr int MAX_SMEM = 227 * 1024;
+template <class F>
+cudaError_t allow_smem(F* fn) {
+    return cudaFuncSetAttribute((const void*)fn, cudaFuncAttributeMaxDynamicSharedMemorySize, MAX_SMEM);
+}
 // frog_search_lean.cu: the trimmed kernel for 384- and 512-byte fp32 and 192- and 256-byte fp16 rows (null: shape not covered)
 frog_kernel_fn lean_kernel(int ef_s, int budget, int row_bytes, bool f16, bool table, bool hook, int queries_per_sm,
                            size_t* smem_per_warp, int* warps_per_cta);

@@ -587,8 +587,8 @@ int plan_launch(const frog_index* ix, int beam_width, const frog_params_t& P, in
             table = false;
         }
     }
-    if (smem > 227 * 1024) return FROG_ERR_UNSUPPORTED;
-    FROG_CUDA_TRY(cudaFuncSetAttribute((const void*)fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+    if (smem > froghost::MAX_SMEM) return FROG_ERR_UNSUPPORTED;
+    FROG_CUDA_TRY(froghost::allow_smem(fn));
     int per_sm = 0;
     FROG_CUDA_TRY(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, (const void*)fn, WARPS_PER_CTA * 32, smem));
     if (per_sm < 1) return FROG_ERR_UNSUPPORTED;
@@ -633,8 +633,8 @@ int plan_team(const frog_index* ix, int beam_width, const frog_params_t& P, int 
     while (bits < (warps == 8 ? 13 : 12) && (1 << bits) < 16 * beam_width) ++bits;
     size_t smem = 0;
     kernel_fn fn = froghost::team_kernel(warps, beam_width, q_len, bits, f16, &smem);
-    if (smem > 227 * 1024) return FROG_ERR_UNSUPPORTED;
-    FROG_CUDA_TRY(cudaFuncSetAttribute((const void*)fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+    if (smem > froghost::MAX_SMEM) return FROG_ERR_UNSUPPORTED;
+    FROG_CUDA_TRY(froghost::allow_smem(fn));
     int per_sm = 0;
     FROG_CUDA_TRY(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, (const void*)fn, warps * 32, smem));
     if (per_sm < 1) return FROG_ERR_UNSUPPORTED;

@@ -278,3 +278,44 @@ def test_the_longest_rows_that_fit_one_query(libs, tmp_path, d):
         lo = rng.integers(0, 15, nq).astype(np.int32)
         _check(gix, ix, rng.integers(0, 3, (nq, d)).astype(np.float32), lo, lo + 5, 10)
     gix.close()
+
+
+def test_two_threads_whose_calls_need_different_shared_memory(libs, tmp_path):
+    """Long and short rows through the same kernels: what one thread allows a kernel, the other does not take back."""
+    import threading
+    work = []
+    for d, n in ((3000, 300), (40, 2000)):
+        rng = np.random.default_rng(d)
+        base = rng.standard_normal((n, d)).astype(np.float32)
+        path = str(tmp_path / ("sm%d.idx" % d))
+        libs.build_index(base, np.arange(n, dtype=np.int32), path, m=4, ef_c=4, n_inv=30)
+        gix = libs.Index.load(path)
+        q = torch.from_numpy(base[:300]).cuda()
+        lo, hi = torch.zeros(300, dtype=torch.int32, device="cuda"), torch.full((300,), n, dtype=torch.int32, device="cuda")
+        calls = []
+        for nq, k, beam in ((300, 400, 0), (300, 40, 0), (100, 400, 0), (8, 400, 0), (50, 10, 290)):
+            a = (q[:nq], lo[:nq], hi[:nq], k) + ((beam,) if beam else ())
+            kw = dict(out_ids=torch.empty((nq, k), dtype=torch.int32, device="cuda"), out_dists=torch.empty((nq, k), device="cuda"))
+            want = [t.clone() for t in (gix.search if beam else gix.exact_search)(*a, **kw)]
+            calls.append((gix.search if beam else gix.exact_search, a, dict(kw, stream=torch.cuda.Stream()), want))
+        work.append((calls, []))
+    torch.cuda.synchronize()
+    gate = threading.Barrier(2)
+
+    def run(calls, errors):
+        gate.wait()
+        try:
+            for _ in range(300):
+                for f, a, kw, want in calls:
+                    f(*a, **kw)
+            torch.cuda.synchronize()
+            assert all(torch.equal(kw["out_ids"], w[0]) and torch.equal(kw["out_dists"], w[1]) for f, a, kw, w in calls)
+        except Exception as e:
+            errors.append(e)
+
+    threads = [threading.Thread(target=run, args=w) for w in work]
+    for t in threads:
+        t.start()
+    for t in threads:
+        t.join()
+    assert [w[1] for w in work] == [[], []]
