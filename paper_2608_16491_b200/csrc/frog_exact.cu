@@ -36,7 +36,7 @@ constexpr int EXACT_GROUP_MIN = 201;
 // 8,000 x 384, 600: 275/203; with k = 100 5,000 x 96, 600: 234/160).
 constexpr long long EXACT_SMALL_BYTES = 4500000;
 constexpr int EXACT_SMALL_K = 32;
-constexpr size_t EXACT_GROW_BYTES = (size_t)64 << 20;   // see exact_scratch
+constexpr size_t EXACT_GROW_BYTES = (size_t)16 << 20;   // see exact_scratch
 constexpr int EXACT_PLAN_MIN = 17;       // from here on the slabs are found by a planning kernel (100,000 x 96, 16 queries: 49 without)
 constexpr int EXACT_STEP = 8 * EXACT_WARPS;    // rows per step of a CTA: two per team
 constexpr int EXACT_BUF = 256;           // keys buffered per query; merged from 64 on, two steps add at most 128
@@ -854,8 +854,9 @@ size_t exact_bytes(size_t nq, const ExactCut& c, bool few) {
 bool exact_scratch(frog_index* ix, FrogExactSet* set, cudaStream_t s, size_t nq, const ExactCut& c, bool few, ExactScratch* out) {
     const size_t bytes = exact_bytes(nq, c, few);
     if (!set->mem || nq > set->queries || bytes > set->bytes) {
-        // Growing takes 0.5-3 ms; on an index this small one scan without scratch costs less than that (up to 64 MB of
-        // rows: 2-3 ms at most for 2,000 queries), so it waits for a second scan that could use it.
+        // Growing takes 0.5-3 ms.  A first scan of 2,000 queries, k = 100, without scratch / with growth: 20,000 x 96 (7.7 MB)
+        // 1,370/1,600 us, 201 queries 490/920; 100,000 x 128 (51 MB) 2,740/1,950.  So on small indexes a scan that would
+        // need more does without, and only a second one grows.
         if (!ix->exact_asked && (size_t)ix->info.n * ix->info.d_pad * 4 <= EXACT_GROW_BYTES) {
             ix->exact_asked = true;
             return false;
