@@ -1,10 +1,12 @@
 // Index handle: file parsing, device residency (paper Sec. 8.1.3: index and vectors stay in GPU
 // memory), error strings, and the host-buffer search call that includes the transfers.
+#include <algorithm>
 #include <atomic>
 #include <cerrno>
 #include <cstdio>
 #include <cstdlib>
 #include <cstring>
+#include <memory>
 #include <new>
 #include <thread>
 
@@ -71,59 +73,40 @@ namespace froghost {
 void set_cuda_error(cudaError_t e) { g_last_cuda_error = (int)e; }
 
 // Copy sections between an index file and device memory.  The page cache is the bound (one thread moves a few
-// GB/s), so up to four threads take 2 MB chunks in turn, each with two page-locked buffers of its own: the
-// bus copy of one chunk overlaps the file access of the next.  A 110 MB index loads in 31 ms instead of 180
-// (a 64 MB page-locked buffer per section took most of that).
+// GB/s), so up to four threads take 2 MB chunks in turn, from 4 MB a thread on.  Their buffers are plain memory: the
+// driver's own staging moves 20 GB/s from such a buffer, where page-locking takes 0.6 ms for every MB of it (16 MB of
+// page-locked buffers: 0.9 MB built in 12-15 ms and loaded in 14-16, 110 MB in 208 and 29; now 6.6 and 3.2, 200 and 11-14).
 int transfer_sections(int fd, int device, const FileSection* sections, int count, bool to_device) {
     constexpr size_t CHUNK = (size_t)2 << 20;
-    size_t chunks = 0;
-    for (int i = 0; i < count; ++i) chunks += (sections[i].bytes + CHUNK - 1) / CHUNK;
-    if (chunks == 0) return FROG_OK;
-    const int threads = (int)(chunks < 4 ? chunks : 4);
-    char* buffers = nullptr;
-    const bool pinned = cudaMallocHost(reinterpret_cast<void**>(&buffers), (size_t)threads * 2 * CHUNK) == cudaSuccess;
-    if (!pinned) {
-        cudaGetLastError();
-        buffers = static_cast<char*>(std::malloc((size_t)threads * 2 * CHUNK));
-        if (!buffers) return FROG_ERR_NOMEM;
-    }
+    size_t bytes = 0;
+    for (int i = 0; i < count; ++i) bytes += sections[i].bytes;
+    const int threads = 1 + (int)std::min<size_t>(3, bytes >> 22);
     std::atomic<size_t> next{0};
     std::atomic<int> failed{FROG_OK}, cuda_error{0};
-    auto work = [&](int t) {
+    auto work = [&]() {
         auto fail = [&](int rc, cudaError_t e) {
             int ok = FROG_OK;
             failed.compare_exchange_strong(ok, rc);
             if (e != cudaSuccess) { cuda_error = (int)e; cudaGetLastError(); }
         };
+        const std::unique_ptr<char[]> buf(new (std::nothrow) char[std::min(CHUNK, bytes)]);
+        if (!buf) return fail(FROG_ERR_NOMEM, cudaSuccess);
         cudaStream_t s = nullptr;
-        cudaEvent_t moved[2] = {nullptr, nullptr};
         cudaError_t e = cudaSetDevice(device);
         if (e == cudaSuccess) e = cudaStreamCreateWithFlags(&s, cudaStreamNonBlocking);
-        for (int b = 0; b < 2 && e == cudaSuccess; ++b) e = cudaEventCreateWithFlags(&moved[b], cudaEventDisableTiming);
-        if (e != cudaSuccess) fail(FROG_ERR_CUDA, e);
-        auto file_io = [&](char* p, size_t bytes, uint64_t off) {
-            while (bytes) {
-                const ssize_t c = to_device ? pread(fd, p, bytes, (off_t)off) : pwrite(fd, p, bytes, (off_t)off);
+        if (e != cudaSuccess) return fail(FROG_ERR_CUDA, e);
+        auto file_io = [&](size_t n, uint64_t off) {
+            for (char* p = buf.get(); n;) {
+                const ssize_t c = to_device ? pread(fd, p, n, (off_t)off) : pwrite(fd, p, n, (off_t)off);
                 if (c < 0 && errno == EINTR) continue;
                 if (c <= 0) return false;
                 p += c;
                 off += (uint64_t)c;
-                bytes -= (size_t)c;
+                n -= (size_t)c;
             }
             return true;
         };
-        struct Chunk { uint64_t off; size_t bytes; bool busy; } held[2] = {{0, 0, false}, {0, 0, false}};
-        // writing: a buffer's chunk goes to the file once it has arrived from the device
-        auto settle = [&](int b) {
-            if (!held[b].busy) return;
-            held[b].busy = false;
-            const cudaError_t w = cudaEventSynchronize(moved[b]);
-            if (w != cudaSuccess) fail(FROG_ERR_CUDA, w);
-            else if (!to_device && failed == FROG_OK &&
-                     !file_io(buffers + (size_t)(2 * t + b) * CHUNK, held[b].bytes, held[b].off)) fail(FROG_ERR_IO, cudaSuccess);
-        };
-        int b = 0;
-        while (e == cudaSuccess && failed == FROG_OK) {
+        while (failed == FROG_OK) {
             size_t i = next++, at = 0;
             int k = 0;
             for (; k < count; ++k) {
@@ -132,34 +115,27 @@ int transfer_sections(int fd, int device, const FileSection* sections, int count
                 i -= n;
             }
             if (k == count) break;
-            settle(b);
-            char* const buf = buffers + (size_t)(2 * t + b) * CHUNK;
             char* const dev = static_cast<char*>(sections[k].dev) + at;
-            held[b] = {sections[k].off + at, sections[k].bytes - at < CHUNK ? sections[k].bytes - at : CHUNK, true};
-            if (to_device && !file_io(buf, held[b].bytes, held[b].off)) { held[b].busy = false; fail(FROG_ERR_IO, cudaSuccess); break; }
-            e = to_device ? cudaMemcpyAsync(dev, buf, held[b].bytes, cudaMemcpyHostToDevice, s)
-                          : cudaMemcpyAsync(buf, dev, held[b].bytes, cudaMemcpyDeviceToHost, s);
-            if (e == cudaSuccess) e = cudaEventRecord(moved[b], s);
-            if (e != cudaSuccess) { held[b].busy = false; fail(FROG_ERR_CUDA, e); break; }
-            b ^= 1;
+            const size_t n = std::min(CHUNK, sections[k].bytes - at);
+            if (to_device && !file_io(n, sections[k].off + at)) { fail(FROG_ERR_IO, cudaSuccess); break; }
+            e = to_device ? cudaMemcpyAsync(dev, buf.get(), n, cudaMemcpyHostToDevice, s)
+                          : cudaMemcpyAsync(buf.get(), dev, n, cudaMemcpyDeviceToHost, s);
+            if (e == cudaSuccess) e = cudaStreamSynchronize(s);
+            if (e != cudaSuccess) { fail(FROG_ERR_CUDA, e); break; }
+            if (!to_device && !file_io(n, sections[k].off + at)) { fail(FROG_ERR_IO, cudaSuccess); break; }
         }
-        settle(b);
-        settle(b ^ 1);
-        if (s) { cudaStreamSynchronize(s); cudaStreamDestroy(s); }
-        for (cudaEvent_t ev : moved) if (ev) cudaEventDestroy(ev);
+        cudaStreamDestroy(s);
     };
     std::thread helpers[3];
     for (int t = 1; t < threads; ++t) {
         try {
-            helpers[t - 1] = std::thread(work, t);
+            helpers[t - 1] = std::thread(work);
         } catch (...) {                                     // no thread to be had: the others do its share
             break;
         }
     }
-    work(0);
+    work();
     for (std::thread& h : helpers) if (h.joinable()) h.join();
-    if (pinned) cudaFreeHost(buffers);
-    else std::free(buffers);
     if (cuda_error) set_cuda_error((cudaError_t)cuda_error.load());
     return failed;
 }
