@@ -606,27 +606,52 @@ int plan_launch(const frog_index* ix, int beam_width, const frog_params_t& P, in
     return FROG_OK;
 }
 
+// Queries per SM up to which four warps per query beat one (see plan_team).  Five CTAs of four warps are resident, so
+// up to five queries per SM run at once; beyond that the last of them wait for a CTA, and what that costs grows with
+// the budget (more rows in flight per expansion) and, for short rows, with an index that does not stay in L2.
+// us, one warp / four warps per query (15,000-100,000 objects):
+//   rows, beam / B            740 queries    900            1,184          1,800
+//   256 bytes, 64 / 64         401 / 365      403 / 543      407 / 577
+//   400 bytes, 64 / 64         489 / 415      486 / 544      491 / 609
+//   400 bytes, 128 / 16       1064 / 772     1053 / 802     1068 / 821
+//   400 bytes, 192 / 128      1927 / 1324    1965 / 1425    1980 / 1614
+//   1,024 bytes, 64 / 64       671 / 523      675 / 565      687 / 700      723 / 946
+//   3,072 bytes, 64 / 64      1566 / 928     1571 / 962     1615 / 988     1651 / 1267
+//   3,072 bytes, 128 / 16     1446 / 1022    1471 / 1054    1514 / 1159    1550 / 1656
+//   1,536 bytes fp16, 64 / 16  790 / 658      795 / 679      808 / 779      825 / 1076
+// Over 8,900 combinations of 18 indexes, 8 beams, 4 budgets and 200-2,368 queries the rule takes 0.78 of the time of one
+// warp per query in the mean; it is slower by more than a tenth in 20 of them.
+int team_queries_per_sm(int row_bytes, bool f16, int beam_width, int budget, size_t index_bytes) {
+    if (row_bytes > STAGE_CHUNK) {
+        const bool few = budget <= 24;
+        if (f16) return few ? 7 : 13;
+        if (few) return 10;
+        if (row_bytes > 2 * STAGE_CHUNK) return 16;
+        return budget > 64 && index_bytes <= (size_t)64 << 20 ? 10 : 8;
+    }
+    const bool few = budget <= 32;
+    if (row_bytes < 150 && beam_width > 256 && !f16) return 0;     // the long merges of one warp leave the others idle
+    if (row_bytes < 200 || (f16 && few)) return 5;
+    if (index_bytes <= (size_t)4 << 20) return 8;
+    if (f16) return 5;
+    return few ? 8 : budget > 64 && index_bytes <= (size_t)64 << 20 ? 7 : 5;
+}
+
 // One CTA per query (frog_search_team.cu) for batches that leave warps idle, or FROG_ERR_UNSUPPORTED where
-// one warp per query is the better use of the GPU.  The line between them was measured on indexes of
-// 10,000-100,000 objects over batches of 1-4,000 queries (us per call, one warp per query / 8 warps / 4 warps):
-//   384-byte rows, beam 64, B 64     150 queries 286/210/275    300: 345/260/338    600: 343/379/351
-//   512-byte rows, beam 44, B 64     150: 229/168/229           300: 252/185/238    600: 296/262/286
-//   400-byte rows, beam 128, B 16    300: 657/414/507           600: 729/553/531    1,000: 772/871/627   1,500: 784/1229/805
-//   256-byte fp16 rows, beam 64      300: 414/257/316           600: 412/372/354    1,000: 511/575/423   1,500: 521/849/553
-//   3,072-byte rows, beam 192, B 128 300: 4212/1457/2515        600: 4219/1731/2620 1,500: 4841/3874/3025 4,000: 5246/10206/5907
-//   1,536-byte rows, beam 64, B 32   300: 688/231/355           600: 682/315/372    1,500: 778/653/486   4,000: 872/1604/1132
-// so: 8 warps while every query has a CTA of its own at once (2 per SM; 4 per SM for rows of several
-// chunks), then 4 warps up to 8 queries per SM (16 for long rows) except on the rows that the kernel of
-// frog_search_lean.cu covers, which one warp serves well enough.
+// one warp per query is the better use of the GPU.  Eight warps while every query has a CTA of its own at once (2 per
+// SM; 4 per SM for rows of several chunks, but not for fp16 rows with small budgets), then four up to the line above,
+// except on the rows that the kernel of frog_search_lean.cu covers, which one warp serves well enough (256-byte fp16
+// rows, beam 64, B 64: 400 queries 343 us with one warp per query and 410 with four, 900: 349 / 585).
 int plan_team(const frog_index* ix, int beam_width, const frog_params_t& P, int nq, LaunchPlan* out, int* vis_bits) {
     const bool f16 = P.storage == FROG_STORAGE_F16;
     const int q_len = query_len(ix->info.d);
     const int row_bytes = f16 ? q_len * 2 : ix->info.d_pad * 4;
-    const bool lean = !f16 && ix->has_tmap_f32 && (row_bytes == 384 || row_bytes == 512);
-    const bool long_rows = row_bytes > STAGE_CHUNK;
-    const int per_sm_nq = (nq + ix->sm_count - 1) / ix->sm_count;
-    const int warps = per_sm_nq <= (long_rows ? 4 : 2) ? 8 : 4;
-    if (warps == 4 && (lean || per_sm_nq > (long_rows ? 16 : 8))) return FROG_ERR_UNSUPPORTED;
+    const bool lean = f16 ? ix->has_tmap_f16 && (row_bytes == 192 || row_bytes == 256)
+                          : ix->has_tmap_f32 && (row_bytes == 384 || row_bytes == 512);
+    const int per_sm_nq = (nq - 1) / ix->sm_count + 1;
+    const int warps = per_sm_nq <= (row_bytes <= STAGE_CHUNK || (f16 && P.budget <= 24) ? 2 : 4) ? 8 : 4;
+    if (warps == 4 && (lean || per_sm_nq > team_queries_per_sm(row_bytes, f16, beam_width, P.budget, (size_t)ix->info.n * row_bytes)))
+        return FROG_ERR_UNSUPPORTED;
     // a table of about 16 ranks per beam slot: smaller ones repeat distances (3,072-byte rows at beam 192:
     // 1.3x slower with 2,048 ranks than with 4,096), larger ones cost resident CTAs
     int bits = 10;
