@@ -185,9 +185,9 @@ int frog_search_ex(const frog_index_t* index, const float* queries, const int32_
 
 /* frog_exact_search: exact filtered kNN (Def. 2 of Sec. 2.1) by scanning the contiguous rank
  * slab of each query (Sec. 4: an attribute range is a contiguous rank interval).  The rows are cut into
- * pieces over the whole GPU: of one query each for up to 200 queries, of a group of eight queries that share
- * them for more.  One CTA per query scans instead, without scratch: more than 200 queries with k <= 32 on an
- * index of at most 4.5 MB of rows, rows too long for eight queries in shared memory, more than 2^30 queries,
+ * pieces over the whole GPU: of one query each for small batches (up to 200 queries), of a group of eight
+ * queries that share them for larger ones.  One CTA per query scans instead, without scratch: where the index
+ * is too small for pieces to pay, rows too long for eight queries in shared memory, more than 2^30 queries,
  * a call under stream capture, and a call whose scratch cannot be had.  The results are the same.
  * Scratch: an index is loaded with what one stream's scans of up to 2,048 queries with k <= 128 need, but
  * no more than a quarter of its own size; a scan on another stream, up to four in flight at once, or one that

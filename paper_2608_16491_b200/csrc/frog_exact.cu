@@ -11,11 +11,11 @@
 //     shared by all pieces of a query through global memory: whatever exceeds the k-th best of ANY piece
 //     cannot be an answer;
 //   * the last CTA to finish a group merges the pieces' lists.
-// Up to EXACT_GROUP_MIN queries are not grouped: all rows are cut into equal pieces, one query each (one launch for
-// fewer than EXACT_PLAN_MIN, else a planning kernel finds the slabs first).  Otherwise queries are ordered by
-// (width, position), grouped by eight, and the groups' rows are cut into pieces of equal size (two small kernels).  The form with one CTA per query
-// and no scratch remains for many queries on small indexes, for captured streams, for rows too long for eight queries in shared memory, and
-// for the case that scratch cannot be had.
+// Few queries are not grouped: all rows are cut into equal pieces, one query each (one launch for fewer than
+// EXACT_PLAN_MIN, else a planning kernel finds the slabs first).  Otherwise queries are ordered by (width, position),
+// grouped by eight, and the groups' rows are cut into pieces of equal size (two small kernels).  The form with one CTA
+// per query and no scratch remains for small indexes, for captured streams, for rows too long for eight queries in
+// shared memory, and for the case that scratch cannot be had.  exact_form says where the lines lie.
 #include <algorithm>
 
 #include "frog_device.cuh"
@@ -27,17 +27,9 @@ namespace {
 
 constexpr int EXACT_WARPS = 8;
 constexpr int EXACT_GROUP = 8;           // queries per group = warps per CTA (one merges each query's buffer)
-// Grouping costs 35 us of planning and pays for itself from about 200 queries on, whatever the rows (us per call,
-// split / grouped, k = 10): 100,000 x 96: 64 queries 129/235, 100: 168/260, 200: 300/358, 600: 1,075/595;
-// 30,000 x 50: 100: 118/138, 200: 169/170, 600: 372/277; 20,000 x 768: 100: 171/216, 200: 263/252, 600: 677/492.
-constexpr int EXACT_GROUP_MIN = 201;
-// Slabs of so few bytes are not worth planning for once there is a query per CTA and lists are short (us, one CTA per
-// query / grouped: 5,000 x 96, 300 queries 93/104, 2,000: 140/163; 8,000 x 128, 600: 169/156, 2,000: 316/349;
-// 8,000 x 384, 600: 275/203; with k = 100 5,000 x 96, 600: 234/160).
-constexpr long long EXACT_SMALL_BYTES = 4500000;
-constexpr int EXACT_SMALL_K = 32;
+constexpr int EXACT_SPLIT_MAX = 200;     // queries that the split form can cut between
 constexpr size_t EXACT_GROW_BYTES = (size_t)16 << 20;   // see exact_scratch
-constexpr int EXACT_PLAN_MIN = 17;       // from here on the slabs are found by a planning kernel (100,000 x 96, 16 queries: 49 without)
+constexpr int EXACT_PLAN_MIN = 17;       // from here on the slabs are found by a planning kernel (100,000 x 96, 16 queries: 49 us without)
 constexpr int EXACT_STEP = 8 * EXACT_WARPS;    // rows per step of a CTA: two per team
 constexpr int EXACT_BUF = 256;           // keys buffered per query; merged from 64 on, two steps add at most 128
 constexpr int EXACT_BINS = 33 * 32;      // (width class, position) bins that queries are ordered by
@@ -440,7 +432,7 @@ __device__ __forceinline__ void exact_piece(const ExactArgs& A, const ExactSmem<
 }
 
 // One CTA per query, no scratch: each warp streams batches of 16 rows and keeps a list of its own, warp 0 merges
-// the lists.  32 warps per SM and no barrier in the loop: the better form for many short slabs (see EXACT_SMALL_BYTES).
+// the lists.  32 warps per SM and no barrier in the loop: the better form for many short slabs (see exact_form).
 template <int EPL>
 __global__ void __launch_bounds__(EXACT_WARPS * 32)
 frog_exact_kernel(const ExactArgs A) {
@@ -504,7 +496,7 @@ struct FewExtra {
 };
 struct SplitExtra {
     unsigned long long rows;
-    int first[EXACT_GROUP_MIN + 1];                          // first piece of each query
+    int first[EXACT_SPLIT_MAX + 1];                          // first piece of each query
     int warp_sum[EXACT_WARPS];
 };
 
@@ -548,7 +540,7 @@ frog_exact_few_kernel(const ExactArgs A) {
     }
 }
 
-// Up to EXACT_GROUP_MIN queries: all rows cut into pieces of equal size, about two per CTA, which evens out their
+// Up to EXACT_SPLIT_MAX queries: all rows cut into pieces of equal size, about two per CTA, which evens out their
 // ends.  Every CTA works out the cut for itself from the slabs that the planning kernel found.
 template <int EPL>
 __global__ void __launch_bounds__(EXACT_WARPS * 32, 2)
@@ -784,6 +776,31 @@ size_t exact_smem(int k, int d_pad) {
          : k <= 128 ? ExactSmem<4, G>::bytes(d_pad) : k <= 256 ? ExactSmem<8, G>::bytes(d_pad) : ExactSmem<16, G>::bytes(d_pad);
 }
 
+// Which form scans.  Two things decide that the host can know, as the slabs' widths are on the device: whether a CTA
+// per query leaves the GPU idle (few queries), and whether the whole index is so short that cutting it costs more
+// than it saves.  us, one CTA per query / split by query / grouped, k = 10, slabs of all rows | log-uniform down to 1/16:
+//                     40 queries                  100                          200                          1,000
+//   1,000 x 96     48/53/84 | 46/52/99        48/77/85 | 46/58/97         49/104/90 | 46/80/95         89/-/100 | 65/-/99
+//   2,000 x 96     63/78/86 | 60/56/96        62/90/87 | 59/77/99         64/123/89 | 60/95/101       120/-/139 | 87/-/116
+//   5,000 x 96     98/73/90 | 95/56/99        99/117/92 | 94/83/101      103/174/95 | 93/116/105      218/-/271 | 151/-/160
+//   20,000 x 96   276/128/111 | 248/96/123   278/220/155 | 269/140/129   293/371/235 | 272/192/164    679/-/678 | 421/-/401
+//   2,000 x 768   137/90/189 | 130/63/176    138/117/190 | 131/93/182    151/175/192 | 140/126/189    359/-/343 | 215/-/201
+//   100,000 x 128      - | 1234/172/280           - | 1284/272/336            - | 1282/446/472             - | 2015/-/1182
+// Long result lists favour pieces (k = 100, second column: 2,000 x 96, 1,000 queries 207/-/121, 5,000 x 96, 100
+// 162/134/122).  Over 3,400 combinations (300 to 1,000,000 objects, 32 to 2,000 dimensions, 1-2,000 queries, k = 10 to
+// 512, three mixes of widths) the rule takes 0.51 of the time of one CTA per query in the mean and is slower by more
+// than a tenth in 1 %; the best form of each would take 0.48.
+enum class ExactForm { OnePerQuery, Few, Split, Grouped };
+ExactForm exact_form(size_t n, size_t row_bytes, int nq, int k) {
+    const size_t bytes = n * row_bytes;
+    if (nq < EXACT_PLAN_MIN) return k <= 32 && bytes <= 500000 ? ExactForm::OnePerQuery : ExactForm::Few;
+    const double work = (double)n * (double)(row_bytes + 384) * (k > 128 ? 3.0 : k > 64 ? 1.4 : 1.0);
+    if (nq <= EXACT_SPLIT_MAX && nq * (n < 8000 ? 45e3 : 100e3) <= work) return ExactForm::Split;
+    if (k > 128) return ExactForm::Grouped;
+    if (n < 3000) return k > 32 && nq >= (k > 64 ? 600 : 1400) ? ExactForm::Grouped : ExactForm::OnePerQuery;
+    return k > 32 || bytes > 4500000 || (n >= 8000 && nq <= 300) ? ExactForm::Grouped : ExactForm::OnePerQuery;
+}
+
 // While another thread captures a stream, event queries and allocations are refused and spoil its capture, unless the
 // calling thread says that they have nothing to do with it.
 struct NoCaptureOfOurs {
@@ -920,13 +937,13 @@ extern "C" int frog_exact_search(const frog_index_t* index, const float* queries
     A.out_dists = out_dists;
     cudaStreamCaptureStatus capture = cudaStreamCaptureStatusNone;
     FROG_CUDA_TRY(cudaStreamIsCapturing(s, &capture));
-    const bool few = nq < EXACT_GROUP_MIN;
-    const bool small = !few && k <= EXACT_SMALL_K && index->info.n * A.d_pad * 4 <= EXACT_SMALL_BYTES;
+    const ExactForm form = exact_form((size_t)index->info.n, (size_t)A.d_pad * 4, nq, k);
+    const bool few = form != ExactForm::Grouped;
     const size_t smem = !few ? exact_smem<EXACT_GROUP>(k, A.d_pad)
-                             : exact_smem<1>(k, A.d_pad) + (nq < EXACT_PLAN_MIN ? sizeof(FewExtra) : sizeof(SplitExtra));
+                             : exact_smem<1>(k, A.d_pad) + (form == ExactForm::Few ? sizeof(FewExtra) : sizeof(SplitExtra));
     // (the planning kernels count queries in ints with some room)
-    if (capture == cudaStreamCaptureStatusNone && !small && smem <= froghost::MAX_SMEM && nq <= 1 << 30) {
-        const exact_fn fn = nq < EXACT_PLAN_MIN ? exact_pick<Few>(k) : few ? exact_pick<Split>(k) : exact_pick<Grouped>(k);
+    if (capture == cudaStreamCaptureStatusNone && form != ExactForm::OnePerQuery && smem <= froghost::MAX_SMEM && nq <= 1 << 30) {
+        const exact_fn fn = form == ExactForm::Few ? exact_pick<Few>(k) : few ? exact_pick<Split>(k) : exact_pick<Grouped>(k);
         FROG_CUDA_TRY(froghost::allow_smem(fn));
         int per_sm = 0;
         FROG_CUDA_TRY(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, (const void*)fn, EXACT_WARPS * 32, smem));
@@ -953,7 +970,7 @@ extern "C" int frog_exact_search(const frog_index_t* index, const float* queries
             A.max_pieces = cut.max_pieces;
             A.min_rows = cut.min_rows;
             set->clean = false;                            // until the launches are under way
-            if (!few || nq >= EXACT_PLAN_MIN) frog_exact_plan_kernel<<<(nq - 1) / 8 + 1, 256, 0, s>>>(A);
+            if (form != ExactForm::Few) frog_exact_plan_kernel<<<(nq - 1) / 8 + 1, 256, 0, s>>>(A);
             if (!few) frog_exact_cut_kernel<<<1, 1024, 0, s>>>(A);
             fn<<<grid, EXACT_WARPS * 32, smem, s>>>(A);
             FROG_CUDA_TRY(cudaGetLastError());

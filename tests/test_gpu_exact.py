@@ -1,6 +1,6 @@
 """The exact filtered scan: grouped, split and one-CTA-per-query forms against the oracle's slab scan, at the
-edges of its pieces, pools and row lengths.  From 201 queries on they are grouped (on
-small indexes only with k > 32), from 17 on planned by a kernel of their own."""
+edges of its pieces, pools and row lengths.  From 17 queries on they are planned by a kernel of their own; which form
+takes them then depends on their number, k and the size of the index, so that these sizes reach all of them."""
 import numpy as np
 import pytest
 
