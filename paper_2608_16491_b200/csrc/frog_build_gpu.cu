@@ -77,7 +77,7 @@ struct BWarp {
     float4* q;
     uint64_t* pool;      // CAND keys
     uint64_t* spool;     // search pool (sibling search only)
-    uint64_t* keys;      // keys of one expansion (sibling search only)
+    uint64_t* keys;      // keys of one expansion (sibling search only): the second half of `pool`, empty until its end
     uint32_t* cand;
     uint64_t* bar;
     float4* stage;       // (sibling search: its table of evaluated ranks)
@@ -85,15 +85,15 @@ struct BWarp {
 constexpr int SEEN_BITS = 10;
 static_assert((4 << SEEN_BITS) == STAGE8, "the table takes the place of the stage buffer");
 __host__ __device__ inline size_t bwarp_bytes(int d_pad, int spool_slots) {
-    return (size_t)d_pad * 4 + CAND * 8 + (size_t)spool_slots * 8 + (spool_slots ? 32 * 8 : 0) + 32 * 4 + 16 + STAGE8;
+    return (size_t)d_pad * 4 + CAND * 8 + (size_t)spool_slots * 8 + 32 * 4 + 16 + STAGE8;
 }
 __device__ __forceinline__ BWarp bwarp_carve(unsigned char* base, int d_pad, int spool_slots) {
     BWarp W;
     W.q = reinterpret_cast<float4*>(base);
     W.pool = reinterpret_cast<uint64_t*>(base + (size_t)d_pad * 4);
     W.spool = W.pool + CAND;
-    W.keys = W.spool + spool_slots;
-    W.cand = reinterpret_cast<uint32_t*>(W.keys + (spool_slots ? 32 : 0));
+    W.keys = W.pool + 32;                       // the m <= 32 nearest of the own child lie before it
+    W.cand = reinterpret_cast<uint32_t*>(W.spool + spool_slots);
     W.bar = reinterpret_cast<uint64_t*>(W.cand + 32);
     W.stage = reinterpret_cast<float4*>(W.bar + 2);
     return W;
@@ -247,6 +247,8 @@ sibling_search_kernel(const BuildArgs A) {
                 if (improved) pat = A.patience;
                 else if (--pat <= 0) break;
             }
+            __syncwarp();
+            W.keys[lane] = KEY_EMPTY;
             __syncwarp();
             uint64_t key = KEY_EMPTY;
             if (lane < A.m) {

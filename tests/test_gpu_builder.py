@@ -71,6 +71,22 @@ def test_enc_arrays_equal_the_host_builder_on_other_shapes(libs, cache_dir, name
     os.remove(pc)
 
 
+def test_the_longest_rows_the_sibling_search_takes(libs, cache_dir):
+    """Rows of 109,424 bytes, the most that two warps' queries and search pools leave shared memory for; four bytes
+    more per row are refused."""
+    rng = np.random.default_rng(8)
+    v = rng.standard_normal((120, 27357)).astype(np.float32)
+    a = rng.integers(0, 90, 120).astype(np.int32)
+    pg, pc = (os.path.join(cache_dir, f"longest_{x}.idx") for x in "gc")
+    libs.build_index_gpu(np.ascontiguousarray(v[:, :27356]), a, pg, n_inv=3)
+    libs.build_index(np.ascontiguousarray(v[:, :27356]), a, pc, n_inv=3)
+    with open(pg, "rb") as f, open(pc, "rb") as g:
+        assert f.read() == g.read()
+    with pytest.raises(libs.FrogError) as e:
+        libs.build_index_gpu(v, a, pg, n_inv=3)
+    assert e.value.code == 6
+
+
 def test_construction_switches_change_the_index_as_described(libs, cache_dir):
     """FROG_BUILD_ENC_FUSION_NEAREST: every ENC row holds the m fusion-nearest of the object's
     candidates, i.e. no row of the default build is fusion-nearer at any position; and the switches
