@@ -564,10 +564,8 @@ int ceil_log2_i64(int64_t n) {
     return b;
 }
 
-}  // namespace
-
-extern "C" int frog_index_build_gpu(const float* vectors, const int32_t* attrs, int64_t n64, int32_t d,
-                                    const frog_build_params_t* params, int device, const char* path) {
+int build_index(const float* vectors, const int32_t* attrs, int64_t n64, int32_t d, const frog_build_params_t* params, int device,
+                const char* path) {
     if (!vectors || !attrs || !path || n64 < 1 || d < 1 || n64 >= ((int64_t)1 << 31) - 1 || device < 0)
         return FROG_ERR_INVALID_ARG;
     frog_build_params_t P{};
@@ -762,4 +760,15 @@ extern "C" int frog_index_build_gpu(const float* vectors, const int32_t* attrs, 
     }
     if (fclose(f) != 0 && rc == FROG_OK) rc = FROG_ERR_IO;
     return rc;
+}
+
+}  // namespace
+
+extern "C" int frog_index_build_gpu(const float* vectors, const int32_t* attrs, int64_t n, int32_t d,
+                                    const frog_build_params_t* params, int device, const char* path) {
+    try {
+        return build_index(vectors, attrs, n, d, params, device, path);
+    } catch (...) {                    // the standard containers' way to say that host memory is short
+        return FROG_ERR_NOMEM;
+    }
 }

@@ -174,7 +174,8 @@ def test_odd_dimension_is_zero_padded(libs, cache_dir):
 
 def test_a_file_without_its_header_is_refused(libs, tiny, tmp_path):
     """The GPU builder writes the header last: zeros in its place mean an unfinished file."""
-    data = bytearray(open(tiny[1], "rb").read())
+    with open(tiny[1], "rb") as f:
+        data = bytearray(f.read())
     data[:256] = bytes(256)
     p = tmp_path / "unfinished.idx"
     p.write_bytes(data)

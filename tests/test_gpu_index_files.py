@@ -1,10 +1,11 @@
 """What ends up in an index file, and what is accepted as one, when file accesses fail: the GPU builder writes the
 two large arrays of a regular file from several threads, the loader reads all four that way.  The failures are
-made on the host, by a stand-in for pread and pwrite that a child process is started with."""
+made on the host, by a stand-in for pread, pwrite and operator new that a child process is started with."""
 import os
 import subprocess
 import sys
 import threading
+from pathlib import Path
 
 import numpy as np
 import pytest
@@ -18,9 +19,14 @@ pytest.importorskip("torch")
 ROOT = os.path.dirname(os.path.dirname(os.path.abspath(__file__)))
 
 # The access at file offset FAULT_OFFSET, if it is a large one, waits until the others are through and fails:
-# a write with ENOSPC, a read as at the end of the file.
+# a write with ENOSPC, a read as at the end of the file.  FAULT_OP = new<i>: the i-th request for exactly FAULT_OFFSET
+# bytes is refused.
 STAND_IN = r"""
+#ifndef _GNU_SOURCE
 #define _GNU_SOURCE
+#endif
+#include <atomic>
+#include <new>
 #include <dlfcn.h>
 #include <errno.h>
 #include <stdlib.h>
@@ -33,16 +39,26 @@ static int hit(const char* op, size_t n, off_t off) {
     usleep(700000);
     return 1;
 }
-ssize_t pwrite(int fd, const void* p, size_t n, off_t off) {
-    ssize_t (*real)(int, const void*, size_t, off_t) = dlsym(RTLD_NEXT, "pwrite");
+extern "C" ssize_t pwrite(int fd, const void* p, size_t n, off_t off) {
+    auto real = (ssize_t (*)(int, const void*, size_t, off_t))dlsym(RTLD_NEXT, "pwrite");
     if (hit("write", n, off)) { errno = ENOSPC; return -1; }
     return real(fd, p, n, off);
 }
-ssize_t pread(int fd, void* p, size_t n, off_t off) {
-    ssize_t (*real)(int, void*, size_t, off_t) = dlsym(RTLD_NEXT, "pread");
+extern "C" ssize_t pread(int fd, void* p, size_t n, off_t off) {
+    auto real = (ssize_t (*)(int, void*, size_t, off_t))dlsym(RTLD_NEXT, "pread");
     return hit("read", n, off) ? 0 : real(fd, p, n, off);
 }
-ssize_t __pread_chk(int fd, void* p, size_t n, off_t off, size_t room) { return pread(fd, p, n, off); }
+extern "C" ssize_t __pread_chk(int fd, void* p, size_t n, off_t off, size_t) { return pread(fd, p, n, off); }
+void* operator new(size_t n) {
+    static std::atomic<int> seen{0};
+    const char *w = getenv("FAULT_OP"), *o = getenv("FAULT_OFFSET");
+    if (w && !strncmp(w, "new", 3) && n == (size_t)atoll(o) && ++seen == atoi(w + 3)) throw std::bad_alloc();
+    void* p = malloc(n ? n : 1);
+    if (!p) throw std::bad_alloc();
+    return p;
+}
+void operator delete(void* p) noexcept { free(p); }
+void operator delete(void* p, size_t) noexcept { free(p); }
 """
 
 CHILD = r"""
@@ -72,8 +88,8 @@ def files(libs, tmp_path_factory):
     np.savez(tmp / "data.npz", base=base, attrs=attrs)
     good = str(tmp / "good.idx")
     libs.build_index_gpu(base, attrs, good, ef_c=16, n_inv=8)
-    (tmp / "stand_in.c").write_text(STAND_IN)
-    subprocess.check_call(["gcc", "-shared", "-fPIC", "-O1", "-o", str(tmp / "stand_in.so"), str(tmp / "stand_in.c"), "-ldl"])
+    (tmp / "stand_in.cpp").write_text(STAND_IN)
+    subprocess.check_call(["g++", "-shared", "-fPIC", "-O1", "-o", str(tmp / "stand_in.so"), str(tmp / "stand_in.cpp"), "-ldl"])
     return tmp, base, attrs, good
 
 
@@ -83,11 +99,11 @@ def _child(files, do, path, op=None, offset=0):
         env["FAULT_OP"] = op
     out = subprocess.run([sys.executable, "-c", CHILD, do, str(files[0] / "data.npz"), path], env=env, cwd=ROOT,
                          stdout=subprocess.PIPE, text=True, timeout=300)
-    return int(out.stdout.split("code ")[1])
+    return int(out.stdout.split("code ")[1]) if out.returncode == 0 else -1
 
 
 def _offsets(path):
-    return [int(x) for x in np.frombuffer(open(path, "rb").read(256)[72:112], np.uint64)]   # attr, id, vec, enc, end
+    return [int(x) for x in np.frombuffer(Path(path).read_bytes()[72:112], np.uint64)]   # attr, id, vec, enc, end
 
 
 def test_a_build_that_fails_late_leaves_nothing_that_loads(libs, files):
@@ -95,13 +111,19 @@ def test_a_build_that_fails_late_leaves_nothing_that_loads(libs, files):
     tmp, good = files[0], files[3]
     path = str(tmp / "hole.idx")
     assert _child(files, "build", path) == 0
-    assert open(path, "rb").read() == open(good, "rb").read()
+    assert Path(path).read_bytes() == Path(good).read_bytes()
     assert _child(files, "build", path, "write", _offsets(good)[2]) == 2
     with pytest.raises(libs.FrogError) as e:
         libs.Index.load(path)
     assert e.value.code == 3
     libs.build_index_gpu(files[1], files[2], path, ef_c=16, n_inv=8)
-    assert open(path, "rb").read() == open(good, "rb").read()
+    assert Path(path).read_bytes() == Path(good).read_bytes()
+
+
+@pytest.mark.parametrize("which", [1, 2, 3])
+def test_a_build_without_host_memory_says_so(files, which):
+    """Arrays of one integer per object: their order, the sorted attributes, the ranks."""
+    assert _child(files, "build", str(files[0] / "none.idx"), "new%d" % which, 4 * 20000) == 4
 
 
 @pytest.mark.parametrize("section", [0, 2, 3])
@@ -115,8 +137,8 @@ def test_a_pipe_gets_the_same_bytes(libs, files):
     fifo = str(tmp / "pipe")
     os.mkfifo(fifo)
     got = []
-    reader = threading.Thread(target=lambda: got.append(open(fifo, "rb").read()))
+    reader = threading.Thread(target=lambda: got.append(Path(fifo).read_bytes()))
     reader.start()
     libs.build_index_gpu(base, attrs, fifo, ef_c=16, n_inv=8)
     reader.join()
-    assert got[0] == open(good, "rb").read()
+    assert got[0] == Path(good).read_bytes()
