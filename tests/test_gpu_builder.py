@@ -71,6 +71,21 @@ def test_enc_arrays_equal_the_host_builder_on_other_shapes(libs, cache_dir, name
     os.remove(pc)
 
 
+@pytest.mark.parametrize("d", [897, 901, 960, 1536, 2050])
+def test_candidate_rows_beyond_shared_memory(libs, cache_dir, d):
+    """64 candidate rows of up to 900 floats are staged for the selection, longer ones are read where they are."""
+    rng = np.random.default_rng(d)
+    v = (rng.standard_normal((3000, d)) * np.arange(1, d + 1) ** -0.4).astype(np.float32)
+    a = rng.integers(0, 1500, 3000).astype(np.int32)
+    pg, pc = (os.path.join(cache_dir, f"rows_{x}_{d}.idx") for x in "gc")
+    libs.build_index_gpu(v, a, pg)
+    libs.build_index(v, a, pc)
+    with open(pg, "rb") as f, open(pc, "rb") as g:
+        assert f.read() == g.read()
+    os.remove(pg)
+    os.remove(pc)
+
+
 def test_the_longest_rows_the_sibling_search_takes(libs, cache_dir):
     """Rows of 109,424 bytes, the most that two warps' queries and search pools leave shared memory for; four bytes
     more per row are refused."""
