@@ -250,8 +250,9 @@ int frog_search_last_status(const frog_index_t* index, void* stream, uint32_t* f
  * this figure leaves out).  Waits for that kernel to finish.  INVALID_ARG if there was no such call. */
 int frog_search_kernel_ms(const frog_index_t* index, void* stream, float* ms);
 
-/* Launch shape of the search kernel for the given beam width (for reporting): CTAs, threads per
- * CTA, dynamic shared memory per CTA, query slots resident per SM. */
+/* Launch shape of the search kernel for the given beam width and a batch that fills the GPU (for
+ * reporting; small batches may run another kernel, see frog_search): CTAs, threads per CTA, dynamic
+ * shared memory per CTA, query slots resident per SM. */
 int frog_search_launch_info(const frog_index_t* index, int beam_width, const frog_params_t* params,
                             int* grid, int* block, int* smem_bytes, int* queries_per_sm);
 

@@ -26,8 +26,8 @@ extern "C" {
  *   attrs    HOST, n int32
  *   params   HOST, may be null; same meaning and defaults as frog_index_build (threads ignored).
  *            Limits of the kernels: m <= 32, ef_c <= 256, leaves of at most 256 objects.
- * Device memory: vectors + ENC array + about 1.2 KB per object of work space + n/8 bytes per
- * resident warp; everything is released before returning.  Returns 0 or a FROG_ERR_* code
+ * Device memory: vectors + ENC array + about 1.5 KB per object of work space (m = 16), and at first a slab
+ * of at most 256 MB of the caller's rows; everything is released before returning.  Returns 0 or a FROG_ERR_* code
  * (1 invalid argument, 2 I/O, 4 out of memory, 5 CUDA error, 6 unsupported parameters).  If a bulk
  * copy of a kernel does not complete within its polling limit the call returns 5 and writes no file.
  * A regular file gets its header last: what an interrupted or failed build leaves behind, of whatever

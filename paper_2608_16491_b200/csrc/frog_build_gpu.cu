@@ -403,7 +403,8 @@ __device__ __forceinline__ uint64_t rng_keep(const SelSmem& S, const char* const
             }
 #pragma unroll
             for (int i = 0; i < 2; ++i)
-                if (sub == 0 && j[i] < na && !(key_dist2(keys[cand[i]]) < d[i])) atomicOr(dead + (pos[i] >> 5), 1u << (pos[i] & 31));
+                if (sub == 0 && j[i] < na && !(key_dist2(keys[cand[i]]) < d[i]))
+                    atomicOr(dead + (pos[i] >> 5), 1u << (pos[i] & 31));
         }
         __syncthreads();
         standing &= ~((uint64_t)dead[0] | (uint64_t)dead[1] << 32);
@@ -450,7 +451,8 @@ select_kernel(const BuildArgs A) {
             for (int r = tid; r < K; r += blockDim.x)
                 if (!A.skip_copies)
                     tma_load_1d(reinterpret_cast<char*>(S.rows) + (size_t)r * row_bytes,
-                                reinterpret_cast<const char*>(A.V) + (size_t)key_rank(S.keys[r]) * row_bytes, (uint32_t)row_bytes, S.bar);
+                                reinterpret_cast<const char*>(A.V) + (size_t)key_rank(S.keys[r]) * row_bytes,
+                                (uint32_t)row_bytes, S.bar);
             wait_copies(A, S.bar, phase);
             phase ^= 1u;
         }
@@ -492,7 +494,8 @@ select_kernel(const BuildArgs A) {
             }
             __syncthreads();
             const uint64_t all = K < 64 ? (1ull << K) - 1ull : ~0ull;
-            uint64_t enc = A.fusion_nearest ? 0ull : rng_keep(S, rows, S.keys, STAGED, row_bytes, K, A.m);   // 0: the m fusion-nearest
+            uint64_t enc = 0ull;                               // as it stands: the m fusion-nearest
+            if (!A.fusion_nearest) enc = rng_keep(S, rows, S.keys, STAGED, row_bytes, K, A.m);
             uint64_t spare = all & ~enc;
             for (int x = __popcll(enc); x < A.m && spare; ++x) {
                 enc |= spare & (0ull - spare);
@@ -631,7 +634,8 @@ int build_index(const float* vectors, const int32_t* attrs, int64_t n64, int32_t
         for (size_t i0 = 0; i0 < (size_t)n; i0 += slab) {
             const size_t rows = std::min(slab, (size_t)n - i0), elems = rows * d_pad;
             FROG_CUDA_TRY(cudaMemcpy(raw, vectors + i0 * d, rows * d * 4, cudaMemcpyHostToDevice));
-            rank_rows_kernel<<<(unsigned)std::min<size_t>((elems + 255) / 256, (size_t)prop.multiProcessorCount * 32), 256>>>(raw, ranks + i0, d, d_pad, elems, dV);
+            const unsigned grid = (unsigned)std::min<size_t>((elems + 255) / 256, (size_t)prop.multiProcessorCount * 32);
+            rank_rows_kernel<<<grid, 256>>>(raw, ranks + i0, d, d_pad, elems, dV);
             FROG_CUDA_TRY(cudaGetLastError());
         }
         FROG_CUDA_TRY(cudaDeviceSynchronize());

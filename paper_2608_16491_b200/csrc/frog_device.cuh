@@ -622,36 +622,33 @@ __device__ __forceinline__ uint32_t merge_batch(uint64_t* pool, uint64_t my_key,
 // key or which old one moves there.  The cost hardly depends on the pool size and little on n, and the
 // dependent chain has no shuffle or vote per key.
 // `entered` tells a lane whether its key is in the pool now and was not before.
-// UNIQUE: the caller guarantees that there are no copies.
-template <int EPL, bool UNIQUE = false>
+template <int EPL>
 __device__ __forceinline__ uint32_t merge_ranked(uint64_t* pool, const uint64_t* keys, int n, int ef_s, int lane,
                                                  bool* entered = nullptr) {
     constexpr int POOL = 32 * EPL;
+    static_assert((POOL & (POOL - 1)) == 0, "the search halves the pool");
     const uint32_t lt_mask = (1u << lane) - 1u;
     uint64_t key = lane < n ? keys[lane] : KEY_EMPTY;
     const uint64_t mk = key | 1ull;
     bool in = mk < (pool[ef_s - 1] | 1ull);             // a full pool rejects what is not better than its worst
     int p = 0;                                          // pool keys below mk (at most ef_s - 1 if it enters)
-    constexpr int TOP = POOL > 256 ? 256 : POOL > 128 ? 128 : POOL / 2;
 #pragma unroll
-    for (int step = TOP; step > 0; step >>= 1)
-        if (((POOL & (POOL - 1)) == 0 || p + step <= POOL) && (pool[p + step - 1] | 1ull) < mk) p += step;
-    if (!UNIQUE) in = in && (pool[p] | 1ull) != mk;     // the pool holds it already
+    for (int step = POOL / 2; step > 0; step >>= 1)
+        if ((pool[p + step - 1] | 1ull) < mk) p += step;
+    in = in && (pool[p] | 1ull) != mk;                  // the pool holds it already
     int r = 0;
     bool copy = false;
 #pragma unroll 4
     for (int j = 0; j < n; ++j) {
         const uint64_t x = keys[j] | 1ull;
         r += x < mk ? 1 : 0;
-        if (!UNIQUE) copy = copy || (x == mk && j < lane);
+        copy = copy || (x == mk && j < lane);
     }
-    if (!UNIQUE) {
-        in = in && !copy;
-        // keys that lie below this one but do not enter: copies only (what the pool rejects lies above)
-        for (uint32_t out = __ballot_sync(FULL, !in && lane < n); out; out &= out - 1) {
-            const uint64_t x = keys[__ffs(out) - 1] | 1ull;
-            r -= x < mk ? 1 : 0;
-        }
+    in = in && !copy;
+    // keys that lie below this one but do not enter: copies only (what the pool rejects lies above)
+    for (uint32_t out = __ballot_sync(FULL, !in && lane < n); out; out &= out - 1) {
+        const uint64_t x = keys[__ffs(out) - 1] | 1ull;
+        r -= x < mk ? 1 : 0;
     }
     const int f = p + r;
     in = in && f < ef_s;

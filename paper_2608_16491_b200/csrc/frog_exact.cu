@@ -29,7 +29,7 @@ constexpr int EXACT_WARPS = 8;
 constexpr int EXACT_GROUP = 8;           // queries per group = warps per CTA (one merges each query's buffer)
 constexpr int EXACT_SPLIT_MAX = 200;     // queries that the split form can cut between
 constexpr size_t EXACT_GROW_BYTES = (size_t)16 << 20;   // see exact_scratch
-constexpr int EXACT_PLAN_MIN = 17;       // from here on the slabs are found by a planning kernel (100,000 x 96, 16 queries: 49 us without)
+constexpr int EXACT_PLAN_MIN = 17;       // from here on a planning kernel finds the slabs (100,000 x 96, 16 queries: 49 us without)
 constexpr int EXACT_STEP = 8 * EXACT_WARPS;    // rows per step of a CTA: two per team
 constexpr int EXACT_BUF = 256;           // keys buffered per query; merged from 64 on, two steps add at most 128
 constexpr int EXACT_BINS = 33 * 32;      // (width class, position) bins that queries are ordered by
@@ -48,9 +48,9 @@ struct ExactArgs {
     // scratch (see exact_scratch); unused by the form with one CTA per query
     int2* ranges;
     int32_t* order;
-    int4* jobs;                      // (group, first row, end row, -)
+    int4* jobs;                      // (group, first row, end row, unused)
     int2* groups;                    // (first piece, pieces)
-    unsigned int* counters;          // [0] pieces of this call, [1] next piece, [2..] bins; zero between calls
+    unsigned int* counters;          // [0] pieces of this call, [1] next piece: set per call; [2..] bins, zero between calls
     unsigned int* done;              // finished pieces per group (or query); zero between calls
     unsigned long long* bound;       // per query: k-th best key of any piece; all ones between calls
     uint64_t* part;                  // per piece and query of the group: k keys
@@ -192,7 +192,8 @@ __device__ __forceinline__ void exact_scan_one(const ExactArgs& A, const ExactSm
 // merge what may be among the k best of the pieces' lists into a single query's pool (one warp); eight loads per
 // lane are in flight at once
 template <int EPL>
-__device__ __forceinline__ void exact_gather(const ExactArgs& A, const ExactSmem<EPL, 1>& S, const unsigned long long* lists, int pieces, int lane) {
+__device__ __forceinline__ void exact_gather(const ExactArgs& A, const ExactSmem<EPL, 1>& S, int first, int pieces, int lane) {
+    const unsigned long long* const lists = reinterpret_cast<const unsigned long long*>(A.part) + (size_t)first * A.k;
     uint64_t* const pool = S.pool;
     uint64_t* const buf = S.buf;
     const unsigned int n = (unsigned int)pieces * (unsigned int)A.k;
@@ -394,7 +395,7 @@ __device__ __forceinline__ void exact_piece(const ExactArgs& A, const ExactSmem<
         __threadfence();
         if constexpr (G == 1) {
             // (this piece's own list is read back too: the merge drops what the pool holds)
-            if (warp == 0) exact_gather<EPL>(A, S, reinterpret_cast<const unsigned long long*>(A.part) + (size_t)first * A.k, pieces, lane);
+            if (warp == 0) exact_gather<EPL>(A, S, first, pieces, lane);
         } else if (warp < G && S.id[warp] >= 0) {
             uint64_t* const pool = S.pool + warp * 32 * EPL;
             uint64_t* const buf = S.buf + warp * EXACT_BUF;
@@ -402,7 +403,8 @@ __device__ __forceinline__ void exact_piece(const ExactArgs& A, const ExactSmem<
             int c = 0;
             for (int p = first; p < first + pieces; ++p) {
                 if (p == piece) continue;
-                const unsigned long long* in = reinterpret_cast<const unsigned long long*>(A.part) + ((size_t)p * G + warp) * A.k;
+                const unsigned long long* in =
+                    reinterpret_cast<const unsigned long long*>(A.part) + ((size_t)p * G + warp) * A.k;
                 for (int off = 0; off < A.k; off += 32) {
                     const uint64_t key = off + lane < A.k ? (uint64_t)__ldcg(in + off + lane) : KEY_EMPTY;
                     const uint32_t M = __ballot_sync(FULL, key != KEY_EMPTY && key <= tau);
@@ -866,9 +868,11 @@ struct ExactScratch {
 size_t up256(size_t x) { return (x + 255) & ~(size_t)255; }
 size_t exact_rest_bytes(size_t queries) { return up256(queries * 8) + up256((EXACT_BINS + 2) * 4) + up256(queries * 4); }
 size_t exact_bytes(size_t nq, const ExactCut& c, bool few) {
-    return up256(nq * 8) + (few ? 0 : up256(nq * 4) + up256(c.groups * 8) + up256((c.pieces + c.groups) * 16)) + up256(c.lists * 8);
+    const size_t grouping = few ? 0 : up256(nq * 4) + up256(c.groups * 8) + up256((c.pieces + c.groups) * 16);
+    return up256(nq * 8) + grouping + up256(c.lists * 8);
 }
-bool exact_scratch(frog_index* ix, FrogExactSet* set, cudaStream_t s, size_t nq, const ExactCut& c, bool few, ExactScratch* out) {
+bool exact_scratch(frog_index* ix, FrogExactSet* set, cudaStream_t s, size_t nq, const ExactCut& c, bool few,
+                   ExactScratch* out) {
     const size_t bytes = exact_bytes(nq, c, few);
     if (!set->mem || nq > set->queries || bytes > set->bytes) {
         // Growing takes 0.5-3 ms.  A first scan of 2,000 queries, k = 100, without scratch / with growth: 20,000 x 96 (7.7 MB)
@@ -942,7 +946,8 @@ extern "C" int frog_exact_search(const frog_index_t* index, const float* queries
     const size_t smem = !few ? exact_smem<EXACT_GROUP>(k, A.d_pad)
                              : exact_smem<1>(k, A.d_pad) + (form == ExactForm::Few ? sizeof(FewExtra) : sizeof(SplitExtra));
     // (the planning kernels count queries in ints with some room)
-    if (capture == cudaStreamCaptureStatusNone && form != ExactForm::OnePerQuery && smem <= froghost::MAX_SMEM && nq <= 1 << 30) {
+    if (capture == cudaStreamCaptureStatusNone && form != ExactForm::OnePerQuery && smem <= froghost::MAX_SMEM &&
+        nq <= 1 << 30) {
         const exact_fn fn = form == ExactForm::Few ? exact_pick<Few>(k) : few ? exact_pick<Split>(k) : exact_pick<Grouped>(k);
         FROG_CUDA_TRY(froghost::allow_smem(fn));
         int per_sm = 0;

@@ -650,7 +650,8 @@ int plan_team(const frog_index* ix, int beam_width, const frog_params_t& P, int 
                           : ix->has_tmap_f32 && (row_bytes == 384 || row_bytes == 512);
     const int per_sm_nq = (nq - 1) / ix->sm_count + 1;
     const int warps = per_sm_nq <= (row_bytes <= STAGE_CHUNK || (f16 && P.budget <= 24) ? 2 : 4) ? 8 : 4;
-    if (warps == 4 && (lean || per_sm_nq > team_queries_per_sm(row_bytes, f16, beam_width, P.budget, (size_t)ix->info.n * row_bytes)))
+    const size_t index_bytes = (size_t)ix->info.n * row_bytes;
+    if (warps == 4 && (lean || per_sm_nq > team_queries_per_sm(row_bytes, f16, beam_width, P.budget, index_bytes)))
         return FROG_ERR_UNSUPPORTED;
     // a table of about 16 ranks per beam slot: smaller ones repeat distances (3,072-byte rows at beam 192:
     // 1.3x slower with 2,048 ranks than with 4,096), larger ones cost resident CTAs
@@ -987,7 +988,8 @@ extern "C" int frog_search_ex(const frog_index_t* index, const float* queries, c
     // (a team launch whose queries all start at once takes no numbers and needs no order)
     if (!team || plan.grid < nq) FROG_CUDA_TRY(cudaMemsetAsync(sc->d_work, 0, 1024, s));
     // planning pass (skipped for tiny batches and when its scratch cannot be had)
-    const bool planned = !(P.debug_flags & 2) && nq >= 64 && (!team || plan.grid < nq) && froghost::ensure_plan(sc, (size_t)nq) == FROG_OK;
+    const bool planned = !(P.debug_flags & 2) && nq >= 64 && (!team || plan.grid < nq) &&
+                         froghost::ensure_plan(sc, (size_t)nq) == FROG_OK;
     if (planned) {
         int2* ranges = reinterpret_cast<int2*>(sc->d_plan);
         int32_t* order = sc->d_plan + 2 * sc->plan_queries;
@@ -1021,7 +1023,8 @@ FrogScratch* last_search_on(frog_index* ix, cudaStream_t s) {
     FrogScratch* last = nullptr;
     for (int i = 0; i < ix->n_scratch; ++i) {
         FrogScratch& sc = ix->scratch[i];
-        if (sc.tick && sc.stream == s && (s != cudaStreamPerThread || sc.stream_id == id) && (!last || sc.tick > last->tick)) last = &sc;
+        const bool same = sc.tick && sc.stream == s && (s != cudaStreamPerThread || sc.stream_id == id);
+        if (same && (!last || sc.tick > last->tick)) last = &sc;
     }
     return last;
 }

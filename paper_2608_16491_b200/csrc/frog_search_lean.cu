@@ -579,8 +579,8 @@ namespace froghost {
 // variant whose visited set is the L2-resident hash table (pools of up to 128 keys only); `hook`: the
 // instantiation whose gathers time out by construction (bitmap form, beams up to 32, budgets up to 64);
 // `queries_per_sm`: of the batch, 0 = not known (a full GPU).
-frog_kernel_fn lean_kernel(int ef_s, int budget, int row_bytes, bool f16, bool table, bool hook, int queries_per_sm, size_t* smem_per_warp,
-                           int* warps_per_cta) {
+frog_kernel_fn lean_kernel(int ef_s, int budget, int row_bytes, bool f16, bool table, bool hook, int queries_per_sm,
+                           size_t* smem_per_warp, int* warps_per_cta) {
     *warps_per_cta = LEAN_WARPS;
     const bool roomy = queries_per_sm > 0 && queries_per_sm <= LEAN_ROOMY_WARPS;
     if (f16) {
