@@ -189,9 +189,9 @@ int frog_search_ex(const frog_index_t* index, const float* queries, const int32_
  * queries that share them for larger ones.  One CTA per query scans instead, without scratch: where the index
  * is too small for pieces to pay, rows too long for eight queries in shared memory, more than 2^30 queries,
  * a call under stream capture, and a call whose scratch cannot be had.  The results are the same.
- * Scratch: an index is loaded with what one stream's scans of up to 2,048 queries with k <= 128 need, but
- * no more than a quarter of its own size; a scan on another stream, up to four in flight at once, or one that
- * needs more allocates with cudaMalloc (0.5-3 ms, kept until frog_index_free) -- on indexes of up to 16 MB of
+ * Scratch: an index is loaded with what one stream's scans of up to 2,048 queries with k <= 128 need (39 MB at
+ * most), but no more than half of its own size; a scan on another stream, up to 16 in flight at once, or one
+ * that needs more allocates with cudaMalloc (0.5-3 ms, kept until frog_index_free) -- on indexes of up to 16 MB of
  * rows only from the second such call on.  None of it is shared with frog_search.
  * Same buffers and conventions as frog_search; 1 <= k <= FROG_MAX_BEAM_WIDTH.  Used for ground truth
  * and as the pre-filtering reference. */

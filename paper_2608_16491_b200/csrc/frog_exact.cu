@@ -995,11 +995,11 @@ extern "C" int frog_exact_search(const frog_index_t* index, const float* queries
     return FROG_OK;
 }
 
-// Scratch for one stream's scans of up to 2,048 queries with k up to 128, but no more than a quarter of the index, so that
-// a first scan has nothing to allocate as a rule.  Not having it is no error.
+// Scratch for one stream's scans of up to 2,048 queries with k up to 128 (39 MB at most), but no more than half of the
+// index, so that a first scan has nothing to allocate as a rule.  Not having it is no error.
 void froghost::reserve_exact(frog_index* ix) {
     const ExactCut cut = exact_cut_of((size_t)ix->info.n, 2048, 128, 2 * ix->sm_count, false);
-    const size_t bytes = std::min(exact_bytes(2048, cut, false), (size_t)ix->info.device_bytes / 4);
+    const size_t bytes = std::min(exact_bytes(2048, cut, false), (size_t)ix->info.device_bytes / 2);
     FrogExactSet& set = ix->exact[0];
     if (cudaEventCreateWithFlags(&set.done, cudaEventDisableTiming) != cudaSuccess) {
         cudaGetLastError();

@@ -42,7 +42,7 @@ struct FrogExactSet {
     unsigned long long stream_id = 0;   // and its stream
     bool used = false;
 };
-constexpr int FROG_EXACT_SETS = 4;
+constexpr int FROG_EXACT_SETS = 16;   // a scan on a further stream in flight does without
 constexpr int FROG_TABLE_BITS = 12;    // 4,096 ranks = 16 KB per resident warp: 78 MB for a full grid, inside L2
 constexpr int FROG_TABLE_BITS_WIDE = 13;   // beam widths 65..128: 8,192 ranks (a query evaluates ~2,000 there)
 

@@ -244,12 +244,12 @@ def test_scans_beside_another_threads_capture(libs, tmp_path):
 
 
 def test_a_first_scan_of_common_size_allocates_nothing(libs, tmp_path):
-    """The scratch of up to 2,048 queries with k up to 128 comes with the index, as far as a quarter of its size."""
+    """The scratch of up to 2,048 queries with k up to 128 comes with the index, as far as half of its size."""
     base, attrs, path = _index(libs, tmp_path, 50000, 96, 3)
     ix = oracle.load_index(path)
     q, lo, hi = _queries(base, attrs, 2048, 8, 6)
     dev = [torch.from_numpy(x).cuda() for x in (q, lo, hi)]
-    for nq, k in ((1, 10), (16, 128), (200, 128), (500, 10), (2048, 10)):
+    for nq, k in ((1, 10), (16, 128), (200, 128), (500, 10), (2048, 10), (2048, 20)):
         gix = libs.Index.load(path)
         out = [torch.empty((nq, k), dtype=t, device="cuda") for t in (torch.int32, torch.float32)]
         part = [x[:nq] for x in dev]
@@ -319,3 +319,26 @@ def test_two_threads_whose_calls_need_different_shared_memory(libs, tmp_path):
     for t in threads:
         t.join()
     assert [w[1] for w in work] == [[], []]
+
+
+def test_more_streams_in_flight_than_scratch_sets(libs, tmp_path):
+    """20 streams: the last of them scan without scratch, with the same results."""
+    base, attrs, path = _index(libs, tmp_path, 60000, 64, 21)
+    gix = libs.Index.load(path)
+    q, lo, hi = _queries(base, attrs, 400, 3, 2)
+    dev = [torch.from_numpy(x).cuda() for x in (q, lo, hi)]
+    want = gix.exact_search(*dev, 50)
+    streams = [torch.cuda.Stream() for _ in range(20)]
+    torch.cuda.synchronize()
+    got = []
+    for i in range(60):
+        n = (400, 60, 9)[i // 20]
+        out = [torch.empty((n, 50), dtype=t, device="cuda") for t in (torch.int32, torch.float32)]
+        got.append(out)
+    torch.cuda.synchronize()
+    for i, out in enumerate(got):
+        gix.exact_search(*(x[:len(out[0])] for x in dev), 50, out_ids=out[0], out_dists=out[1], stream=streams[i % 20])
+    torch.cuda.synchronize()
+    for g in got:
+        assert torch.equal(g[0], want[0][:len(g[0])]) and torch.equal(g[1], want[1][:len(g[0])])
+    gix.close()
