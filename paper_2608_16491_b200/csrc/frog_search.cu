@@ -642,7 +642,9 @@ int team_queries_per_sm(int row_bytes, bool f16, int beam_width, int budget, siz
 // SM; 4 per SM for rows of several chunks, but not for fp16 rows with small budgets), then four up to the line above,
 // except on the rows that the kernel of frog_search_lean.cu covers, which one warp serves well enough (256-byte fp16
 // rows, beam 64, B 64: 400 queries 343 us with one warp per query and 410 with four, 900: 349 / 585).
-int plan_team(const frog_index* ix, int beam_width, const frog_params_t& P, int nq, LaunchPlan* out, int* vis_bits) {
+// `any_batch`: also where one warp per query would be faster (this kernel needs no visited slabs).
+int plan_team(const frog_index* ix, int beam_width, const frog_params_t& P, int nq, LaunchPlan* out, int* vis_bits,
+              bool any_batch = false) {
     const bool f16 = P.storage == FROG_STORAGE_F16;
     const int q_len = query_len(ix->info.d);
     const int row_bytes = f16 ? q_len * 2 : ix->info.d_pad * 4;
@@ -651,7 +653,8 @@ int plan_team(const frog_index* ix, int beam_width, const frog_params_t& P, int 
     const int per_sm_nq = (nq - 1) / ix->sm_count + 1;
     const int warps = per_sm_nq <= (row_bytes <= STAGE_CHUNK || (f16 && P.budget <= 24) ? 2 : 4) ? 8 : 4;
     const size_t index_bytes = (size_t)ix->info.n * row_bytes;
-    if (warps == 4 && (lean || per_sm_nq > team_queries_per_sm(row_bytes, f16, beam_width, P.budget, index_bytes)))
+    if (!any_batch && warps == 4 &&
+        (lean || per_sm_nq > team_queries_per_sm(row_bytes, f16, beam_width, P.budget, index_bytes)))
         return FROG_ERR_UNSUPPORTED;
     // a table of about 16 ranks per beam slot: smaller ones repeat distances (3,072-byte rows at beam 192:
     // 1.3x slower with 2,048 ranks than with 4,096), larger ones cost resident CTAs
@@ -914,8 +917,8 @@ extern "C" int frog_search_ex(const frog_index_t* index, const float* queries, c
     // one CTA per query where that pays; any explicit choice of the visited set, ablation or test hook keeps
     // the kernels it names
     int vis_bits = 0;
-    const bool team = mode == MODE_FAST && P.visited == FROG_VISITED_AUTO && !P.eager_hash && !(P.debug_flags & ~(2 | 16)) &&
-                      plan_team(index, beam_width, P, nq, &plan, &vis_bits) == FROG_OK;
+    const bool may_team = mode == MODE_FAST && P.visited == FROG_VISITED_AUTO && !P.eager_hash && !(P.debug_flags & ~(2 | 16));
+    bool team = may_team && plan_team(index, beam_width, P, nq, &plan, &vis_bits) == FROG_OK;
     if (team) bitmap = false;
     else rc = plan_launch(index, beam_width, P, mode, bitmap, nq, &plan);
     if (rc) return rc;
@@ -928,9 +931,14 @@ extern "C" int frog_search_ex(const frog_index_t* index, const float* queries, c
     if (bitmap) {
         rc = froghost::ensure_bitmap(index, sc, (size_t)plan.grid * WARPS_PER_CTA);
         if (rc == FROG_ERR_NOMEM && P.visited == FROG_VISITED_AUTO) {
-            // no room for the slabs: fall back to the shared-memory table
+            // no room for the slabs: fall back to the shared-memory table, or for fp16 rows, which its kernels do not
+            // read, to the form with one CTA per query
             bitmap = false;
             rc = plan_launch(index, beam_width, P, mode, false, nq, &plan);
+            if (rc == FROG_ERR_UNSUPPORTED && may_team) {
+                rc = plan_team(index, beam_width, P, nq, &plan, &vis_bits, true);
+                team = rc == FROG_OK;
+            }
         }
         if (rc) return rc;
     }

@@ -46,3 +46,44 @@ def test_every_pool(libs, tmp_path, d, storage, copies):
             other = gix.search_static(*q1, 10, ef, params=libs.Params(budget=budget, storage=storage))
             assert torch.equal(other[0], ids) and torch.equal(other[1], dists)
     gix.close()
+
+
+def test_fp16_batch_without_room_for_visited_slabs(libs):
+    """600 queries need 170 MB of slabs on this index; where they cannot be had, the form that needs none runs."""
+    import ctypes
+    n, d, nq = 2_000_000, 96, 600
+    vec = (np.arange(n * d, dtype=np.int32) * 7919 % 1021).astype(np.float32).reshape(n, d)
+    rank = np.arange(n, dtype=np.int32)
+    enc = np.full((n, 4), 0xFFFFFFFF, dtype=np.uint32)
+    enc[:, 0] = (np.arange(n, dtype=np.int64) * 31 + 7) % n
+    shape = libs.IndexInfo(n=n, d=d, d_pad=d, H=1, m=4)
+    ptr = lambda x: x.ctypes.data_as(ctypes.c_void_p)
+
+    def load():
+        h = ctypes.c_void_p()
+        assert libs._lib.frog_index_from_host(ptr(rank), ptr(rank), ptr(vec), ptr(enc), ctypes.byref(shape), 0, ctypes.byref(h)) == 0
+        gix = libs.Index(h)
+        gix.enable_f16()
+        return gix
+
+    g = torch.Generator(device="cuda").manual_seed(1)
+    q = torch.randint(0, 1000, (nq, d), generator=g, device="cuda").float()
+    lo = torch.randint(0, n // 2, (nq,), generator=g, device="cuda", dtype=torch.int32)
+    hi = lo + n // 3
+    prm = libs.Params(budget=64, storage=1)
+    out = [torch.empty((nq, 10), dtype=t, device="cuda") for t in (torch.int32, torch.float32)]
+    gix = load()
+    want = [t.clone() for t in gix.search(q, lo, hi, 10, 64, params=prm)]
+    torch.cuda.synchronize()
+    gix.close()
+    gix = load()
+    torch.cuda.empty_cache()
+    fill = [torch.empty(torch.cuda.mem_get_info()[0] - (120 << 20), dtype=torch.uint8, device="cuda")]
+    try:
+        gix.search(q, lo, hi, 10, 64, params=prm, out_ids=out[0], out_dists=out[1])
+        torch.cuda.synchronize()
+    finally:
+        fill.clear()
+        torch.cuda.empty_cache()
+    assert torch.equal(out[0], want[0]) and torch.equal(out[1], want[1])
+    gix.close()
