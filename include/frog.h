@@ -242,12 +242,14 @@ int frog_search_static(const frog_index_t* index, const float* queries, const in
  * that concern the whole launch rather than one query: today FROG_ST_COPY_TIMEOUT (some row of the
  * result was written as padding because a bulk copy never completed; never expected).  Lets a caller
  * that passes no `status` array notice it.  Waits for that launch to finish.  INVALID_ARG if there
- * was no launch on the stream.  frog_search_static keeps no such word. */
+ * was no launch on the stream, or if a later search on another stream has taken over its scratch set
+ * (see frog_search), with which the word goes.  frog_search_static keeps no such word. */
 int frog_search_last_status(const frog_index_t* index, void* stream, uint32_t* flags);
 
 /* Device time, in milliseconds, of the search kernel of the last frog_search_ex call on `stream` that
  * was made with params->debug_flags bit 4 set (the call also runs two small planning kernels, which
- * this figure leaves out).  Waits for that kernel to finish.  INVALID_ARG if there was no such call. */
+ * this figure leaves out).  Waits for that kernel to finish.  INVALID_ARG if there was no such call, or as
+ * for frog_search_last_status. */
 int frog_search_kernel_ms(const frog_index_t* index, void* stream, float* ms);
 
 /* Launch shape of the search kernel for the given beam width and a batch that fills the GPU (for
