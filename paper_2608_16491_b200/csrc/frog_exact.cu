@@ -11,6 +11,7 @@
 //     shared by all pieces of a query through global memory: whatever exceeds the k-th best of ANY piece
 //     cannot be an answer;
 //   * the last CTA to finish a group merges the pieces' lists.
+// Many queries on all but small indexes are filtered first (frog_exact_filter.cu).
 // Few queries are not grouped: all rows are cut into equal pieces, one query each (one launch for fewer than
 // EXACT_PLAN_MIN, else a planning kernel finds the slabs first).  Otherwise queries are ordered by (width, position),
 // grouped by eight, and the groups' rows are cut into pieces of equal size (two small kernels).  The form with one CTA
@@ -19,6 +20,7 @@
 #include <algorithm>
 
 #include "frog_device.cuh"
+#include "frog_exact_filter.h"
 #include "frog_internal.h"
 
 using namespace frogdev;
@@ -792,9 +794,23 @@ size_t exact_smem(int k, int d_pad) {
 // 162/134/122).  Over 3,400 combinations (300 to 1,000,000 objects, 32 to 2,000 dimensions, 1-2,000 queries, k = 10 to
 // 512, three mixes of widths) the rule takes 0.51 of the time of one CTA per query in the mean and is slower by more
 // than a tenth in 1 %; the best form of each would take 0.48.
-enum class ExactForm { OnePerQuery, Few, Split, Grouped };
-ExactForm exact_form(size_t n, size_t row_bytes, int nq, int k) {
+// More queries than a line that depends on rows and k, on 4,000 rows or more, are filtered (frog_exact_filter.cu): six
+// launches and two passes of products, which take 50-110 us in any case and hardly grow with the queries.  us, the
+// form of the lines above / filtered, log-uniform widths down to 2^-10 | all rows:
+//                      40 queries, k = 10      100, k = 10           400, k = 10            2,000, k = 100
+//   3,000 x 96      34/55 | 58/48         50/55 | 54/48          54/60 | 66/53        120/123 | 369/136
+//   5,000 x 128     33/56 | 51/52         74/58 | 84/51          82/62 | 104/60       168/135 | 546/517
+//   20,000 x 50     51/54 | 100/50        68/54 | 188/54         240/59 | 282/88      423/170 | 1,270/347
+//   5,000 x 768     43/110 | 76/100       69/112 | 165/104       179/123 | 321/135    345/290 | 1,391/1,461
+//   20,000 x 768    72/121 | 212/117      120/120 | 464/137      283/128 | 1,071/294  1,032/435 | 4,720/1,461
+//   100,000 x 128   90/100 | 253/105      149/107 | 555/129      411/128 | 1,190/259  1,262/324 | -
+//   400,000 x 96    155/207 | 1,200/251   352/246 | 2,926/302    1,032/327 | -        3,802/808 | -
+enum class ExactForm { OnePerQuery, Few, Split, Grouped, Filter };
+ExactForm exact_form(size_t n, size_t row_bytes, int nq, int k, bool filter) {
     const size_t bytes = n * row_bytes;
+    if (filter && n >= 4000 && row_bytes <= 16384 &&
+        nq >= (row_bytes > 1024 ? (n >= 16000 ? 128 : 400) : n < 16000 ? 100 : k <= 32 ? 80 : n < 64000 ? 40 : EXACT_PLAN_MIN))
+        return ExactForm::Filter;
     if (nq < EXACT_PLAN_MIN) return k <= 32 && bytes <= 500000 ? ExactForm::OnePerQuery : ExactForm::Few;
     const double work = (double)n * (double)(row_bytes + 384) * (k > 128 ? 3.0 : k > 64 ? 1.4 : 1.0);
     if (nq <= EXACT_SPLIT_MAX && nq * (n < 8000 ? 45e3 : 100e3) <= work) return ExactForm::Split;
@@ -871,9 +887,8 @@ size_t exact_bytes(size_t nq, const ExactCut& c, bool few) {
     const size_t grouping = few ? 0 : up256(nq * 4) + up256(c.groups * 8) + up256((c.pieces + c.groups) * 16);
     return up256(nq * 8) + grouping + up256(c.lists * 8);
 }
-bool exact_scratch(frog_index* ix, FrogExactSet* set, cudaStream_t s, size_t nq, const ExactCut& c, bool few,
-                   ExactScratch* out) {
-    const size_t bytes = exact_bytes(nq, c, few);
+// make sure the set has `bytes` beside what `nq` queries keep between calls
+bool exact_room(frog_index* ix, FrogExactSet* set, size_t nq, size_t bytes) {
     if (!set->mem || nq > set->queries || bytes > set->bytes) {
         // Growing takes 0.5-3 ms.  A first scan of 2,000 queries, k = 100, without scratch / with growth: 20,000 x 96 (7.7 MB)
         // 1,370/1,600 us, 201 queries 490/920; 100,000 x 128 (51 MB) 2,740/1,950.  So on small indexes a scan that would
@@ -897,6 +912,11 @@ bool exact_scratch(frog_index* ix, FrogExactSet* set, cudaStream_t s, size_t nq,
         set->bytes = new_bytes;
         set->clean = false;
     }
+    return true;
+}
+bool exact_scratch(frog_index* ix, FrogExactSet* set, cudaStream_t s, size_t nq, const ExactCut& c, bool few,
+                   ExactScratch* out) {
+    if (!exact_room(ix, set, nq, exact_bytes(nq, c, few))) return false;
     out->bound = set->mem;
     out->counters = out->bound + up256(set->queries * 8);
     out->done = out->counters + up256((EXACT_BINS + 2) * 4);
@@ -941,7 +961,43 @@ extern "C" int frog_exact_search(const frog_index_t* index, const float* queries
     A.out_dists = out_dists;
     cudaStreamCaptureStatus capture = cudaStreamCaptureStatusNone;
     FROG_CUDA_TRY(cudaStreamIsCapturing(s, &capture));
-    const ExactForm form = exact_form((size_t)index->info.n, (size_t)A.d_pad * 4, nq, k);
+    ExactForm form = exact_form((size_t)index->info.n, (size_t)A.d_pad * 4, nq, k, capture == cudaStreamCaptureStatusNone);
+    if (form == ExactForm::Filter) {
+        // (scratch of the sets' part that has no state at rest; where it cannot be had, the other forms)
+        frog_index* mix = const_cast<frog_index*>(index);
+        std::lock_guard<std::mutex> lock(mix->exact_mu);
+        const froghost::FilterRoom room = froghost::filter_room((size_t)index->info.n, (size_t)nq, k, A.d_pad);
+        const size_t want = std::min(room.most, std::max(room.least, std::max((size_t)index->info.device_bytes / 2, (size_t)32 << 20)));
+        FrogExactSet* set = nullptr;
+        {
+            const NoCaptureOfOurs relaxed;
+            set = exact_set(mix, s);
+            if (set && set->bytes < room.least && !exact_room(mix, set, 0, want)) set = nullptr;
+        }
+        if (set) {
+            froghost::FilterArgs F{};
+            F.sorted_attr = A.sorted_attr;
+            F.rank2id = A.rank2id;
+            F.vectors = A.vectors;
+            F.n = A.n;
+            F.d = A.d;
+            F.d_pad = A.d_pad;
+            F.queries = queries;
+            F.lo = lo;
+            F.hi = hi;
+            F.nq = nq;
+            F.k = k;
+            F.out_ids = out_ids;
+            F.out_dists = out_dists;
+            froghost::filter_scratch(set->mem + exact_rest_bytes(set->queries), std::min(set->bytes, room.most), &F);
+            FROG_CUDA_TRY(froghost::filter_launch(F, index->sm_count, s));
+            FROG_CUDA_TRY(cudaEventRecord(set->done, s));
+            FROG_CUDA_TRY(cudaStreamGetId(s, &set->stream_id));
+            set->used = true;
+            return FROG_OK;
+        }
+        form = exact_form((size_t)index->info.n, (size_t)A.d_pad * 4, nq, k, false);
+    }
     const bool few = form != ExactForm::Grouped;
     const size_t smem = !few ? exact_smem<EXACT_GROUP>(k, A.d_pad)
                              : exact_smem<1>(k, A.d_pad) + (form == ExactForm::Few ? sizeof(FewExtra) : sizeof(SplitExtra));

@@ -1,0 +1,619 @@
+// The exact scan of many queries: tensor cores rule rows out, what is left is compared in fp32.
+//
+// A row's distance to a query enters the answer only if it is among the k smallest, and of the rows of a slab all but a
+// few can be told apart from those with a rough distance.  |x|^2 + |q|^2 - 2 x.q with x.q from tf32 matrix
+// instructions is such a distance, for 128 rows and 128 queries at a time, and its error is bounded (row_error):
+//   * bounds: for every query and every 8 (wide slabs: 32) rows the smallest upper bound of a distance.  The k-th
+//     smallest of these belongs to k different rows, so no answer lies beyond it;
+//   * masks: the same products again, one bit per row and query: the lower bound does not exceed that;
+//   * the rows whose bit is set, a little more than k, are compared as frog_exact.cu compares all: fp32, in the fixed
+//     order.  Ids and distances are therefore those of a scan of all rows, bit for bit.
+// Products are computed twice, the second time only for tiles that a bound of the first says may hold an answer, because
+// storing them would take 4 bytes per row and query.  2,000 queries, k = 100, on 100,000 x 128, log-uniform widths:
+// 1,290 us by groups of eight in fp32, 325 filtered: 132 first pass, 17 bounds, 101 second pass, 93 comparison (k = 10:
+// 250).  The passes are bound by fragment loads from shared memory (24 for 16 matrix instructions) and their
+// epilogues, not by the matrix unit (60 TFLOP/s): tiles are as deep as a vector, 32 to 768.  Hence mma.sync, whose
+// accumulators are where the epilogue needs them.
+#include <algorithm>
+
+#include "frog_device.cuh"
+#include "frog_exact_filter.h"
+#include "frog_internal.h"
+
+using namespace frogdev;
+using froghost::FilterArgs;
+
+namespace {
+
+constexpr int TILE = 128;                // rows, and queries, of a tile of products
+constexpr int KC = 32;                   // elements of a row per pipeline stage
+constexpr int KP = KC + 4;               // their stride in shared memory: fragment loads without bank conflicts
+constexpr int STAGES = 2;
+constexpr int SEG = 2048;                // queries listed at a time
+constexpr int THREADS = 256;             // 4 x 2 warps of 32 rows x 64 queries
+
+struct FilterSmem {
+    float a[STAGES][TILE * KP];
+    float b[STAGES][TILE * KP];
+    int list[SEG];                       // queries whose slab meets the tile
+    float row_norm[TILE];
+    int l[TILE], r[TILE];                // of the batch's queries
+    float norm[TILE], tau[TILE];
+    uint32_t off[TILE];
+    int count;
+};
+
+__device__ __forceinline__ uint32_t to_tf32(float x) {
+    uint32_t y;
+    asm("cvt.rna.tf32.f32 %0, %1;" : "=r"(y) : "f"(x));
+    return y;
+}
+__device__ __forceinline__ void mma_tf32(float (&c)[4], const uint32_t (&a)[4], uint32_t b0, uint32_t b1) {
+    asm volatile("mma.sync.aligned.m16n8k8.row.col.f32.tf32.tf32.f32 {%0,%1,%2,%3}, {%4,%5,%6,%7}, {%8,%9}, {%0,%1,%2,%3};"
+                 : "+f"(c[0]), "+f"(c[1]), "+f"(c[2]), "+f"(c[3])
+                 : "r"(a[0]), "r"(a[1]), "r"(a[2]), "r"(a[3]), "r"(b0), "r"(b1));
+}
+// 16 bytes to shared memory, zeros unless `on`
+__device__ __forceinline__ void copy16(void* dst, const void* src, bool on) {
+    const int bytes = on ? 16 : 0;
+    asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(smem_u32(dst)), "l"(src), "r"(bytes) : "memory");
+}
+
+// Values of a query per 32 rows in the first pass: one where its slab is so wide that they are still many more than k
+__device__ __forceinline__ int values_per_block(int w, int k) { return w >= 128 * k ? 1 : 4; }
+// Narrower slabs have hardly k values to choose from: their rows are all compared
+__device__ __forceinline__ bool filtered(int w, int k) { return w >= max(10 * k, 128); }
+
+// slabs of the queries, their norms, and the queries themselves rounded to tf32 (one warp per query)
+__global__ void __launch_bounds__(256)
+filter_plan_kernel(const FilterArgs A) {
+    const unsigned int q = blockIdx.x * 8u + (threadIdx.x >> 5);
+    const int lane = lane_id();
+    if (q >= (unsigned int)A.nq) return;
+    const int32_t lo = __ldg(A.lo + q), hi = __ldg(A.hi + q);
+    int l_q, r_q;
+    warp_rank_interval(A.sorted_attr, A.n, lo, hi, lane, l_q, r_q);
+    float s = 0.f;
+    for (int i = lane; i < A.d_pad; i += 32) {
+        const float x = i < A.d ? __ldg(A.queries + (size_t)q * A.d + i) : 0.f;
+        s = fmaf(x, x, s);
+        A.rounded[(size_t)q * A.d_pad + i] = __uint_as_float(to_tf32(x));
+    }
+    for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(FULL, s, o);
+    if (lane == 0) {
+        A.slab[q] = lo > hi || r_q < l_q ? make_int2(1, 0) : make_int2(l_q, r_q);
+        A.norm[q] = s;
+    }
+}
+
+// where each query's values and masks lie (one CTA); BOT: the query is not filtered
+__global__ void __launch_bounds__(1024)
+filter_offsets_kernel(const FilterArgs A) {
+    __shared__ unsigned long long warp_sum[32];
+    __shared__ unsigned long long base;
+    const int t = threadIdx.x, lane = lane_id(), warp = t >> 5;
+    if (t == 0) base = 0;
+    for (int i = t; i * TILE < A.n; i += 1024) A.tile_norm[i] = 0u;
+    __syncthreads();
+    for (int q0 = 0; q0 < A.nq; q0 += 1024) {
+        const int q = q0 + t;
+        unsigned long long need = 0;                             // 32-bit words: the values, then the masks
+        uint32_t nv = 0;
+        if (q < A.nq) {
+            const int2 s = A.slab[q];
+            const int w = s.y - s.x + 1;
+            if (filtered(w, A.k)) {
+                const uint32_t nb = (uint32_t)((s.y >> 5) - (s.x >> 5) + 1);
+                nv = nb * values_per_block(w, A.k);
+                need = nv + nb;
+            }
+        }
+        unsigned long long x = need;
+        for (int o = 1; o < 32; o <<= 1) {
+            const unsigned long long y = __shfl_up_sync(FULL, x, o);
+            if (lane >= o) x += y;
+        }
+        if (lane == 31) warp_sum[warp] = x;
+        __syncthreads();
+        unsigned long long at = base + x - need;
+        for (int w = 0; w < warp; ++w) at += warp_sum[w];
+        if (q < A.nq) A.off[q] = need != 0 && at + need <= A.words ? (uint32_t)at : BOT;
+        __syncthreads();
+        if (t == 1023) base = at + need;
+        __syncthreads();
+    }
+}
+
+// Bound of the error of a rough distance, and of what separates the fp32 distance of the scan from the true one.
+// With u = 2^-11 the rounding of an operand: |x~.q~ - x.q| <= (2u + u^2) |x| |q|; the sums of d products, of the norms
+// and of the scan are within d 2^-22 of their magnitude each (twice what rounding to nearest gives); the last two terms
+// cover what underflows.  Anything not finite makes the comparisons with it false, which rules nothing out.
+struct RowError {
+    float c1, c2;
+    __device__ __forceinline__ explicit RowError(int d) : c1(0.00197f + d * 0x1p-20f), c2(0x1p-19f + d * 0x1p-21f) {}
+    __device__ __forceinline__ float operator()(float nx, float x, float nq, float q) const {
+        return c1 * x * q + c2 * (nx + nq) + 1e-30f * (x + q) + 1e-34f;
+    }
+};
+
+// PASS 0: bounds, PASS 1: masks.  One CTA per 128 rows and per share of the queries: those whose number is blockIdx.y
+// modulo gridDim.y (the order in which a CTA lists its queries is not that of another).
+template <int PASS>
+__global__ void __launch_bounds__(THREADS, 2)
+filter_tile_kernel(const FilterArgs A) {
+    extern __shared__ __align__(16) unsigned char smem_raw[];
+    FilterSmem& S = *reinterpret_cast<FilterSmem*>(smem_raw);
+    const int t = threadIdx.x, lane = lane_id(), warp = t >> 5;
+    const int wm = warp >> 1, wn = warp & 1;                     // this warp's rows and queries of the tile
+    const int g = lane >> 2, p = lane & 3;                       // fragment coordinates
+    const int row0 = blockIdx.x * TILE, row_end = min(row0 + TILE, A.n);
+    const int chunks = (A.d_pad + KC - 1) / KC;
+    const RowError error(A.d);
+    const float tile_norm = PASS == 1 ? __uint_as_float(A.tile_norm[blockIdx.x]) : 0.f, tile_sqrt = __fsqrt_rn(tile_norm);
+    bool have_norms = false;
+
+    for (int q0 = 0; q0 < A.nq; q0 += SEG) {
+        __syncthreads();
+        if (t == 0) S.count = 0;
+        __syncthreads();
+        for (int i = t; i < SEG; i += THREADS) {                 // (SEG is a multiple of THREADS)
+            const int q = q0 + i;
+            bool hit = false;
+            if (q < A.nq && q % gridDim.y == blockIdx.y && A.off[q] != BOT) {
+                const int2 s = A.slab[q];
+                hit = s.x < row_end && s.y >= row0;
+                if (PASS == 1 && hit) {
+                    // The second pass is for tiles with a row that may be an answer: a value of the first is a lower bound
+                    // too, less twice the error.  (The infinite ones say nothing.)  The masks of the others are zero.
+                    const int w = s.y - s.x + 1, per = values_per_block(w, A.k), all = (s.y >> 5) - (s.x >> 5) + 1;
+                    const int from = max((row0 >> 5) - (s.x >> 5), 0), to = min(((row0 + TILE) >> 5) - (s.x >> 5), all);
+                    const float nq = A.norm[q], tau = A.tau[q], e = 2.f * error(tile_norm, tile_sqrt, nq, __fsqrt_rn(nq));
+                    const uint32_t* const v = A.store + A.off[q];
+                    hit = false;
+                    for (int x = from * per; x < to * per; ++x) {
+                        const float least = __uint_as_float(v[x]);
+                        hit = hit || !(least - e > tau) || !(least < __int_as_float(0x7F800000));
+                    }
+                    if (!hit)
+                        for (int x = from; x < to; ++x) A.store[A.off[q] + all * per + x] = 0u;
+                }
+            }
+            const uint32_t M = __ballot_sync(FULL, hit);
+            int at = 0;
+            if (lane == 0 && M) at = atomicAdd(&S.count, __popc(M));
+            at = __shfl_sync(FULL, at, 0);
+            if (hit) S.list[at + __popc(M & ((1u << lane) - 1u))] = q;
+        }
+        __syncthreads();
+        const int count = S.count;
+        for (int b0 = 0; b0 < count; b0 += TILE) {
+            const int nb = min(TILE, count - b0);
+            __syncthreads();                                     // the batch before is done with the tables
+            if (t < TILE) {
+                const int q = S.list[b0 + min(t, nb - 1)];
+                const int2 s = t < nb ? A.slab[q] : make_int2(1, -1);
+                const int w = s.y - s.x + 1;
+                S.l[t] = s.x;
+                S.r[t] = s.y;
+                S.norm[t] = A.norm[q];
+                if (PASS == 1) {
+                    const int blocks = (s.y >> 5) - (s.x >> 5) + 1;
+                    S.tau[t] = A.tau[q];
+                    S.off[t] = A.off[q] + (t < nb ? (uint32_t)(blocks * values_per_block(w, A.k)) : 0u);
+                } else {
+                    S.off[t] = A.off[q];
+                    S.tau[t] = __int_as_float(t < nb ? values_per_block(w, A.k) : 0);
+                }
+            }
+            float acc[2][8][4];
+#pragma unroll
+            for (int m = 0; m < 2; ++m)
+#pragma unroll
+                for (int x = 0; x < 8; ++x)
+#pragma unroll
+                    for (int c = 0; c < 4; ++c) acc[m][x][c] = 0.f;
+            auto fetch = [&](int chunk) {
+                const int st = chunk % STAGES;
+#pragma unroll
+                for (int x = 0; x < TILE * (KC / 4) / THREADS; ++x) {
+                    const int i = x * THREADS + t, r = i / (KC / 4), c = (i % (KC / 4)) * 4;
+                    const bool in = chunk * KC + c < A.d_pad;
+                    const bool ra = in && row0 + r < A.n, rb = in && r < nb;
+                    copy16(&S.a[st][r * KP + c], A.vectors + (ra ? (size_t)(row0 + r) * A.d_pad + chunk * KC + c : 0), ra);
+                    copy16(&S.b[st][r * KP + c], A.rounded + (rb ? (size_t)S.list[b0 + r] * A.d_pad + chunk * KC + c : 0), rb);
+                }
+            };
+#pragma unroll
+            for (int x = 0; x < STAGES - 1; ++x) {
+                if (x < chunks) fetch(x);
+                asm volatile("cp.async.commit_group;" ::: "memory");
+            }
+            float part = 0.f;                                    // of the norm of row t / 2
+            for (int chunk = 0; chunk < chunks; ++chunk) {
+                asm volatile("cp.async.wait_group %0;" ::"n"(STAGES - 2) : "memory");
+                __syncthreads();
+                if (chunk + STAGES - 1 < chunks) fetch(chunk + STAGES - 1);
+                asm volatile("cp.async.commit_group;" ::: "memory");
+                const float* const a = S.a[chunk % STAGES];
+                const float* const b = S.b[chunk % STAGES];
+                if (!have_norms) {
+                    const float4* const x = reinterpret_cast<const float4*>(a + (t >> 1) * KP + (t & 1) * (KC / 2));
+#pragma unroll
+                    for (int c = 0; c < KC / 8; ++c) {
+                        const float4 v = x[c];
+                        part = fmaf(v.x, v.x, part);
+                        part = fmaf(v.y, v.y, part);
+                        part = fmaf(v.z, v.z, part);
+                        part = fmaf(v.w, v.w, part);
+                    }
+                }
+                if (wn * 64 < nb) {
+#pragma unroll
+                    for (int k0 = 0; k0 < KC; k0 += 8) {
+                        uint32_t fa[2][4];
+#pragma unroll
+                        for (int m = 0; m < 2; ++m) {
+                            const float* const x = a + (wm * 32 + m * 16 + g) * KP + k0 + p;
+                            fa[m][0] = to_tf32(x[0]);
+                            fa[m][1] = to_tf32(x[8 * KP]);
+                            fa[m][2] = to_tf32(x[4]);
+                            fa[m][3] = to_tf32(x[8 * KP + 4]);
+                        }
+#pragma unroll
+                        for (int x = 0; x < 8; ++x) {
+                            const float* const y = b + (wn * 64 + x * 8 + g) * KP + k0 + p;
+                            const uint32_t b0f = __float_as_uint(y[0]), b1f = __float_as_uint(y[4]);
+                            mma_tf32(acc[0][x], fa[0], b0f, b1f);
+                            mma_tf32(acc[1][x], fa[1], b0f, b1f);
+                        }
+                    }
+                }
+            }
+            asm volatile("cp.async.wait_group 0;" ::: "memory");
+            if (!have_norms) {
+                part += __shfl_xor_sync(FULL, part, 1);
+                if ((t & 1) == 0) S.row_norm[t >> 1] = part;
+                have_norms = true;
+                if (PASS == 0) {
+                    const uint32_t most = __reduce_max_sync(FULL, __float_as_uint(part));
+                    if (lane == 0) atomicMax(A.tile_norm + blockIdx.x, most);
+                }
+                __syncthreads();
+            }
+            if (wn * 64 < nb) {
+                // this thread's rows are base + g + 8 j, its queries 8 x + 2 p and the next one
+                const int base = row0 + wm * 32;
+                bool finite = true;
+                float nx[4], sx[4];
+#pragma unroll
+                for (int j = 0; j < 4; ++j) {
+                    nx[j] = S.row_norm[wm * 32 + g + 8 * j];
+                    sx[j] = __fsqrt_rn(nx[j]);
+                }
+#pragma unroll
+                for (int x = 0; x < 8; ++x) {
+                    uint32_t bits[2][4];
+#pragma unroll
+                    for (int c = 0; c < 2; ++c) {
+                        const int i = wn * 64 + x * 8 + 2 * p + c;
+                        const int l = S.l[i], r = S.r[i];
+                        const float nq = S.norm[i], sq = __fsqrt_rn(nq), tau = S.tau[i];
+                        float least = __int_as_float(0x7F800000);
+#pragma unroll
+                        for (int j = 0; j < 4; ++j) {
+                            const int row = base + g + 8 * j;
+                            const float rough = fmaf(-2.f, acc[j >> 1][x][(j & 1) * 2 + c], nx[j] + nq);
+                            const float e = error(nx[j], sx[j], nq, sq);
+                            const bool in = row >= l && row <= r;
+                            if (PASS == 0) {
+                                if (in && rough + e < least) least = rough + e;
+                                finite = finite && (!in || rough + e < __int_as_float(0x7F800000));
+                            } else {
+                                bits[c][j] = __ballot_sync(FULL, in && !(rough - e > tau));
+                            }
+                        }
+                        if (PASS == 0) {
+                            least = least > 0.f ? least : 0.f;
+                            least = fminf(least, __shfl_xor_sync(FULL, least, 4));
+                            const float wide = fminf(least, __shfl_xor_sync(FULL, least, 8));
+                            const float all = fminf(wide, __shfl_xor_sync(FULL, wide, 16));
+                            const int block = (base >> 5) - (l >> 5), per = __float_as_int(tau);
+                            if (block >= 0 && base <= r) {
+                                if (per == 4 && (g & 1) == 0) A.store[S.off[i] + 4 * block + (g >> 1)] = __float_as_uint(least);
+                                if (per == 1 && g == 0) A.store[S.off[i] + block] = __float_as_uint(all);
+                            }
+                        }
+                    }
+                    if (PASS == 1 && lane < 8) {
+                        // query 8 x + lane: lanes 4 g + lane / 2 of the ballots of its parity; bit 4 g + j is row g + 8 j
+                        uint32_t word = 0;
+#pragma unroll
+                        for (int j = 0; j < 4; ++j)
+                            word |= ((((lane & 1) ? bits[1][j] : bits[0][j]) >> (lane >> 1)) & 0x11111111u) << j;
+                        const int i = wn * 64 + x * 8 + lane;
+                        const int block = (base >> 5) - (S.l[i] >> 5);
+                        if (block >= 0 && base <= S.r[i]) A.store[S.off[i] + block] = word;
+                    }
+                }
+                if (PASS == 0 && !finite) atomicMax(A.tile_norm + blockIdx.x, 0x7F800000u);
+            }
+        }
+    }
+}
+
+// Per query: an upper bound, within 2^-14, of the k-th smallest of its values.  Two passes over the values, eleven bits
+// of the (non-negative) numbers each.
+__global__ void __launch_bounds__(256)
+filter_bound_kernel(const FilterArgs A) {
+    __shared__ unsigned int bins[2048];
+    __shared__ unsigned int warp_sum[8];
+    __shared__ unsigned int found[2];                            // the bin that holds the k-th, values below it
+    const int q = blockIdx.x, t = threadIdx.x, lane = lane_id(), warp = t >> 5;
+    const uint32_t off = A.off[q];
+    if (off == BOT) return;
+    const int2 s = A.slab[q];
+    const int nv = ((s.y >> 5) - (s.x >> 5) + 1) * values_per_block(s.y - s.x + 1, A.k);
+    unsigned int want = (unsigned int)A.k, prefix = 0;
+    for (int pass = 0; pass < 2; ++pass) {
+        for (int i = t; i < 2048; i += 256) bins[i] = 0u;
+        if (t == 0) found[0] = 0x7F8u;
+        __syncthreads();
+        for (int i = t; i < nv; i += 256) {
+            const uint32_t v = A.store[off + i];
+            if (pass == 0) atomicAdd(&bins[v >> 20], 1u);
+            else if ((v >> 20) == prefix) atomicAdd(&bins[(v >> 9) & 0x7FFu], 1u);
+        }
+        __syncthreads();
+        unsigned int mine = 0;
+        for (int i = 0; i < 8; ++i) mine += bins[8 * t + i];
+        unsigned int x = mine;
+        for (int o = 1; o < 32; o <<= 1) {
+            const unsigned int y = __shfl_up_sync(FULL, x, o);
+            if (lane >= o) x += y;
+        }
+        if (lane == 31) warp_sum[warp] = x;
+        __syncthreads();
+        unsigned int below = x - mine;
+        for (int w = 0; w < warp; ++w) below += warp_sum[w];
+        if (below < want && below + mine >= want) {
+            int i = 8 * t;
+            while (below + bins[i] < want) below += bins[i++];
+            found[0] = (unsigned int)i;
+            found[1] = below;
+        }
+        __syncthreads();
+        if (pass == 0) {
+            prefix = found[0];
+            if (prefix >= 0x7F8u) break;                         // fewer than k finite values
+            want -= found[1];
+            __syncthreads();
+        }
+    }
+    if (t == 0) A.tau[q] = prefix >= 0x7F8u ? __int_as_float(0x7F800000) : __uint_as_float(prefix << 20 | found[0] << 9 | 0x1FFu);
+}
+
+// The rows that are left, one CTA of four warps per query, so that those of 2,000 queries are resident together; four
+// rows per team in flight, as a step is a round trip.
+constexpr int REFINE_WARPS = 4, REFINE_BUF = 192, REFINE_STEP = REFINE_WARPS * 16;
+constexpr int REFINE_MORE = 1024;        // rows listed before they are compared; as many as 128 masks give come on top
+constexpr int REFINE_LIST = REFINE_MORE + REFINE_WARPS * 32 * 32;
+template <int EPL>
+struct RefineSmem {
+    uint64_t pool[32 * EPL];
+    uint64_t buf[REFINE_BUF];            // merged from 128 on, a step adds at most 64
+    uint64_t bound;                      // keys from here on are not wanted
+    uint16_t list[REFINE_LIST];          // rows to compare, from a base on
+    int count, kept;                     // entries of list, of buf
+};
+
+template <int EPL>
+__global__ void __launch_bounds__(REFINE_WARPS * 32)
+filter_refine_kernel(const FilterArgs A) {
+    extern __shared__ __align__(16) unsigned char smem_raw[];
+    RefineSmem<EPL>& S = *reinterpret_cast<RefineSmem<EPL>*>(smem_raw);
+    const float4* const qs = reinterpret_cast<const float4*>(smem_raw + (sizeof(RefineSmem<EPL>) + 15) / 16 * 16);
+    const int q = blockIdx.x, t = threadIdx.x, lane = lane_id(), warp = t >> 5;
+    const int team = t >> 3, sub = lane & 7, groups = A.d_pad >> 2;
+    const int2 slab = A.slab[q];
+    const int w = slab.y - slab.x + 1;
+    const uint32_t off = A.off[q];
+    {
+        float* qf = reinterpret_cast<float*>(smem_raw + (sizeof(RefineSmem<EPL>) + 15) / 16 * 16);
+        for (int i = t; i < A.d_pad; i += REFINE_WARPS * 32) qf[i] = i < A.d ? __ldg(A.queries + (size_t)q * A.d + i) : 0.f;
+        for (int i = t; i < 32 * EPL; i += REFINE_WARPS * 32) S.pool[i] = KEY_EMPTY;
+        if (t == 0) {
+            S.kept = 0;
+            S.bound = KEY_EMPTY;
+            if (off != BOT && A.tau[q] < __int_as_float(0x7F800000)) S.bound = (uint64_t)__float_as_uint(A.tau[q]) << 32 | 0xFFFFFFFFu;
+        }
+    }
+    auto flush = [&]() {                                         // warp 0
+        for (int x = 0; x < S.kept; x += 32) merge_ranked<EPL>(S.pool, S.buf + x, min(32, S.kept - x), A.k, lane);
+        __syncwarp();
+        if (lane == 0) {
+            S.bound = min(S.bound, S.pool[A.k - 1]);
+            S.kept = 0;
+        }
+    };
+    // rows first + list[0..n), or first + [0..n)
+    auto compare = [&](int n, int first, bool listed) {
+        for (int j0 = 0; j0 < n; j0 += REFINE_STEP) {
+            int row[4];
+            float acc[4] = {0.f, 0.f, 0.f, 0.f};
+            const float4* src[4];
+            bool on[4];
+#pragma unroll
+            for (int r = 0; r < 4; ++r) {
+                const int j = j0 + r * (REFINE_WARPS * 4) + team;
+                on[r] = j < n;
+                row[r] = on[r] ? (first + (listed ? (int)S.list[j] : j)) : 0;
+                src[r] = reinterpret_cast<const float4*>(A.vectors + (size_t)row[r] * (size_t)A.d_pad) + sub;
+            }
+#pragma unroll 1
+            for (int g0 = 0; g0 < groups; g0 += 32) {
+                float4 x[4][4];
+                const int left = groups - g0 - sub;
+#pragma unroll
+                for (int r = 0; r < 4; ++r)
+#pragma unroll
+                    for (int c = 0; c < 4; ++c) {
+                        x[r][c] = make_float4(0.f, 0.f, 0.f, 0.f);
+                        if (on[r] && 8 * c < left) x[r][c] = __ldg(src[r] + g0 + 8 * c);
+                    }
+#pragma unroll
+                for (int c = 0; c < 4; ++c) {
+                    if (8 * c < left) {
+                        const float4 v = qs[g0 + sub + 8 * c];
+#pragma unroll
+                        for (int r = 0; r < 4; ++r) {
+                            float u;
+                            u = x[r][c].x - v.x; acc[r] = fmaf(u, u, acc[r]);
+                            u = x[r][c].y - v.y; acc[r] = fmaf(u, u, acc[r]);
+                            u = x[r][c].z - v.z; acc[r] = fmaf(u, u, acc[r]);
+                            u = x[r][c].w - v.w; acc[r] = fmaf(u, u, acc[r]);
+                        }
+                    }
+                }
+            }
+            // the butterfly 4, 2, 1 over the team, every lane handing on the sums it does not keep
+            const bool up4 = (sub & 4) != 0, up2 = (sub & 2) != 0;
+            float s1[2];
+#pragma unroll
+            for (int r = 0; r < 2; ++r) {
+                const float give = up4 ? acc[r] : acc[r + 2], keep = up4 ? acc[r + 2] : acc[r];
+                s1[r] = keep + __shfl_xor_sync(FULL, give, 4);
+            }
+            const float give = up2 ? s1[0] : s1[1], keep = up2 ? s1[1] : s1[0];
+            float d = keep + __shfl_xor_sync(FULL, give, 2);
+            d = d + __shfl_xor_sync(FULL, d, 1);
+            const int mine = up4 ? (up2 ? row[3] : row[2]) : (up2 ? row[1] : row[0]);
+            const bool have = up4 ? (up2 ? on[3] : on[2]) : (up2 ? on[1] : on[0]);
+            if ((sub & 1) == 0 && have && __float_as_uint(d) <= (uint32_t)(S.bound >> 32)) {
+                const uint64_t key = make_key(d, (uint32_t)__ldg(A.rank2id + mine), 1u);
+                if (key < S.bound) S.buf[atomicAdd(&S.kept, 1)] = key;
+            }
+            __syncthreads();
+            const bool full = S.kept >= REFINE_BUF - REFINE_STEP;
+            __syncthreads();
+            if (full) {
+                if (warp == 0) flush();
+                __syncthreads();
+            }
+        }
+    };
+    __syncthreads();
+    if (off == BOT) {
+        compare(w, slab.x, false);
+    } else {
+        const int blocks = (slab.y >> 5) - (slab.x >> 5) + 1, block0 = slab.x >> 5;
+        const uint32_t* const mask = A.store + off + (uint32_t)(blocks * values_per_block(w, A.k));
+        constexpr int MASKS = REFINE_WARPS * 32;
+        if (t == 0) S.count = 0;
+        __syncthreads();
+        for (int m0 = 0; m0 < blocks; m0 += 4 * MASKS) {
+            uint32_t word[4];
+#pragma unroll
+            for (int x = 0; x < 4; ++x) word[x] = m0 + x * MASKS + t < blocks ? __ldcg(mask + m0 + x * MASKS + t) : 0u;
+#pragma unroll 1
+            for (int x = 0; x < 4 && m0 + x * MASKS < blocks; ++x) {
+                uint32_t m = x == 0 ? word[0] : x == 1 ? word[1] : x == 2 ? word[2] : word[3];
+                int sum = __popc(m);
+                const int own = sum;
+                for (int o = 1; o < 32; o <<= 1) {
+                    const int y = __shfl_up_sync(FULL, sum, o);
+                    if (lane >= o) sum += y;
+                }
+                int at = 0;
+                if (lane == 31 && sum) at = atomicAdd(&S.count, sum);
+                at = __shfl_sync(FULL, at, 31) + sum - own;
+                for (; m; m &= m - 1) {                          // bit 4 g + j: row g + 8 j of the mask's 32
+                    const int bit = __ffs(m) - 1;
+                    S.list[at++] = (uint16_t)((x * MASKS + t) * 32 + (bit >> 2) + 8 * (bit & 3));
+                }
+                __syncthreads();
+                const int n = S.count;
+                if (n > REFINE_MORE || x == 3 || m0 + (x + 1) * MASKS >= blocks) {
+                    compare(n, (block0 + m0) * 32, true);
+                    __syncthreads();
+                    if (t == 0) S.count = 0;
+                }
+                __syncthreads();
+            }
+        }
+    }
+    __syncthreads();
+    if (warp == 0) flush();
+    __syncthreads();
+    for (int j = t; j < A.k; j += REFINE_WARPS * 32) {
+        const uint64_t key = S.pool[j];
+        int32_t oid = -1;
+        float dist = __int_as_float(0x7F800000);
+        if (key != KEY_EMPTY) {
+            oid = (int32_t)key_rank(key);
+            dist = __fsqrt_rn(key_dist2(key));
+        }
+        A.out_ids[(size_t)q * A.k + j] = oid;
+        A.out_dists[(size_t)q * A.k + j] = dist;
+    }
+}
+
+}  // namespace
+namespace froghost {
+
+namespace {
+size_t up16(size_t x) { return (x + 15) & ~(size_t)15; }
+typedef void (*filter_fn)(const FilterArgs);
+size_t refine_smem(int k, int d_pad, filter_fn* fn) {
+    const size_t q = (size_t)d_pad * 4;
+    if (k <= 32) { *fn = filter_refine_kernel<1>; return up16(sizeof(RefineSmem<1>)) + q; }
+    if (k <= 64) { *fn = filter_refine_kernel<2>; return up16(sizeof(RefineSmem<2>)) + q; }
+    if (k <= 128) { *fn = filter_refine_kernel<4>; return up16(sizeof(RefineSmem<4>)) + q; }
+    if (k <= 256) { *fn = filter_refine_kernel<8>; return up16(sizeof(RefineSmem<8>)) + q; }
+    *fn = filter_refine_kernel<16>;
+    return up16(sizeof(RefineSmem<16>)) + q;
+}
+size_t filter_fixed_bytes(size_t n, size_t nq, int d_pad) {
+    return nq * ((size_t)d_pad * 4 + 8 + 4 + 4 + 4) + (n / TILE + 1) * 4 + 64;
+}
+}  // namespace
+
+FilterRoom filter_room(size_t n, size_t nq, int k, int d_pad) {
+    const size_t narrow = std::min(n, (size_t)128 * k);
+    const size_t words = nq * std::max(2 * (n / 32 + 2), 5 * (narrow / 32 + 2));
+    const size_t fixed = filter_fixed_bytes(n, nq, d_pad);
+    return {fixed + words, fixed + words * 4};
+}
+
+void filter_scratch(char* mem, size_t bytes, FilterArgs* A) {
+    const size_t nq = (size_t)A->nq;
+    A->rounded = reinterpret_cast<float*>(mem);
+    A->slab = reinterpret_cast<int2*>(mem + nq * A->d_pad * 4);
+    A->norm = reinterpret_cast<float*>(A->slab + nq);
+    A->off = reinterpret_cast<uint32_t*>(A->norm + nq);
+    A->tau = reinterpret_cast<float*>(A->off + nq);
+    A->tile_norm = reinterpret_cast<uint32_t*>(A->tau + nq);
+    A->store = A->tile_norm + A->n / TILE + 1;
+    A->words = std::min<size_t>((bytes - filter_fixed_bytes((size_t)A->n, nq, A->d_pad)) / 4, 0xFFFFFFF0u);
+}
+
+cudaError_t filter_launch(const FilterArgs& A, int sm_count, cudaStream_t s) {
+    filter_fn refine;
+    const size_t smem = refine_smem(A.k, A.d_pad, &refine);
+    cudaError_t e;
+    if ((e = allow_smem(refine)) != cudaSuccess || (e = allow_smem(filter_tile_kernel<0>)) != cudaSuccess ||
+        (e = allow_smem(filter_tile_kernel<1>)) != cudaSuccess)
+        return e;
+    const int tiles = (A.n - 1) / TILE + 1;
+    // two CTAs per SM; several share a tile's queries where there are fewer tiles than that
+    const int parts = std::max(1, std::min((A.nq - 1) / TILE + 1, 2 * sm_count / tiles));
+    const dim3 grid((unsigned)tiles, (unsigned)parts);
+    filter_plan_kernel<<<(A.nq - 1) / 8 + 1, 256, 0, s>>>(A);
+    filter_offsets_kernel<<<1, 1024, 0, s>>>(A);
+    filter_tile_kernel<0><<<grid, THREADS, sizeof(FilterSmem), s>>>(A);
+    filter_bound_kernel<<<A.nq, 256, 0, s>>>(A);
+    filter_tile_kernel<1><<<grid, THREADS, sizeof(FilterSmem), s>>>(A);
+    refine<<<A.nq, REFINE_WARPS * 32, smem, s>>>(A);
+    return cudaGetLastError();
+}
+
+}  // namespace froghost

@@ -69,6 +69,56 @@ def test_matches_the_oracle(libs, tmp_path, n, d):
     gix.close()
 
 
+# Filtered scans (4,000 rows and more, many queries): rows that fill no tile of 128 or block of 32, row lengths on both
+# sides of a pipeline stage, more queries than a tile has and than are listed at a time, k on both sides of what makes
+# a slab wide, and an index too small for the bounds of all queries.
+@pytest.mark.parametrize("n,d,nq", [(4000, 3, 129), (4127, 33, 260), (20011, 50, 100), (16001, 128, 2300), (5000, 260, 400), (70001, 8, 40)])
+def test_filtered_scans(libs, tmp_path, n, d, nq):
+    base, attrs, path = _index(libs, tmp_path, n, d, n)
+    ix = oracle.load_index(path)
+    gix = libs.Index.load(path)
+    for narrow in (0, 4, 11) if nq < 2000 else (9,):
+        q, lo, hi = _queries(base, attrs, nq, nq, narrow)
+        for k in (1, 10, 40, 129, 512) if nq < 300 else (10, 100):
+            _check(gix, ix, q, lo, hi, k)
+    gix.close()
+
+
+@pytest.mark.parametrize("scale", [1.0, 1e-21, 3e17, 1e19])
+def test_filtered_scans_of_extreme_values(libs, tmp_path, scale):
+    """Products that underflow, overflow or are not numbers rule nothing out: same results, bit for bit, as the captured
+    scan, which compares all rows."""
+    rng = np.random.default_rng(8)
+    n, d, nq = 9000, 40, 300
+    base = (rng.standard_normal((n, d)) * scale).astype(np.float32)
+    base[17, 3], base[18, 0], base[5000:5040, 1], base[77] = np.nan, np.inf, -np.inf, 3e38
+    base[6000:6010] *= np.float32(1e6)
+    attrs = rng.integers(0, n, n).astype(np.int32)
+    path = str(tmp_path / "x.idx")
+    libs.build_index_gpu(base, attrs, path, m=4, ef_c=4, patience=1, n_inv=30)
+    gix = libs.Index.load(path)
+    q = (rng.standard_normal((nq, d)) * scale).astype(np.float32)
+    q[3, 5], q[4], q[5, 0], q[6], q[7] = np.inf, np.nan, -np.inf, 2e38, 0.0
+    q[8] = base[6003]
+    w = np.maximum(1, (n * 2.0 ** -rng.uniform(0, 5, nq)).astype(int))
+    w[:9] = n
+    s = (rng.random(nq) * (n - w + 1)).astype(int)
+    a = np.sort(attrs)
+    dev = [torch.from_numpy(np.ascontiguousarray(x)).cuda() for x in (q, a[s], a[s + w - 1])]
+    for k in (1, 10, 100):
+        want = [torch.empty((nq, k), dtype=t, device="cuda") for t in (torch.int32, torch.float32)]
+        graph = torch.cuda.CUDAGraph()
+        with torch.cuda.graph(graph):
+            gix.exact_search(*dev, k, out_ids=want[0], out_dists=want[1])
+        graph.replay()
+        for _ in range(2):
+            got = gix.exact_search(*dev, k)
+            torch.cuda.synchronize()
+            assert torch.equal(got[0], want[0]) and torch.equal(got[1].view(torch.int32), want[1].view(torch.int32))
+        graph.reset()
+    gix.close()
+
+
 def test_groups_with_gaps_streams_and_capture(libs, tmp_path):
     """Slabs that share no rows (a group's pieces jump the gaps), calls on two streams, and a captured call."""
     base, attrs, path = _index(libs, tmp_path, 30000, 24, 11)
