@@ -621,9 +621,9 @@ __device__ __forceinline__ uint32_t merge_batch(uint64_t* pool, uint64_t my_key,
 // positions of the new keys, as one bit mask per 32 positions, tell each position whether it takes a new
 // key or which old one moves there.  The cost hardly depends on the pool size and little on n, and the
 // dependent chain has no shuffle or vote per key.
-// `entered` tells a lane whether its key is in the pool now and was not before.
+// `entered` tells a lane whether its key is in the pool now and was not before.  Keys that do not enter are emptied.
 template <int EPL>
-__device__ __forceinline__ uint32_t merge_ranked(uint64_t* pool, const uint64_t* keys, int n, int ef_s, int lane,
+__device__ __forceinline__ uint32_t merge_ranked(uint64_t* pool, uint64_t* keys, int n, int ef_s, int lane,
                                                  bool* entered = nullptr) {
     constexpr int POOL = 32 * EPL;
     static_assert((POOL & (POOL - 1)) == 0, "the search halves the pool");
@@ -636,20 +636,14 @@ __device__ __forceinline__ uint32_t merge_ranked(uint64_t* pool, const uint64_t*
     for (int step = POOL / 2; step > 0; step >>= 1)
         if ((pool[p + step - 1] | 1ull) < mk) p += step;
     in = in && (pool[p] | 1ull) != mk;                  // the pool holds it already
+    // of equal keys the first one goes on (their ranks are equal, and the other lanes' are made different)
+    const uint32_t same = __match_any_sync(FULL, lane < n ? key_rank(key) : 0x80000000u | (uint32_t)lane);
+    in = in && (same & lt_mask) == 0;
+    if (lane < n && !in) keys[lane] = KEY_EMPTY;        // not below any other
+    __syncwarp();
     int r = 0;
-    bool copy = false;
-#pragma unroll 4
-    for (int j = 0; j < n; ++j) {
-        const uint64_t x = keys[j] | 1ull;
-        r += x < mk ? 1 : 0;
-        copy = copy || (x == mk && j < lane);
-    }
-    in = in && !copy;
-    // keys that lie below this one but do not enter: copies only (what the pool rejects lies above)
-    for (uint32_t out = __ballot_sync(FULL, !in && lane < n); out; out &= out - 1) {
-        const uint64_t x = keys[__ffs(out) - 1] | 1ull;
-        r -= x < mk ? 1 : 0;
-    }
+#pragma unroll 8
+    for (int j = 0; j < n; ++j) r += (keys[j] | 1ull) < mk ? 1 : 0;
     const int f = p + r;
     in = in && f < ef_s;
     if (entered) *entered = in;
