@@ -182,6 +182,7 @@ extern "C" void frog_index_free(frog_index_t* ix) {
             cudaEventDestroy(ix->exact[i].done);
         }
         cudaFree(ix->d_stage);
+        cudaFreeHost(ix->h_stage);
     }
     delete ix;
 }
@@ -282,18 +283,54 @@ extern "C" int frog_search_host(frog_index_t* ix, const float* queries, const in
     if (!queries || !lo || !hi || !out_ids || !out_dists) return FROG_ERR_INVALID_ARG;
     FROG_CUDA_TRY(cudaSetDevice(ix->info.device));
     cudaStream_t s = static_cast<cudaStream_t>(stream);
+    auto up = [](size_t x) { return (x + 255) & ~(size_t)255; };
+    const size_t b_q = up((size_t)nq * ix->info.d * 4), b_r = up((size_t)nq * 4), b_o = up((size_t)nq * k * 4);
     // Pinned (page-locked, device-mapped) host buffers need no staging: the kernels read each query
     // and write each result row across the bus themselves, so the transfers overlap the search
-    // instead of bracketing it.  Pageable buffers take the staged path below.
+    // instead of bracketing it.  A few pageable ones pass through a page-locked buffer of the index in the same way: a
+    // copy by the driver is a launch each, and up to five of them were a third of a small call (16 queries on 100,000 x
+    // 96, beam 64).  Larger pageable buffers take the staged path below.
+    std::unique_lock<std::mutex> stage_lock(ix->stage_mu, std::defer_lock);
     {
         const void* host[5] = {queries, lo, hi, out_ids, out_dists};
+        const size_t bytes[5] = {b_q, b_r, b_r, b_o, b_o};
+        char* pageable[5] = {nullptr, nullptr, nullptr, nullptr, nullptr};
         void* dev[5] = {nullptr, nullptr, nullptr, nullptr, nullptr};
-        bool mapped = true;
-        for (int i = 0; i < 5 && mapped; ++i) {
+        size_t staged = 0;
+        bool known = true;                                     // each is pinned or pageable
+        for (int i = 0; i < 5 && known; ++i) {
             cudaPointerAttributes at;
-            if (cudaPointerGetAttributes(&at, host[i]) != cudaSuccess) { cudaGetLastError(); mapped = false; break; }
-            mapped = at.type == cudaMemoryTypeHost && at.devicePointer != nullptr;
-            dev[i] = at.devicePointer;
+            if (cudaPointerGetAttributes(&at, host[i]) != cudaSuccess) { cudaGetLastError(); known = false; break; }
+            if (at.type == cudaMemoryTypeHost && at.devicePointer != nullptr) dev[i] = at.devicePointer;
+            else if (at.type == cudaMemoryTypeUnregistered) staged += bytes[i];
+            else known = false;
+        }
+        bool mapped = known && staged == 0;
+        if (known && !mapped && staged <= FROG_HOST_STAGE) {
+            stage_lock.lock();
+            if (!ix->h_stage && !ix->no_h_stage &&
+                cudaHostAlloc((void**)&ix->h_stage, FROG_HOST_STAGE, cudaHostAllocMapped) != cudaSuccess) {
+                cudaGetLastError();
+                ix->h_stage = nullptr;
+                ix->no_h_stage = true;
+            }
+            char* base = nullptr;
+            if (ix->h_stage && cudaHostGetDevicePointer((void**)&base, ix->h_stage, 0) != cudaSuccess) { cudaGetLastError(); base = nullptr; }
+            if (base) {
+                mapped = true;
+                size_t at = 0;
+                for (int i = 0; i < 5; ++i) {
+                    if (dev[i]) continue;
+                    pageable[i] = ix->h_stage + at;
+                    dev[i] = base + at;
+                    at += bytes[i];
+                }
+                if (pageable[0]) std::memcpy(pageable[0], queries, (size_t)nq * ix->info.d * 4);
+                if (pageable[1]) std::memcpy(pageable[1], lo, (size_t)nq * 4);
+                if (pageable[2]) std::memcpy(pageable[2], hi, (size_t)nq * 4);
+            } else {
+                stage_lock.unlock();
+            }
         }
         if (mapped) {
             int rc = frog_search_ex(ix, static_cast<const float*>(dev[0]), static_cast<const int32_t*>(dev[1]),
@@ -302,12 +339,12 @@ extern "C" int frog_search_host(frog_index_t* ix, const float* queries, const in
                                     nullptr, 0, stream);
             if (rc != FROG_OK) return rc;
             FROG_CUDA_TRY(cudaStreamSynchronize(s));
+            if (pageable[3]) std::memcpy(out_ids, pageable[3], (size_t)nq * k * 4);
+            if (pageable[4]) std::memcpy(out_dists, pageable[4], (size_t)nq * k * 4);
             return FROG_OK;
         }
     }
-    std::lock_guard<std::mutex> stage_lock(ix->stage_mu);
-    auto up = [](size_t x) { return (x + 255) & ~(size_t)255; };
-    const size_t b_q = up((size_t)nq * ix->info.d * 4), b_r = up((size_t)nq * 4), b_o = up((size_t)nq * k * 4);
+    stage_lock.lock();
     const size_t need = b_q + 2 * b_r + 2 * b_o;
     if (need > ix->stage_bytes) {
         FROG_CUDA_TRY(cudaStreamSynchronize(s));

@@ -43,6 +43,7 @@ struct FrogExactSet {
     bool used = false;
 };
 constexpr int FROG_EXACT_SETS = 16;   // a scan on a further stream in flight does without
+constexpr size_t FROG_HOST_STAGE = (size_t)256 << 10;
 constexpr int FROG_TABLE_BITS = 12;    // 4,096 ranks = 16 KB per resident warp: 78 MB for a full grid, inside L2
 constexpr int FROG_TABLE_BITS_WIDE = 13;   // beam widths 65..128: 8,192 ranks (a query evaluates ~2,000 there)
 
@@ -71,6 +72,8 @@ struct frog_index {
     // staging for frog_search_host, grown on demand
     void* d_stage = nullptr;
     size_t stage_bytes = 0;
+    char* h_stage = nullptr;         // FROG_HOST_STAGE bytes of page-locked memory for small calls
+    bool no_h_stage = false;         // it cannot be had
     std::mutex stage_mu;             // one staged host call at a time
     int sm_count = 0;
 };
