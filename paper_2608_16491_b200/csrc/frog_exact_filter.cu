@@ -10,10 +10,10 @@
 //     order.  Ids and distances are therefore those of a scan of all rows, bit for bit.
 // Products are computed twice, the second time only for tiles that a bound of the first says may hold an answer, because
 // storing them would take 4 bytes per row and query.  2,000 queries, k = 100, on 100,000 x 128, log-uniform widths:
-// 1,290 us by groups of eight in fp32, 325 filtered: 132 first pass, 17 bounds, 101 second pass, 93 comparison (k = 10:
-// 250).  The passes are bound by fragment loads from shared memory (24 for 16 matrix instructions) and their
-// epilogues, not by the matrix unit (60 TFLOP/s): tiles are as deep as a vector, 32 to 768.  Hence mma.sync, whose
-// accumulators are where the epilogue needs them.
+// 1,290 us by groups of eight in fp32, 288 filtered: 116 first pass, 17 bounds, 89 second pass, 81 comparison (k = 10:
+// 222).  The passes are bound by issue and the latency of fragment loads (24 for 16 matrix instructions) and of their
+// epilogues, the matrix unit is active for a quarter of the time: tiles are as deep as a vector, 32 to 768.  Hence
+// mma.sync, whose accumulators are where the epilogue needs them.
 #include <algorithm>
 
 #include "frog_device.cuh"
@@ -26,19 +26,24 @@ using froghost::FilterArgs;
 namespace {
 
 constexpr int TILE = 128;                // rows, and queries, of a tile of products
-constexpr int KC = 32;                   // elements of a row per pipeline stage
-constexpr int KP = KC + 4;               // their stride in shared memory: fragment loads without bank conflicts
-constexpr int STAGES = 2;
 constexpr int SEG = 2048;                // queries listed at a time
 constexpr int THREADS = 256;             // 4 x 2 warps of 32 rows x 64 queries
 
+// KC: elements of a row per pipeline stage, 64 in all.  Short rows have few stages, so more of them in flight count
+// (100,000 x 32: 201 us with two stages of 32, 172 with four of 16), long ones pay for each stage's barrier (20,000 x
+// 768: 277 and 299).
+template <int KC>
 struct FilterSmem {
+    static constexpr int KP = KC + 4;    // stride of a row's part: fragment loads without bank conflicts
+    static constexpr int STAGES = 64 / KC;
     float a[STAGES][TILE * KP];
     float b[STAGES][TILE * KP];
     int list[SEG];                       // queries whose slab meets the tile
     float row_norm[TILE];
-    int l[TILE], r[TILE];                // of the batch's queries
-    float norm[TILE], tau[TILE];
+    // of the batch's queries: first rank and how many follow it, blocks of 32 rows (0: no query), values per block
+    uint32_t l[TILE], span[TILE], blocks[TILE];
+    int per[TILE];
+    float norm[TILE], root[TILE], tau[TILE];     // squared norm with its part of the bound, norm, bound of the answers
     uint32_t off[TILE];
     int count;
 };
@@ -128,21 +133,24 @@ filter_offsets_kernel(const FilterArgs A) {
 // With u = 2^-11 the rounding of an operand: |x~.q~ - x.q| <= (2u + u^2) |x| |q|; the sums of d products, of the norms
 // and of the scan are within d 2^-22 of their magnitude each (twice what rounding to nearest gives); the last two terms
 // cover what underflows.  Anything not finite makes the comparisons with it false, which rules nothing out.
+// (x and q are the norms, c1 x q + own(x) + own(q) the bound.)
 struct RowError {
     float c1, c2;
     __device__ __forceinline__ explicit RowError(int d) : c1(0.00197f + d * 0x1p-20f), c2(0x1p-19f + d * 0x1p-21f) {}
+    __device__ __forceinline__ float own(float nx, float x) const { return c2 * nx + (1e-30f * x + 1e-34f); }
     __device__ __forceinline__ float operator()(float nx, float x, float nq, float q) const {
-        return c1 * x * q + c2 * (nx + nq) + 1e-30f * (x + q) + 1e-34f;
+        return c1 * x * q + (own(nx, x) + own(nq, q));
     }
 };
 
 // PASS 0: bounds, PASS 1: masks.  One CTA per 128 rows and per share of the queries: those whose number is blockIdx.y
 // modulo gridDim.y (the order in which a CTA lists its queries is not that of another).
-template <int PASS>
+template <int PASS, int KC>
 __global__ void __launch_bounds__(THREADS, 2)
 filter_tile_kernel(const FilterArgs A) {
     extern __shared__ __align__(16) unsigned char smem_raw[];
-    FilterSmem& S = *reinterpret_cast<FilterSmem*>(smem_raw);
+    FilterSmem<KC>& S = *reinterpret_cast<FilterSmem<KC>*>(smem_raw);
+    constexpr int KP = FilterSmem<KC>::KP, STAGES = FilterSmem<KC>::STAGES;
     const int t = threadIdx.x, lane = lane_id(), warp = t >> 5;
     const int wm = warp >> 1, wn = warp & 1;                     // this warp's rows and queries of the tile
     const int g = lane >> 2, p = lane & 3;                       // fragment coordinates
@@ -156,11 +164,26 @@ filter_tile_kernel(const FilterArgs A) {
         __syncthreads();
         if (t == 0) S.count = 0;
         __syncthreads();
-        for (int i = t; i < SEG; i += THREADS) {                 // (SEG is a multiple of THREADS)
-            const int q = q0 + i;
+        constexpr int EACH = SEG / THREADS;                      // queries per thread, in flight together
+        int2 slabs[EACH];
+        uint32_t offs[EACH];
+#pragma unroll
+        for (int x = 0; x < EACH; ++x) {
+            const int q = q0 + x * THREADS + t;
+            const bool mine = q < A.nq && q % gridDim.y == blockIdx.y;
+            offs[x] = mine ? A.off[q] : BOT;
+            slabs[x] = mine ? A.slab[q] : make_int2(1, 0);
+        }
+#pragma unroll 1
+        for (int i = 0; i < EACH; ++i) {
+            const int q = q0 + i * THREADS + t;
+            int2 s = slabs[0];
+            uint32_t off = offs[0];
+#pragma unroll
+            for (int x = 1; x < EACH; ++x)
+                if (x == i) { s = slabs[x]; off = offs[x]; }
             bool hit = false;
-            if (q < A.nq && q % gridDim.y == blockIdx.y && A.off[q] != BOT) {
-                const int2 s = A.slab[q];
+            if (off != BOT) {
                 hit = s.x < row_end && s.y >= row0;
                 if (PASS == 1 && hit) {
                     // The second pass is for tiles with a row that may be an answer: a value of the first is a lower bound
@@ -168,14 +191,14 @@ filter_tile_kernel(const FilterArgs A) {
                     const int w = s.y - s.x + 1, per = values_per_block(w, A.k), all = (s.y >> 5) - (s.x >> 5) + 1;
                     const int from = max((row0 >> 5) - (s.x >> 5), 0), to = min(((row0 + TILE) >> 5) - (s.x >> 5), all);
                     const float nq = A.norm[q], tau = A.tau[q], e = 2.f * error(tile_norm, tile_sqrt, nq, __fsqrt_rn(nq));
-                    const uint32_t* const v = A.store + A.off[q];
+                    const uint32_t* const v = A.store + off;
                     hit = false;
                     for (int x = from * per; x < to * per; ++x) {
                         const float least = __uint_as_float(v[x]);
                         hit = hit || !(least - e > tau) || !(least < __int_as_float(0x7F800000));
                     }
                     if (!hit)
-                        for (int x = from; x < to; ++x) A.store[A.off[q] + all * per + x] = 0u;
+                        for (int x = from; x < to; ++x) A.store[off + all * per + x] = 0u;
                 }
             }
             const uint32_t M = __ballot_sync(FULL, hit);
@@ -191,19 +214,18 @@ filter_tile_kernel(const FilterArgs A) {
             __syncthreads();                                     // the batch before is done with the tables
             if (t < TILE) {
                 const int q = S.list[b0 + min(t, nb - 1)];
-                const int2 s = t < nb ? A.slab[q] : make_int2(1, -1);
-                const int w = s.y - s.x + 1;
-                S.l[t] = s.x;
-                S.r[t] = s.y;
-                S.norm[t] = A.norm[q];
-                if (PASS == 1) {
-                    const int blocks = (s.y >> 5) - (s.x >> 5) + 1;
-                    S.tau[t] = A.tau[q];
-                    S.off[t] = A.off[q] + (t < nb ? (uint32_t)(blocks * values_per_block(w, A.k)) : 0u);
-                } else {
-                    S.off[t] = A.off[q];
-                    S.tau[t] = __int_as_float(t < nb ? values_per_block(w, A.k) : 0);
-                }
+                const int2 s = A.slab[q];
+                const float n = A.norm[q], root = __fsqrt_rn(n), own = error.own(n, root);
+                const uint32_t blocks = (uint32_t)((s.y >> 5) - (s.x >> 5) + 1);
+                const int per = values_per_block(s.y - s.x + 1, A.k);
+                S.l[t] = t < nb ? (uint32_t)s.x : 0x80000000u;           // no row lies in the slab of none
+                S.span[t] = t < nb ? (uint32_t)(s.y - s.x) : 0u;
+                S.blocks[t] = t < nb ? blocks : 0u;
+                S.per[t] = per;
+                S.norm[t] = PASS == 0 ? n + own : n - own;
+                S.root[t] = root;
+                if (PASS == 1) S.tau[t] = A.tau[q];
+                S.off[t] = A.off[q] + (PASS == 1 ? blocks * per : 0u);
             }
             float acc[2][8][4];
 #pragma unroll
@@ -283,12 +305,14 @@ filter_tile_kernel(const FilterArgs A) {
             if (wn * 64 < nb) {
                 // this thread's rows are base + g + 8 j, its queries 8 x + 2 p and the next one
                 const int base = row0 + wm * 32;
-                bool finite = true;
+                float finite = 0.f;                                  // or not a number
+                // a bound is |x|^2 +- own(x) + |q|^2 +- own(q) +- c1 |x| |q| - 2 x.q
                 float nx[4], sx[4];
 #pragma unroll
                 for (int j = 0; j < 4; ++j) {
-                    nx[j] = S.row_norm[wm * 32 + g + 8 * j];
-                    sx[j] = __fsqrt_rn(nx[j]);
+                    const float n = S.row_norm[wm * 32 + g + 8 * j], s = __fsqrt_rn(n), own = error.own(n, s);
+                    nx[j] = PASS == 0 ? n + own : n - own;
+                    sx[j] = PASS == 0 ? error.c1 * s : -error.c1 * s;
                 }
 #pragma unroll
                 for (int x = 0; x < 8; ++x) {
@@ -296,20 +320,18 @@ filter_tile_kernel(const FilterArgs A) {
 #pragma unroll
                     for (int c = 0; c < 2; ++c) {
                         const int i = wn * 64 + x * 8 + 2 * p + c;
-                        const int l = S.l[i], r = S.r[i];
-                        const float nq = S.norm[i], sq = __fsqrt_rn(nq), tau = S.tau[i];
+                        const uint32_t l = S.l[i], span = S.span[i], at = (uint32_t)(base + g) - l;
+                        const float nq = S.norm[i], sq = S.root[i], tau = S.tau[i];
                         float least = __int_as_float(0x7F800000);
 #pragma unroll
                         for (int j = 0; j < 4; ++j) {
-                            const int row = base + g + 8 * j;
-                            const float rough = fmaf(-2.f, acc[j >> 1][x][(j & 1) * 2 + c], nx[j] + nq);
-                            const float e = error(nx[j], sx[j], nq, sq);
-                            const bool in = row >= l && row <= r;
+                            const float bound = fmaf(sx[j], sq, fmaf(-2.f, acc[j >> 1][x][(j & 1) * 2 + c], nx[j] + nq));
+                            const bool in = at + 8u * j <= span;
                             if (PASS == 0) {
-                                if (in && rough + e < least) least = rough + e;
-                                finite = finite && (!in || rough + e < __int_as_float(0x7F800000));
+                                if (in && bound < least) least = bound;
+                                finite = fmaf(bound, 0.f, finite);
                             } else {
-                                bits[c][j] = __ballot_sync(FULL, in && !(rough - e > tau));
+                                bits[c][j] = __ballot_sync(FULL, in && !(bound > tau));
                             }
                         }
                         if (PASS == 0) {
@@ -317,8 +339,9 @@ filter_tile_kernel(const FilterArgs A) {
                             least = fminf(least, __shfl_xor_sync(FULL, least, 4));
                             const float wide = fminf(least, __shfl_xor_sync(FULL, least, 8));
                             const float all = fminf(wide, __shfl_xor_sync(FULL, wide, 16));
-                            const int block = (base >> 5) - (l >> 5), per = __float_as_int(tau);
-                            if (block >= 0 && base <= r) {
+                            const uint32_t block = (uint32_t)(base >> 5) - (l >> 5);
+                            if (block < S.blocks[i]) {
+                                const int per = S.per[i];
                                 if (per == 4 && (g & 1) == 0) A.store[S.off[i] + 4 * block + (g >> 1)] = __float_as_uint(least);
                                 if (per == 1 && g == 0) A.store[S.off[i] + block] = __float_as_uint(all);
                             }
@@ -331,11 +354,11 @@ filter_tile_kernel(const FilterArgs A) {
                         for (int j = 0; j < 4; ++j)
                             word |= ((((lane & 1) ? bits[1][j] : bits[0][j]) >> (lane >> 1)) & 0x11111111u) << j;
                         const int i = wn * 64 + x * 8 + lane;
-                        const int block = (base >> 5) - (S.l[i] >> 5);
-                        if (block >= 0 && base <= S.r[i]) A.store[S.off[i] + block] = word;
+                        const uint32_t block = (uint32_t)(base >> 5) - (S.l[i] >> 5);
+                        if (block < S.blocks[i]) A.store[S.off[i] + block] = word;
                     }
                 }
-                if (PASS == 0 && !finite) atomicMax(A.tile_norm + blockIdx.x, 0x7F800000u);
+                if (PASS == 0 && !(finite == 0.f)) atomicMax(A.tile_norm + blockIdx.x, 0x7F800000u);
             }
         }
     }
@@ -395,14 +418,14 @@ filter_bound_kernel(const FilterArgs A) {
 // The rows that are left, one CTA of four warps per query, so that those of 2,000 queries are resident together; four
 // rows per team in flight, as a step is a round trip.
 constexpr int REFINE_WARPS = 4, REFINE_BUF = 192, REFINE_STEP = REFINE_WARPS * 16;
-constexpr int REFINE_MORE = 1024;        // rows listed before they are compared; as many as 128 masks give come on top
+constexpr int REFINE_MORE = 512;         // rows listed before they are compared; as many as 128 masks give come on top
 constexpr int REFINE_LIST = REFINE_MORE + REFINE_WARPS * 32 * 32;
 template <int EPL>
 struct RefineSmem {
     uint64_t pool[32 * EPL];
     uint64_t buf[REFINE_BUF];            // merged from 128 on, a step adds at most 64
     uint64_t bound;                      // keys from here on are not wanted
-    uint16_t list[REFINE_LIST];          // rows to compare, from a base on
+    int list[REFINE_LIST];               // rows to compare
     int count, kept;                     // entries of list, of buf
 };
 
@@ -435,7 +458,7 @@ filter_refine_kernel(const FilterArgs A) {
             S.kept = 0;
         }
     };
-    // rows first + list[0..n), or first + [0..n)
+    // rows list[0..n), or first + [0..n)
     auto compare = [&](int n, int first, bool listed) {
         for (int j0 = 0; j0 < n; j0 += REFINE_STEP) {
             int row[4];
@@ -446,7 +469,7 @@ filter_refine_kernel(const FilterArgs A) {
             for (int r = 0; r < 4; ++r) {
                 const int j = j0 + r * (REFINE_WARPS * 4) + team;
                 on[r] = j < n;
-                row[r] = on[r] ? (first + (listed ? (int)S.list[j] : j)) : 0;
+                row[r] = on[r] ? (listed ? S.list[j] : first + j) : 0;
                 src[r] = reinterpret_cast<const float4*>(A.vectors + (size_t)row[r] * (size_t)A.d_pad) + sub;
             }
 #pragma unroll 1
@@ -528,12 +551,12 @@ filter_refine_kernel(const FilterArgs A) {
                 at = __shfl_sync(FULL, at, 31) + sum - own;
                 for (; m; m &= m - 1) {                          // bit 4 g + j: row g + 8 j of the mask's 32
                     const int bit = __ffs(m) - 1;
-                    S.list[at++] = (uint16_t)((x * MASKS + t) * 32 + (bit >> 2) + 8 * (bit & 3));
+                    S.list[at++] = (block0 + m0 + x * MASKS + t) * 32 + (bit >> 2) + 8 * (bit & 3);
                 }
                 __syncthreads();
                 const int n = S.count;
-                if (n > REFINE_MORE || x == 3 || m0 + (x + 1) * MASKS >= blocks) {
-                    compare(n, (block0 + m0) * 32, true);
+                if (n > REFINE_MORE || m0 + (x + 1) * MASKS >= blocks) {
+                    compare(n, 0, true);
                     __syncthreads();
                     if (t == 0) S.count = 0;
                 }
@@ -599,9 +622,12 @@ void filter_scratch(char* mem, size_t bytes, FilterArgs* A) {
 cudaError_t filter_launch(const FilterArgs& A, int sm_count, cudaStream_t s) {
     filter_fn refine;
     const size_t smem = refine_smem(A.k, A.d_pad, &refine);
+    const bool deep = A.d_pad >= 384;
+    const filter_fn bounds = deep ? filter_tile_kernel<0, 32> : filter_tile_kernel<0, 16>;
+    const filter_fn masks = deep ? filter_tile_kernel<1, 32> : filter_tile_kernel<1, 16>;
+    const size_t tile_smem = deep ? sizeof(FilterSmem<32>) : sizeof(FilterSmem<16>);
     cudaError_t e;
-    if ((e = allow_smem(refine)) != cudaSuccess || (e = allow_smem(filter_tile_kernel<0>)) != cudaSuccess ||
-        (e = allow_smem(filter_tile_kernel<1>)) != cudaSuccess)
+    if ((e = allow_smem(refine)) != cudaSuccess || (e = allow_smem(bounds)) != cudaSuccess || (e = allow_smem(masks)) != cudaSuccess)
         return e;
     const int tiles = (A.n - 1) / TILE + 1;
     // two CTAs per SM; several share a tile's queries where there are fewer tiles than that
@@ -609,9 +635,9 @@ cudaError_t filter_launch(const FilterArgs& A, int sm_count, cudaStream_t s) {
     const dim3 grid((unsigned)tiles, (unsigned)parts);
     filter_plan_kernel<<<(A.nq - 1) / 8 + 1, 256, 0, s>>>(A);
     filter_offsets_kernel<<<1, 1024, 0, s>>>(A);
-    filter_tile_kernel<0><<<grid, THREADS, sizeof(FilterSmem), s>>>(A);
+    bounds<<<grid, THREADS, tile_smem, s>>>(A);
     filter_bound_kernel<<<A.nq, 256, 0, s>>>(A);
-    filter_tile_kernel<1><<<grid, THREADS, sizeof(FilterSmem), s>>>(A);
+    masks<<<grid, THREADS, tile_smem, s>>>(A);
     refine<<<A.nq, REFINE_WARPS * 32, smem, s>>>(A);
     return cudaGetLastError();
 }
