@@ -132,6 +132,7 @@ cudaError_t allow_smem(F* fn) {
 // frog_search_lean.cu: the trimmed kernel for 384- and 512-byte fp32 and 192- and 256-byte fp16 rows (null: shape not covered)
 frog_kernel_fn lean_kernel(int ef_s, int budget, int row_bytes, bool f16, bool table, bool hook, int queries_per_sm,
                            size_t* smem_per_warp, int* warps_per_cta);
+bool lean_row(int row_bytes, bool f16);          // the rows it covers
 // frog_search_team.cu: one CTA of `warps` warps per query (see there)
 frog_kernel_fn team_kernel(int warps, int ef_s, int q_len, int vis_bits, bool f16, size_t* smem);
 void set_cuda_error(cudaError_t e);

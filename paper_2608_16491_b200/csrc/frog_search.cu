@@ -648,8 +648,7 @@ int plan_team(const frog_index* ix, int beam_width, const frog_params_t& P, int 
     const bool f16 = P.storage == FROG_STORAGE_F16;
     const int q_len = query_len(ix->info.d);
     const int row_bytes = f16 ? q_len * 2 : ix->info.d_pad * 4;
-    const bool lean = f16 ? ix->has_tmap_f16 && (row_bytes == 192 || row_bytes == 256)
-                          : ix->has_tmap_f32 && (row_bytes == 384 || row_bytes == 512);
+    const bool lean = (f16 ? ix->has_tmap_f16 : ix->has_tmap_f32) && froghost::lean_row(row_bytes, f16);
     const int per_sm_nq = (nq - 1) / ix->sm_count + 1;
     const int warps = per_sm_nq <= (row_bytes <= STAGE_CHUNK || (f16 && P.budget <= 24) ? 2 : 4) ? 8 : 4;
     const size_t index_bytes = (size_t)ix->info.n * row_bytes;

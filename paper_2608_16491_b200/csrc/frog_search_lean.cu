@@ -1,4 +1,4 @@
-// The search kernel for the common case: fp32 or fp16 rows of 96 or 128 elements, an exact
+// The search kernel for the common case: fp32 or fp16 rows of 32, 64, 96 or 128 elements, an exact
 // visited set in global scratch (bitmap slab, or for large indexes a hash table of ranks), rows
 // fetched four at a time by the copy engine's tile::gather4, no counters and no trace.  It
 // computes exactly what frog_search_kernel computes (paper Alg. 2 with Alg. 3 once per query and
@@ -574,6 +574,10 @@ frog_kernel_fn lean_pick(int ef_s, int budget, bool table, bool roomy, bool hook
 
 namespace froghost {
 
+// The rows are those whose 4-element groups fill whole teams.  Against the generic kernel on 50,000 rows (beam / B, us):
+//   128 bytes   10,000 queries 32 / 16  333 -> 244   64 / 64  736 -> 550   160 / 128 2,152 -> 1,643   1,500, 64 / 64  328 -> 272
+//   256 bytes                           354 -> 266            759 -> 568             2,286 -> 1,688                   344 -> 286
+//   64 and 128 bytes of fp16                              733 -> 555 and 762 -> 572                                   330 -> 281
 // The lean kernel for this beam width and row size, or null if the shape is not covered (the caller
 // then uses the generic kernel).  Needs the row tensor map and the bitmap visited set.  `table`: the
 // variant whose visited set is the L2-resident hash table (pools of up to 128 keys only); `hook`: the
@@ -584,13 +588,22 @@ frog_kernel_fn lean_kernel(int ef_s, int budget, int row_bytes, bool f16, bool t
     *warps_per_cta = LEAN_WARPS;
     const bool roomy = queries_per_sm > 0 && queries_per_sm <= LEAN_ROOMY_WARPS;
     if (f16) {
+        if (row_bytes == 64) return lean_pick<RowF16<64>>(ef_s, budget, table, roomy, hook, smem_per_warp);
+        if (row_bytes == 128) return lean_pick<RowF16<128>>(ef_s, budget, table, roomy, hook, smem_per_warp);
         if (row_bytes == 192) return lean_pick<RowF16<192>>(ef_s, budget, table, roomy, hook, smem_per_warp);
         if (row_bytes == 256) return lean_pick<RowF16<256>>(ef_s, budget, table, roomy, hook, smem_per_warp);
         return nullptr;
     }
+    if (row_bytes == 128) return lean_pick<RowF32<128>>(ef_s, budget, table, roomy, hook, smem_per_warp);
+    if (row_bytes == 256) return lean_pick<RowF32<256>>(ef_s, budget, table, roomy, hook, smem_per_warp);
     if (row_bytes == 384) return lean_pick<RowF32<384>>(ef_s, budget, table, roomy, hook, smem_per_warp);
     if (row_bytes == 512) return lean_pick<RowF32<512>>(ef_s, budget, table, roomy, hook, smem_per_warp);
     return nullptr;
+}
+
+bool lean_row(int row_bytes, bool f16) {
+    return f16 ? row_bytes == 64 || row_bytes == 128 || row_bytes == 192 || row_bytes == 256
+               : row_bytes == 128 || row_bytes == 256 || row_bytes == 384 || row_bytes == 512;
 }
 
 }  // namespace froghost

@@ -48,6 +48,37 @@ def test_every_pool(libs, tmp_path, d, storage, copies):
     gix.close()
 
 
+# rows of 32 and 64 elements, two of them with padding; pools and budgets on both sides of the instantiations
+@pytest.mark.parametrize("d,storage", [(32, 0), (30, 1), (64, 0), (61, 0), (64, 1)])
+def test_rows_of_32_and_64(libs, tmp_path, d, storage):
+    rng = np.random.default_rng(d)
+    n, nq = 4000, 50
+    base = rng.standard_normal((n, d)).astype(np.float32)
+    attrs = rng.integers(0, n, n).astype(np.int32)
+    path = str(tmp_path / "x.idx")
+    libs.build_index_gpu(base, attrs, path, ef_c=48)
+    ix = oracle.load_index(path)
+    gix = libs.Index.load(path)
+    if storage:
+        gix.enable_f16()
+        ix = oracle.rounded_to_f16(ix)
+    q = (base[rng.integers(0, n, nq)] + 0.2 * rng.standard_normal((nq, d))).astype(np.float32)
+    a = np.sort(attrs)
+    w = (n * 2.0 ** -rng.uniform(0, 6, nq)).astype(int)
+    s = (rng.random(nq) * (n - w)).astype(int)
+    lo, hi = a[s], a[s + w - 1]
+    for ef, budget in ((16, 16), (33, 64), (65, 128), (128, 64), (192, 128), (256, 64), (512, 32)):
+        ref = oracle.search(ix, q, lo, hi, 10, ef, B=budget)
+        for copies in (1, 80):                                           # one query per SM, and 28
+            dev = [torch.from_numpy(np.ascontiguousarray(np.tile(x, (copies,) + (1,) * (x.ndim - 1)))).cuda() for x in (q, lo, hi)]
+            for visited, flags in ((libs.VISITED_BITMAP, 0), (libs.VISITED_AUTO, 8)):      # bitmap, hash table where there is one
+                ids, dists = gix.search(*dev, 10, ef, params=libs.Params(budget=budget, storage=storage, visited=visited, debug_flags=flags))
+                torch.cuda.synchronize()
+                assert np.array_equal(ids.cpu().numpy(), np.tile(ref.ids, (copies, 1)))
+                assert np.array_equal(dists.cpu().numpy().view(np.uint32), np.tile(ref.dists.view(np.uint32), (copies, 1)))
+    gix.close()
+
+
 def test_fp16_batch_without_room_for_visited_slabs(libs):
     """600 queries need 170 MB of slabs on this index; where they cannot be had, the form that needs none runs."""
     import ctypes
