@@ -642,6 +642,12 @@ int team_queries_per_sm(int row_bytes, bool f16, int beam_width, int budget, siz
 // SM; 4 per SM for rows of several chunks, but not for fp16 rows with small budgets), then four up to the line above,
 // except on the rows that the kernel of frog_search_lean.cu covers, which one warp serves well enough (256-byte fp16
 // rows, beam 64, B 64: 400 queries 343 us with one warp per query and 410 with four, 900: 349 / 585).
+// A query with an SM of its own and a budget whose candidates keep them busy has sixteen: us, eight / sixteen warps, beam / B
+//   rows          queries   64 / 16     64 / 32     64 / 64     160 / 128     32 / 64
+//   384 bytes          1   167 / 176   163 / 167   156 / 154    446 / 411    86 / 83
+//   384 bytes        148   276 / 286   199 / 202   195 / 190    513 / 475   106 / 99
+//   128 bytes         16   150 / 157   152 / 155   163 / 158    439 / 414    89 / 84
+//   3,072 bytes       16   285 / 289   421 / 422   373 / 341  1,095 / 861   215 / 218
 // `any_batch`: also where one warp per query would be faster (this kernel needs no visited slabs).
 int plan_team(const frog_index* ix, int beam_width, const frog_params_t& P, int nq, LaunchPlan* out, int* vis_bits,
               bool any_batch = false) {
@@ -650,7 +656,7 @@ int plan_team(const frog_index* ix, int beam_width, const frog_params_t& P, int 
     const int row_bytes = f16 ? q_len * 2 : ix->info.d_pad * 4;
     const bool lean = (f16 ? ix->has_tmap_f16 : ix->has_tmap_f32) && froghost::lean_row(row_bytes, f16);
     const int per_sm_nq = (nq - 1) / ix->sm_count + 1;
-    const int warps = per_sm_nq <= (row_bytes <= STAGE_CHUNK || (f16 && P.budget <= 24) ? 2 : 4) ? 8 : 4;
+    const int warps = per_sm_nq <= 1 && P.budget >= 48 ? 16 : per_sm_nq <= (row_bytes <= STAGE_CHUNK || (f16 && P.budget <= 24) ? 2 : 4) ? 8 : 4;
     const size_t index_bytes = (size_t)ix->info.n * row_bytes;
     if (!any_batch && warps == 4 &&
         (lean || per_sm_nq > team_queries_per_sm(row_bytes, f16, beam_width, P.budget, index_bytes)))
@@ -658,7 +664,7 @@ int plan_team(const frog_index* ix, int beam_width, const frog_params_t& P, int 
     // a table of about 16 ranks per beam slot: smaller ones repeat distances (3,072-byte rows at beam 192:
     // 1.3x slower with 2,048 ranks than with 4,096), larger ones cost resident CTAs
     int bits = 10;
-    while (bits < (warps == 8 ? 13 : 12) && (1 << bits) < 16 * beam_width) ++bits;
+    while (bits < (warps >= 8 ? 13 : 12) && (1 << bits) < 16 * beam_width) ++bits;
     size_t smem = 0;
     kernel_fn fn = froghost::team_kernel(warps, beam_width, q_len, bits, f16, &smem);
     if (smem > froghost::MAX_SMEM) return FROG_ERR_UNSUPPORTED;

@@ -80,7 +80,7 @@ __device__ __forceinline__ float add_sq(float acc, const float4& x, const float4
 }
 
 template <int EPL, int W, int SPEC, bool F16>
-__global__ void __launch_bounds__(W * 32, W == 8 ? 2 : 5)
+__global__ void __launch_bounds__(W * 32, W == 16 ? 1 : W == 8 ? 2 : 5)
 frog_search_team_kernel(const __grid_constant__ FrogSearchArgs A) {
     using L = TeamLayout<EPL, SPEC>;
     extern __shared__ __align__(128) unsigned char smem_raw[];
@@ -456,6 +456,7 @@ frog_kernel_fn team_pick(int ef_s, int q_len, int vis_bits, size_t* smem) {
 namespace froghost {
 
 frog_kernel_fn team_kernel(int warps, int ef_s, int q_len, int vis_bits, bool f16, size_t* smem) {
+    if (warps == 16) return f16 ? team_pick<16, true>(ef_s, q_len, vis_bits, smem) : team_pick<16, false>(ef_s, q_len, vis_bits, smem);
     if (warps == 8) return f16 ? team_pick<8, true>(ef_s, q_len, vis_bits, smem) : team_pick<8, false>(ef_s, q_len, vis_bits, smem);
     return f16 ? team_pick<4, true>(ef_s, q_len, vis_bits, smem) : team_pick<4, false>(ef_s, q_len, vis_bits, smem);
 }

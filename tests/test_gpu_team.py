@@ -75,6 +75,22 @@ def test_every_batch_size(libs, tmp_path, d, storage):
     gix.close()
 
 
+# the lines between sixteen, eight and four warps per query and one, by batch size, budget and beam width
+@pytest.mark.parametrize("d,storage", [(96, 0), (64, 1), (200, 0)])
+def test_lines_between_the_forms(libs, tmp_path, d, storage):
+    base, attrs, path = _index(libs, tmp_path, 4000, d, d)
+    gix = libs.Index.load(path)
+    gix.enable_f16()
+    q, lo, hi = _queries(base, attrs, 900, 4)
+    for budget, ef in ((47, 40), (48, 40), (128, 96), (128, 97), (64, 300)):
+        for nq in (1, 148, 149, 297, 740, 741, 900):
+            a = _run(libs, gix, q[:nq], lo[:nq], hi[:nq], 10, ef, budget=budget, storage=storage)
+            b = _run(libs, gix, q[:nq], lo[:nq], hi[:nq], 10, ef, budget=budget, storage=storage, visited=libs.VISITED_BITMAP)
+            for x, y in zip(a, b):
+                assert np.array_equal(x.view(np.uint32), y.view(np.uint32))
+    gix.close()
+
+
 @pytest.mark.parametrize("kw,okw", [(dict(max_iters=1), dict(max_iters=1)), (dict(max_iters=7, budget=24), dict(max_iters=7, B=24)),
                                     (dict(epn=1), dict(epn=1)), (dict(epn=32, budget=1), dict(epn=32, B=1)),
                                     (dict(no_hotspot=1, budget=100), dict(no_hotspot=1, B=100)),
