@@ -639,9 +639,14 @@ int team_queries_per_sm(int row_bytes, bool f16, int beam_width, int budget, siz
 
 // One CTA per query (frog_search_team.cu) for batches that leave warps idle, or FROG_ERR_UNSUPPORTED where
 // one warp per query is the better use of the GPU.  Eight warps while every query has a CTA of its own at once (2 per
-// SM; 4 per SM for rows of several chunks, but not for fp16 rows with small budgets), then four up to the line above,
-// except on the rows that the kernel of frog_search_lean.cu covers, which one warp serves well enough (256-byte fp16
-// rows, beam 64, B 64: 400 queries 343 us with one warp per query and 410 with four, 900: 349 / 585).
+// SM; 4 per SM for rows of several chunks, but not for fp16 rows with small budgets), then four up to the line above.
+// The rows that the kernel of frog_search_lean.cu covers are served well enough by one warp where the pool is small;
+// the merges of larger ones pay up to the five CTAs per SM that are resident.  us, one warp / four, beam / B:
+//   rows           queries   64 / 64    100 / 64    128 / 16    160 / 64     160 / 128     192 / 128
+//   384 bytes          300  298 / 309   438 / 415   687 / 648   677 / 606   1,101 / 889   1,288 / 1,085
+//   384 bytes          740  305 / 344   449 / 441   674 / 656   682 / 630   1,095 / 943   1,287 / 1,139
+//   512 bytes          740  322 / 354   440 / 436   698 / 687   682 / 652   1,096 / 976   1,301 / 1,204
+//   128 bytes          740  281 / 290   425 / 396   412 / 401   653 / 586   1,024 / 833   1,193 / 1,042
 // A query with an SM of its own and a budget whose candidates keep them busy has sixteen: us, eight / sixteen warps, beam / B
 //   rows          queries   64 / 16     64 / 32     64 / 64     160 / 128     32 / 64
 //   384 bytes          1   167 / 176   163 / 167   156 / 154    446 / 411    86 / 83
@@ -659,7 +664,8 @@ int plan_team(const frog_index* ix, int beam_width, const frog_params_t& P, int 
     const int warps = per_sm_nq <= 1 && P.budget >= 48 ? 16 : per_sm_nq <= (row_bytes <= STAGE_CHUNK || (f16 && P.budget <= 24) ? 2 : 4) ? 8 : 4;
     const size_t index_bytes = (size_t)ix->info.n * row_bytes;
     if (!any_batch && warps == 4 &&
-        (lean || per_sm_nq > team_queries_per_sm(row_bytes, f16, beam_width, P.budget, index_bytes)))
+        (lean ? beam_width <= 96 || per_sm_nq > 5
+              : per_sm_nq > team_queries_per_sm(row_bytes, f16, beam_width, P.budget, index_bytes)))
         return FROG_ERR_UNSUPPORTED;
     // a table of about 16 ranks per beam slot: smaller ones repeat distances (3,072-byte rows at beam 192:
     // 1.3x slower with 2,048 ranks than with 4,096), larger ones cost resident CTAs
