@@ -631,10 +631,16 @@ __device__ __forceinline__ uint32_t merge_ranked(uint64_t* pool, uint64_t* keys,
     uint64_t key = lane < n ? keys[lane] : KEY_EMPTY;
     const uint64_t mk = key | 1ull;
     bool in = mk < (pool[ef_s - 1] | 1ull);             // a full pool rejects what is not better than its worst
-    int p = 0;                                          // pool keys below mk (at most ef_s - 1 if it enters)
+    // Pool keys below mk (at most ef_s - 1 if it enters): a quarter of what is left per step, as three reads take no longer
+    // than one (16 queries, beam 64, B 16: 187 -> 184 us; 148, beam 32, B 64: 139 -> 137), after a half where that leaves a power of four.
+    constexpr bool HALF = POOL == 32 || POOL == 128 || POOL == 512;
+    int p = HALF && (pool[POOL / 2 - 1] | 1ull) < mk ? POOL / 2 : 0;
 #pragma unroll
-    for (int step = POOL / 2; step > 0; step >>= 1)
-        if ((pool[p + step - 1] | 1ull) < mk) p += step;
+    for (int step = HALF ? POOL / 8 : POOL / 4; step > 0; step >>= 2) {
+        const bool a = (pool[p + step - 1] | 1ull) < mk, b = (pool[p + 2 * step - 1] | 1ull) < mk,
+                   c = (pool[p + 3 * step - 1] | 1ull) < mk;
+        p += a ? (b ? (c ? 3 * step : 2 * step) : step) : 0;
+    }
     in = in && (pool[p] | 1ull) != mk;                  // the pool holds it already
     // of equal keys the first one goes on (their ranks are equal, and the other lanes' are made different)
     const uint32_t same = __match_any_sync(FULL, lane < n ? key_rank(key) : 0x80000000u | (uint32_t)lane);
