@@ -79,7 +79,7 @@ typedef struct {
                                   waits give up after 64 polls, so every gather ends as a copy time-out would,
                                   with nothing in flight: the affected rows are padding, their status carries
                                   FROG_ST_COPY_TIMEOUT, frog_search_last_status reports it, and the next call
-                                  works.  Honoured by the kernel for 384- and 512-byte rows (bitmap visited set,
+                                  works.  Honoured by the kernel for fp32 rows of 128, 256, 384 and 512 bytes (bitmap visited set,
                                   beam widths up to 32, budgets up to 64) and, when `stats` is given, by the
                                   general kernel; ignored otherwise;
                            bits 8-11: log2 of that table's slots, 6..12 (0 = 12), to make queries outgrow it */
@@ -192,7 +192,9 @@ int frog_search_ex(const frog_index_t* index, const float* queries, const int32_
  * Scratch: an index is loaded with what one stream's scans of up to 2,048 queries with k <= 128 need (39 MB at
  * most), but no more than half of its own size; a scan on another stream, up to 16 in flight at once, or one
  * that needs more allocates with cudaMalloc (0.5-3 ms, kept until frog_index_free) -- on indexes of up to 16 MB of
- * rows only from the second such call on.  None of it is shared with frog_search.
+ * rows only from the second such call on.  The scan of many queries on 4,000 objects and more asks for the larger of
+ * 32 MB and half of the index at most, and makes do with a quarter of what it could use.  None of it is shared
+ * with frog_search.
  * Same buffers and conventions as frog_search; 1 <= k <= FROG_MAX_BEAM_WIDTH.  Used for ground truth
  * and as the pre-filtering reference. */
 int frog_exact_search(const frog_index_t* index, const float* queries, const int32_t* lo, const int32_t* hi,
@@ -202,8 +204,9 @@ int frog_exact_search(const frog_index_t* index, const float* queries, const int
  * query vectors and ranges, then execution).  All pointers are HOST memory.  If all five buffers
  * are page-locked and device-mapped (cudaHostAlloc / cudaHostRegister) the kernels read the inputs
  * and write the results across the bus themselves, overlapping the transfers with the search;
- * otherwise the call copies in through staging buffers owned by the index (grown on first use),
- * searches and copies the results out.  Either way it returns after synchronising the stream. */
+ * otherwise up to 256 KB of pageable buffers pass through a page-locked block of the index (allocated on first use)
+ * in the same way, and larger calls copy in through staging buffers owned by the index (grown on first use),
+ * search and copy the results out.  Either way it returns after synchronising the stream. */
 int frog_search_host(frog_index_t* index, const float* queries, const int32_t* lo, const int32_t* hi,
                      int nq, int k, int beam_width, const frog_params_t* params /* HOST, may be null */,
                      int32_t* out_ids, float* out_dists, void* stream);

@@ -129,7 +129,7 @@ template <class F>
 cudaError_t allow_smem(F* fn) {
     return cudaFuncSetAttribute((const void*)fn, cudaFuncAttributeMaxDynamicSharedMemorySize, MAX_SMEM);
 }
-// frog_search_lean.cu: the trimmed kernel for 384- and 512-byte fp32 and 192- and 256-byte fp16 rows (null: shape not covered)
+// frog_search_lean.cu: the trimmed kernel for short rows, 128 to 512 bytes fp32 and 64 to 256 bytes fp16 (null: shape not covered)
 frog_kernel_fn lean_kernel(int ef_s, int budget, int row_bytes, bool f16, bool table, bool hook, int queries_per_sm,
                            size_t* smem_per_warp, int* warps_per_cta);
 bool lean_row(int row_bytes, bool f16);          // the rows it covers
