@@ -43,7 +43,7 @@ struct FilterSmem {
     // of the batch's queries: first rank and how many follow it, blocks of 32 rows (0: no query), values per block
     uint32_t l[TILE], span[TILE], blocks[TILE];
     int per[TILE];
-    float norm[TILE], root[TILE], tau[TILE];     // squared norm with its part of the bound, norm, bound of the answers
+    float norm[TILE], root[TILE], tau[TILE];     // half the squared norm with its part of the bound, norm, half the bound of the answers
     uint32_t off[TILE];
     int count;
 };
@@ -132,8 +132,10 @@ filter_offsets_kernel(const FilterArgs A) {
 // Bound of the error of a rough distance, and of what separates the fp32 distance of the scan from the true one.
 // With u = 2^-11 the rounding of an operand: |x~.q~ - x.q| <= (2u + u^2) |x| |q|; the sums of d products, of the norms
 // and of the scan are within d 2^-22 of their magnitude each (twice what rounding to nearest gives); the last two terms
-// cover what underflows.  Anything not finite makes the comparisons with it false, which rules nothing out.
-// (x and q are the norms, c1 x q + own(x) + own(q) the bound.)
+// cover what underflows.  (x and q are the norms, c1 x q + own(x) + own(q) the bound.)
+// The epilogue computes HALF of a bound, which two finite norms cannot take beyond the range of fp32: it is infinite only
+// where x.q is below -2^128, and then so is the distance.  A norm that is not finite makes it not a number, and the
+// comparison with it false, which rules nothing out.
 struct RowError {
     float c1, c2;
     __device__ __forceinline__ explicit RowError(int d) : c1(0.00197f + d * 0x1p-20f), c2(0x1p-19f + d * 0x1p-21f) {}
@@ -222,9 +224,9 @@ filter_tile_kernel(const FilterArgs A) {
                 S.span[t] = t < nb ? (uint32_t)(s.y - s.x) : 0u;
                 S.blocks[t] = t < nb ? blocks : 0u;
                 S.per[t] = per;
-                S.norm[t] = PASS == 0 ? n + own : n - own;
+                S.norm[t] = PASS == 0 ? 0.5f * n + 0.5f * own : 0.5f * n - 0.5f * own;
                 S.root[t] = root;
-                if (PASS == 1) S.tau[t] = A.tau[q];
+                if (PASS == 1) S.tau[t] = 0.5f * A.tau[q];
                 S.off[t] = A.off[q] + (PASS == 1 ? blocks * per : 0u);
             }
             float acc[2][8][4];
@@ -306,13 +308,13 @@ filter_tile_kernel(const FilterArgs A) {
                 // this thread's rows are base + g + 8 j, its queries 8 x + 2 p and the next one
                 const int base = row0 + wm * 32;
                 float finite = 0.f;                                  // or not a number
-                // a bound is |x|^2 +- own(x) + |q|^2 +- own(q) +- c1 |x| |q| - 2 x.q
+                // half a bound is (|x|^2 +- own(x) + |q|^2 +- own(q) +- c1 |x| |q|) / 2 - x.q
                 float nx[4], sx[4];
 #pragma unroll
                 for (int j = 0; j < 4; ++j) {
                     const float n = S.row_norm[wm * 32 + g + 8 * j], s = __fsqrt_rn(n), own = error.own(n, s);
-                    nx[j] = PASS == 0 ? n + own : n - own;
-                    sx[j] = PASS == 0 ? error.c1 * s : -error.c1 * s;
+                    nx[j] = PASS == 0 ? 0.5f * n + 0.5f * own : 0.5f * n - 0.5f * own;
+                    sx[j] = PASS == 0 ? 0.5f * error.c1 * s : -0.5f * error.c1 * s;
                 }
 #pragma unroll
                 for (int x = 0; x < 8; ++x) {
@@ -325,7 +327,7 @@ filter_tile_kernel(const FilterArgs A) {
                         float least = __int_as_float(0x7F800000);
 #pragma unroll
                         for (int j = 0; j < 4; ++j) {
-                            const float bound = fmaf(sx[j], sq, fmaf(-2.f, acc[j >> 1][x][(j & 1) * 2 + c], nx[j] + nq));
+                            const float bound = fmaf(sx[j], sq, (nx[j] + nq) - acc[j >> 1][x][(j & 1) * 2 + c]);
                             const bool in = at + 8u * j <= span;
                             if (PASS == 0) {
                                 if (in && bound < least) least = bound;
@@ -335,7 +337,7 @@ filter_tile_kernel(const FilterArgs A) {
                             }
                         }
                         if (PASS == 0) {
-                            least = least > 0.f ? least : 0.f;
+                            least = least > 0.f ? 2.f * least : 0.f;
                             least = fminf(least, __shfl_xor_sync(FULL, least, 4));
                             const float wide = fminf(least, __shfl_xor_sync(FULL, least, 8));
                             const float all = fminf(wide, __shfl_xor_sync(FULL, wide, 16));

@@ -119,6 +119,28 @@ def test_filtered_scans_of_extreme_values(libs, tmp_path, scale):
     gix.close()
 
 
+def test_filtered_scans_of_norms_whose_sum_overflows(libs, tmp_path):
+    """|q|^2 = 2e38: both norms and all distances are finite, the sum of the norms of q and a row like it is not."""
+    rng = np.random.default_rng(2)
+    n, d, nq = 6000, 40, 200
+    q = rng.standard_normal((nq, d))
+    q = (q * np.sqrt(2e38 / (q * q).sum(1, keepdims=True))).astype(np.float32)
+    base = (rng.standard_normal((n, d)) * 5e17).astype(np.float32)
+    for j, t in enumerate((1.0, 0.97, 0.5, 0.0, -0.3)):
+        base[j:5 * nq:5] = np.float32(t) * q
+    path = str(tmp_path / "x.idx")
+    libs.build_index_gpu(base, rng.permutation(n).astype(np.int32), path, m=4, ef_c=4, patience=1, n_inv=30)
+    ix, gix = oracle.load_index(path), libs.Index.load(path)
+    lo, hi = np.zeros(nq, np.int32), np.full(nq, n, np.int32)
+    hi[::7] = n // 2
+    ids = gix.exact_search(*(torch.from_numpy(x).cuda() for x in (q, lo, hi)), 1)[0].cpu().numpy()[:, 0]
+    all_rows = np.arange(nq) % 7 != 0
+    assert np.array_equal(ids[all_rows], (5 * np.arange(nq))[all_rows])
+    for k in (1, 3, 10):
+        _check(gix, ix, q, lo, hi, k)
+    gix.close()
+
+
 def test_groups_with_gaps_streams_and_capture(libs, tmp_path):
     """Slabs that share no rows (a group's pieces jump the gaps), calls on two streams, and a captured call."""
     base, attrs, path = _index(libs, tmp_path, 30000, 24, 11)
