@@ -208,7 +208,7 @@ sibling_search_kernel(const BuildArgs A) {
                 W.keys[0] = make_key(d2, ep, 0u);
             }
             __syncwarp();
-            int first = (int)merge_ranked<EPL>(W.spool, W.keys, 1, A.ef_c, lane);
+            int first = (int)merge_ranked<EPL, true>(W.spool, W.keys, 1, A.ef_c, lane);
             int pat = A.patience;
             for (int it = 0; first < A.ef_c && it < 4 * A.ef_c; ++it) {
                 const uint32_t x = key_rank(W.spool[first]);
@@ -239,7 +239,7 @@ sibling_search_kernel(const BuildArgs A) {
                 if (close) W.keys[__popc(C & lt_mask)] = key;
                 __syncwarp();
                 bool entered = false;
-                if (C) first = (int)merge_ranked<EPL>(W.spool, W.keys, __popc(C), A.ef_c, lane, &entered);
+                if (C) first = (int)merge_ranked<EPL, true>(W.spool, W.keys, __popc(C), A.ef_c, lane, &entered);
                 else first = (int)next_open<EPL>(W.spool, first, lane);
                 // something enters the top m
                 const bool improved = __any_sync(FULL, entered && (W.keys[lane] | 1ull) < (mth | 1ull));

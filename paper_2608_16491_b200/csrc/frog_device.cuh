@@ -622,7 +622,9 @@ __device__ __forceinline__ uint32_t merge_batch(uint64_t* pool, uint64_t my_key,
 // key or which old one moves there.  The cost hardly depends on the pool size and little on n, and the
 // dependent chain has no shuffle or vote per key.
 // `entered` tells a lane whether its key is in the pool now and was not before.  Keys that do not enter are emptied.
-template <int EPL>
+// ROWS: a key's rank is that of a row, so that keys of one rank are equal (matching half a key: one query 143.5 -> 142 us).
+// In an exact scan it is an object id, and an object may have several vectors.
+template <int EPL, bool ROWS = false>
 __device__ __forceinline__ uint32_t merge_ranked(uint64_t* pool, uint64_t* keys, int n, int ef_s, int lane,
                                                  bool* entered = nullptr) {
     constexpr int POOL = 32 * EPL;
@@ -642,8 +644,9 @@ __device__ __forceinline__ uint32_t merge_ranked(uint64_t* pool, uint64_t* keys,
         p += a ? (b ? (c ? 3 * step : 2 * step) : step) : 0;
     }
     in = in && (pool[p] | 1ull) != mk;                  // the pool holds it already
-    // of equal keys the first one goes on (their ranks are equal, and the other lanes' are made different)
-    const uint32_t same = __match_any_sync(FULL, lane < n ? key_rank(key) : 0x80000000u | (uint32_t)lane);
+    // of equal keys the first one goes on (the other lanes' are made different)
+    const uint32_t same = ROWS ? __match_any_sync(FULL, lane < n ? key_rank(key) : 0x80000000u | (uint32_t)lane)
+                               : __match_any_sync(FULL, lane < n ? mk : 0xFFFFFFFF00000000ull | (uint64_t)lane);
     in = in && (same & lt_mask) == 0;
     if (lane < n && !in) keys[lane] = KEY_EMPTY;        // not below any other
     __syncwarp();

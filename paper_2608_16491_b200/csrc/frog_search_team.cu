@@ -198,7 +198,7 @@ frog_search_team_kernel(const __grid_constant__ FrogSearchArgs A) {
                 *vis_slot(key_rank(key)) = key_rank(key);
             }
             __syncwarp();
-            merge_ranked<EPL>(pool, ctl.batch, min(32, n - off), A.ef_s, lane);
+            merge_ranked<EPL, true>(pool, ctl.batch, min(32, n - off), A.ef_s, lane);
         }
     };
 

@@ -276,6 +276,33 @@ def test_more_queries_than_a_planning_kernel_has_32_bit_threads(libs, tmp_path):
     gix.close()
 
 
+@pytest.mark.parametrize("n,d", [(300, 12), (9000, 33)])
+def test_objects_of_several_vectors(libs, n, d):
+    """An id that occurs several times, each time at another distance, is listed as often: in every form, and as in the
+    scan of all rows."""
+    import ctypes
+    rng = np.random.default_rng(n)
+    d_pad = (d + 3) // 4 * 4
+    vec = np.zeros((n, d_pad), np.float32)
+    vec[:, :d] = rng.standard_normal((n, d))
+    attr, ids = np.arange(n, dtype=np.int32), rng.integers(0, n // 40, n).astype(np.int32)
+    enc = np.full((n, 1, 4), 0xFFFFFFFF, np.uint32)
+    shape = libs.IndexInfo(n=n, d=d, d_pad=d_pad, H=1, m=4)
+    h = ctypes.c_void_p()
+    assert libs._lib.frog_index_from_host(*[a.ctypes.data_as(ctypes.c_void_p) for a in (attr, ids, vec, enc)], ctypes.byref(shape), 0,
+                                          ctypes.byref(h)) == 0
+    gix = libs.Index(h)
+    ix = oracle.OracleIndex(n=n, d=d, d_pad=d_pad, H=1, m=4, n_inv=0, ef_c=4, patience=1, beta=0.0, gamma=1.0, seed=0, sorted_attr=attr,
+                            rank2id=ids, vectors=vec, enc=enc)
+    q = rng.standard_normal((600, d)).astype(np.float32)
+    lo = rng.integers(0, n // 2, 600).astype(np.int32)
+    hi = (lo + rng.integers(0, n // 2, 600)).astype(np.int32)
+    for nq in (1, 6, 30, 250, 600):
+        for k in (10, 60, 300):
+            _check(gix, ix, q[:nq], lo[:nq], hi[:nq], k)
+    gix.close()
+
+
 def test_scans_beside_another_threads_capture(libs, tmp_path):
     """A thread captures a graph; another one scans an index for the first time, which allocates.  The scan works
     and the capture is not spoilt."""
