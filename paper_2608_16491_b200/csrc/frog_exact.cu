@@ -819,14 +819,6 @@ ExactForm exact_form(size_t n, size_t row_bytes, int nq, int k, bool filter) {
     return k > 32 || bytes > 4500000 || (n >= 8000 && nq <= 300) ? ExactForm::Grouped : ExactForm::OnePerQuery;
 }
 
-// While another thread captures a stream, event queries and allocations are refused and spoil its capture, unless the
-// calling thread says that they have nothing to do with it.
-struct NoCaptureOfOurs {
-    cudaStreamCaptureMode mode = cudaStreamCaptureModeRelaxed;
-    NoCaptureOfOurs() { cudaThreadExchangeStreamCaptureMode(&mode); }
-    ~NoCaptureOfOurs() { cudaThreadExchangeStreamCaptureMode(&mode); }
-};
-
 // A set for a scan on stream s: the one it used last, an idle one, a new one, or null when all are busy with other
 // streams' scans (the caller does without: a wait for another stream is not made here).  Called with exact_mu held.
 FrogExactSet* exact_set(frog_index* ix, cudaStream_t s) {
@@ -970,7 +962,7 @@ extern "C" int frog_exact_search(const frog_index_t* index, const float* queries
         const size_t want = std::min(room.most, std::max(room.least, std::max((size_t)index->info.device_bytes / 2, (size_t)32 << 20)));
         FrogExactSet* set = nullptr;
         {
-            const NoCaptureOfOurs relaxed;
+            const froghost::NoCaptureOfOurs relaxed;
             set = exact_set(mix, s);
             if (set && set->bytes < room.least && !exact_room(mix, set, 0, want)) set = nullptr;
         }
@@ -1015,7 +1007,7 @@ extern "C" int frog_exact_search(const frog_index_t* index, const float* queries
         FrogExactSet* set = nullptr;
         ExactScratch X;
         {
-            const NoCaptureOfOurs relaxed;
+            const froghost::NoCaptureOfOurs relaxed;
             set = exact_set(mix, s);
             if (set && !exact_scratch(mix, set, s, (size_t)nq, cut, few, &X)) set = nullptr;
         }

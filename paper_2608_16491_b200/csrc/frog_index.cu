@@ -282,6 +282,7 @@ extern "C" int frog_search_host(frog_index_t* ix, const float* queries, const in
     if (nq == 0) return FROG_OK;
     if (!queries || !lo || !hi || !out_ids || !out_dists) return FROG_ERR_INVALID_ARG;
     FROG_CUDA_TRY(cudaSetDevice(ix->info.device));
+    const froghost::NoCaptureOfOurs relaxed;               // the allocations and the wait at the end
     cudaStream_t s = static_cast<cudaStream_t>(stream);
     auto up = [](size_t x) { return (x + 255) & ~(size_t)255; };
     const size_t b_q = up((size_t)nq * ix->info.d * 4), b_r = up((size_t)nq * 4), b_o = up((size_t)nq * k * 4);
@@ -308,11 +309,13 @@ extern "C" int frog_search_host(frog_index_t* ix, const float* queries, const in
         bool mapped = known && staged == 0;
         if (known && !mapped && staged <= FROG_HOST_STAGE) {
             stage_lock.lock();
-            if (!ix->h_stage && !ix->no_h_stage &&
-                cudaHostAlloc((void**)&ix->h_stage, FROG_HOST_STAGE, cudaHostAllocMapped) != cudaSuccess) {
-                cudaGetLastError();
-                ix->h_stage = nullptr;
-                ix->no_h_stage = true;
+            if (!ix->h_stage && !ix->no_h_stage) {
+                const cudaError_t e = cudaHostAlloc((void**)&ix->h_stage, FROG_HOST_STAGE, cudaHostAllocMapped);
+                if (e != cudaSuccess) {
+                    cudaGetLastError();
+                    ix->h_stage = nullptr;
+                    ix->no_h_stage = e == cudaErrorMemoryAllocation;       // not asked for again
+                }
             }
             char* base = nullptr;
             if (ix->h_stage && cudaHostGetDevicePointer((void**)&base, ix->h_stage, 0) != cudaSuccess) { cudaGetLastError(); base = nullptr; }

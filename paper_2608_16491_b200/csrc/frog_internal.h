@@ -129,6 +129,13 @@ template <class F>
 cudaError_t allow_smem(F* fn) {
     return cudaFuncSetAttribute((const void*)fn, cudaFuncAttributeMaxDynamicSharedMemorySize, MAX_SMEM);
 }
+// While another thread captures a stream, waits, event queries and allocations are refused and spoil its capture, unless the
+// calling thread says that they have nothing to do with it.
+struct NoCaptureOfOurs {
+    cudaStreamCaptureMode mode = cudaStreamCaptureModeRelaxed;
+    NoCaptureOfOurs() { cudaThreadExchangeStreamCaptureMode(&mode); }
+    ~NoCaptureOfOurs() { cudaThreadExchangeStreamCaptureMode(&mode); }
+};
 // frog_search_lean.cu: the trimmed kernel for short rows, 128 to 512 bytes fp32 and 64 to 256 bytes fp16 (null: shape not covered)
 frog_kernel_fn lean_kernel(int ef_s, int budget, int row_bytes, bool f16, bool table, bool hook, int queries_per_sm,
                            size_t* smem_per_warp, int* warps_per_cta);

@@ -52,3 +52,48 @@ def test_pinned_and_pageable_buffers(libs, tmp_path):
         t.join()
     assert not bad
     gix.close()
+
+
+def _small(libs, tmp_path):
+    rng = np.random.default_rng(5)
+    n, d = 3000, 32
+    base = rng.standard_normal((n, d)).astype(np.float32)
+    path = str(tmp_path / "s.idx")
+    libs.build_index_gpu(base, np.arange(n, dtype=np.int32), path, ef_c=32)
+    return base, libs.Index.load(path)
+
+
+@pytest.mark.parametrize("nq", [20, 2000])
+def test_first_calls_beside_another_threads_capture(libs, tmp_path, nq):
+    """The page-locked block, or the staging buffers of a larger call, are allocated while another thread captures a graph:
+    the call works and the capture is not spoilt."""
+    base, gix = _small(libs, tmp_path)
+    side = torch.cuda.Stream()
+    # the stream's scratch is there; pinned buffers need no block
+    pinned = [torch.from_numpy(x).pin_memory() for x in (base[:nq] + 0.1, np.zeros(nq, np.int32), np.full(nq, 900, np.int32))]
+    held = [torch.empty((nq, 5), dtype=t).pin_memory() for t in (torch.int32, torch.float32)]
+    want = [x.clone() for x in gix.search_host(*pinned, 5, 32, out_ids=held[0], out_dists=held[1], stream=side)]
+    plain = [x.clone() for x in pinned]
+    out = [torch.zeros((nq, 5), dtype=t) for t in (torch.int32, torch.float32)]
+    x, errors = torch.zeros(1000, device="cuda"), []
+    torch.cuda.synchronize()
+
+    def call():
+        try:
+            gix.search_host(*plain, 5, 32, out_ids=out[0], out_dists=out[1], stream=side)
+        except libs.FrogError as e:
+            errors.append(e)
+
+    graph = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(graph, capture_error_mode="global"):
+        x += 1
+        t = threading.Thread(target=call)
+        t.start()
+        t.join()
+        x += 1
+    graph.replay()
+    torch.cuda.synchronize()
+    assert not errors and float(x[0]) == 2.0
+    assert torch.equal(out[0], want[0]) and torch.equal(out[1], want[1])
+    graph.reset()
+    gix.close()
