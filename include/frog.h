@@ -193,8 +193,8 @@ int frog_search_ex(const frog_index_t* index, const float* queries, const int32_
  * most), but no more than half of its own size; a scan on another stream, up to 16 in flight at once, or one
  * that needs more allocates with cudaMalloc (0.5-3 ms, kept until frog_index_free) -- on indexes of up to 16 MB of
  * rows only from the second such call on.  The scan of many queries on 4,000 objects and more asks for the larger of
- * 32 MB and half of the index at most, and makes do with a quarter of what it could use.  None of it is shared
- * with frog_search.
+ * 64 MB and half of the index at most, and takes a batch that needs more in rounds.  None of it is shared with
+ * frog_search.
  * Same buffers and conventions as frog_search; 1 <= k <= FROG_MAX_BEAM_WIDTH.  Used for ground truth
  * and as the pre-filtering reference. */
 int frog_exact_search(const frog_index_t* index, const float* queries, const int32_t* lo, const int32_t* hi,

@@ -806,11 +806,14 @@ size_t exact_smem(int k, int d_pad) {
 //   100,000 x 128   90/100 | 253/105      149/107 | 555/129      411/128 | 1,190/259  1,262/324 | -
 //   400,000 x 96    155/207 | 1,200/251   352/246 | 2,926/302    1,032/327 | -        3,802/808 | -
 enum class ExactForm { OnePerQuery, Few, Split, Grouped, Filter };
+int filter_line(size_t n, size_t row_bytes, int k) {
+    if (n < 4000 || row_bytes > 16384) return 0x7FFFFFFF;
+    if (row_bytes > 1024) return n >= 16000 ? 128 : 400;
+    return n < 16000 ? 100 : k <= 32 ? 80 : n < 64000 ? 40 : EXACT_PLAN_MIN;
+}
 ExactForm exact_form(size_t n, size_t row_bytes, int nq, int k, bool filter) {
     const size_t bytes = n * row_bytes;
-    if (filter && n >= 4000 && row_bytes <= 16384 &&
-        nq >= (row_bytes > 1024 ? (n >= 16000 ? 128 : 400) : n < 16000 ? 100 : k <= 32 ? 80 : n < 64000 ? 40 : EXACT_PLAN_MIN))
-        return ExactForm::Filter;
+    if (filter && nq >= filter_line(n, row_bytes, k)) return ExactForm::Filter;
     if (nq < EXACT_PLAN_MIN) return k <= 32 && bytes <= 500000 ? ExactForm::OnePerQuery : ExactForm::Few;
     const double work = (double)n * (double)(row_bytes + 384) * (k > 128 ? 3.0 : k > 64 ? 1.4 : 1.0);
     if (nq <= EXACT_SPLIT_MAX && nq * (n < 8000 ? 45e3 : 100e3) <= work) return ExactForm::Split;
@@ -955,18 +958,31 @@ extern "C" int frog_exact_search(const frog_index_t* index, const float* queries
     FROG_CUDA_TRY(cudaStreamIsCapturing(s, &capture));
     ExactForm form = exact_form((size_t)index->info.n, (size_t)A.d_pad * 4, nq, k, capture == cudaStreamCaptureStatusNone);
     if (form == ExactForm::Filter) {
-        // (scratch of the sets' part that has no state at rest; where it cannot be had, the other forms)
+        // Scratch of the sets' part that has no state at rest, for slabs of any width, as these are on the device, up to the
+        // larger of 64 MB and half of the index.  A batch for which that may not be enough goes in rounds, where these are
+        // few or each is large (one that has nothing to do takes 15-25 us, and the grouped form 27 us for 1,000 queries of
+        // 50 rows); where scratch cannot be had, the other forms.  Batches over all rows, us, by the forms below / filtered
+        // with one CTA for a query that there was no room for / in rounds: 2,000 queries, k = 10, on 100,000 x 128
+        // 4,990 / 3,980 / 803, 400,000 x 96 17,200 / 15,300 / 2,650; 100 on 4,000,000 x 32 23,100 / 55,900 / 1,760.
         frog_index* mix = const_cast<frog_index*>(index);
         std::lock_guard<std::mutex> lock(mix->exact_mu);
-        const froghost::FilterRoom room = froghost::filter_room((size_t)index->info.n, (size_t)nq, k, A.d_pad);
-        const size_t want = std::min(room.most, std::max(room.least, std::max((size_t)index->info.device_bytes / 2, (size_t)32 << 20)));
+        const size_t n = (size_t)index->info.n;
+        const size_t want = std::min(froghost::filter_bytes(n, (size_t)nq, k, A.d_pad),
+                                     std::max((size_t)index->info.device_bytes / 2, (size_t)64 << 20));
         FrogExactSet* set = nullptr;
+        froghost::FilterFit fit{};
         {
             const froghost::NoCaptureOfOurs relaxed;
             set = exact_set(mix, s);
-            if (set && set->bytes < room.least && !exact_room(mix, set, 0, want)) set = nullptr;
+            if (set && set->mem) fit = froghost::filter_fit(n, (size_t)nq, set->bytes, k, A.d_pad);
+            if (set && set->bytes < want) {
+                // (what takes the batch in four rounds will do for the first call of its kind)
+                if (fit.queries && fit.parts * fit.rounds <= 4 && !mix->exact_asked) mix->exact_asked = true;
+                else if (exact_room(mix, set, 0, want)) fit = froghost::filter_fit(n, (size_t)nq, set->bytes, k, A.d_pad);
+            }
         }
-        if (set) {
+        if (fit.queries && fit.per_round >= (size_t)filter_line(n, (size_t)A.d_pad * 4, k) &&
+            (fit.parts * fit.rounds <= 4 || (fit.per_round >= 512 && fit.parts <= 64))) {
             froghost::FilterArgs F{};
             F.sorted_attr = A.sorted_attr;
             F.rank2id = A.rank2id;
@@ -974,15 +990,20 @@ extern "C" int frog_exact_search(const frog_index_t* index, const float* queries
             F.n = A.n;
             F.d = A.d;
             F.d_pad = A.d_pad;
-            F.queries = queries;
-            F.lo = lo;
-            F.hi = hi;
-            F.nq = nq;
             F.k = k;
-            F.out_ids = out_ids;
-            F.out_dists = out_dists;
-            froghost::filter_scratch(set->mem + exact_rest_bytes(set->queries), std::min(set->bytes, room.most), &F);
-            FROG_CUDA_TRY(froghost::filter_launch(F, index->sm_count, s));
+            F.rounds = (int)fit.rounds;
+            F.step = fit.step;
+            for (size_t p = 0; p < fit.parts; ++p) {
+                const size_t q0 = (size_t)nq * p / fit.parts, q1 = (size_t)nq * (p + 1) / fit.parts;
+                F.queries = queries + q0 * A.d;
+                F.lo = lo + q0;
+                F.hi = hi + q0;
+                F.nq = (int)(q1 - q0);
+                F.out_ids = out_ids + q0 * k;
+                F.out_dists = out_dists + q0 * k;
+                froghost::filter_scratch(set->mem + exact_rest_bytes(set->queries), &F);
+                FROG_CUDA_TRY(froghost::filter_launch(F, index->sm_count, s));
+            }
             FROG_CUDA_TRY(cudaEventRecord(set->done, s));
             FROG_CUDA_TRY(cudaStreamGetId(s, &set->stream_id));
             set->used = true;

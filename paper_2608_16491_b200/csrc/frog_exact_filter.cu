@@ -91,7 +91,9 @@ filter_plan_kernel(const FilterArgs A) {
     }
 }
 
-// where each query's values and masks lie (one CTA); BOT: the query is not filtered
+// Where each query's values lie (one CTA); BOT: the query is not filtered.  The store holds the values of some queries at a
+// time, as the widths, which are on the device, allow: a round takes those whose values, laid end to end, begin in its
+// share of A.step.
 __global__ void __launch_bounds__(1024)
 filter_offsets_kernel(const FilterArgs A) {
     __shared__ unsigned long long warp_sum[32];
@@ -103,15 +105,11 @@ filter_offsets_kernel(const FilterArgs A) {
     for (int q0 = 0; q0 < A.nq; q0 += 1024) {
         const int q = q0 + t;
         unsigned long long need = 0;                             // 32-bit words: the values, then the masks
-        uint32_t nv = 0;
         if (q < A.nq) {
             const int2 s = A.slab[q];
             const int w = s.y - s.x + 1;
-            if (filtered(w, A.k)) {
-                const uint32_t nb = (uint32_t)((s.y >> 5) - (s.x >> 5) + 1);
-                nv = nb * values_per_block(w, A.k);
-                need = nv + nb;
-            }
+            if (filtered(w, A.k))
+                need = (unsigned long long)((s.y >> 5) - (s.x >> 5) + 1) * (values_per_block(w, A.k) + 1);
         }
         unsigned long long x = need;
         for (int o = 1; o < 32; o <<= 1) {
@@ -122,7 +120,12 @@ filter_offsets_kernel(const FilterArgs A) {
         __syncthreads();
         unsigned long long at = base + x - need;
         for (int w = 0; w < warp; ++w) at += warp_sum[w];
-        if (q < A.nq) A.off[q] = need != 0 && at + need <= A.words ? (uint32_t)at : BOT;
+        if (q < A.nq) {
+            const unsigned long long round = at / A.step, next = q + 1 < A.nq ? (at + need) / A.step : (unsigned long long)A.rounds;
+            A.off[q] = need != 0 ? (uint32_t)(at - round * A.step) : BOT;
+            if (q == 0) A.first[0] = 0;
+            for (unsigned long long r = round + 1; r <= next; ++r) A.first[r] = q + 1;
+        }
         __syncthreads();
         if (t == 1023) base = at + need;
         __syncthreads();
@@ -147,9 +150,12 @@ struct RowError {
 
 // PASS 0: bounds, PASS 1: masks.  One CTA per 128 rows and per share of the queries: those whose number is blockIdx.y
 // modulo gridDim.y (the order in which a CTA lists its queries is not that of another).
+__device__ __forceinline__ int2 round_queries(const FilterArgs& A, int round) {      // first and end
+    return A.rounds == 1 ? make_int2(0, A.nq) : make_int2(__ldg(A.first + round), __ldg(A.first + round + 1));
+}
 template <int PASS, int KC>
 __global__ void __launch_bounds__(THREADS, 2)
-filter_tile_kernel(const FilterArgs A) {
+filter_tile_kernel(const FilterArgs A, int round) {
     extern __shared__ __align__(16) unsigned char smem_raw[];
     FilterSmem<KC>& S = *reinterpret_cast<FilterSmem<KC>*>(smem_raw);
     constexpr int KP = FilterSmem<KC>::KP, STAGES = FilterSmem<KC>::STAGES;
@@ -162,7 +168,8 @@ filter_tile_kernel(const FilterArgs A) {
     const float tile_norm = PASS == 1 ? __uint_as_float(A.tile_norm[blockIdx.x]) : 0.f, tile_sqrt = __fsqrt_rn(tile_norm);
     bool have_norms = false;
 
-    for (int q0 = 0; q0 < A.nq; q0 += SEG) {
+    const int2 queries = round_queries(A, round);
+    for (int q0 = queries.x; q0 < queries.y; q0 += SEG) {
         __syncthreads();
         if (t == 0) S.count = 0;
         __syncthreads();
@@ -172,7 +179,7 @@ filter_tile_kernel(const FilterArgs A) {
 #pragma unroll
         for (int x = 0; x < EACH; ++x) {
             const int q = q0 + x * THREADS + t;
-            const bool mine = q < A.nq && q % gridDim.y == blockIdx.y;
+            const bool mine = q < queries.y && q % gridDim.y == blockIdx.y;
             offs[x] = mine ? A.off[q] : BOT;
             slabs[x] = mine ? A.slab[q] : make_int2(1, 0);
         }
@@ -193,14 +200,14 @@ filter_tile_kernel(const FilterArgs A) {
                     const int w = s.y - s.x + 1, per = values_per_block(w, A.k), all = (s.y >> 5) - (s.x >> 5) + 1;
                     const int from = max((row0 >> 5) - (s.x >> 5), 0), to = min(((row0 + TILE) >> 5) - (s.x >> 5), all);
                     const float nq = A.norm[q], tau = A.tau[q], e = 2.f * error(tile_norm, tile_sqrt, nq, __fsqrt_rn(nq));
-                    const uint32_t* const v = A.store + off;
+                    uint32_t* const v = A.store + off;
                     hit = false;
                     for (int x = from * per; x < to * per; ++x) {
                         const float least = __uint_as_float(v[x]);
                         hit = hit || !(least - e > tau) || !(least < __int_as_float(0x7F800000));
                     }
                     if (!hit)
-                        for (int x = from; x < to; ++x) A.store[off + all * per + x] = 0u;
+                        for (int x = from; x < to; ++x) v[all * per + x] = 0u;
                 }
             }
             const uint32_t M = __ballot_sync(FULL, hit);
@@ -369,12 +376,13 @@ filter_tile_kernel(const FilterArgs A) {
 // Per query: an upper bound, within 2^-14, of the k-th smallest of its values.  Two passes over the values, eleven bits
 // of the (non-negative) numbers each.
 __global__ void __launch_bounds__(256)
-filter_bound_kernel(const FilterArgs A) {
+filter_bound_kernel(const FilterArgs A, int round) {
     __shared__ unsigned int bins[2048];
     __shared__ unsigned int warp_sum[8];
     __shared__ unsigned int found[2];                            // the bin that holds the k-th, values below it
-    const int q = blockIdx.x, t = threadIdx.x, lane = lane_id(), warp = t >> 5;
-    const uint32_t off = A.off[q];
+    const int2 queries = round_queries(A, round);
+    const int q = queries.x + blockIdx.x, t = threadIdx.x, lane = lane_id(), warp = t >> 5;
+    const uint32_t off = q < queries.y ? A.off[q] : BOT;
     if (off == BOT) return;
     const int2 s = A.slab[q];
     const int nv = ((s.y >> 5) - (s.x >> 5) + 1) * values_per_block(s.y - s.x + 1, A.k);
@@ -433,11 +441,13 @@ struct RefineSmem {
 
 template <int EPL>
 __global__ void __launch_bounds__(REFINE_WARPS * 32)
-filter_refine_kernel(const FilterArgs A) {
+filter_refine_kernel(const FilterArgs A, int round) {
     extern __shared__ __align__(16) unsigned char smem_raw[];
     RefineSmem<EPL>& S = *reinterpret_cast<RefineSmem<EPL>*>(smem_raw);
     const float4* const qs = reinterpret_cast<const float4*>(smem_raw + (sizeof(RefineSmem<EPL>) + 15) / 16 * 16);
-    const int q = blockIdx.x, t = threadIdx.x, lane = lane_id(), warp = t >> 5;
+    const int2 queries = round_queries(A, round);
+    const int q = queries.x + blockIdx.x, t = threadIdx.x, lane = lane_id(), warp = t >> 5;
+    if (q >= queries.y) return;
     const int team = t >> 3, sub = lane & 7, groups = A.d_pad >> 2;
     const int2 slab = A.slab[q];
     const int w = slab.y - slab.x + 1;
@@ -587,7 +597,7 @@ namespace froghost {
 
 namespace {
 size_t up16(size_t x) { return (x + 15) & ~(size_t)15; }
-typedef void (*filter_fn)(const FilterArgs);
+typedef void (*filter_fn)(const FilterArgs, int);
 size_t refine_smem(int k, int d_pad, filter_fn* fn) {
     const size_t q = (size_t)d_pad * 4;
     if (k <= 32) { *fn = filter_refine_kernel<1>; return up16(sizeof(RefineSmem<1>)) + q; }
@@ -597,19 +607,45 @@ size_t refine_smem(int k, int d_pad, filter_fn* fn) {
     *fn = filter_refine_kernel<16>;
     return up16(sizeof(RefineSmem<16>)) + q;
 }
-size_t filter_fixed_bytes(size_t n, size_t nq, int d_pad) {
-    return nq * ((size_t)d_pad * 4 + 8 + 4 + 4 + 4) + (n / TILE + 1) * 4 + 64;
-}
+// of a part (the CTAs of its queries, 0.9 ns each, are launched in a round that has nothing to do too)
+constexpr size_t MOST_ROUNDS = 1000, MOST_QUERIES = 16384;
+// words of the slab that has most
+size_t most_words(size_t n, int k) { return std::max(2 * (n / 32 + 2), 5 * (std::min(n, (size_t)128 * k) / 32 + 2)); }
+// the arrays of FilterArgs
+size_t query_bytes(int d_pad) { return (size_t)d_pad * 4 + 8 + 4 + 4 + 4; }
+size_t fixed_bytes(size_t n) { return (n / TILE + 1) * 4 + (MOST_ROUNDS + 1) * 4; }
 }  // namespace
 
-FilterRoom filter_room(size_t n, size_t nq, int k, int d_pad) {
-    const size_t narrow = std::min(n, (size_t)128 * k);
-    const size_t words = nq * std::max(2 * (n / 32 + 2), 5 * (narrow / 32 + 2));
-    const size_t fixed = filter_fixed_bytes(n, nq, d_pad);
-    return {fixed + words, fixed + words * 4};
+size_t filter_bytes(size_t n, size_t nq, int k, int d_pad) {
+    return fixed_bytes(n) + std::min(nq, MOST_QUERIES) * (query_bytes(d_pad) + 4 * most_words(n, k));
 }
 
-void filter_scratch(char* mem, size_t bytes, FilterArgs* A) {
+FilterFit filter_fit(size_t n, size_t nq, size_t bytes, int k, int d_pad) {
+    FilterFit f{};
+    if (bytes < 2 * fixed_bytes(n)) return f;
+    f.queries = std::min(nq, MOST_QUERIES);
+    if (filter_bytes(n, nq, k, d_pad) > bytes) f.queries = std::min(f.queries, bytes / 4 / query_bytes(d_pad));
+    if (f.queries == 0) return f;
+    f.parts = (nq + f.queries - 1) / f.queries;
+    const size_t each = most_words(n, k);
+    // (offsets are 32-bit)
+    const size_t words = std::min<size_t>((bytes - fixed_bytes(n) - f.queries * query_bytes(d_pad)) / 4, 0xFFFFFFF0u);
+    if (f.queries * each <= words) {
+        f.step = words + 1;
+        f.rounds = 1;
+        f.per_round = f.queries;
+    } else if (words > each) {
+        f.step = words - each;
+        f.rounds = (f.queries - 1) * each / f.step + 1;
+        f.per_round = f.step / each;
+        if (f.rounds > MOST_ROUNDS) f.queries = 0;
+    } else {
+        f.queries = 0;
+    }
+    return f;
+}
+
+void filter_scratch(char* mem, FilterArgs* A) {
     const size_t nq = (size_t)A->nq;
     A->rounded = reinterpret_cast<float*>(mem);
     A->slab = reinterpret_cast<int2*>(mem + nq * A->d_pad * 4);
@@ -617,8 +653,8 @@ void filter_scratch(char* mem, size_t bytes, FilterArgs* A) {
     A->off = reinterpret_cast<uint32_t*>(A->norm + nq);
     A->tau = reinterpret_cast<float*>(A->off + nq);
     A->tile_norm = reinterpret_cast<uint32_t*>(A->tau + nq);
-    A->store = A->tile_norm + A->n / TILE + 1;
-    A->words = std::min<size_t>((bytes - filter_fixed_bytes((size_t)A->n, nq, A->d_pad)) / 4, 0xFFFFFFF0u);
+    A->first = reinterpret_cast<int*>(A->tile_norm + A->n / TILE + 1);
+    A->store = reinterpret_cast<uint32_t*>(A->first + MOST_ROUNDS + 1);
 }
 
 cudaError_t filter_launch(const FilterArgs& A, int sm_count, cudaStream_t s) {
@@ -637,10 +673,12 @@ cudaError_t filter_launch(const FilterArgs& A, int sm_count, cudaStream_t s) {
     const dim3 grid((unsigned)tiles, (unsigned)parts);
     filter_plan_kernel<<<(A.nq - 1) / 8 + 1, 256, 0, s>>>(A);
     filter_offsets_kernel<<<1, 1024, 0, s>>>(A);
-    bounds<<<grid, THREADS, tile_smem, s>>>(A);
-    filter_bound_kernel<<<A.nq, 256, 0, s>>>(A);
-    masks<<<grid, THREADS, tile_smem, s>>>(A);
-    refine<<<A.nq, REFINE_WARPS * 32, smem, s>>>(A);
+    for (int r = 0; r < A.rounds; ++r) {
+        bounds<<<grid, THREADS, tile_smem, s>>>(A, r);
+        filter_bound_kernel<<<A.nq, 256, 0, s>>>(A, r);
+        masks<<<grid, THREADS, tile_smem, s>>>(A, r);
+        refine<<<A.nq, REFINE_WARPS * 32, smem, s>>>(A, r);
+    }
     return cudaGetLastError();
 }
 

@@ -24,16 +24,21 @@ struct FilterArgs {
     uint32_t* off;           // where its values, then its masks, begin in `store`
     float* tau;              // no answer is farther
     uint32_t* tile_norm;     // per 128 rows: the largest squared norm (bits); infinite where a rough distance is not finite
+    int* first;              // per round: its first query; then the number of queries
     uint32_t* store;
-    size_t words;            // of `store`
+    int rounds;
+    unsigned long long step; // a round's share of the words of all queries, laid end to end
 };
 
-// Scratch bytes of a call: what it cannot do without (the rest is used as far as it goes) and what covers every case.
-struct FilterRoom {
-    size_t least, most;
+// Scratch for nq queries of any width in one round.
+size_t filter_bytes(size_t n, size_t nq, int k, int d_pad);
+// How so many bytes serve: a call goes in parts of `queries` (0: not at all), a part in rounds, of which as many do
+// something as the widths ask for; per_round: queries of the widest slabs in a round.
+struct FilterFit {
+    size_t queries, parts, rounds, per_round, step;
 };
-FilterRoom filter_room(size_t n, size_t nq, int k, int d_pad);
-void filter_scratch(char* mem, size_t bytes, FilterArgs* A);
+FilterFit filter_fit(size_t n, size_t nq, size_t bytes, int k, int d_pad);
+void filter_scratch(char* mem, FilterArgs* A);
 cudaError_t filter_launch(const FilterArgs& A, int sm_count, cudaStream_t s);
 
 }  // namespace froghost

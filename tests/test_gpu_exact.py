@@ -119,6 +119,36 @@ def test_filtered_scans_of_extreme_values(libs, tmp_path, scale):
     gix.close()
 
 
+@pytest.mark.parametrize("n,d,nq,k", [(100_000, 8, 9_001, 10), (20_011, 33, 20_003, 100), (400_003, 3, 2_001, 10)])
+def test_filtered_scans_in_parts(libs, tmp_path, n, d, nq, k):
+    """Batches over all rows that need several times the scratch there may be: bit for bit the captured scan, which
+    compares all rows, and no more memory than the larger of 64 MB and half of the index."""
+    rng = np.random.default_rng(n)
+    base = rng.standard_normal((n, d)).astype(np.float32)
+    path = str(tmp_path / "parts.idx")
+    libs.build_index_gpu(base, rng.integers(0, n, n).astype(np.int32), path, m=4, ef_c=4, patience=1, n_inv=12)
+    gix = libs.Index.load(path)
+    q = torch.from_numpy(rng.standard_normal((nq, d)).astype(np.float32)).cuda()
+    lo, hi = torch.zeros(nq, dtype=torch.int32, device="cuda"), torch.full((nq,), n, dtype=torch.int32, device="cuda")
+    hi[::5] = n // 3
+    hi[3::50] = 40
+    out = [[torch.empty((nq, k), dtype=t, device="cuda") for t in (torch.int32, torch.float32)] for _ in range(2)]
+    graph = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(graph):
+        gix.exact_search(q, lo, hi, k, out_ids=out[0][0], out_dists=out[0][1])
+    graph.replay()
+    gix.exact_search(q[:1], lo[:1], hi[:1], k)
+    torch.cuda.synchronize()
+    before = torch.cuda.mem_get_info()[0]
+    for _ in range(3):
+        gix.exact_search(q, lo, hi, k, out_ids=out[1][0], out_dists=out[1][1])
+    torch.cuda.synchronize()
+    assert before - torch.cuda.mem_get_info()[0] <= max(64 << 20, gix.info.device_bytes // 2) + (4 << 20)
+    assert torch.equal(out[0][0], out[1][0]) and torch.equal(out[0][1].view(torch.int32), out[1][1].view(torch.int32))
+    graph.reset()
+    gix.close()
+
+
 def test_filtered_scans_of_norms_whose_sum_overflows(libs, tmp_path):
     """|q|^2 = 2e38: both norms and all distances are finite, the sum of the norms of q and a row like it is not."""
     rng = np.random.default_rng(2)
