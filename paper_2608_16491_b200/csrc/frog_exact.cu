@@ -882,14 +882,15 @@ size_t exact_bytes(size_t nq, const ExactCut& c, bool few) {
     const size_t grouping = few ? 0 : up256(nq * 4) + up256(c.groups * 8) + up256((c.pieces + c.groups) * 16);
     return up256(nq * 8) + grouping + up256(c.lists * 8);
 }
-// make sure the set has `bytes` beside what `nq` queries keep between calls
-bool exact_room(frog_index* ix, FrogExactSet* set, size_t nq, size_t bytes) {
+bool exact_small(const frog_index* ix) { return (size_t)ix->info.n * ix->info.d_pad * 4 <= EXACT_GROW_BYTES; }
+// make sure the set has `bytes` beside what `nq` queries keep between calls; `refused`: this call has been told to do without
+bool exact_room(frog_index* ix, FrogExactSet* set, size_t nq, size_t bytes, bool* refused) {
     if (!set->mem || nq > set->queries || bytes > set->bytes) {
         // Growing takes 0.5-3 ms.  A first scan of 2,000 queries, k = 100, without scratch / with growth: 20,000 x 96 (7.7 MB)
         // 1,370/1,600 us, 201 queries 490/920; 100,000 x 128 (51 MB) 2,740/1,950.  So on small indexes a scan that would
-        // need more does without, and only a second one grows.
-        if (!ix->exact_asked && (size_t)ix->info.n * ix->info.d_pad * 4 <= EXACT_GROW_BYTES) {
-            ix->exact_asked = true;
+        // need more does without, whichever forms it asks for, and only a second one grows.
+        if (*refused || (!ix->exact_asked && exact_small(ix))) {
+            ix->exact_asked = *refused = true;
             return false;
         }
         const size_t new_queries = std::max(nq, set->queries), new_bytes = std::max(bytes, set->bytes);
@@ -910,8 +911,8 @@ bool exact_room(frog_index* ix, FrogExactSet* set, size_t nq, size_t bytes) {
     return true;
 }
 bool exact_scratch(frog_index* ix, FrogExactSet* set, cudaStream_t s, size_t nq, const ExactCut& c, bool few,
-                   ExactScratch* out) {
-    if (!exact_room(ix, set, nq, exact_bytes(nq, c, few))) return false;
+                   bool* refused, ExactScratch* out) {
+    if (!exact_room(ix, set, nq, exact_bytes(nq, c, few), refused)) return false;
     out->bound = set->mem;
     out->counters = out->bound + up256(set->queries * 8);
     out->done = out->counters + up256((EXACT_BINS + 2) * 4);
@@ -957,6 +958,7 @@ extern "C" int frog_exact_search(const frog_index_t* index, const float* queries
     cudaStreamCaptureStatus capture = cudaStreamCaptureStatusNone;
     FROG_CUDA_TRY(cudaStreamIsCapturing(s, &capture));
     ExactForm form = exact_form((size_t)index->info.n, (size_t)A.d_pad * 4, nq, k, capture == cudaStreamCaptureStatusNone);
+    bool refused = false;
     if (form == ExactForm::Filter) {
         // Scratch of the sets' part that has no state at rest, for slabs of any width, as these are on the device, up to the
         // larger of 64 MB and half of the index.  A batch for which that may not be enough goes in rounds, where these are
@@ -977,8 +979,12 @@ extern "C" int frog_exact_search(const frog_index_t* index, const float* queries
             if (set && set->mem) fit = froghost::filter_fit(n, (size_t)nq, set->bytes, k, A.d_pad);
             if (set && set->bytes < want) {
                 // (what takes the batch in four rounds will do for the first call of its kind)
-                if (fit.queries && fit.parts * fit.rounds <= 4 && !mix->exact_asked) mix->exact_asked = true;
-                else if (exact_room(mix, set, 0, want)) fit = froghost::filter_fit(n, (size_t)nq, set->bytes, k, A.d_pad);
+                if (fit.queries && fit.parts * fit.rounds <= 4 && !mix->exact_asked) {
+                    mix->exact_asked = true;
+                    refused = exact_small(mix);
+                } else if (exact_room(mix, set, 0, want, &refused)) {
+                    fit = froghost::filter_fit(n, (size_t)nq, set->bytes, k, A.d_pad);
+                }
             }
         }
         if (fit.queries && fit.per_round >= (size_t)filter_line(n, (size_t)A.d_pad * 4, k) &&
@@ -1030,7 +1036,7 @@ extern "C" int frog_exact_search(const frog_index_t* index, const float* queries
         {
             const froghost::NoCaptureOfOurs relaxed;
             set = exact_set(mix, s);
-            if (set && !exact_scratch(mix, set, s, (size_t)nq, cut, few, &X)) set = nullptr;
+            if (set && !exact_scratch(mix, set, s, (size_t)nq, cut, few, &refused, &X)) set = nullptr;
         }
         if (set) {
             A.ranges = reinterpret_cast<int2*>(X.ranges);

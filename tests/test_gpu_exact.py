@@ -395,6 +395,28 @@ def test_a_first_scan_of_common_size_allocates_nothing(libs, tmp_path):
         gix.close()
 
 
+@pytest.mark.parametrize("n,d,nq,k", [(5000, 128, 2000, 100), (8000, 8, 400, 512)])
+def test_a_first_scan_of_a_small_index_allocates_nothing(libs, tmp_path, n, d, nq, k):
+    """It needs more than came with the index, and does without whichever form it takes."""
+    base, attrs, path = _index(libs, tmp_path, n, d, 5)
+    ix = oracle.load_index(path)
+    q, lo, hi = _queries(base, attrs, nq, 8, 6)
+    dev = [torch.from_numpy(x).cuda() for x in (q, lo, hi)]
+    out = [torch.empty((nq, k), dtype=t, device="cuda") for t in (torch.int32, torch.float32)]
+    ids, _ = oracle.exact_slab(ix, q, lo, hi, k, mode=1)[:2]
+    for load in range(2):                                   # the first loads the library's kernels
+        gix = libs.Index.load(path)
+        free = []
+        for call in range(3):
+            torch.cuda.synchronize()
+            free.append(torch.cuda.mem_get_info()[0])
+            out[0].zero_()
+            gix.exact_search(*dev, k, out_ids=out[0], out_dists=out[1])
+            assert np.array_equal(out[0].cpu().numpy(), ids)
+        gix.close()
+    assert free[1] == free[0]
+
+
 @pytest.mark.parametrize("d", [57300, 57520])
 def test_the_longest_rows_that_fit_one_query(libs, tmp_path, d):
     """Rows of 229,200 and 230,080 bytes: the scan without pieces needs 2,048 bytes of shared memory besides."""
