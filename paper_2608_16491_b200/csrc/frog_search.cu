@@ -647,21 +647,25 @@ int team_queries_per_sm(int row_bytes, bool f16, int beam_width, int budget, siz
 //   384 bytes          740  305 / 344   449 / 441   674 / 656   682 / 630   1,095 / 943   1,287 / 1,139
 //   512 bytes          740  322 / 354   440 / 436   698 / 687   682 / 652   1,096 / 976   1,301 / 1,204
 //   128 bytes          740  281 / 290   425 / 396   412 / 401   653 / 586   1,024 / 833   1,193 / 1,042
-// A query with an SM of its own and a budget whose candidates keep them busy has sixteen: us, eight / sixteen warps, beam / B
+// A query with an SM to itself and a budget whose candidates keep them busy has sixteen: us, eight / sixteen warps, beam / B
 //   rows          queries   64 / 16     64 / 32     64 / 64     160 / 128     32 / 64
 //   384 bytes          1   167 / 176   163 / 167   156 / 154    446 / 411    86 / 83
 //   384 bytes        148   276 / 286   199 / 202   195 / 190    513 / 475   106 / 99
 //   128 bytes         16   150 / 157   152 / 155   163 / 158    439 / 414    89 / 84
 //   3,072 bytes       16   285 / 289   421 / 422   373 / 341  1,095 / 861   215 / 218
+// Sixteen warps leave room for nothing else on their SM, eight for as many.  So up to sm_count / FROG_SCRATCH_SETS queries
+// only, as that many searches of an index run at once, and with none in flight (`alone`): us, eight / sixteen, rows of 384
+// bytes, beam 64, B 64, searches x queries  4 x 37 181 / 178, 4 x 74 190 / 213, 2 x 148 183 / 229, 4 x 148 227 / 413; one query
+// beside 740 (beam 160) 157 / 326, beside 3,000 145 / 199.
 // `any_batch`: also where one warp per query would be faster (this kernel needs no visited slabs).
-int plan_team(const frog_index* ix, int beam_width, const frog_params_t& P, int nq, LaunchPlan* out, int* vis_bits,
+int plan_team(const frog_index* ix, int beam_width, const frog_params_t& P, int nq, bool alone, LaunchPlan* out, int* vis_bits,
               bool any_batch = false) {
     const bool f16 = P.storage == FROG_STORAGE_F16;
     const int q_len = query_len(ix->info.d);
     const int row_bytes = f16 ? q_len * 2 : ix->info.d_pad * 4;
     const bool lean = (f16 ? ix->has_tmap_f16 : ix->has_tmap_f32) && froghost::lean_row(row_bytes, f16);
     const int per_sm_nq = (nq - 1) / ix->sm_count + 1;
-    const int warps = per_sm_nq <= 1 && P.budget >= 48 ? 16 : per_sm_nq <= (row_bytes <= STAGE_CHUNK || (f16 && P.budget <= 24) ? 2 : 4) ? 8 : 4;
+    const int warps = alone ? 16 : per_sm_nq <= (row_bytes <= STAGE_CHUNK || (f16 && P.budget <= 24) ? 2 : 4) ? 8 : 4;
     const size_t index_bytes = (size_t)ix->info.n * row_bytes;
     if (!any_batch && warps == 4 &&
         (lean ? beam_width <= 96 || per_sm_nq > 5
@@ -823,6 +827,20 @@ int acquire_scratch(frog_index* ix, cudaStream_t s, FrogScratch** out) {
     return FROG_OK;
 }
 
+// Whether a search on stream s has no other search of the index beside it.
+bool no_search_beside(frog_index* ix, cudaStream_t s) {
+    const NoCaptureOfOurs relaxed;
+    std::lock_guard<std::mutex> lock(ix->mu);
+    unsigned long long id = 0;
+    bool alone = cudaStreamGetId(s, &id) == cudaSuccess;
+    for (int i = 0; i < ix->n_scratch && alone; ++i) {
+        const FrogScratch& sc = ix->scratch[i];
+        alone = !sc.tick || sc.stream_id == id || cudaEventQuery(sc.done) == cudaSuccess;
+    }
+    if (!alone) cudaGetLastError();
+    return alone;
+}
+
 // Make sure the set owns a visited slab for `slots` resident warps.  Grows (cudaFree + cudaMalloc,
 // after synchronising the device) only when a launch needs more slots than any launch before it.
 int ensure_bitmap(const frog_index* ix, FrogScratch* sc, size_t slots) {
@@ -929,12 +947,13 @@ extern "C" int frog_search_ex(const frog_index_t* index, const float* queries, c
     // the kernels it names
     int vis_bits = 0;
     const bool may_team = mode == MODE_FAST && P.visited == FROG_VISITED_AUTO && !P.eager_hash && !(P.debug_flags & ~(2 | 16));
-    bool team = may_team && plan_team(index, beam_width, P, nq, &plan, &vis_bits) == FROG_OK;
+    cudaStream_t s = static_cast<cudaStream_t>(stream);
+    frog_index* mix = const_cast<frog_index*>(index);      // the scratch sets are the index's only mutable part
+    const bool alone = may_team && P.budget >= 48 && nq <= index->sm_count / FROG_SCRATCH_SETS && froghost::no_search_beside(mix, s);
+    bool team = may_team && plan_team(index, beam_width, P, nq, alone, &plan, &vis_bits) == FROG_OK;
     if (team) bitmap = false;
     else rc = plan_launch(index, beam_width, P, mode, bitmap, nq, &plan);
     if (rc) return rc;
-    cudaStream_t s = static_cast<cudaStream_t>(stream);
-    frog_index* mix = const_cast<frog_index*>(index);      // the scratch sets are the index's only mutable part
     std::lock_guard<std::mutex> lock(mix->mu);
     FrogScratch* sc = nullptr;
     rc = froghost::acquire_scratch(mix, s, &sc);
@@ -947,7 +966,7 @@ extern "C" int frog_search_ex(const frog_index_t* index, const float* queries, c
             bitmap = false;
             rc = plan_launch(index, beam_width, P, mode, false, nq, &plan);
             if (rc == FROG_ERR_UNSUPPORTED && may_team) {
-                rc = plan_team(index, beam_width, P, nq, &plan, &vis_bits, true);
+                rc = plan_team(index, beam_width, P, nq, false, &plan, &vis_bits, true);
                 team = rc == FROG_OK;
             }
         }

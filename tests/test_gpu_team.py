@@ -1,5 +1,7 @@
 """The one-CTA-per-query search kernel (small batches) against the CPU oracle, at the edges of its pools, row
 lengths, batch sizes and options.  ``visited=VISITED_AUTO`` takes it for these batch sizes."""
+import json
+
 import numpy as np
 import pytest
 
@@ -88,6 +90,67 @@ def test_lines_between_the_forms(libs, tmp_path, d, storage):
             b = _run(libs, gix, q[:nq], lo[:nq], hi[:nq], 10, ef, budget=budget, storage=storage, visited=libs.VISITED_BITMAP)
             for x, y in zip(a, b):
                 assert np.array_equal(x.view(np.uint32), y.view(np.uint32))
+    gix.close()
+
+
+def _kernels(tmp, call):
+    """(name, threads of a CTA) of the kernels that `call` launches."""
+    from torch.profiler import ProfilerActivity, profile
+    with profile(activities=[ProfilerActivity.CUDA]) as prof:
+        call()
+        torch.cuda.synchronize()
+    prof.export_chrome_trace(str(tmp / "trace.json"))
+    events = json.loads((tmp / "trace.json").read_text())["traceEvents"]
+    return [(e["name"], e["args"]["block"][0]) for e in events if e.get("cat") == "kernel"]
+
+
+# sixteen warps per query, which take their SM whole: every pool and row length
+@pytest.mark.parametrize("d,storage", [(30, 0), (96, 1), (128, 0), (300, 0), (768, 1)])
+def test_sixteen_warps(libs, tmp_path, d, storage):
+    base, attrs, path = _index(libs, tmp_path, 3000, d, d)
+    ix = oracle.load_index(path)
+    gix = libs.Index.load(path)
+    if storage:
+        gix.enable_f16()
+        ix = oracle.rounded_to_f16(ix)
+    q, lo, hi = _queries(base, attrs, 37, d + 1)
+    for ef in (1, 33, 65, 129, 257, 512):
+        for budget, nq in ((48, 37), (128, 5)):
+            got = _run(libs, gix, q[:nq], lo[:nq], hi[:nq], min(ef, 10), ef, budget=budget, storage=storage)
+            ref = oracle.search(ix, q[:nq], lo[:nq], hi[:nq], min(ef, 10), ef, B=budget)
+            assert np.array_equal(got[0], ref.ids) and np.array_equal(got[2], ref.status)
+            assert np.array_equal(got[1].view(np.uint32), ref.dists.view(np.uint32))
+    gix.close()
+
+
+def test_sixteen_warps_only_beside_nothing(libs, tmp_path):
+    """... so: a quarter of the SMs at most, and no other stream's search in flight."""
+    base, attrs, path = _index(libs, tmp_path, 4000, 96, 1)
+    gix = libs.Index.load(path)
+    q, lo, hi = (torch.from_numpy(x).cuda() for x in _queries(base, attrs, 6000, 4))
+    quarter = torch.cuda.get_device_properties(0).multi_processor_count // 4
+    other = torch.cuda.Stream()
+    kept = [torch.empty((6000, 10), dtype=t, device="cuda") for t in (torch.int32, torch.float32)]
+    params = libs.Params(budget=64)
+    want = gix.search(q[:1], lo[:1], hi[:1], 10, 40, params=libs.Params(budget=64, visited=libs.VISITED_BITMAP))
+
+    def threads(nq, before=lambda: None):
+        def call():
+            before()
+            out.append(gix.search(q[:nq], lo[:nq], hi[:nq], 10, 40, params=params))
+        out = []
+        found = [n for name, n in _kernels(tmp_path, call) if "team" in name]
+        assert torch.equal(out[0][0][:1], want[0]) and torch.equal(out[0][1][:1], want[1])
+        return found
+
+    def busy():                                              # some milliseconds of the general kernel
+        torch.cuda.synchronize()
+        gix.search(q, lo, hi, 10, 512, stream=other, params=libs.Params(budget=64, visited=libs.VISITED_HASH), out_ids=kept[0], out_dists=kept[1])
+
+    assert threads(1) == [512] and threads(quarter) == [512] and threads(quarter + 1) == [256] and threads(148) == [256]
+    assert threads(1, busy) == [256] and threads(quarter, busy) == [256]
+    torch.cuda.synchronize()
+    assert threads(1) == [512]
     gix.close()
 
 
