@@ -611,7 +611,6 @@ int plan_launch(const frog_index* ix, int beam_width, const frog_params_t& P, in
 // the budget (more rows in flight per expansion) and, for short rows, with an index that does not stay in L2.
 // us, one warp / four warps per query (15,000-100,000 objects):
 //   rows, beam / B            740 queries    900            1,184          1,800
-//   256 bytes, 64 / 64         401 / 365      403 / 543      407 / 577
 //   400 bytes, 64 / 64         489 / 415      486 / 544      491 / 609
 //   400 bytes, 128 / 16       1064 / 772     1053 / 802     1068 / 821
 //   400 bytes, 192 / 128      1927 / 1324    1965 / 1425    1980 / 1614
@@ -637,16 +636,25 @@ int team_queries_per_sm(int row_bytes, bool f16, int beam_width, int budget, siz
     return few ? 8 : budget > 64 && index_bytes <= (size_t)64 << 20 ? 7 : 5;
 }
 
+// Whether four warps per query, up to the five CTAs per SM that are resident, beat one warp of the kernel for short rows: time
+// of four warps / of one, 300 and 740 queries on 50,000 rows, B 64 | B 96 | B 128:
+//   beam                   128                              257                              384
+//   512 bytes              1.00 1.12 | 1.00 1.06 |  .89  .93  1.03 1.07 |  .78  .82 |  .73  .76  1.17 1.17 |  .90  .96 |  .82  .90
+//   384 bytes               .96 1.08 | 1.06 1.13 |  .97 1.02  1.07 1.10 |  .83  .89 |  .79  .84  1.25 1.24 |  .99 1.04 |  .92  .95
+//   384, long chains       1.14 1.24 | 1.05 1.18 |  .97 1.04  1.12 1.19 |  .85  .97 |  .76  .87  1.24 1.26 |  .99 1.04 |  .86  .97
+//   128 bytes              1.10 1.24 | 1.10 1.11 |  .92 1.00  1.15 1.14 |  .91  .95 |  .83  .86  1.35 1.32 | 1.10 1.11 |  .98 1.01
+//   256 fp16               1.08 1.20 | 1.09 1.13 |  .97 1.01  1.14 1.15 |  .80  .85 |  .77  .79  1.29 1.25 |  .94  .98 |  .87  .93
+//   192 fp16, long chains  1.23 1.35 | 1.15 1.24 | 1.04 1.09  1.23 1.27 |  .86  .97 |  .78  .88  1.34 1.34 | 1.01 1.06 |  .90  .99
+// B 16 and 32 are like B 64, beams 192 and 256 like 128; beam 512 takes 1.10-1.95 of one warp's time, B 128 .94-1.21.
+bool team_lean(bool f16, int beam_width, int budget) {
+    return beam_width > 256 ? budget > 64 && beam_width <= 384 : !f16 && beam_width > 96 && budget > 96;
+}
+
 // One CTA per query (frog_search_team.cu) for batches that leave warps idle, or FROG_ERR_UNSUPPORTED where
 // one warp per query is the better use of the GPU.  Eight warps while every query has a CTA of its own at once (2 per
 // SM; 4 per SM for rows of several chunks, but not for fp16 rows with small budgets), then four up to the line above.
-// The rows that the kernel of frog_search_lean.cu covers are served well enough by one warp where the pool is small;
-// the merges of larger ones pay up to the five CTAs per SM that are resident.  us, one warp / four, beam / B:
-//   rows           queries   64 / 64    100 / 64    128 / 16    160 / 64     160 / 128     192 / 128
-//   384 bytes          300  298 / 309   438 / 415   687 / 648   677 / 606   1,101 / 889   1,288 / 1,085
-//   384 bytes          740  305 / 344   449 / 441   674 / 656   682 / 630   1,095 / 943   1,287 / 1,139
-//   512 bytes          740  322 / 354   440 / 436   698 / 687   682 / 652   1,096 / 976   1,301 / 1,204
-//   128 bytes          740  281 / 290   425 / 396   412 / 401   653 / 586   1,024 / 833   1,193 / 1,042
+// The rows that the kernel of frog_search_lean.cu covers are served well enough by one warp, except where expansions are fat
+// and pools large (team_lean).
 // A query with an SM to itself and a budget whose candidates keep them busy has sixteen: us, eight / sixteen warps, beam / B
 //   rows          queries   64 / 16     64 / 32     64 / 64     160 / 128     32 / 64
 //   384 bytes          1   167 / 176   163 / 167   156 / 154    446 / 411    86 / 83
@@ -668,7 +676,7 @@ int plan_team(const frog_index* ix, int beam_width, const frog_params_t& P, int 
     const int warps = alone ? 16 : per_sm_nq <= (row_bytes <= STAGE_CHUNK || (f16 && P.budget <= 24) ? 2 : 4) ? 8 : 4;
     const size_t index_bytes = (size_t)ix->info.n * row_bytes;
     if (!any_batch && warps == 4 &&
-        (lean ? beam_width <= 96 || per_sm_nq > 5
+        (lean ? !team_lean(f16, beam_width, P.budget) || per_sm_nq > 5
               : per_sm_nq > team_queries_per_sm(row_bytes, f16, beam_width, P.budget, index_bytes)))
         return FROG_ERR_UNSUPPORTED;
     // a table of about 16 ranks per beam slot: smaller ones repeat distances (3,072-byte rows at beam 192:

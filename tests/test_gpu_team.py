@@ -154,6 +154,24 @@ def test_sixteen_warps_only_beside_nothing(libs, tmp_path):
     gix.close()
 
 
+# four warps per query or one, on rows that the short-row kernel covers
+@pytest.mark.parametrize("storage,ef,budget,team", [(0, 96, 128, 0), (0, 97, 97, 1), (0, 160, 96, 0), (0, 256, 64, 0), (0, 257, 65, 1), (0, 384, 128, 1),
+                                                    (0, 385, 128, 0), (0, 512, 64, 0), (1, 160, 128, 0), (1, 257, 65, 1), (1, 257, 64, 0)])
+def test_lines_on_short_rows(libs, tmp_path, storage, ef, budget, team):
+    base, attrs, path = _index(libs, tmp_path, 4000, 96, 2)
+    gix = libs.Index.load(path)
+    gix.enable_f16()
+    q, lo, hi = _queries(base, attrs, 740, 4)
+    for nq in (297, 740):
+        found = []
+        kernels = _kernels(tmp_path, lambda: found.append(_run(libs, gix, q[:nq], lo[:nq], hi[:nq], 10, ef, budget=budget, storage=storage)))
+        assert [n for name, n in kernels if "team" in name] == [128] * team
+        want = _run(libs, gix, q[:nq], lo[:nq], hi[:nq], 10, ef, budget=budget, storage=storage, visited=libs.VISITED_BITMAP)
+        for x, y in zip(found[0], want):
+            assert np.array_equal(x.view(np.uint32), y.view(np.uint32))
+    gix.close()
+
+
 @pytest.mark.parametrize("kw,okw", [(dict(max_iters=1), dict(max_iters=1)), (dict(max_iters=7, budget=24), dict(max_iters=7, B=24)),
                                     (dict(epn=1), dict(epn=1)), (dict(epn=32, budget=1), dict(epn=32, B=1)),
                                     (dict(no_hotspot=1, budget=100), dict(no_hotspot=1, B=100)),
