@@ -805,6 +805,16 @@ size_t exact_smem(int k, int d_pad) {
 //   20,000 x 768    72/121 | 212/117      120/120 | 464/137      283/128 | 1,071/294  1,032/435 | 4,720/1,461
 //   100,000 x 128   90/100 | 253/105      149/107 | 555/129      411/128 | 1,190/259  1,262/324 | -
 //   400,000 x 96    155/207 | 1,200/251   352/246 | 2,926/302    1,032/327 | -        3,802/808 | -
+// Slabs of fewer than 10 k rows are not filtered.  Where no slab is wider, all that the form does is to scan each with one CTA,
+// which up to EXACT_SPLIT_MAX queries still beats the form that splits them and after that loses to the grouped one; us, the
+// same columns:
+//                          100, k = 512          200                  400                  2,000
+//   5,119 x 32           189/187 | 362/194    166/188 | 198/195    172/190 | 266/202    232/270 | 716/740
+//   5,119 x 128          186/203 | 375/207    284/205 | 369/215    182/205 | 281/232    245/293 | 794/861
+//   4,096 x 200          148/210 | 379/218    281/215 | 393/231    186/217 | 270/252    236/313 | 811/957
+//   5,119 x 768          208/400 | 422/410    299/406 | 525/456    279/414 | 471/520    410/590 | 1,663/2,024
+//   8,000 x 128          322/222 | 406/101         -               227/236 | 385/114    344/342 | 1,055/366
+//   64,000 x 128         582/249 | 839/140         -               560/269 | 1,388/263  1,264/533 | 4,506/1,087
 enum class ExactForm { OnePerQuery, Few, Split, Grouped, Filter };
 int filter_line(size_t n, size_t row_bytes, int k) {
     if (n < 4000 || row_bytes > 16384) return 0x7FFFFFFF;
@@ -813,7 +823,7 @@ int filter_line(size_t n, size_t row_bytes, int k) {
 }
 ExactForm exact_form(size_t n, size_t row_bytes, int nq, int k, bool filter) {
     const size_t bytes = n * row_bytes;
-    if (filter && nq >= filter_line(n, row_bytes, k)) return ExactForm::Filter;
+    if (filter && nq >= filter_line(n, row_bytes, k) && (n >= (size_t)10 * k || nq <= EXACT_SPLIT_MAX)) return ExactForm::Filter;
     if (nq < EXACT_PLAN_MIN) return k <= 32 && bytes <= 500000 ? ExactForm::OnePerQuery : ExactForm::Few;
     const double work = (double)n * (double)(row_bytes + 384) * (k > 128 ? 3.0 : k > 64 ? 1.4 : 1.0);
     if (nq <= EXACT_SPLIT_MAX && nq * (n < 8000 ? 45e3 : 100e3) <= work) return ExactForm::Split;

@@ -84,6 +84,25 @@ def test_filtered_scans(libs, tmp_path, n, d, nq):
     gix.close()
 
 
+# slabs of fewer than 10 k rows are not filtered: without wider ones the form is for 100 (rows above 1 KB: 400) to 200 queries
+@pytest.mark.parametrize("n,d,k,counts,filtered", [(5119, 20, 512, (100, 200, 201, 600), (1, 1, 0, 0)), (5120, 20, 512, (201, 600), (1, 1)),
+                                                   (4000, 20, 401, (200, 201), (1, 0)), (4500, 260, 512, (200, 400), (0, 0))])
+def test_long_lists_from_few_rows(libs, tmp_path, n, d, k, counts, filtered):
+    from torch.profiler import ProfilerActivity, profile
+    base, attrs, path = _index(libs, tmp_path, n, d, n)
+    ix = oracle.load_index(path)
+    gix = libs.Index.load(path)
+    q, lo, hi = _queries(base, attrs, max(counts), 7, 6)
+    for nq, want in zip(counts, filtered):
+        _check(gix, ix, q[:nq], lo[:nq], hi[:nq], k)                     # (its scratch is there from here on)
+        dev = [torch.from_numpy(x[:nq]).cuda() for x in (q, lo, hi)]
+        with profile(activities=[ProfilerActivity.CUDA]) as prof:
+            gix.exact_search(*dev, k)
+            torch.cuda.synchronize()
+        assert any("filter_refine" in e.name for e in prof.events()) == bool(want)
+    gix.close()
+
+
 @pytest.mark.parametrize("scale", [1.0, 1e-21, 3e17, 1e19])
 def test_filtered_scans_of_extreme_values(libs, tmp_path, scale):
     """Products that underflow, overflow or are not numbers rule nothing out: same results, bit for bit, as the captured
