@@ -46,3 +46,33 @@ def build_scaled(libs, cache_dir, name, n, nq, **kw):
     if not os.path.exists(path):
         libs.build_index(wl.vectors, wl.attrs, path, seed=wl.seed, **kw)
     return wl, path, oracle.load_index(path)
+
+
+@pytest.fixture
+def launches(tmp_path):
+    """launches(call): (name, threads of a CTA) of this library's kernels that `call` launches, by torch's profiler.  That
+    drops what seems to lie outside its window, hence the pauses and the repetition."""
+    import json
+    import time
+    import warnings
+    import torch
+    from torch.profiler import ProfilerActivity, profile
+
+    def record(call):
+        for _ in range(5):
+            torch.cuda.synchronize()
+            with warnings.catch_warnings():
+                warnings.simplefilter("ignore")
+                with profile(activities=[ProfilerActivity.CUDA]) as prof:
+                    time.sleep(0.02)
+                    call()
+                    torch.cuda.synchronize()
+                    time.sleep(0.02)
+            prof.export_chrome_trace(str(tmp_path / "trace.json"))
+            events = json.loads((tmp_path / "trace.json").read_text())["traceEvents"]
+            found = [(e["name"], e["args"]["block"][0]) for e in events
+                     if e.get("cat") == "kernel" and ("frog_" in e["name"] or "filter_" in e["name"])]
+            if found:
+                return found
+        pytest.skip("the profiler records no kernels")
+    return record

@@ -1,7 +1,5 @@
 """The one-CTA-per-query search kernel (small batches) against the CPU oracle, at the edges of its pools, row
 lengths, batch sizes and options.  ``visited=VISITED_AUTO`` takes it for these batch sizes."""
-import json
-
 import numpy as np
 import pytest
 
@@ -93,17 +91,6 @@ def test_lines_between_the_forms(libs, tmp_path, d, storage):
     gix.close()
 
 
-def _kernels(tmp, call):
-    """(name, threads of a CTA) of the kernels that `call` launches."""
-    from torch.profiler import ProfilerActivity, profile
-    with profile(activities=[ProfilerActivity.CUDA]) as prof:
-        call()
-        torch.cuda.synchronize()
-    prof.export_chrome_trace(str(tmp / "trace.json"))
-    events = json.loads((tmp / "trace.json").read_text())["traceEvents"]
-    return [(e["name"], e["args"]["block"][0]) for e in events if e.get("cat") == "kernel"]
-
-
 # sixteen warps per query, which take their SM whole: every pool and row length
 @pytest.mark.parametrize("d,storage", [(30, 0), (96, 1), (128, 0), (300, 0), (768, 1)])
 def test_sixteen_warps(libs, tmp_path, d, storage):
@@ -123,7 +110,7 @@ def test_sixteen_warps(libs, tmp_path, d, storage):
     gix.close()
 
 
-def test_sixteen_warps_only_beside_nothing(libs, tmp_path):
+def test_sixteen_warps_only_beside_nothing(libs, tmp_path, launches):
     """... so: a quarter of the SMs at most, and no other stream's search in flight."""
     base, attrs, path = _index(libs, tmp_path, 4000, 96, 1)
     gix = libs.Index.load(path)
@@ -139,7 +126,7 @@ def test_sixteen_warps_only_beside_nothing(libs, tmp_path):
             before()
             out.append(gix.search(q[:nq], lo[:nq], hi[:nq], 10, 40, params=params))
         out = []
-        found = [n for name, n in _kernels(tmp_path, call) if "team" in name]
+        found = [n for name, n in launches(call) if "team" in name]
         assert torch.equal(out[0][0][:1], want[0]) and torch.equal(out[0][1][:1], want[1])
         return found
 
@@ -157,14 +144,14 @@ def test_sixteen_warps_only_beside_nothing(libs, tmp_path):
 # four warps per query or one, on rows that the short-row kernel covers
 @pytest.mark.parametrize("storage,ef,budget,team", [(0, 96, 128, 0), (0, 97, 97, 1), (0, 160, 96, 0), (0, 256, 64, 0), (0, 257, 65, 1), (0, 384, 128, 1),
                                                     (0, 385, 128, 0), (0, 512, 64, 0), (1, 160, 128, 0), (1, 257, 65, 1), (1, 257, 64, 0)])
-def test_lines_on_short_rows(libs, tmp_path, storage, ef, budget, team):
+def test_lines_on_short_rows(libs, tmp_path, launches, storage, ef, budget, team):
     base, attrs, path = _index(libs, tmp_path, 4000, 96, 2)
     gix = libs.Index.load(path)
     gix.enable_f16()
     q, lo, hi = _queries(base, attrs, 740, 4)
     for nq in (297, 740):
         found = []
-        kernels = _kernels(tmp_path, lambda: found.append(_run(libs, gix, q[:nq], lo[:nq], hi[:nq], 10, ef, budget=budget, storage=storage)))
+        kernels = launches(lambda: found.append(_run(libs, gix, q[:nq], lo[:nq], hi[:nq], 10, ef, budget=budget, storage=storage)))
         assert [n for name, n in kernels if "team" in name] == [128] * team
         want = _run(libs, gix, q[:nq], lo[:nq], hi[:nq], 10, ef, budget=budget, storage=storage, visited=libs.VISITED_BITMAP)
         for x, y in zip(found[0], want):
