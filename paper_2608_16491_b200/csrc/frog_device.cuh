@@ -645,8 +645,8 @@ __device__ __forceinline__ uint32_t merge_ranked(uint64_t* pool, uint64_t* keys,
     }
     in = in && (pool[p] | 1ull) != mk;                  // the pool holds it already
     // of equal keys the first one goes on (the other lanes' are made different)
-    const uint32_t same = ROWS ? __match_any_sync(FULL, lane < n ? key_rank(key) : 0x80000000u | (uint32_t)lane)
-                               : __match_any_sync(FULL, lane < n ? mk : 0xFFFFFFFF00000000ull | (uint64_t)lane);
+    uint32_t same = __match_any_sync(FULL, lane < n ? key_rank(key) : 0x80000000u | (uint32_t)lane);
+    if (!ROWS && __any_sync(FULL, (same & lt_mask) != 0)) same &= __match_any_sync(FULL, (uint32_t)(key >> 32));
     in = in && (same & lt_mask) == 0;
     if (lane < n && !in) keys[lane] = KEY_EMPTY;        // not below any other
     __syncwarp();
