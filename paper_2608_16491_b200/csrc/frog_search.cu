@@ -658,7 +658,7 @@ bool team_lean(bool f16, int beam_width, int budget) {
 // A query with an SM to itself and a budget whose candidates keep them busy has sixteen: us, eight / sixteen warps, beam / B
 //   rows          queries   64 / 16     64 / 32     64 / 64     160 / 128     32 / 64
 //   384 bytes          1   167 / 176   163 / 167   156 / 154    446 / 411    86 / 83
-//   384 bytes        148   276 / 286   199 / 202   195 / 190    513 / 475   106 / 99
+//   384 bytes         37      -           -        167 / 164    450 / 426    85 / 83
 //   128 bytes         16   150 / 157   152 / 155   163 / 158    439 / 414    89 / 84
 //   3,072 bytes       16   285 / 289   421 / 422   373 / 341  1,095 / 861   215 / 218
 // Sixteen warps leave room for nothing else on their SM, eight for as many.  So up to sm_count / FROG_SCRATCH_SETS queries
