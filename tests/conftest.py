@@ -50,29 +50,21 @@ def build_scaled(libs, cache_dir, name, n, nq, **kw):
 
 @pytest.fixture
 def launches(tmp_path):
-    """launches(call): (name, threads of a CTA) of this library's kernels that `call` launches, by torch's profiler.  That
-    drops what seems to lie outside its window, hence the pauses and the repetition."""
+    """launches(index file, q, lo, hi, steps): per step, (name, threads of a CTA) of this library's kernels (record_launches.py)."""
     import json
-    import time
-    import warnings
-    import torch
-    from torch.profiler import ProfilerActivity, profile
+    import subprocess
+    import numpy as np
 
-    def record(call):
-        for _ in range(5):
-            torch.cuda.synchronize()
-            with warnings.catch_warnings():
-                warnings.simplefilter("ignore")
-                with profile(activities=[ProfilerActivity.CUDA]) as prof:
-                    time.sleep(0.02)
-                    call()
-                    torch.cuda.synchronize()
-                    time.sleep(0.02)
-            prof.export_chrome_trace(str(tmp_path / "trace.json"))
-            events = json.loads((tmp_path / "trace.json").read_text())["traceEvents"]
-            found = [(e["name"], e["args"]["block"][0]) for e in events
-                     if e.get("cat") == "kernel" and ("frog_" in e["name"] or "filter_" in e["name"])]
-            if found:
+    def record(path, q, lo, hi, steps):
+        np.savez(str(tmp_path / "queries.npz"), q=q, lo=lo, hi=hi)
+        script = os.path.join(ROOT, "tests", "record_launches.py")
+        for _ in range(3):
+            r = subprocess.run([sys.executable, script, path, str(tmp_path / "queries.npz"), json.dumps(steps)],
+                               capture_output=True, text=True, timeout=300)
+            assert r.returncode == 0, r.stderr
+            found = [json.loads(line[9:]) for line in r.stdout.splitlines() if line.startswith("LAUNCHES ")]
+            assert len(found) == len(steps)
+            if all(found):
                 return found
         pytest.skip("the profiler records no kernels")
     return record

@@ -92,11 +92,12 @@ def test_long_lists_from_few_rows(libs, tmp_path, launches, n, d, k, counts, fil
     ix = oracle.load_index(path)
     gix = libs.Index.load(path)
     q, lo, hi = _queries(base, attrs, max(counts), 7, 6)
-    for nq, want in zip(counts, filtered):
-        _check(gix, ix, q[:nq], lo[:nq], hi[:nq], k)                     # (its scratch is there from here on)
-        dev = [torch.from_numpy(x[:nq]).cuda() for x in (q, lo, hi)]
-        assert any("filter_refine" in name for name, _ in launches(lambda: gix.exact_search(*dev, k))) == bool(want)
+    for nq in counts:
+        _check(gix, ix, q[:nq], lo[:nq], hi[:nq], k)
     gix.close()
+    found = launches(path, q, lo, hi, [dict(nq=nq, k=k) for nq in counts])
+    assert all(found)
+    assert [any("filter_refine" in name for name, _ in kernels) for kernels in found] == [bool(x) for x in filtered]
 
 
 @pytest.mark.parametrize("scale", [1.0, 1e-21, 3e17, 1e19])

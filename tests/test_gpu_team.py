@@ -113,50 +113,36 @@ def test_sixteen_warps(libs, tmp_path, d, storage):
 def test_sixteen_warps_only_beside_nothing(libs, tmp_path, launches):
     """... so: a quarter of the SMs at most, and no other stream's search in flight."""
     base, attrs, path = _index(libs, tmp_path, 4000, 96, 1)
-    gix = libs.Index.load(path)
-    q, lo, hi = (torch.from_numpy(x).cuda() for x in _queries(base, attrs, 6000, 4))
     quarter = torch.cuda.get_device_properties(0).multi_processor_count // 4
-    other = torch.cuda.Stream()
-    kept = [torch.empty((6000, 10), dtype=t, device="cuda") for t in (torch.int32, torch.float32)]
-    params = libs.Params(budget=64)
-    want = gix.search(q[:1], lo[:1], hi[:1], 10, 40, params=libs.Params(budget=64, visited=libs.VISITED_BITMAP))
-
-    def threads(nq, before=lambda: None):
-        def call():
-            before()
-            out.append(gix.search(q[:nq], lo[:nq], hi[:nq], 10, 40, params=params))
-        out = []
-        found = [n for name, n in launches(call) if "team" in name]
-        assert torch.equal(out[0][0][:1], want[0]) and torch.equal(out[0][1][:1], want[1])
-        return found
-
-    def busy():                                              # some milliseconds of the general kernel
-        torch.cuda.synchronize()
-        gix.search(q, lo, hi, 10, 512, stream=other, params=libs.Params(budget=64, visited=libs.VISITED_HASH), out_ids=kept[0], out_dists=kept[1])
-
-    assert threads(1) == [512] and threads(quarter) == [512] and threads(quarter + 1) == [256] and threads(148) == [256]
-    assert threads(1, busy) == [256] and threads(quarter, busy) == [256]
-    torch.cuda.synchronize()
-    assert threads(1) == [512]
-    gix.close()
+    steps = [dict(nq=nq, ef=40, budget=64, beside=beside) for nq, beside in
+             ((1, 0), (quarter, 0), (quarter + 1, 0), (148, 0), (1, 1), (quarter, 1), (1, 0))]
+    found = launches(path, *_queries(base, attrs, 6000, 4), steps)
+    assert [[n for name, n in kernels if "team" in name] for kernels in found] == [[512], [512], [256], [256], [256], [256], [512]]
 
 
-# four warps per query or one, on rows that the short-row kernel covers
-@pytest.mark.parametrize("storage,ef,budget,team", [(0, 96, 128, 0), (0, 97, 97, 1), (0, 160, 96, 0), (0, 256, 64, 0), (0, 257, 65, 1), (0, 384, 128, 1),
-                                                    (0, 385, 128, 0), (0, 512, 64, 0), (1, 160, 128, 0), (1, 257, 65, 1), (1, 257, 64, 0)])
-def test_lines_on_short_rows(libs, tmp_path, launches, storage, ef, budget, team):
+# four warps per query or one, on rows that the short-row kernel covers: storage, beam, budget, whether four
+SHORT_ROWS = [(0, 96, 128, 0), (0, 97, 97, 1), (0, 160, 96, 0), (0, 256, 64, 0), (0, 257, 65, 1), (0, 384, 128, 1), (0, 385, 128, 0),
+              (0, 512, 64, 0), (1, 160, 128, 0), (1, 257, 65, 1), (1, 257, 64, 0)]
+
+
+def test_lines_on_short_rows(libs, tmp_path, launches):
     base, attrs, path = _index(libs, tmp_path, 4000, 96, 2)
     gix = libs.Index.load(path)
     gix.enable_f16()
     q, lo, hi = _queries(base, attrs, 740, 4)
-    for nq in (297, 740):
-        found = []
-        kernels = launches(lambda: found.append(_run(libs, gix, q[:nq], lo[:nq], hi[:nq], 10, ef, budget=budget, storage=storage)))
-        assert [n for name, n in kernels if "team" in name] == [128] * team
-        want = _run(libs, gix, q[:nq], lo[:nq], hi[:nq], 10, ef, budget=budget, storage=storage, visited=libs.VISITED_BITMAP)
-        for x, y in zip(found[0], want):
-            assert np.array_equal(x.view(np.uint32), y.view(np.uint32))
+    steps = []
+    for storage, ef, budget, _ in SHORT_ROWS:
+        for nq in (297, 740):
+            steps.append(dict(nq=nq, ef=ef, budget=budget, storage=storage))
+            a = _run(libs, gix, q[:nq], lo[:nq], hi[:nq], 10, ef, budget=budget, storage=storage)
+            b = _run(libs, gix, q[:nq], lo[:nq], hi[:nq], 10, ef, budget=budget, storage=storage, visited=libs.VISITED_BITMAP)
+            for x, y in zip(a, b):
+                assert np.array_equal(x.view(np.uint32), y.view(np.uint32))
     gix.close()
+    found = launches(path, q, lo, hi, steps)
+    assert all(found)
+    for step, kernels, team in zip(steps, found, np.repeat([x[3] for x in SHORT_ROWS], 2)):
+        assert [n for name, n in kernels if "team" in name] == [128] * team, step
 
 
 @pytest.mark.parametrize("kw,okw", [(dict(max_iters=1), dict(max_iters=1)), (dict(max_iters=7, budget=24), dict(max_iters=7, B=24)),
