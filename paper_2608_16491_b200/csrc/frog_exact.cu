@@ -803,8 +803,8 @@ size_t exact_smem(int k, int d_pad) {
 //   20,000 x 50     51/54 | 100/50        68/54 | 188/54         240/59 | 282/88      423/170 | 1,270/347
 //   5,000 x 768     43/110 | 76/100       69/112 | 165/104       179/123 | 321/135    345/290 | 1,391/1,461
 //   20,000 x 768    72/121 | 212/117      120/120 | 464/137      283/128 | 1,071/294  1,032/435 | 4,720/1,461
-//   100,000 x 128   90/100 | 253/105      149/107 | 555/129      411/128 | 1,190/259  1,262/324 | -
-//   400,000 x 96    155/207 | 1,200/251   352/246 | 2,926/302    1,032/327 | -        3,802/808 | -
+//   100,000 x 128   90/100 | 253/105      149/107 | 555/129      411/128 | 1,190/259  1,262/324 | 5,075/873
+//   400,000 x 96    155/207 | 1,200/251   352/246 | 2,926/302    1,032/327 | 3,497/663  3,802/808 | 16,761/2,978
 // Slabs of fewer than 10 k rows are not filtered.  Where no slab is wider, all that the form does is to scan each with one CTA,
 // which up to EXACT_SPLIT_MAX queries still beats the form that splits them and after that loses to the grouped one; us, the
 // same columns:
@@ -814,6 +814,8 @@ size_t exact_smem(int k, int d_pad) {
 //   4,096 x 200          148/210 | 379/218    281/215 | 393/231    186/217 | 270/252    236/313 | 811/957
 //   5,119 x 768          208/400 | 422/410    299/406 | 525/456    279/414 | 471/520    410/590 | 1,663/2,024
 //   8,000 x 128          322/222 | 406/101         -               227/236 | 385/114    344/342 | 1,055/366
+//   100,000 x 128            - | 1,051/167        -                    - | 1,890/325    - | 6,428/1,255
+//   400,000 x 96             - | 3,577/383        -                    - | 4,872/750    - | 19,502/3,306
 //   64,000 x 128         582/249 | 839/140         -               560/269 | 1,388/263  1,264/533 | 4,506/1,087
 enum class ExactForm { OnePerQuery, Few, Split, Grouped, Filter };
 int filter_line(size_t n, size_t row_bytes, int k) {
