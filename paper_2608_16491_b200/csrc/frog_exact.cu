@@ -799,11 +799,11 @@ size_t exact_smem(int k, int d_pad) {
 // form of the lines above / filtered, log-uniform widths down to 2^-10 | all rows:
 //                      40 queries, k = 10      100, k = 10           400, k = 10            2,000, k = 100
 //   3,000 x 96      34/55 | 58/48         50/55 | 54/48          54/60 | 66/53        120/123 | 369/136
-//   5,000 x 128     33/56 | 51/52         74/58 | 84/51          82/62 | 104/60       168/135 | 546/517
-//   20,000 x 50     51/54 | 100/50        68/54 | 188/54         240/59 | 282/88      423/170 | 1,270/347
-//   5,000 x 768     43/110 | 76/100       69/112 | 165/104       179/123 | 321/135    345/290 | 1,391/1,461
-//   20,000 x 768    72/121 | 212/117      120/120 | 464/137      283/128 | 1,071/294  1,032/435 | 4,720/1,461
-//   100,000 x 128   90/100 | 253/105      149/107 | 555/129      411/128 | 1,190/259  1,262/324 | 5,075/873
+//   5,000 x 128     33/56 | 51/52         74/58 | 84/51          82/62 | 104/60       149/118 | 488/157
+//   20,000 x 50     51/54 | 100/50        68/54 | 188/54         240/59 | 282/88      370/145 | 1,137/288
+//   5,000 x 768     43/110 | 76/100       69/112 | 165/104       179/123 | 321/135    321/248 | 1,303/417
+//   20,000 x 768    72/121 | 212/117      120/120 | 464/137      283/128 | 1,071/294  953/411 | 4,521/1,451
+//   100,000 x 128   90/100 | 253/105      149/107 | 555/129      411/128 | 1,190/259  1,163/294 | 5,075/873
 //   400,000 x 96    155/207 | 1,200/251   352/246 | 2,926/302    1,032/327 | 3,497/663  3,802/808 | 16,761/2,978
 // Slabs of fewer than 10 k rows are not filtered.  Where no slab is wider, all that the form does is to scan each with one CTA,
 // which up to EXACT_SPLIT_MAX queries still beats the form that splits them and after that loses to the grouped one; us, the
